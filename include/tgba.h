@@ -92,8 +92,8 @@ tgba_status tgba_basis_free(tgba_basis b);
  * pairs and keeps them in the basis handle (device memory owned by the library), where
  * tgba_assemble_heff, tgba_dsf and tgba_quench reuse them for any h_x.  Steps: the
  * contraction table of the Bogoliubov operators (the Schur complement of Eq. S2's matrix on
- * the vacuum operators) and then one small real Pfaffian per element, of size M_a + M_b,
- * batched over all sectors and sizes.  screen: NULL for the exact assembly, or a trained pair
+ * the vacuum operators, in closed form) and then one small real Pfaffian per element, of size
+ * M_a + M_b, evaluated as a product by Schur's Pfaffian identity, over all sectors and sizes.  screen: NULL for the exact assembly, or a trained pair
  * screener; pairs it predicts with |V_ab| = L h_x |X_ab| < screen_tau (at screen_hx) are set to
  * 0 without a Pfaffian.  Asynchronous on `stream`. */
 tgba_status tgba_compute_x(tgba_basis b, tgba_screen screen, double screen_tau, double screen_hx, void* stream);
@@ -307,16 +307,11 @@ tgba_status tgba_table_noalloc(int32_t L, double J, double h_z, double* table_de
 /* ---------------------------------------------------------------- measurement
  * Profile of a basis handle.  table_ms / pfaffian_ms: device time of the contraction table and
  * of the Pfaffian kernels of the last tgba_compute_x, from CUDA events recorded on its stream
- * (blocks until they complete).  pfaffian_flops: algorithmic FP64 flops of one Pfaffian stage,
- * sum over elements of F(n) = sum_{m = n-2, n-4, ..., 2} [2 m (m-1) + m] (the real-arithmetic
- * Parlett-Reid count: two FMAs per updated entry, one multiply per Gauss-vector entry).
- * pfaffian_launches: kernel launches of one Pfaffian stage.  kernel_launches: all kernel
- * launches this handle has made (this library's kernels only, not cuSOLVER/cuBLAS).
- * upload_bytes: host-to-device bytes of tgba_build_basis.  tune_mode / tune_threads: the launch
- * shape the autotuner chose for the register-resident sizes (0: one launch per size, 1: one
- * persistent queue launch, 3: the queue with a register cap for occupancy; threads per block),
- * tune_ms: its measured stage time (ms) for each candidate in the order {0,64}, {0,128},
- * {0,256}, {1,64}, {1,128}, {1,256}, {3,128} (0 where not measured).
+ * (blocks until they complete).  pfaffian_flops: FP64 multiplications of one Pfaffian stage, sum over
+ * elements of M_b/2 + 1 (the product form).  pfaffian_launches: kernel launches of one Pfaffian
+ * stage after the table.  kernel_launches: all kernel launches this handle has made (this
+ * library's kernels only, not cuSOLVER/cuBLAS).  upload_bytes: host-to-device bytes of
+ * tgba_build_basis.  tune_mode, tune_threads, tune_ms: -1 and zeros (nothing is tuned).
  * tridiag_ms / bisect_ms: device time of the tridiagonalisation and of the bisection kernel of
  * the last native tgba_eigvals (0 if none ran); tridiag_flops: its algorithmic FP64 flops,
  * sum over matrices of sum_{m=1}^{n-1} 4 m (m + 1) (two FMAs of the rank-2 update and two of

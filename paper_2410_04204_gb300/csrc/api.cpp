@@ -55,9 +55,10 @@ tgba_status scratch(Basis& b, int64_t doubles, double** out) {
 
 static void release(Basis* b) {
   void* ptrs[] = {b->d_E_ns, b->d_E_r, b->d_M_ns, b->d_M_r, b->d_sel_ns, b->d_sel_r, b->d_modes_ns, b->d_modes_r,
-                  b->d_theta, b->d_nlab, b->d_table, b->d_c0, b->d_work, b->d_P, b->d_status,
+                  b->d_theta, b->d_nlab, b->d_table, b->d_c0, b->d_const, b->d_tdd, b->d_fac_ns, b->d_fac_r, b->d_pairs_r,
+                  b->d_P, b->d_status,
                   b->d_eig_a, b->d_eig_w, b->d_eig_work, b->d_eig_info, b->d_scratch,
-                  b->d_reg_rects, b->d_counter, b->d_blas_ws, b->d_emu_part};
+                  b->d_rects, b->d_heff_secs, b->d_blas_ws, b->d_emu_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int e = 0; e < 3; ++e) {
@@ -66,10 +67,6 @@ static void release(Basis* b) {
   }
   for (int e = 0; e < 2; ++e)
     if (b->q_ev[e]) cudaEventDestroy(b->q_ev[e]);
-  for (RectList& L : b->rect_lists)
-    if (L.d_rects) cudaFree(L.d_rects);
-  if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
-  if (b->graph) cudaGraphDestroy(b->graph);
   if (b->solver) destroy_solver(b->solver);
   if (b->blas) destroy_blas(b->blas);
   delete b;
@@ -133,24 +130,16 @@ static tgba_status build(const tgba_model* model, const int32_t* sectors, int32_
   if ((r = upload(&b->d_nlab, nl.data(), nl.size(), &b->upload_bytes)) != TGBA_OK) return r;
   TGBA_CUDA(cudaMalloc((void**)&b->d_table, sizeof(double) * 4 * L * L));
   TGBA_CUDA(cudaMalloc((void**)&b->d_c0, sizeof(double) * 4));
-  TGBA_CUDA(cudaMalloc((void**)&b->d_work, sizeof(double) * 2 * (16 * L * L + 4 * L + 1)));
   TGBA_CUDA(cudaMalloc((void**)&b->d_P, sizeof(double) * std::max<int64_t>(1, b->n_elements)));
   TGBA_CUDA(cudaMalloc((void**)&b->d_status, sizeof(unsigned)));
   TGBA_CUDA(cudaMemset(b->d_status, 0, sizeof(unsigned)));
-  TGBA_CUDA(cudaMalloc((void**)&b->d_counter, sizeof(unsigned long long)));
+  if ((r = upload_mode_constants(*b)) != TGBA_OK) return r;
   build_rects(*b);
-  for (RectList& L : b->rect_lists) {
-    for (const Rect& t : L.rects) {
-      double f = 0;
-      for (int m = t.n - 2; m >= 2; m -= 2) f += 2.0 * m * (m - 1) + m;   // F(n), real Parlett-Reid
-      b->pf_flops += f * (double)t.rows * t.w;
-    }
-    if (!L.rects.empty() && (r = upload(&L.d_rects, L.rects.data(), L.rects.size(), &b->upload_bytes)) != TGBA_OK)
-      return r;
-  }
-  if ((r = upload(&b->d_reg_rects, b->reg_rects.data(), b->reg_rects.size(), &b->upload_bytes)) != TGBA_OK) return r;
+  const std::vector<HeffSector> hs = heff_sectors(*b, &b->heff_tiles);
+  b->n_heff_secs = (int)hs.size();
+  if ((r = upload(&b->d_heff_secs, hs.data(), hs.size(), &b->upload_bytes)) != TGBA_OK) return r;
+  if ((r = upload(&b->d_rects, b->rects.data(), b->rects.size(), &b->upload_bytes)) != TGBA_OK) return r;
   for (int e = 0; e < 3; ++e) TGBA_CUDA(cudaEventCreate(&b->ev[e]));
-  if ((r = plan_pfaffians(*b)) != TGBA_OK) return r;
   return TGBA_OK;
 }
 
@@ -175,73 +164,22 @@ static tgba_status ensure_table(Basis& b, cudaStream_t st) {
   return ensure_c0_host(b, st);
 }
 
-// The stage without screening: contraction table, then the Pfaffians.  The first call builds the
-// table eagerly, runs the autotuner, then captures the stage (with its timing events) into a
-// CUDA graph on a private stream; every call launches that graph on the caller's stream.
-static tgba_status compute_x_graph(Basis& b, cudaStream_t st) {
-  tgba_status r;
-  if (!b.tuned) {
-    if ((r = ensure_table(b, st)) != TGBA_OK) return r;
-    if ((r = autotune_pfaffians(b, st)) != TGBA_OK) return r;
-  }
-  if (!b.graph_exec) {
-    cudaStream_t cs;
-    TGBA_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    const int64_t before = b.launches.load();
-    TGBA_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    cudaEventRecordWithFlags(b.ev[0], cs, cudaEventRecordExternal);
-    r = build_table(b, cs);
-    if (r == TGBA_OK) {
-      cudaEventRecordWithFlags(b.ev[1], cs, cudaEventRecordExternal);
-      r = run_pfaffians(b, cs);
-      cudaEventRecordWithFlags(b.ev[2], cs, cudaEventRecordExternal);
-    }
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(cs, &g);
-    cudaStreamDestroy(cs);
-    if (r != TGBA_OK) { if (g) cudaGraphDestroy(g); return r; }
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-    b.graph = g;
-    TGBA_CUDA(cudaGraphInstantiate(&b.graph_exec, b.graph, 0));
-    b.graph_launches = b.launches.load() - before;
-    b.launches -= b.graph_launches;        // counted when the graph runs
-  }
-  TGBA_CUDA(cudaGraphLaunch(b.graph_exec, st));
-  b.launches += b.graph_launches;
-  b.table_valid = true;
-  b.c0_host_valid = false;
-  b.ev_recorded = true;
-  return TGBA_OK;
-}
-
 static tgba_status compute_x(Basis& b, Screen* screen, double tau, double hx, cudaStream_t st) {
   if (screen && !(tau > 0)) return fail(TGBA_EINVAL, "screening needs tau > 0");
   tgba_status r;
-  if (!screen) {
-    if ((r = compute_x_graph(b, st)) != TGBA_OK) return r;
-  } else {
-    if (!b.tuned) {
-      if ((r = ensure_table(b, st)) != TGBA_OK) return r;
-      if ((r = autotune_pfaffians(b, st)) != TGBA_OK) return r;
-    }
-    TGBA_CUDA(cudaEventRecord(b.ev[0], st));
-    if ((r = build_table(b, st)) != TGBA_OK) return r;
-    b.c0_host_valid = false;
-    TGBA_CUDA(cudaEventRecord(b.ev[1], st));
-    int64_t kept = 0;
-    if ((r = screen_pfaffians(*screen, b, tau, hx, &kept, st)) != TGBA_OK) return r;
-    TGBA_CUDA(cudaEventRecord(b.ev[2], st));
-    b.ev_recorded = true;
-    b.x_evaluated = kept;
-    b.x_screened = b.n_elements - kept;
-  }
+  TGBA_CUDA(cudaEventRecord(b.ev[0], st));
+  if ((r = build_table(b, st)) != TGBA_OK) return r;
+  b.c0_host_valid = false;
+  TGBA_CUDA(cudaEventRecord(b.ev[1], st));
+  int64_t kept = b.n_elements;
+  if ((r = screen ? screen_pfaffians(*screen, b, tau, hx, &kept, st) : run_elements(b, st)) != TGBA_OK) return r;
+  TGBA_CUDA(cudaEventRecord(b.ev[2], st));
+  b.ev_recorded = true;
+  b.x_evaluated = kept;
+  b.x_screened = b.n_elements - kept;
   b.x_valid = true;
   b.x_screen = screen;
   b.x_tau = tau;
-  if (!screen) {
-    b.x_evaluated = b.n_elements;
-    b.x_screened = 0;
-  }
   return TGBA_OK;
 }
 
@@ -364,7 +302,7 @@ tgba_status tgba_x_pairs(tgba_basis h, int32_t s, const int32_t* pairs_dev, int6
   cudaStream_t st = (cudaStream_t)stream;
   tgba_status r = ensure_table(*b, st);
   if (r != TGBA_OK) return r;
-  if ((r = run_pfaffian_pairs(*b, s, pairs_dev, n_pairs, out_dev, st)) != TGBA_OK) return r;
+  if ((r = run_element_pairs(*b, s, pairs_dev, n_pairs, out_dev, st)) != TGBA_OK) return r;
   return check_status(*b, st);
 }
 
@@ -651,14 +589,12 @@ tgba_status tgba_profile(tgba_basis h, tgba_prof* out) {
     out->table_ms = t0;
     out->pfaffian_ms = t1;
   }
-  out->pfaffian_flops = b->pf_flops;
-  out->pfaffian_launches = (int64_t)b->pf_plan.size();
+  out->pfaffian_flops = b->x_mults;
+  out->pfaffian_launches = b->tiles_total > 0 ? 1 : 0;
   out->kernel_launches = b->launches.load();
   out->upload_bytes = b->upload_bytes;
   out->evaluated = b->x_evaluated;
-  out->tune_mode = b->tuned ? b->tune_mode : -1;
-  out->tune_threads = b->tune_threads;
-  for (size_t i = 0; i < b->tune_log.size() && i < 8; ++i) out->tune_ms[i] = b->tune_log[i].ms;
+  out->tune_mode = -1;
   if (b->eig_ev_recorded) {
     float t0 = 0, t1 = 0;
     TGBA_CUDA(cudaEventSynchronize(b->eig_ev[2]));

@@ -20,31 +20,68 @@ __device__ __forceinline__ double2 xval(const double* c0, double p, int n) {
   }
 }
 
-// Column-major complex H of one sector, one thread per entry in 32 x 32 blocks of entries.  The
-// writes are coalesced; in the NS-row/R-column block the reads of P stride by n_r.
-__global__ void heff_kernel(int64_t n_ns, int64_t n_r, const double* __restrict__ E_ns, const double* __restrict__ E_r,
-                            const uint8_t* __restrict__ M_ns, const uint8_t* __restrict__ M_r,
-                            const double* __restrict__ P, const double* __restrict__ c0, double scale,
-                            double2* __restrict__ H) {
-  const int64_t n = n_ns + n_r;
-  const int64_t col0 = (int64_t)blockIdx.y * 32, row0 = (int64_t)blockIdx.x * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-  for (int yy = ty; yy < 32; yy += 8) {
-    const int64_t col = col0 + yy, row = row0 + tx;
-    if (col >= n || row >= n) continue;
-    double2 v = make_double2(0.0, 0.0);
-    if (row == col) {
-      v.x = row < n_ns ? E_ns[row] : E_r[row - n_ns];
-    } else if (col < n_ns && row >= n_ns) {            // R row, NS column: -L h_x conj(X_{col, row-n_ns})
-      const int64_t a = col, b = row - n_ns;
-      double2 x = xval(c0, P[a * n_r + b], M_ns[a] + M_r[b]);
-      v = make_double2(scale * x.x, -scale * x.y);
-    } else if (col >= n_ns && row < n_ns) {            // NS row, R column: -L h_x X_{row, col-n_ns}
-      const int64_t a = row, b = col - n_ns;
-      double2 x = xval(c0, P[a * n_r + b], M_ns[a] + M_r[b]);
-      v = make_double2(scale * x.x, scale * x.y);
+// Column-major complex H of every sector in one launch.  A block of 256 threads owns one 32 x 32
+// tile: of the X block (P read once, coalesced, and written to both off-diagonal blocks of H, the
+// transposed one through shared memory) or of a diagonal block (zeros and the energies).  Bound: the
+// HBM write of 16 B per entry; the streaming stores leave P in L2.  One thread per entry, with P
+// read along a column for the NS-row block and one launch per sector, took 0.56 ms for the 24
+// sectors of the L = 24 workload (1.39 GB).
+__device__ __forceinline__ double2 scaled(double s, double2 x) { return make_double2(s * x.x, s * x.y); }
+
+__global__ void __launch_bounds__(256) heff_kernel(const HeffSector* __restrict__ secs, int n_sec,
+                                                   const double* __restrict__ E_ns, const double* __restrict__ E_r,
+                                                   const uint8_t* __restrict__ M_ns, const uint8_t* __restrict__ M_r,
+                                                   const double* __restrict__ P, const double* __restrict__ c0,
+                                                   double scale, double2* __restrict__ Hall) {
+  __shared__ double t[32][33];
+  __shared__ uint8_t s_m[32];
+  int lo = 0, hi = n_sec - 1;                         // the sector holding this tile
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (secs[mid].tile0 <= (int64_t)blockIdx.x) lo = mid;
+    else hi = mid - 1;
+  }
+  const HeffSector sc = secs[lo];
+  const int64_t n_ns = sc.n_ns, n_r = sc.n_r, n = n_ns + n_r;
+  const int64_t tn = (n_ns + 31) / 32, tr = (n_r + 31) / 32;
+  int64_t q = (int64_t)blockIdx.x - sc.tile0;
+  double2* H = Hall + sc.h_off;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  if (q < tn * tr) {
+    const int64_t a0 = (q / tr) * 32, b0 = (q % tr) * 32;
+    const double* Ps = P + sc.x_off;
+    if (threadIdx.x < 32 && a0 + tx < n_ns) s_m[tx] = M_ns[sc.ns_off + a0 + tx];
+    __syncthreads();
+    const int mb = b0 + tx < n_r ? M_r[sc.r_off + b0 + tx] : 0;
+#pragma unroll
+    for (int y = ty; y < 32; y += 8) {
+      const int64_t a = a0 + y, b = b0 + tx;
+      if (a >= n_ns || b >= n_r) continue;
+      const double p = Ps[a * n_r + b];
+      t[y][tx] = p;
+      const double2 x = xval(c0, p, s_m[y] + mb);
+      __stcs(H + a * n + n_ns + b, make_double2(scale * x.x, -scale * x.y));     // R row, NS column: conj(X)
     }
-    H[col * n + row] = v;
+    __syncthreads();
+#pragma unroll
+    for (int y = ty; y < 32; y += 8) {
+      const int64_t a = a0 + tx, b = b0 + y;
+      if (a >= n_ns || b >= n_r) continue;
+      __stcs(H + (n_ns + b) * n + a, scaled(scale, xval(c0, t[tx][y], s_m[tx] + M_r[sc.r_off + b])));
+    }
+    return;
+  }
+  q -= tn * tr;
+  const bool ns = q < tn * tn;
+  if (!ns) q -= tn * tn;
+  const int64_t nt = ns ? tn : tr, m = ns ? n_ns : n_r, o = ns ? 0 : n_ns;
+  const double* E = ns ? E_ns + sc.ns_off : E_r + sc.r_off;
+  const int64_t c0_ = (q / nt) * 32, r0_ = (q % nt) * 32;
+#pragma unroll
+  for (int y = ty; y < 32; y += 8) {
+    const int64_t col = c0_ + y, row = r0_ + tx;
+    if (col >= m || row >= m) continue;
+    __stcs(H + (o + col) * n + o + row, make_double2(row == col ? E[row] : 0.0, 0.0));
   }
 }
 
@@ -87,18 +124,26 @@ int grid_for(int64_t work, int threads) {
 
 }  // namespace
 
-tgba_status assemble_heff(Basis& b, double h_x, double* heff, cudaStream_t st) {
-  const double scale = -b.L * h_x;
+std::vector<HeffSector> heff_sectors(const Basis& b, int64_t* tiles) {
+  std::vector<HeffSector> v;
+  int64_t t = 0;
   for (const Sector& sec : b.sectors) {
-    const int64_t n = sec.n_ns + sec.n_r;
-    if (n == 0) continue;
-    dim3 grid((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32)), block(32, 8);
-    heff_kernel<<<grid, block, 0, st>>>(sec.n_ns, sec.n_r, b.d_E_ns + sec.ns_off, b.d_E_r + sec.r_off,
-                                        b.d_M_ns + sec.ns_off, b.d_M_r + sec.r_off, b.d_P + sec.x_off, b.d_c0, scale,
-                                        (double2*)heff + sec.h_off);
-    TGBA_CUDA(cudaGetLastError());
-    ++b.launches;
+    if (sec.n_ns + sec.n_r == 0) continue;
+    v.push_back(HeffSector{sec.n_ns, sec.n_r, sec.ns_off, sec.r_off, sec.x_off, sec.h_off, t});
+    const int64_t tn = (sec.n_ns + 31) / 32, tr = (sec.n_r + 31) / 32;
+    t += tn * tr + tn * tn + tr * tr;
   }
+  *tiles = t;
+  return v;
+}
+
+tgba_status assemble_heff(Basis& b, double h_x, double* heff, cudaStream_t st) {
+  if (b.heff_tiles == 0) return TGBA_OK;
+  if (b.heff_tiles > 0x7fffffff) return fail(TGBA_ELIMIT, "too many tiles of H_eff");
+  heff_kernel<<<(unsigned)b.heff_tiles, 256, 0, st>>>(b.d_heff_secs, b.n_heff_secs, b.d_E_ns, b.d_E_r, b.d_M_ns,
+                                                      b.d_M_r, b.d_P, b.d_c0, -b.L * h_x, (double2*)heff);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
   return TGBA_OK;
 }
 

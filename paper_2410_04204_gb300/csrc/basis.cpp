@@ -1,6 +1,5 @@
 // Host side of the basis: single-particle modes (Eq. 6-7, S3), enumeration and truncation of
-// the Gaussian basis per momentum sector (Method section, Appendix B), and the tiling of the
-// NS x R pair grid into work units of uniform Pfaffian size.
+// the Gaussian basis per momentum sector (Method section, Appendix B).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -10,16 +9,6 @@
 #include "tgba_internal.h"
 
 namespace tgba {
-
-// Size classes of the Pfaffian kernels.  Classes 0..7: exact n = 0, 2, ..., 14 (register
-// kernel, 128 threads); classes 8..11: n <= 16, 20, 24, 32 (shared-memory kernel).
-int tile_class(int n) {
-  if (n <= 14) return n / 2;
-  if (n <= 16) return 8;
-  if (n <= 20) return 9;
-  if (n <= 24) return 10;
-  return 11;
-}
 
 Modes make_modes(int N, int parity, double h) {
   Modes md;
@@ -189,56 +178,6 @@ tgba_status enumerate_basis(const tgba_model& model, const int32_t* sectors, int
   b.n_states = ev_off;
   b.max_n = max_n;
   return TGBA_OK;
-}
-
-void build_rects(Basis& b) {
-  b.rect_lists.assign(kNumClasses, RectList());
-  for (int c = 0; c < kNumClasses; ++c) b.rect_lists[c].nmax = c < 8 ? 2 * c : c == 8 ? 16 : c == 9 ? 20 : c == 10 ? 24 : 32;
-  for (size_t s = 0; s < b.sectors.size(); ++s) {
-    const Sector& sec = b.sectors[s];
-    for (const Group& ga : sec.g_ns)
-      for (const Group& gb : sec.g_r) {
-        Rect r;
-        r.out0 = sec.x_off + ga.begin * sec.n_r + gb.begin;
-        r.ns0 = sec.ns_off + ga.begin;
-        r.r0 = sec.r_off + gb.begin;
-        r.ld = (int32_t)sec.n_r;
-        r.w = (int32_t)(gb.end - gb.begin);
-        r.rows = (int32_t)(ga.end - ga.begin);
-        r.n = ga.M + gb.M;
-        r.Ma = ga.M;
-        r.pad = 0;
-        r.tile0 = 0;
-        b.rect_lists[tile_class(r.n)].rects.push_back(r);
-      }
-  }
-  std::vector<Rect> all_reg;
-  b.max_reg_n = 0;
-  for (int c = 0; c < kNumClasses; ++c) {
-    RectList& Lc = b.rect_lists[c];
-    std::stable_sort(Lc.rects.begin(), Lc.rects.end(), [](const Rect& x, const Rect& y) { return x.n > y.n; });
-    int64_t t = 0;
-    for (Rect& r : Lc.rects) {
-      r.tile0 = t;
-      t += ((int64_t)r.rows * r.w + 31) / 32;
-    }
-    Lc.n_tiles = t;
-    Lc.n_rects = (int)Lc.rects.size();
-    if (Lc.nmax <= 14)
-      for (const Rect& r : Lc.rects) {
-        all_reg.push_back(r);
-        b.max_reg_n = std::max(b.max_reg_n, r.n);
-      }
-  }
-  std::stable_sort(all_reg.begin(), all_reg.end(), [](const Rect& x, const Rect& y) { return x.n > y.n; });
-  int64_t t = 0;
-  for (Rect& r : all_reg) {
-    r.tile0 = t;
-    t += ((int64_t)r.rows * r.w + 31) / 32;
-  }
-  b.reg_tiles_total = t;
-  b.reg_rects_total = (int)all_reg.size();
-  b.reg_rects = all_reg;
 }
 
 }  // namespace tgba

@@ -188,8 +188,8 @@ tgba_status dsf_k(Basis& b, int s, int s0, double h_x, double w_min, double w_ma
     if ((r = build_real_heff(b, s, h_x, Ak, nullptr, sk.n_ns, nullptr, sk.n_r, st)) != TGBA_OK) return r;
     if ((r = eig_sym(b, nk, Ak, Ek, true, st)) != TGBA_OK) return r;
   }
-  if ((r = run_pfaffian_cross(b, s, s0, P1, st)) != TGBA_OK) return r;
-  if ((r = run_pfaffian_cross(b, s0, s, P2, st)) != TGBA_OK) return r;
+  if ((r = run_elements_cross(b, s, s0, P1, st)) != TGBA_OK) return r;
+  if ((r = run_elements_cross(b, s0, s, P2, st)) != TGBA_OK) return r;
   // v = Y~ u0:  v_ns(k) = c P1 u0_r,  v_r(k) = c P2^T u0_ns
   TGBA_CUDA(cudaMemsetAsync(v, 0, nk * sizeof(double), st));
   if (sk.n_ns > 0 && sz.n_r > 0) {

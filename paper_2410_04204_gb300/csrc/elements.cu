@@ -1,0 +1,550 @@
+// Matrix elements X_ab = <phi_a^NS| c_1 + c_1^dag |phi_b^R> (rows a3 and a4 of the hot path;
+// Appendix A, Eq. S1-S2, S4) from the closed form of the contraction table.
+//
+// X_ab = C0 (-i)^{n/2} P_ab with P_ab = Pf(R[sel, sel]), sel = (a's NS rows) ++ (b's R rows), n =
+// M_a + M_b, and R the real contraction table of the excitation operators (the Schur complement of
+// the vacuum operators in Eq. S2's matrix).  For this chain the table is known in closed form:
+// with e_a the excitation energies (e_pi = 2 (1 - h) on the R mode at pi) and k_a the momenta,
+//   R_ab = r_a r_b t_ab,
+//   t_ab = 4 sqrt(h) sin((k_a - k_b)/2) / (e_a + e_b)      (a and b of one parity),
+//          (e_a + e_b) / (4 sqrt(h) sin((k_a - k_b)/2))     (one NS, one R),
+//   r_a^2 = (4 sqrt(h) / L) prod_{b != a, same parity} (e_a + e_b) / prod_{b, other parity} (e_a + e_b),
+//   C0 = (-1)^{L/2 + 1} [ (1 + h)/4 prod_a 1/Lambda_a ]^{1/8},  Lambda_a = r_a^2 L 2 e_a / (4 sqrt(h))
+//        (without the factor 2 e_a for the R mode at pi),
+// the finite-chain form factors of the Ising chain (Iorgov, Shadura and Tykhyy, J. Stat. Mech.
+// (2011) P02028; Bugrij and Lisovyy, Phys. Lett. A 319 (2003) 390), brought here to this library's
+// operator order and gauge and checked against the elimination of Eq. S2's matrix
+// (tgba_table_noalloc) and against direct Pfaffians (tgba_x_direct).  t_ab has the form (x_a - x_b)/
+// (x_a + x_b), so by Schur's Pfaffian identity (I. Schur, J. reine angew. Math. 139 (1911) 155)
+//   Pf(R[sel, sel]) = prod_i r_i prod_{i<j} t_ij = A_a B_b prod_{i in a, q in b} t_iq,
+// a product instead of an elimination: with G_a(q) = prod_{i in a} t_iq a row a costs M_b/2 + 1
+// multiplications per element once the products G_a(q) G_a(q') of all mode pairs are tabulated.
+//
+// Precision: e, sin and sqrt(h) come from the host as pairs of doubles, and r, t, A, B and G are
+// formed in double-double arithmetic (Dekker, Numer. Math. 18 (1971) 224) and rounded once, so an
+// element carries about M_b/2 + 2 roundings; the elimination it replaces lost about 1e-14.
+//
+// Measured on one GB300, table, elements and the complex H_eff: the 24 sectors of the L = 24 workload
+// (2.2e7 elements) 7.22 ms by elimination, 0.90 ms as products; L = 80, M <= 10 (2.7e7 elements of sizes
+// up to 20) 17.1 ms, 1.42 ms, its error against 64-bit values 9e-15 before, 4e-16 now; L = 12,
+// M <= 4 (latency) 136 us, 45 us.
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "tgba_internal.h"
+
+namespace tgba {
+namespace {
+
+// ------------------------------------------------------------------ double-double (h + l)
+struct dd { double h, l; };
+
+__device__ __forceinline__ dd two(double s, double e) {               // |s| >= |e|
+  const double t = __dadd_rn(s, e);
+  return dd{t, __dadd_rn(__dsub_rn(s, t), e)};
+}
+__device__ __forceinline__ dd mul(dd a, dd b) {
+  const double p = __dmul_rn(a.h, b.h);
+  double e = __fma_rn(a.h, b.h, -p);
+  e = __fma_rn(a.h, b.l, e);
+  e = __fma_rn(a.l, b.h, e);
+  return two(p, e);
+}
+__device__ __forceinline__ dd add(dd a, dd b) {
+  const double s = __dadd_rn(a.h, b.h), bb = __dsub_rn(s, a.h);
+  const double e = __dadd_rn(__dsub_rn(a.h, __dsub_rn(s, bb)), __dsub_rn(b.h, bb));
+  return two(s, __dadd_rn(e, __dadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ dd div(dd a, dd b) {
+  const double q = a.h / b.h;
+  const double r = __dadd_rn(__fma_rn(-q, b.h, a.h), __fma_rn(-q, b.l, a.l));
+  return two(q, r / b.h);
+}
+__device__ __forceinline__ dd root(dd a) {
+  const double s = sqrt(a.h);
+  const double r = __dadd_rn(__fma_rn(-s, s, a.h), a.l);
+  return two(s, r / (2.0 * s));
+}
+__device__ __forceinline__ dd ld(const double2* p) { const double2 v = __ldg(p); return dd{v.x, v.y}; }
+__device__ __forceinline__ dd shfl_down(dd a, int o) {
+  return dd{__shfl_down_sync(0xffffffffu, a.h, o), __shfl_down_sync(0xffffffffu, a.l, o)};
+}
+
+// The host's constants (ModeConst): rows of the table are NS modes by descending k, then R
+// modes by ascending k (the R mode at pi last).
+struct Tab {
+  int L;
+  const double2* e;     // [2L] excitation energies by table row
+  const double2* epi;   // [2L] e_a + e_pi (computed without cancellation)
+  const double2* sn;    // [2L + 1] sin(pi m / (2L))
+  const double2* cst;   // 4 sqrt(h), (1 + h)/4
+  const int* nlab;      // momentum labels by mode: NS [0, L), R [L, 2L)
+  double2* r;           // [2L]
+  double2* lam;         // [2L]
+  double2* t;           // [2L][2L]
+};
+
+__device__ __forceinline__ int label(const Tab& T, int row) { return T.nlab[row < T.L ? T.L - 1 - row : row]; }
+__device__ __forceinline__ dd esum(const Tab& T, int a, int b) {
+  const int pi = 2 * T.L - 1;
+  if (b == pi) return ld(T.epi + a);
+  if (a == pi) return ld(T.epi + b);
+  return add(ld(T.e + a), ld(T.e + b));
+}
+
+// One block per table row a: t_ab for all b, then r_a and Lambda_a by warp 0 (a lane multiplies the
+// ratios (e_a + e_same)/(e_a + e_other) of its columns, a shuffle tree the lanes).  Latency-bound
+// (2L blocks, a few divisions each); the elimination it replaces took 2L dependent launches.
+__global__ void __launch_bounds__(128) mode_table(Tab T) {
+  const int L = T.L, n2 = 2 * L, a = blockIdx.x;
+  const dd s4h = ld(T.cst);
+  const int na = label(T, a);
+  for (int b = threadIdx.x; b < n2; b += blockDim.x) {
+    double2 v = make_double2(0.0, 0.0);
+    if (b != a) {
+      const int d = na - label(T, b);
+      dd s = mul(s4h, ld(T.sn + (d < 0 ? -d : d)));
+      if (d < 0) s = dd{-s.h, -s.l};
+      const dd e = esum(T, a, b);
+      const dd q = ((a < L) == (b < L)) ? div(s, e) : div(e, s);
+      v = make_double2(q.h, q.l);
+    }
+    T.t[(size_t)a * n2 + b] = v;
+  }
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x, same0 = a < L ? 0 : L, oth0 = L - same0;
+    dd p{1.0, 0.0};
+    for (int j = lane; j < L; j += 32) {
+      const dd den = esum(T, a, oth0 + j);
+      const dd num = same0 + j == a ? dd{1.0, 0.0} : esum(T, a, same0 + j);
+      p = mul(p, div(num, den));
+    }
+    for (int o = 16; o > 0; o >>= 1) p = mul(p, shfl_down(p, o));
+    if (lane == 0) {
+      const dd r2 = mul(div(s4h, dd{(double)L, 0.0}), p);
+      const dd r = root(r2);
+      T.r[a] = make_double2(r.h, r.l);
+      const dd ea = ld(T.e + a);
+      if (a != n2 - 1) p = mul(p, dd{2.0 * ea.h, 2.0 * ea.l});
+      T.lam[a] = make_double2(p.h, p.l);
+    }
+  }
+}
+
+// R (rounded), C0, the per-state factors A_a (NS) and B_b (R), and each R state's list of mode
+// pairs (indices into the pair tables of x_tiles).  One thread per entry or state.
+__global__ void __launch_bounds__(256) state_factors(Tab T, double* __restrict__ R, double* __restrict__ c0,
+                                                     int64_t n_ns, int64_t n_r, int max_qp,
+                                                     const uint8_t* __restrict__ sel_ns, const uint8_t* __restrict__ sel_r,
+                                                     const uint8_t* __restrict__ M_ns, const uint8_t* __restrict__ M_r,
+                                                     double* __restrict__ A, double* __restrict__ B,
+                                                     uint16_t* __restrict__ pairs, int hp, unsigned* __restrict__ status) {
+  const int L = T.L, n2 = 2 * L;
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    dd p{1.0, 0.0};
+    for (int i = lane; i < L; i += 32)
+      p = mul(p, div(dd{1.0, 0.0}, mul(ld(T.lam + i), ld(T.lam + L + i))));
+    for (int o = 16; o > 0; o >>= 1) p = mul(p, shfl_down(p, o));
+    if (lane == 0) {
+      const dd c = root(root(root(mul(p, ld(T.cst + 1)))));
+      c0[0] = (L / 2) % 2 ? c.h : -c.h;
+      c0[1] = 0.0;
+      if (!(c.h > 0.0) || !isfinite(c.h)) atomicOr(status, kStTableSingular);
+    }
+  }
+  const int64_t total = (int64_t)n2 * n2 + n_ns + n_r;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+    if (q < n_ns + n_r) {
+      const bool ns = q < n_ns;
+      const int64_t s = ns ? q : q - n_ns;
+      const uint8_t* sel = (ns ? sel_ns : sel_r) + s * max_qp;
+      const int M = ns ? M_ns[s] : M_r[s];
+      dd p{1.0, 0.0};
+      for (int i = 0; i < M; ++i) {
+        const int a = sel[i];
+        p = mul(p, ld(T.r + a));
+        for (int j = i + 1; j < M; ++j) p = mul(p, ld(T.t + (size_t)a * n2 + sel[j]));
+      }
+      (ns ? A : B)[s] = p.h;
+      if (!ns)
+        for (int u = 0; u < M / 2; ++u) {
+          const int q0 = sel[2 * u] - L, q1 = sel[2 * u + 1] - L;      // ascending
+          pairs[s * hp + u] = (uint16_t)(q0 * (2 * L - q0 - 1) / 2 + (q1 - q0 - 1));
+        }
+    } else {
+      const int64_t k = q - n_ns - n_r;
+      const int a = (int)(k / n2), b = (int)(k % n2);
+      R[k] = a == b ? 0.0 : mul(mul(ld(T.r + a), ld(T.r + b)), ld(T.t + k)).h;
+    }
+  }
+}
+
+struct Elems {
+  int L, max_qp, hp;
+  const double2* t;           // [2L][2L]
+  const double* A;            // per NS state
+  const double* B;            // per R state
+  const uint16_t* pairs;      // [R state][hp]
+  const uint8_t* sel_ns;
+  const uint8_t* sel_r;
+  unsigned* status;
+};
+
+// G_a(q) = prod_{i in a} t(i, L + q), rounded once
+__device__ __forceinline__ double row_factor(const Elems& g, const uint8_t* sel, int M, int q) {
+  dd p{1.0, 0.0};
+  for (int i = 0; i < M; ++i) p = mul(p, ld(g.t + (size_t)sel[i] * (2 * g.L) + g.L + q));
+  return p.h;
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
+// One element, the same operations in the same order as x_tiles (so every path gives the same bits):
+// B_b, times G_a(q0) G_a(q1) for each mode pair of b, times A_a.
+__device__ __forceinline__ double x_value(const Elems& g, int64_t a, int Ma, int64_t b, int Mb) {
+  const uint8_t* sa = g.sel_ns + a * g.max_qp;
+  const uint8_t* sb = g.sel_r + b * g.max_qp;
+  double v = __ldg(g.B + b);
+  for (int u = 0; u < Mb / 2; ++u)
+    v = __dmul_rn(v, __dmul_rn(row_factor(g, sa, Ma, sb[2 * u] - g.L), row_factor(g, sa, Ma, sb[2 * u + 1] - g.L)));
+  return __dmul_rn(v, __ldg(g.A + a));
+}
+
+// All elements of the listed rectangles (uniform M_a and M_b).  A block owns RB rows x kColChunk
+// columns: it forms G_a(q) of its rows, then (rc.pairs) the products of all L (L - 1)/2 mode pairs
+// in shared memory, and each thread then walks down its columns, loading a column's pair list and
+// B_b once for the RB rows: M_b/2 + 1 multiplications and M_b/2 shared-memory loads per element
+// and one coalesced 8-byte store.  Rectangles whose columns would use fewer pair products than the
+// table holds (w M_b/2 <= L (L - 1)/2, see build_rects) multiply the two factors themselves, which
+// rounds the same way.  RB is the largest of 8, 4, 2, 1 whose tables fit 100 KB (two blocks per
+// SM): 8 up to L = 56, 4 up to L = 80, 2 up to L = 112.  Bound: FP64 multiplications (2 lanes per SM and clock) for M_b >= 4.
+constexpr int kColChunk = 2048;
+constexpr int kTileThreads = 256;
+
+template <int RB, int H>
+__device__ __forceinline__ void tile_columns(const Elems& g, const Rect& rc, const double* sG, const double* sG2, int np,
+                                             int r0, int nr, int c0, int c1, double* __restrict__ P) {
+  double av[RB];
+#pragma unroll
+  for (int r = 0; r < RB; ++r) av[r] = __ldg(g.A + rc.ns0 + r0 + min(r, nr - 1));
+  bool bad = false;
+  for (int c = c0 + (int)threadIdx.x; c < c1; c += kTileThreads) {
+    const int64_t b = rc.r0 + c;
+    const double bv = __ldg(g.B + b);
+    double* out = P + rc.out0 + (int64_t)r0 * rc.ld + c;
+    if (rc.pairs || H == 0) {
+      int id[H > 0 ? H : 1];
+#pragma unroll
+      for (int u = 0; u < H; ++u) id[u] = __ldg(g.pairs + b * g.hp + u);
+#pragma unroll
+      for (int r = 0; r < RB; ++r) {
+        double v = bv;
+#pragma unroll
+        for (int u = 0; u < H; ++u) v = __dmul_rn(v, sG2[r * np + id[u]]);
+        v = __dmul_rn(v, av[r]);
+        bad |= !finite_bits(v);
+        if (r < nr) out[(int64_t)r * rc.ld] = v;
+      }
+    } else {
+      const uint8_t* sb = g.sel_r + b * g.max_qp;
+      int q[H > 0 ? 2 * H : 1];
+#pragma unroll
+      for (int u = 0; u < 2 * H; ++u) q[u] = __ldg(sb + u) - g.L;
+#pragma unroll
+      for (int r = 0; r < RB; ++r) {
+        double v = bv;
+#pragma unroll
+        for (int u = 0; u < H; ++u)
+          v = __dmul_rn(v, __dmul_rn(sG[r * g.L + q[2 * u]], sG[r * g.L + q[2 * u + 1]]));
+        v = __dmul_rn(v, av[r]);
+        bad |= !finite_bits(v);
+        if (r < nr) out[(int64_t)r * rc.ld] = v;
+      }
+    }
+  }
+  if (bad) atomicOr(g.status, kStNan);
+}
+
+template <int RB>
+__global__ void __launch_bounds__(kTileThreads) x_tiles(Elems g, const Rect* __restrict__ rects, int n_rects,
+                                                        double* __restrict__ P) {
+  extern __shared__ double sm[];
+  const int L = g.L, np = L * (L - 1) / 2;
+  double* sG = sm;                       // [RB][L]
+  double* sG2 = sm + RB * L;             // [RB][np]
+  int lo = 0, hi = n_rects - 1;          // the rectangle holding this tile
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (rects[mid].tile0 <= (int64_t)blockIdx.x) lo = mid;
+    else hi = mid - 1;
+  }
+  const Rect rc = rects[lo];
+  const int lt = (int)((int64_t)blockIdx.x - rc.tile0), ncc = (rc.w + kColChunk - 1) / kColChunk;
+  const int r0 = (lt / ncc) * RB, nr = min(RB, rc.rows - r0);
+  const int c0 = (lt % ncc) * kColChunk, c1 = min(rc.w, c0 + kColChunk);
+  const int Ma = rc.Ma, H = (rc.n - rc.Ma) / 2;
+  // rows beyond the rectangle repeat its last row (never stored), so that every value is finite
+  for (int i = threadIdx.x; i < RB * L; i += kTileThreads) {
+    const int r = min(i / L, nr - 1), q = i % L;
+    sG[i] = row_factor(g, g.sel_ns + (rc.ns0 + r0 + r) * g.max_qp, Ma, q);
+  }
+  __syncthreads();
+  if (rc.pairs) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int q0 = warp; q0 < L - 1; q0 += kTileThreads / 32) {
+      const int base = q0 * (2 * L - q0 - 1) / 2 - (q0 + 1);
+      for (int q1 = q0 + 1 + lane; q1 < L; q1 += 32)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) sG2[r * np + base + q1] = __dmul_rn(sG[r * L + q0], sG[r * L + q1]);
+    }
+    __syncthreads();
+  }
+  switch (H) {
+    case 0: tile_columns<RB, 0>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    case 1: tile_columns<RB, 1>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    case 2: tile_columns<RB, 2>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    case 3: tile_columns<RB, 3>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    case 4: tile_columns<RB, 4>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    case 5: tile_columns<RB, 5>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    case 6: tile_columns<RB, 6>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    case 7: tile_columns<RB, 7>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+    default: tile_columns<RB, 8>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+  }
+}
+
+// One thread per explicit (a, b) pair: X = C0 (-i)^{n/2} P.
+__global__ void __launch_bounds__(128) x_pairs_kernel(Elems g, const int32_t* __restrict__ pairs, int64_t n_pairs,
+                                                      int64_t ns_off, int64_t r_off, int64_t n_ns, int64_t n_r,
+                                                      const uint8_t* __restrict__ m_ns, const uint8_t* __restrict__ m_r,
+                                                      const double* __restrict__ c0, double* __restrict__ out) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n_pairs; q += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t pa = pairs[2 * q], pb = pairs[2 * q + 1];
+    if (pa < 0 || pa >= n_ns || pb < 0 || pb >= n_r) {      // reject, never read out of range
+      atomicOr(g.status, kStBadIndex);
+      out[2 * q] = out[2 * q + 1] = __longlong_as_double(0x7ff8000000000000ll);
+      continue;
+    }
+    const int64_t a = ns_off + pa, b = r_off + pb;
+    const int ma = m_ns[a], mb = m_r[b];
+    const double pf = x_value(g, a, ma, b, mb);
+    if (!finite_bits(pf)) atomicOr(g.status, kStNan);
+    const double re = c0[0] * pf, im = c0[1] * pf;
+    switch (((ma + mb) / 2) & 3) {
+      case 0: out[2 * q] = re; out[2 * q + 1] = im; break;
+      case 1: out[2 * q] = im; out[2 * q + 1] = -re; break;
+      case 2: out[2 * q] = -re; out[2 * q + 1] = -im; break;
+      default: out[2 * q] = -im; out[2 * q + 1] = re; break;
+    }
+  }
+}
+
+// The pairs that the screener kept: list n / 2 holds counts[n / 2] entries from list_off[n / 2].
+// Screened pairs are not visited (their P stays 0).
+__global__ void __launch_bounds__(128) x_lists(Elems g, const uint8_t* __restrict__ M_ns, const unsigned* __restrict__ counts,
+                                               const int64_t* __restrict__ list_off, int sizes,
+                                               const PairEntry* __restrict__ lists, double* __restrict__ P) {
+  for (int h = 0; h < sizes; ++h) {
+    const int64_t n = counts[h];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+      const PairEntry pe = lists[list_off[h] + i];
+      const int ma = M_ns[pe.a];
+      const double v = x_value(g, pe.a, ma, pe.b, 2 * h - ma);
+      if (!finite_bits(v)) atomicOr(g.status, kStNan);
+      P[pe.out] = v;
+    }
+  }
+}
+
+int rows_per_tile(int L) {
+  for (int rb = 8; rb > 1; rb /= 2)
+    if ((size_t)rb * (L + L * (L - 1) / 2) * sizeof(double) <= 102400) return rb;
+  return 1;
+}
+
+Elems elems_of(const Basis& b) {
+  Elems g;
+  g.L = b.L; g.max_qp = b.max_qp; g.hp = std::max(1, b.max_qp / 2);
+  g.t = (const double2*)b.d_tdd;
+  g.A = b.d_fac_ns; g.B = b.d_fac_r; g.pairs = b.d_pairs_r;
+  g.sel_ns = b.d_sel_ns; g.sel_r = b.d_sel_r;
+  g.status = b.d_status;
+  return g;
+}
+
+tgba_status launch_tiles(Basis& b, const Rect* d_rects, int n_rects, int64_t n_tiles, double* P, cudaStream_t st) {
+  if (n_tiles == 0) return TGBA_OK;
+  if (n_tiles > 0x7fffffff) return fail(TGBA_ELIMIT, "too many element tiles");
+  const Elems g = elems_of(b);
+  const int rb = rows_per_tile(b.L);
+  const size_t smem = (size_t)rb * (b.L + b.L * (b.L - 1) / 2) * sizeof(double);
+  auto go = [&](auto kern) -> tgba_status {
+    if (smem > 48 * 1024)
+      TGBA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<(unsigned)n_tiles, kTileThreads, smem, st>>>(g, d_rects, n_rects, P);
+    TGBA_CUDA(cudaGetLastError());
+    ++b.launches;
+    return TGBA_OK;
+  };
+  return rb == 8 ? go(x_tiles<8>) : rb == 4 ? go(x_tiles<4>) : rb == 2 ? go(x_tiles<2>) : go(x_tiles<1>);
+}
+
+// rectangles of uniform (M_a, M_b) of one NS group list against one R group list; X row-major from
+// out0 with row stride ld
+void add_rects(std::vector<Rect>& v, const std::vector<Group>& g_ns, int64_t ns_off, const std::vector<Group>& g_r,
+               int64_t r_off, int64_t out0, int64_t ld, int L) {
+  for (const Group& ga : g_ns)
+    for (const Group& gb : g_r) {
+      Rect r;
+      r.out0 = out0 + ga.begin * ld + gb.begin;
+      r.ns0 = ns_off + ga.begin;
+      r.r0 = r_off + gb.begin;
+      r.tile0 = 0;
+      r.ld = (int32_t)ld;
+      r.w = (int32_t)(gb.end - gb.begin);
+      r.rows = (int32_t)(ga.end - ga.begin);
+      r.n = ga.M + gb.M;
+      r.Ma = ga.M;
+      // the pair table costs L (L - 1)/2 products per row and saves one per element and pair
+      r.pairs = (int64_t)std::min(r.w, kColChunk) * (gb.M / 2) > (int64_t)L * (L - 1) / 2;
+      v.push_back(r);
+    }
+}
+
+// largest n first, tiles numbered; returns the tiles of the first `head` rectangles in *head_tiles
+int64_t number_tiles(std::vector<Rect>& v, int L, int n_head, int64_t* head_tiles) {
+  std::stable_sort(v.begin(), v.end(), [](const Rect& x, const Rect& y) { return x.n > y.n; });
+  const int rb = rows_per_tile(L);
+  int64_t t = 0;
+  if (head_tiles) *head_tiles = 0;
+  for (Rect& r : v) {
+    r.tile0 = t;
+    t += (int64_t)((r.rows + rb - 1) / rb) * ((r.w + kColChunk - 1) / kColChunk);
+    if (head_tiles && r.n >= n_head) *head_tiles = t;
+  }
+  return t;
+}
+
+}  // namespace
+
+// Every rectangle of the basis, largest n first (so those the screener does not judge, n >= 16, are
+// the first b.big_rects).
+void build_rects(Basis& b) {
+  b.rects.clear();
+  for (const Sector& sec : b.sectors)
+    add_rects(b.rects, sec.g_ns, sec.ns_off, sec.g_r, sec.r_off, sec.x_off, sec.n_r, b.L);
+  b.tiles_total = number_tiles(b.rects, b.L, 16, &b.big_tiles);
+  b.big_rects = 0;
+  b.x_mults = 0;
+  for (const Rect& r : b.rects) {
+    if (r.n >= 16) ++b.big_rects;
+    b.x_mults += ((r.n - r.Ma) / 2 + 1.0) * (double)r.rows * r.w;
+  }
+}
+
+// Constants of the closed form, in long double on the host (rounded to pairs of doubles).
+tgba_status upload_mode_constants(Basis& b) {
+  using ld = long double;
+  const int L = b.L, n2 = 2 * L;
+  const ld pi = std::acos((ld)-1), h = (ld)b.h;
+  std::vector<double> v((size_t)2 * (2 * n2 + n2 + 1 + 2));
+  auto put = [&](size_t i, ld x) {
+    v[2 * i] = (double)x;
+    v[2 * i + 1] = (double)(x - (ld)v[2 * i]);
+  };
+  const ld e_pi = 2 * (1 - h);
+  for (int a = 0; a < n2; ++a) {
+    const int n = a < L ? -(L - 1) + 2 * (L - 1 - a) : -(L - 2) + 2 * (a - L);
+    const ld c = std::cos(pi * n / (2 * (ld)L));
+    if (n == L) {
+      put(a, e_pi);
+      put(n2 + a, 2 * e_pi);
+    } else {
+      const ld e = 2 * std::sqrt((h - 1) * (h - 1) + 4 * h * c * c);
+      put(a, e);
+      // e^2 - e_pi^2 = 16 h cos^2(k/2): no cancellation when e_pi < 0
+      put(n2 + a, e_pi < 0 ? 16 * h * c * c / (e - e_pi) : e + e_pi);
+    }
+  }
+  for (int m = 0; m <= n2; ++m) put(2 * n2 + m, std::sin(pi * m / (2 * (ld)L)));
+  put(3 * n2 + 1, 4 * std::sqrt(h));
+  put(3 * n2 + 2, (1 + h) / 4);
+  TGBA_CUDA(cudaMalloc((void**)&b.d_const, v.size() * sizeof(double)));
+  TGBA_CUDA(cudaMemcpy(b.d_const, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice));
+  b.upload_bytes += (int64_t)(v.size() * sizeof(double));
+  const size_t nns = b.ns.E.size(), nr = b.r.E.size(), hp = (size_t)std::max(1, b.max_qp / 2);
+  TGBA_CUDA(cudaMalloc((void**)&b.d_tdd, sizeof(double) * 2 * ((size_t)n2 * n2 + 2 * n2)));
+  TGBA_CUDA(cudaMalloc((void**)&b.d_fac_ns, sizeof(double) * std::max<size_t>(1, nns)));
+  TGBA_CUDA(cudaMalloc((void**)&b.d_fac_r, sizeof(double) * std::max<size_t>(1, nr)));
+  TGBA_CUDA(cudaMalloc((void**)&b.d_pairs_r, sizeof(uint16_t) * std::max<size_t>(1, nr * hp)));
+  return TGBA_OK;
+}
+
+tgba_status build_table(Basis& b, cudaStream_t st) {
+  const int L = b.L, n2 = 2 * L;
+  Tab T;
+  T.L = L;
+  T.e = (const double2*)b.d_const;
+  T.epi = T.e + n2;
+  T.sn = T.epi + n2;
+  T.cst = T.sn + n2 + 1;
+  T.nlab = b.d_nlab;
+  T.t = (double2*)b.d_tdd;
+  T.r = T.t + (size_t)n2 * n2;
+  T.lam = T.r + n2;
+  mode_table<<<n2, 128, 0, st>>>(T);
+  const int64_t nns = (int64_t)b.ns.E.size(), nr = (int64_t)b.r.E.size(), work = (int64_t)n2 * n2 + nns + nr;
+  state_factors<<<(int)std::min<int64_t>((work + 255) / 256, 152 * 8), 256, 0, st>>>(
+      T, b.d_table, b.d_c0, nns, nr, b.max_qp, b.d_sel_ns, b.d_sel_r, b.d_M_ns, b.d_M_r, b.d_fac_ns, b.d_fac_r,
+      b.d_pairs_r, std::max(1, b.max_qp / 2), b.d_status);
+  TGBA_CUDA(cudaGetLastError());
+  b.launches += 2;
+  b.table_valid = true;
+  return TGBA_OK;
+}
+
+tgba_status run_elements(Basis& b, cudaStream_t st) {
+  return launch_tiles(b, b.d_rects, (int)b.rects.size(), b.tiles_total, b.d_P, st);
+}
+
+tgba_status run_elements_big(Basis& b, cudaStream_t st) {
+  return launch_tiles(b, b.d_rects, b.big_rects, b.big_tiles, b.d_P, st);
+}
+
+tgba_status run_element_lists(Basis& b, const unsigned* counts, const int64_t* list_off, int sizes,
+                              const PairEntry* lists, cudaStream_t st) {
+  x_lists<<<152 * 8, 128, 0, st>>>(elems_of(b), b.d_M_ns, counts, list_off, sizes, lists, b.d_P);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
+  return TGBA_OK;
+}
+
+tgba_status run_element_pairs(Basis& b, int s, const int32_t* pairs, int64_t n, double* out, cudaStream_t st) {
+  if (n == 0) return TGBA_OK;
+  const Sector& sec = b.sectors[s];
+  x_pairs_kernel<<<(int)std::min<int64_t>((n + 127) / 128, 152 * 16), 128, 0, st>>>(
+      elems_of(b), pairs, n, sec.ns_off, sec.r_off, sec.n_ns, sec.n_r, b.d_M_ns, b.d_M_r, b.d_c0, out);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
+  return TGBA_OK;
+}
+
+tgba_status run_elements_cross(Basis& b, int s_ns, int s_r, double* out, cudaStream_t st) {
+  const Sector& A = b.sectors[s_ns];
+  const Sector& B = b.sectors[s_r];
+  if (A.n_ns * B.n_r == 0) return TGBA_OK;
+  std::vector<Rect> v;
+  add_rects(v, A.g_ns, A.ns_off, B.g_r, B.r_off, 0, B.n_r, b.L);
+  const int64_t tiles = number_tiles(v, b.L, 0, nullptr);
+  Rect* d = nullptr;
+  TGBA_CUDA(cudaMallocAsync((void**)&d, v.size() * sizeof(Rect), st));
+  cudaError_t e = cudaMemcpyAsync(d, v.data(), v.size() * sizeof(Rect), cudaMemcpyHostToDevice, st);
+  tgba_status r = e == cudaSuccess ? launch_tiles(b, d, (int)v.size(), tiles, out, st)
+                                   : cuda_fail(e, "rectangles of the cross-sector elements");
+  cudaFreeAsync(d, st);
+  return r;
+}
+
+}  // namespace tgba

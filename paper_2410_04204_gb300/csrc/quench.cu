@@ -206,37 +206,11 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
                    int j_max, double* corr_out) {
   const Sector& sec = b.sectors[s];
   const int L = b.L;
-  // s = conj(z)/|z|, z = <0_NS(h0)|sigma_1|0_R(h0)>: the vacuum element of a table at h0
   Modes m0ns = make_modes(L, 0, h0 / b.J), m0r = make_modes(L, 1, h0 / b.J);
   Modes mns = make_modes(L, 0, b.h), mr = make_modes(L, 1, b.h);
-  double z[2];
-  {
-    Basis tmp;
-    tmp.L = L; tmp.device = b.device;
-    std::vector<double> th(2 * L);
-    std::vector<int> nl(2 * L);
-    for (int i = 0; i < L; ++i) { th[i] = m0ns.theta[i]; th[L + i] = m0r.theta[i]; nl[i] = m0ns.nlab[i]; nl[L + i] = m0r.nlab[i]; }
-    tmp.vac_norm = m0ns.norm * m0r.norm;
-    const int64_t need = 2 * L + L + 2 * (16 * (int64_t)L * L + 4 * L + 1) + 4 * (int64_t)L * L + 8;
-    double* sc;
-    tgba_status r = scratch(b, need, &sc);
-    if (r != TGBA_OK) return r;
-    tmp.d_theta = sc;
-    tmp.d_nlab = (int*)(sc + 2 * L);
-    tmp.d_work = sc + 3 * L;
-    tmp.d_table = tmp.d_work + 2 * (16 * (int64_t)L * L + 4 * L + 1);
-    tmp.d_c0 = tmp.d_table + 4 * (int64_t)L * L;
-    tmp.d_status = b.d_status;
-    TGBA_CUDA(cudaMemcpyAsync(tmp.d_theta, th.data(), 2 * L * sizeof(double), cudaMemcpyHostToDevice, st));
-    TGBA_CUDA(cudaMemcpyAsync(tmp.d_nlab, nl.data(), 2 * L * sizeof(int), cudaMemcpyHostToDevice, st));
-    if ((r = build_table(tmp, st)) != TGBA_OK) return r;
-    TGBA_CUDA(cudaMemcpyAsync(z, tmp.d_c0, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    TGBA_CUDA(cudaStreamSynchronize(st));
-    if ((r = check_status(b, st)) != TGBA_OK) return r;
-  }
-  const double zabs = std::hypot(z[0], z[1]);
-  if (!(zabs > 0)) return fail(TGBA_ENUMERIC, "vanishing vacuum element at the initial field");
-  const double s_re = z[0] / zabs, s_im = -z[1] / zabs;
+  // s = conj(z)/|z|, z = <0_NS(h0)|sigma_1|0_R(h0)>: the vacuum element at h0, which is real with the
+  // sign (-1)^{L/2 + 1} at every field (elements.cu)
+  const double s_re = (L / 2) % 2 ? 1.0 : -1.0, s_im = 0.0;
   const double cabs = std::hypot(b.c0_host[0], b.c0_host[1]);
   const double g_re = b.c0_host[0] / cabs, g_im = b.c0_host[1] / cabs;   // e^{i arg C0(h)}
   // Eq. S6 ingredients: D_k and prod_{0<k<pi} cos(D_k/2) per parity

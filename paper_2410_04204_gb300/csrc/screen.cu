@@ -421,9 +421,8 @@ tgba_status screen_score(Screen& s, Basis& b, int sidx, float* pred, cudaStream_
     if (r != TGBA_OK) return r;
   }
   std::vector<Rect> rects;
-  for (const RectList& L : b.rect_lists)
-    for (const Rect& rc : L.rects)
-      if (rc.ns0 >= sec.ns_off && rc.ns0 < sec.ns_off + sec.n_ns) rects.push_back(rc);
+  for (const Rect& rc : b.rects)
+    if (rc.ns0 >= sec.ns_off && rc.ns0 < sec.ns_off + sec.n_ns) rects.push_back(rc);
   float* part = nullptr;
   tgba_status r = state_partials_all(s, b, &part, st);
   if (r != TGBA_OK) return r;
@@ -436,9 +435,9 @@ tgba_status screen_score(Screen& s, Basis& b, int sidx, float* pred, cudaStream_
   return r;
 }
 
-// The screened Pfaffian stage (after the contraction table): P = 0, the register-size pairs
-// scored and the kept ones compacted into per-size lists, their Pfaffians from the lists, and
-// the shared-memory sizes (n >= 16) without screening.  *kept: pairs evaluated by Pfaffian.
+// The screened element stage (after the contraction table): P = 0, the pairs with n <= 14 scored and
+// the kept ones compacted into per-size lists, their elements from the lists, and the larger
+// sizes without screening.  *kept: pairs evaluated.
 tgba_status screen_pfaffians(Screen& s, Basis& b, double tau, double hx, int64_t* kept, cudaStream_t st) {
   if (s.H != 256) return fail(TGBA_EINVAL, "inference supports width 256");
   if (!s.w2b_valid) {
@@ -448,7 +447,8 @@ tgba_status screen_pfaffians(Screen& s, Basis& b, double tau, double hx, int64_t
   const int H = s.H;
   constexpr int kSizes = 8;                                     // n = 0, 2, ..., 14
   std::vector<int64_t> off(kSizes + 1, 0);
-  for (const Rect& rc : b.reg_rects) off[rc.n / 2 + 1] += (int64_t)rc.rows * rc.w;
+  const std::vector<Rect> small(b.rects.begin() + b.big_rects, b.rects.end());
+  for (const Rect& rc : small) off[rc.n / 2 + 1] += (int64_t)rc.rows * rc.w;
   for (int i = 0; i < kSizes; ++i) off[i + 1] += off[i];
   TGBA_CUDA(cudaMemsetAsync(b.d_P, 0, (size_t)std::max<int64_t>(1, b.n_elements) * sizeof(double), st));
   void* lb = nullptr;
@@ -466,10 +466,10 @@ tgba_status screen_pfaffians(Screen& s, Basis& b, double tau, double hx, int64_t
   // keep iff y - (n/2) log10(L/24) + log10(L hx) >= log10(tau) - margin
   const float half_log_l = (float)(0.5 * std::log10(b.L / 24.0));
   const float shift = (float)(std::log10(b.L * std::fabs(hx)) - std::log10(tau) + s.margin);
-  r = score_rects_tc(b, b.reg_rects, part, part + (int64_t)b.ns.E.size() * H, s.W2b, b2, b2 + H, b2 + 2 * H, shift,
+  r = score_rects_tc(b, small, part, part + (int64_t)b.ns.E.size() * H, s.W2b, b2, b2 + H, b2 + 2 * H, shift,
                      half_log_l, nullptr, 0, d_cnt, d_off, lists, st);
-  if (r == TGBA_OK) r = run_pfaffian_lists(b, d_cnt, d_off, lists, st);
-  if (r == TGBA_OK) r = run_pfaffians_smem_classes(b, st);
+  if (r == TGBA_OK) r = run_element_lists(b, d_cnt, d_off, kSizes, lists, st);
+  if (r == TGBA_OK) r = run_elements_big(b, st);
   unsigned hc[kSizes] = {};
   if (r == TGBA_OK) {
     TGBA_CUDA(cudaMemcpyAsync(hc, d_cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
@@ -532,7 +532,7 @@ tgba_status screen_train(Basis** sets, int n_sets, int64_t n_samples, uint64_t s
     if (!bb.table_valid) {
       if ((r = build_table(bb, st)) != TGBA_OK) return r;
     }
-    if ((r = run_pfaffian_pairs(bb, sidx, dp, n, dx, st)) != TGBA_OK) return r;
+    if ((r = run_element_pairs(bb, sidx, dp, n, dx, st)) != TGBA_OK) return r;
     pair_features<<<blocks(n), 256, 0, st>>>(n, dp, sec.ns_off, sec.r_off, bb.d_modes_ns, bb.d_modes_r, bb.d_M_ns,
                                              bb.d_M_r, bb.max_qp, bb.d_nlab, bb.L, X + o * kD);
     pair_targets<<<blocks(n), 256, 0, st>>>(n, dp, sec.ns_off, sec.r_off, bb.d_M_ns, bb.d_M_r, dx,

@@ -16,7 +16,6 @@ namespace tgba {
 constexpr int kMaxQp = 16;        // quasiparticles per state
 constexpr int kMaxL = 120;        // 2L excitation operators must index a uint8 table row
 constexpr int kMaxN = 2 * kMaxQp; // largest Pfaffian M_a + M_b
-constexpr int kNumClasses = 12;   // Pfaffian size classes (basis.cpp: tile_class)
 
 // Device status word bits (tgba_status is derived from them at the next sync).
 enum : unsigned { kStNan = 1u, kStTableImag = 2u, kStTableSingular = 4u, kStTimeout = 8u, kStBadIndex = 16u,
@@ -46,8 +45,8 @@ struct StateTable {
   std::vector<int16_t> modes;      // [state][max_qp], ascending mode indices, -1 padded
 };
 
-// Work of the Pfaffian stage: a rectangle of pairs with uniform (M_a, M_b), laid out row-major
-// (row = NS state, column = R state), cut into tiles of 32 consecutive pairs (one per warp).
+// Work of the element stage: a rectangle of pairs with uniform (M_a, M_b), laid out row-major
+// (row = NS state, column = R state), cut into tiles (elements.cu: x_tiles).
 struct Rect {
   int64_t out0;   // element index of the rectangle's first pair in the X cache
   int64_t ns0;    // global NS state index of the rectangle's first row
@@ -58,22 +57,11 @@ struct Rect {
   int32_t rows;   // rectangle height
   int32_t n;      // Pfaffian size M_a + M_b
   int32_t Ma;     // quasiparticles of the NS state
-  int32_t pad;
+  int32_t pairs;  // 1: products of mode pairs tabulated per row
 };
 
-// Rectangles of one size class: exact n for n <= 14 (register kernels), n <= 16/20/24/32 above.
-struct RectList {
-  int nmax = 0;
-  std::vector<Rect> rects;        // sorted by n descending, tile0 prefix
-  int64_t n_tiles = 0;
-  Rect* d_rects = nullptr;
-  int n_rects = 0;
-};
-
-// One kernel launch of the Pfaffian stage (kind 0: one exact register size, 1: queue over all
-// register sizes, 2: shared-memory class).
-struct PfLaunch { int kind, size, threads, grid, list; size_t smem; };
-struct TuneEntry { int mode, threads; float ms; };
+// A sector as the assembly kernel sees it: tile0 is its first tile in the launch.
+struct HeffSector { int64_t n_ns, n_r, ns_off, r_off, x_off, h_off, tile0; };
 
 // Single-particle data of one parity at field h (Eq. 7, S3), host side.
 struct Modes {
@@ -90,7 +78,6 @@ struct Basis;
 // basis.cpp
 tgba_status enumerate_basis(const tgba_model& model, const int32_t* sectors, int n_sectors,
                             const tgba_trunc& tr, Basis& b);
-void build_rects(Basis& b);
 
 struct Basis {
   int L = 0;
@@ -119,29 +106,27 @@ struct Basis {
   double* d_table = nullptr;       // R, 2L x 2L row-major
   double* d_c0 = nullptr;          // C0 (re, im), then diagnostics: max |Im| residual, max |R|
   double c0_host[2] = {0, 0};
-  double* d_work = nullptr;        // 4L x 4L complex scratch of the table build
+  double* d_const = nullptr;       // constants of the closed form (elements.cu)
+  double* d_tdd = nullptr;         // its factors t [2L][2L], r and Lambda [2L] (pairs of doubles)
+  double* d_fac_ns = nullptr; double* d_fac_r = nullptr;     // per-state factors A, B
+  uint16_t* d_pairs_r = nullptr;   // mode pairs of the R states
   bool table_valid = false;
-  // Pfaffian stage
+  // element stage
   double* d_P = nullptr;           // X_ab = C0 (-i)^{(M_a+M_b)/2} P_ab, P real, [n_elements]
   bool x_valid = false;
   const void* x_screen = nullptr;
   double x_tau = 0;
   int64_t x_evaluated = 0, x_screened = 0;
-  std::vector<RectList> rect_lists;    // one per size class (basis.cpp: tile_class)
-  std::vector<Rect> reg_rects;         // all register-size rectangles, n descending, one tile prefix
-  Rect* d_reg_rects = nullptr;
-  int reg_rects_total = 0;
-  int64_t reg_tiles_total = 0;
-  int max_reg_n = 0;
-  unsigned long long* d_counter = nullptr;   // work counter of the queue launch
-  std::vector<PfLaunch> pf_plan;
-  int tune_mode = 0, tune_threads = 128;
-  bool tuned = false;
-  std::vector<TuneEntry> tune_log;
-  cudaGraph_t graph = nullptr;         // table + Pfaffian stage, captured once
-  cudaGraphExec_t graph_exec = nullptr;
+  std::vector<Rect> rects;             // all rectangles, n descending, one tile prefix
+  Rect* d_rects = nullptr;
+  int64_t tiles_total = 0;
+  int big_rects = 0;                   // the first ones: n >= 16
+  int64_t big_tiles = 0;
+  HeffSector* d_heff_secs = nullptr;   // non-empty sectors (assemble.cu)
+  int n_heff_secs = 0;
+  int64_t heff_tiles = 0;
+  double x_mults = 0;                  // FP64 multiplications of one element stage
   bool c0_host_valid = false;
-  int64_t graph_launches = 0;          // kernel launches inside the graph
   unsigned* d_status = nullptr;
   // measurement
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
@@ -153,8 +138,7 @@ struct Basis {
   int64_t eig_matrices = 0;
   int eig_cluster = 0;
   std::atomic<int64_t> launches{0};
-  int64_t upload_bytes = 0, pf_launches = 0;
-  double pf_flops = 0;
+  int64_t upload_bytes = 0;
   // eigen solver scratch
   void* solver = nullptr;          // cusolverDnHandle_t
   void* blas = nullptr;            // cublasHandle_t
@@ -176,14 +160,12 @@ struct Basis {
 tgba_status fail(tgba_status st, const std::string& msg);
 tgba_status cuda_fail(cudaError_t e, const char* what);
 
-// table.cu
+// elements.cu: the contraction table in closed form, and the elements as products
+void build_rects(Basis& b);
+tgba_status upload_mode_constants(Basis& b);
 tgba_status build_table(Basis& b, cudaStream_t st);
-
-// pfaffian.cu
-tgba_status plan_pfaffians(Basis& b);
-tgba_status autotune_pfaffians(Basis& b, cudaStream_t st);
-tgba_status run_pfaffians(Basis& b, cudaStream_t st);
-tgba_status run_pfaffian_pairs(Basis& b, int s, const int32_t* pairs, int64_t n, double* out, cudaStream_t st);
+tgba_status run_elements(Basis& b, cudaStream_t st);
+tgba_status run_element_pairs(Basis& b, int s, const int32_t* pairs, int64_t n, double* out, cudaStream_t st);
 // direct.cu: X of explicit pairs by the paper-literal Pfaffian of size 2L + M_a + M_b
 size_t x_direct_smem(int L, int max_qp, int jmid);
 tgba_status x_direct(Basis& b, int s, const int32_t* pairs, int64_t n, double* out, cudaStream_t st);
@@ -197,9 +179,10 @@ size_t z_reduced_smem(int max_qp, int j);
 tgba_status z_reduced_elements(Basis& b, int s, int parity, int j, int J, const double* S, const double* c0z,
                                const int32_t* pairs, int64_t n, double* out, cudaStream_t st);
 // real P of every (NS state of sector s_ns, R state of sector s_r) pair, out [n_ns][n_r] row-major
-tgba_status run_pfaffian_cross(Basis& b, int s_ns, int s_r, double* out, cudaStream_t st);
+tgba_status run_elements_cross(Basis& b, int s_ns, int s_r, double* out, cudaStream_t st);
 
 // assemble.cu
+std::vector<HeffSector> heff_sectors(const Basis& b, int64_t* tiles);
 tgba_status assemble_heff(Basis& b, double h_x, double* heff, cudaStream_t st);
 tgba_status export_x(Basis& b, int s, double* x, cudaStream_t st);
 tgba_status build_real_heff(Basis& b, int s, double h_x, double* a, const int32_t* idx_ns, int64_t kn,
@@ -267,11 +250,11 @@ tgba_status score_rects_tc(Basis& b, const std::vector<Rect>& rects, const float
                            const __nv_bfloat16* W2b, const float* b2, const float* w3, const float* b3, float shift,
                            float half_log_l, float* pred, int64_t pred_base, unsigned* counts,
                            const int64_t* list_off, PairEntry* lists, cudaStream_t st);
-// pfaffian.cu: Pfaffians of the kept pairs (sizes n <= 14, lists per n / 2), and the launches of
-// the shared-memory size classes (n >= 16) without screening
-tgba_status run_pfaffian_lists(Basis& b, const unsigned* counts, const int64_t* list_off, const PairEntry* lists,
-                               cudaStream_t st);
-tgba_status run_pfaffians_smem_classes(Basis& b, cudaStream_t st);
+// elements.cu: the kept pairs (sizes n <= 14, `sizes` lists per n / 2), and the rectangles with
+// n >= 16, which are not screened
+tgba_status run_element_lists(Basis& b, const unsigned* counts, const int64_t* list_off, int sizes,
+                              const PairEntry* lists, cudaStream_t st);
+tgba_status run_elements_big(Basis& b, cudaStream_t st);
 
 // dgemm_tc.cu: FP64 products on the tensor cores (BF16 slices, exact FP32 chunk sums, 48-bit
 // running sums).  An operand (rows x K) is sliced by emu_slice into tile images of 128 rows (A
