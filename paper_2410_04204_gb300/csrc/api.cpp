@@ -58,7 +58,7 @@ static void release(Basis* b) {
                   b->d_theta, b->d_nlab, b->d_table, b->d_c0, b->d_const, b->d_tdd, b->d_fac_ns, b->d_fac_r, b->d_pairs_r,
                   b->d_P, b->d_status,
                   b->d_eig_a, b->d_eig_w, b->d_eig_work, b->d_eig_info, b->d_scratch,
-                  b->d_rects, b->d_heff_secs, b->d_blas_ws, b->d_emu_part};
+                  b->d_rects, b->d_heff_secs, b->d_mirror, b->d_blas_ws, b->d_emu_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int e = 0; e < 3; ++e) {
@@ -95,6 +95,7 @@ static tgba_status build(const tgba_model* model, const int32_t* sectors, int32_
                          Basis* b) {
   tgba_status r = enumerate_basis(*model, sectors, n_sectors, *trunc, *b);
   if (r != TGBA_OK) return r;
+  find_mirrors(*b);
   TGBA_CUDA(cudaGetDevice(&b->device));
   const int L = b->L, q = b->max_qp;
   const size_t nns = b->ns.E.size(), nr = b->r.E.size();
@@ -135,6 +136,13 @@ static tgba_status build(const tgba_model* model, const int32_t* sectors, int32_
   TGBA_CUDA(cudaMemset(b->d_status, 0, sizeof(unsigned)));
   if ((r = upload_mode_constants(*b)) != TGBA_OK) return r;
   build_rects(*b);
+  std::vector<MirrorPair> mp;
+  for (const SectorSym& y : b->sym)
+    for (int p = 0; p < 2; ++p) {
+      mp.insert(mp.end(), y.even[p].begin(), y.even[p].end());
+      mp.insert(mp.end(), y.odd[p].begin(), y.odd[p].end());
+    }
+  if ((r = upload(&b->d_mirror, mp.data(), mp.size(), &b->upload_bytes)) != TGBA_OK) return r;
   const std::vector<HeffSector> hs = heff_sectors(*b, &b->heff_tiles);
   b->n_heff_secs = (int)hs.size();
   if ((r = upload(&b->d_heff_secs, hs.data(), hs.size(), &b->upload_bytes)) != TGBA_OK) return r;

@@ -180,4 +180,89 @@ tgba_status enumerate_basis(const tgba_model& model, const int32_t* sectors, int
   return TGBA_OK;
 }
 
+// Images of all states under k -> -k.  A mode's image has its excitation energy to the bit, so a
+// state and its image have bitwise equal energies, and runs of equal (M, E) of a sector correspond to
+// those of its partner.  Why P_{a'b'} = P_{ab}: the table entries change sign under k -> -k except
+// those of the R mode at pi (its own image), which gives (-1)^{n/2} (-1)^{#pi}; reversing the order
+// of the NS rows gives (-1)^{M_a/2}, of the R rows other than pi (-1)^{M_b/2} (-1)^{#pi}; the product
+// is +1.
+void find_mirrors(Basis& b) {
+  const int L = b.L, q = b.max_qp;
+  b.sym.assign(b.sectors.size(), SectorSym());
+  b.n_mirror = 0;
+  for (size_t s = 0; s < b.sectors.size(); ++s) {
+    SectorSym& y = b.sym[s];
+    int p = -1;
+    for (size_t t = 0; t < b.sectors.size(); ++t)
+      if (b.sectors[t].m == (L - b.sectors[s].m) % L) p = (int)t;
+    if (p < 0) continue;
+    if (p < (int)s) {                                   // the inverse of the partner's map
+      const SectorSym& z = b.sym[p];
+      if (z.partner != (int)s) continue;
+      for (int par = 0; par < 2; ++par) {
+        y.img[par].resize(z.img[par].size());
+        for (size_t i = 0; i < z.img[par].size(); ++i) y.img[par][z.img[par][i]] = (int32_t)i;
+      }
+      y.partner = p;
+      continue;
+    }
+    bool ok = true;
+    for (int par = 0; par < 2 && ok; ++par) {
+      const StateTable& T = par ? b.r : b.ns;
+      const Sector &A = b.sectors[s], &B = b.sectors[p];
+      const int64_t na = par ? A.n_r : A.n_ns, nb = par ? B.n_r : B.n_ns;
+      const int64_t oa = par ? A.r_off : A.ns_off, ob = par ? B.r_off : B.ns_off;
+      if (na != nb) { ok = false; break; }
+      y.img[par].assign(na, -1);
+      for (int64_t i0 = 0; i0 < na && ok;) {
+        int64_t i1 = i0;                              // the run of equal (M, E), the same range in the partner
+        while (i1 < na && T.M[oa + i1] == T.M[oa + i0] && T.E[oa + i1] == T.E[oa + i0]) ++i1;
+        const int M = T.M[oa + i0];
+        if (T.M[ob + i0] != M || T.M[ob + i1 - 1] != M || T.E[ob + i0] != T.E[oa + i0] ||
+            T.E[ob + i1 - 1] != T.E[oa + i0]) {
+          ok = false;
+          break;
+        }
+        for (int64_t i = i0; i < i1 && ok; ++i) {
+          // the image's modes, ascending: the labels reversed (the R mode at pi stays last)
+          int16_t im[kMaxQp];
+          const int16_t* md = T.modes.data() + (oa + i) * q;
+          const int k = par == 1 && M > 0 && md[M - 1] == L - 1 ? M - 1 : M;
+          for (int u = 0; u < k; ++u) im[u] = (int16_t)((par == 0 ? L - 1 : L - 2) - md[k - 1 - u]);
+          if (k < M) im[k] = (int16_t)(L - 1);
+          int64_t lo = i0, hi = i1;                   // modes ascend within the partner's run
+          while (lo < hi) {
+            const int64_t mid = (lo + hi) / 2;
+            const int16_t* c = T.modes.data() + (ob + mid) * q;
+            if (std::lexicographical_compare(c, c + M, im, im + M)) lo = mid + 1;
+            else hi = mid;
+          }
+          if (lo < i1 && std::equal(im, im + M, T.modes.data() + (ob + lo) * q)) y.img[par][i] = (int32_t)lo;
+          else ok = false;
+        }
+        i0 = i1;
+      }
+    }
+    if (!ok) {
+      y = SectorSym();
+      continue;
+    }
+    y.partner = p;
+    if (p != (int)s) continue;
+    y.split = true;
+    for (int par = 0; par < 2; ++par) {
+      for (size_t i = 0; i < y.img[par].size(); ++i) {
+        const int32_t j = y.img[par][i];
+        if ((int32_t)i > j) continue;
+        y.even[par].push_back(MirrorPair{(int32_t)i, j});
+        if ((int32_t)i != j) y.odd[par].push_back(MirrorPair{(int32_t)i, j});
+      }
+      y.even_off[par] = b.n_mirror;
+      b.n_mirror += (int64_t)y.even[par].size();
+      y.odd_off[par] = b.n_mirror;
+      b.n_mirror += (int64_t)y.odd[par].size();
+    }
+  }
+}
+
 }  // namespace tgba

@@ -135,9 +135,17 @@ tgba_status eig_all_sectors(Basis& b, const double* hx, int n_hx, double* evals,
   int64_t n_max = 0;
   for (const Sector& s : b.sectors) n_max = std::max(n_max, s.n_ns + s.n_r);
   const bool fits = (n_max + 31) / 32 * 32 <= kMaxNativeLd;
+  // a self-mirrored sector is solved as two blocks, so the automatic choice looks at their sizes
+  int64_t blk_max = 0;
+  for (size_t s = 0; s < b.sectors.size(); ++s) {
+    const SectorSym& y = b.sym[s];
+    const bool split = b.x_screen == nullptr && y.split;
+    blk_max = std::max(blk_max, split ? (int64_t)(y.even[0].size() + y.even[1].size()) : b.sectors[s].n_ns + b.sectors[s].n_r);
+  }
+  const bool blocks_fit = (blk_max + 31) / 32 * 32 <= kMaxNativeLd;
   if (method == 1 && !fits)
     return fail(TGBA_EINVAL, "the native eigen-solver takes sectors of at most " + std::to_string(kMaxNativeLd) + " states");
-  if (method == 1 || (method == 0 && fits)) return eig_all_sectors_native(b, hx, n_hx, evals, st);
+  if (method == 1 || (method == 0 && blocks_fit)) return eig_all_sectors_native(b, hx, n_hx, evals, st);
   return eig_all_sectors_lib(b, hx, n_hx, evals, st);
 }
 

@@ -455,9 +455,11 @@ tgba_status upload_mode_constants(Basis& b) {
     v[2 * i + 1] = (double)(x - (ld)v[2 * i]);
   };
   const ld e_pi = 2 * (1 - h);
+  std::vector<ld> sn(n2 + 1);                       // sin(pi m / (2L)), symmetric about m = L
+  for (int m = 0; m <= L; ++m) sn[m] = sn[n2 - m] = std::sin(pi * m / (2 * (ld)L));
   for (int a = 0; a < n2; ++a) {
     const int n = a < L ? -(L - 1) + 2 * (L - 1 - a) : -(L - 2) + 2 * (a - L);
-    const ld c = std::cos(pi * n / (2 * (ld)L));
+    const ld c = sn[L - (n < 0 ? -n : n)];          // cos(k / 2), k = pi n / L
     if (n == L) {
       put(a, e_pi);
       put(n2 + a, 2 * e_pi);
@@ -468,7 +470,7 @@ tgba_status upload_mode_constants(Basis& b) {
       put(n2 + a, e_pi < 0 ? 16 * h * c * c / (e - e_pi) : e + e_pi);
     }
   }
-  for (int m = 0; m <= n2; ++m) put(2 * n2 + m, std::sin(pi * m / (2 * (ld)L)));
+  for (int m = 0; m <= n2; ++m) put(2 * n2 + m, sn[m]);
   put(3 * n2 + 1, 4 * std::sqrt(h));
   put(3 * n2 + 2, (1 + h) / 4);
   TGBA_CUDA(cudaMalloc((void**)&b.d_const, v.size() * sizeof(double)));

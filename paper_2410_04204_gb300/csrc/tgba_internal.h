@@ -45,6 +45,26 @@ struct StateTable {
   std::vector<int16_t> modes;      // [state][max_qp], ascending mode indices, -1 padded
 };
 
+// A state and its mirror image (all momenta reversed) in a sector that the reflection maps to
+// itself (m = 0 or L/2): indices within the sector's states of one parity; equal for a state that
+// is its own image.
+struct MirrorPair { int32_t a, b; };
+
+// Reflection symmetry of the chain.  In the real gauge the elements satisfy P_{a'b'} = P_{ab} for the
+// images a', b' (every sign of the table under k -> -k cancels for even M, see basis.cpp), and a
+// state and its image have the same energy.  So sector L - m has the spectrum of sector m, and H~ of
+// a self-mirrored sector splits into the blocks of the even and the odd combinations
+// (a +- a')/sqrt 2.  Truncations by energy or quasiparticle number are closed under the
+// reflection; a cap on the number of states may not be (then nothing is used).
+struct SectorSym {
+  int partner = -1;                 // sector index of L - m when present and its states are the images
+  bool split = false;               // partner == itself: the even/odd lists below
+  std::vector<int32_t> img[2];      // image of every state (index in the partner), per parity
+  std::vector<MirrorPair> even[2];  // one entry per self-image or pair, in the states' order
+  std::vector<MirrorPair> odd[2];   // the pairs
+  int64_t even_off[2] = {0, 0}, odd_off[2] = {0, 0};   // their places in d_mirror
+};
+
 // Work of the element stage: a rectangle of pairs with uniform (M_a, M_b), laid out row-major
 // (row = NS state, column = R state), cut into tiles (elements.cu: x_tiles).
 struct Rect {
@@ -78,6 +98,7 @@ struct Basis;
 // basis.cpp
 tgba_status enumerate_basis(const tgba_model& model, const int32_t* sectors, int n_sectors,
                             const tgba_trunc& tr, Basis& b);
+void find_mirrors(Basis& b);
 
 struct Basis {
   int L = 0;
@@ -88,6 +109,9 @@ struct Basis {
   double e_ns_vac = 0;             // NS vacuum energy (in units of J)
   std::vector<Sector> sectors;
   StateTable ns, r;
+  std::vector<SectorSym> sym;      // per sector
+  MirrorPair* d_mirror = nullptr;  // the even and odd lists of the split sectors
+  int64_t n_mirror = 0;
   int64_t n_elements = 0, n_heff = 0, n_states = 0;
   int max_n = 0;                   // largest M_a + M_b in the basis
 

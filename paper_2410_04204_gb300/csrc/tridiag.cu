@@ -69,8 +69,24 @@ struct TriSlot {
   int64_t tk_off;   // the matrix's step tickets (one counter per step) in the counter array
   int64_t p_off;    // p = tau A v [ld], then one dot partial per CTA of the group [16]
   int64_t de_off;   // diagonal d [n], off-diagonal e [n]
-  int64_t out_off;  // first eigenvalue in the caller's output
+  int64_t out_off;  // first eigenvalue in the workspace's list (merge_evals brings them to the caller)
   int32_t n, ld;
+};
+
+// What a slot's matrix holds: H~ of a (field, sector), whole (ns = r = nullptr) or the block of the
+// even (sgn = 1) or odd (sgn = -1) combinations of mirror images listed in ns and r.
+struct FillSlot {
+  const MirrorPair* ns;
+  const MirrorPair* r;
+  const double *E_ns, *E_r, *P;   // the sector's energies and X block
+  double scale, sgn;
+  int64_t n_r, kn;                // row stride of P; NS entries of the matrix
+};
+
+// One output (field, sector): the eigenvalues of one block, or of two merged.
+struct MergeJob {
+  int64_t out, a, b;
+  int32_t na, nb;
 };
 
 __device__ __forceinline__ double isel(bool s, double y, double x) {   // s ? y : x, integer halves
@@ -798,27 +814,96 @@ sturm_bisect(const TriSlot* __restrict__ slots, const int2* __restrict__ items, 
   }
 }
 
-// Real-gauge H~ of one (field, sector) slot, full symmetric, ld x ld in 32 x 16 tiles (see
-// blk_off); padding rows and columns n .. ld - 1 are zero.  Consecutive threads write
-// consecutive doubles of the tiled array.
-__global__ void fill_sym(int64_t kn, int64_t kr, int ld, const double* __restrict__ E_ns,
-                         const double* __restrict__ E_r, const double* __restrict__ Pm,
-                         const double* __restrict__ c0, double scale, double* __restrict__ A) {
-  const int64_t n = kn + kr;
-  const int LB = ld >> 5;
-  const double c = scale * sqrt(c0[0] * c0[0] + c0[1] * c0[1]);
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < (int64_t)ld * ld;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t blk = idx >> 9, in = idx & 511;
-    const int64_t g = blk / LB, rb = blk - g * LB;
-    const int64_t row = rb * 32 + (in & 31), col = g * 16 + (in >> 5);
-    double v = 0.0;
-    if (row < n && col < n) {
-      if (row == col) v = row < kn ? E_ns[row] : E_r[row - kn];
-      else if (row < kn && col >= kn) v = c * Pm[row * kr + (col - kn)];
-      else if (row >= kn && col < kn) v = c * Pm[col * kr + (row - kn)];
+// The lower triangle of every slot's matrix (blocks on and below the diagonal, see blk_off; rows
+// and columns n .. ld - 1 zero), all slots in one launch: a warp writes 32 x 16 blocks down a column
+// group, a lane per row, so both the tiled stores and the reads of P's rows are coalesced.  Between
+// combinations of mirror images, with x = (a, a'), y = (b, b'): P_ab for two self-images, sqrt 2 P_ab
+// for a self-image and a pair, P_ab +- P_ab' for two pairs.  Writing every block of the square, one
+// launch per matrix and a 64-bit division per entry, took 2.6 ms for the 48 matrices of the L = 24 workload.
+__device__ __forceinline__ double coupling(const FillSlot& f, int64_t x, int64_t y) {   // NS entry x, R entry y
+  if (f.ns == nullptr) return f.P[x * f.n_r + y];
+  const MirrorPair p = f.ns[x], q = f.r[y];
+  const double* row = f.P + (int64_t)p.a * f.n_r;
+  const double v = row[q.a];
+  if (p.a == p.b) return q.a == q.b ? v : M_SQRT2 * v;
+  if (q.a == q.b) return M_SQRT2 * v;
+  return fma(f.sgn, row[q.b], v);
+}
+
+__global__ void __launch_bounds__(256) fill_lower(const TriSlot* __restrict__ slots, const FillSlot* __restrict__ fill,
+                                                  const double* __restrict__ c0, double* __restrict__ ws) {
+  const TriSlot S = slots[blockIdx.y];
+  const int LB = S.ld >> 5, G = S.ld / kCols, lane = threadIdx.x & 31;
+  const FillSlot f = fill[blockIdx.y];
+  const double c = f.scale * sqrt(c0[0] * c0[0] + c0[1] * c0[1]);
+  const int kn = (int)f.kn;
+  double* A = ws + S.a_off;
+  for (int g = blockIdx.x; g < G; g += gridDim.x)
+    for (int rb = (g >> 1) + (threadIdx.x >> 5); rb < LB; rb += 8) {
+      const int row = 32 * rb + lane;
+      double* out = A + blk_off(g, rb, LB) + lane;
+#pragma unroll 4
+      for (int kk = 0; kk < kCols; ++kk) {
+        const int col = kCols * g + kk;
+        double v = 0.0;
+        if (row < S.n && col < S.n) {
+          if (row == col) {
+            const int64_t x = row < kn ? row : row - kn;
+            const int64_t i = f.ns == nullptr ? x : (row < kn ? f.ns[x].a : f.r[x].a);
+            v = row < kn ? f.E_ns[i] : f.E_r[i];
+          } else if (row >= kn && col < kn) {
+            v = c * coupling(f, col, row - kn);
+          } else if (row < kn && col >= kn) {            // above the diagonal, in a diagonal block
+            v = c * coupling(f, row, col - kn);
+          }
+        }
+        out[32 * kk] = v;
+      }
     }
-    A[idx] = v;
+}
+
+// The caller's eigenvalues of one (field, sector) per block: list a, or lists a and b merged (each
+// ascending; made monotone first, because neighbours of a near-degenerate pair may come out of the
+// bisection a rounding apart in the other order).  An entry's place is its index plus the number of
+// entries of the other list before it (ties: list a first).
+__device__ void make_monotone(double* v, int n, double* part) {
+  const int T = blockDim.x, per = (n + T - 1) / T, i0 = min(n, (int)threadIdx.x * per), i1 = min(n, i0 + per);
+  double m = -INFINITY;
+  for (int i = i0; i < i1; ++i) m = fmax(m, v[i]);
+  part[threadIdx.x] = m;
+  __syncthreads();
+  m = -INFINITY;
+  for (int t = 0; t < (int)threadIdx.x; ++t) m = fmax(m, part[t]);
+  for (int i = i0; i < i1; ++i) {
+    if (v[i] < m) v[i] = m;
+    else if (v[i] > m) m = v[i];
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(256) merge_evals(const MergeJob* __restrict__ jobs, double* __restrict__ list,
+                                                   double* __restrict__ evals) {
+  __shared__ double part[256];
+  const MergeJob j = jobs[blockIdx.x];
+  double *a = list + j.a, *b = list + j.b, *out = evals + j.out;
+  if (j.nb == 0) {
+    for (int i = threadIdx.x; i < j.na; i += blockDim.x) out[i] = a[i];
+    return;
+  }
+  make_monotone(a, j.na, part);
+  make_monotone(b, j.nb, part);
+  for (int i = threadIdx.x; i < j.na + j.nb; i += blockDim.x) {
+    const bool first = i < j.na;
+    const int k = first ? i : i - j.na;
+    const double v = first ? a[k] : b[k];
+    const double* o = first ? b : a;
+    int lo = 0, hi = first ? j.nb : j.na;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (first ? o[mid] < v : o[mid] <= v) lo = mid + 1;
+      else hi = mid;
+    }
+    out[k + lo] = v;
   }
 }
 
@@ -836,28 +921,74 @@ int64_t max_chunks(int ld) {
 
 tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double* evals, cudaStream_t st,
                                    const WaitCheck* check) {
+  // The matrices to solve.  With the elements as they are (not screened, which breaks the reflection
+  // symmetry), a sector whose mirror sector comes earlier takes that one's eigenvalues, and a
+  // self-mirrored sector is solved as its even and its odd block: for the 24 sectors of the L = 24
+  // workload 11 whole sectors and 4 blocks of half the size instead of 24 sectors (table, elements
+  // and both fields' eigenvalues 514 -> 274 ms); the k = 0 sector of L = 40 with 2697 states as two
+  // blocks 345 -> 85 ms.
   std::vector<TriSlot> slots;
-  std::vector<std::pair<int, int>> who;     // (field, sector)
-  int64_t total = 0, tk_total = 0;
+  std::vector<FillSlot> fills;
+  std::vector<MergeJob> jobs;
+  int64_t total = 0, tk_total = 0, ev_total = 0;
   int n_max = 0;
-  for (int h = 0; h < n_hx; ++h)
-    for (size_t s = 0; s < b.sectors.size(); ++s) {
-      const int64_t n = b.sectors[s].n_ns + b.sectors[s].n_r;
-      if (n == 0) continue;
-      TriSlot t{};
-      t.n = (int32_t)n;
-      t.ld = (int32_t)round32(n);
-      t.out_off = (int64_t)h * b.n_states + b.sectors[s].ev_off;
-      t.a_off = total;            total += round32((int64_t)t.ld * t.ld);
-      t.rp_off = total;           total += round32((int64_t)(t.ld / kCols) * t.ld);
-      t.cp_off = total;           total += round32((int64_t)kCols * max_chunks(t.ld));
-      t.tk_off = tk_total;        tk_total += t.ld;
-      t.p_off = total;            total += round32(t.ld + kMaxGroup);
-      t.de_off = total;           total += round32(2 * n);
-      slots.push_back(t);
-      who.emplace_back(h, (int)s);
-      n_max = std::max(n_max, (int)n);
+  // (A withheld CTA is named by its (field, sector) matrix: then every sector is solved whole.)
+  const bool symmetric = b.x_screen == nullptr && (check == nullptr || check->withhold_matrix < 0);
+  auto add = [&](int h, int s, int kind) {        // kind 0: the whole sector, 1: even, 2: odd block
+    const Sector& sec = b.sectors[s];
+    const SectorSym& y = b.sym[s];
+    FillSlot f{nullptr, nullptr, b.d_E_ns + sec.ns_off, b.d_E_r + sec.r_off, b.d_P + sec.x_off, -b.L * hx[h], 1.0,
+               sec.n_r, sec.n_ns};
+    int64_t n = sec.n_ns + sec.n_r;
+    if (kind > 0) {
+      const bool even = kind == 1;
+      f.ns = b.d_mirror + (even ? y.even_off[0] : y.odd_off[0]);
+      f.r = b.d_mirror + (even ? y.even_off[1] : y.odd_off[1]);
+      f.sgn = even ? 1.0 : -1.0;
+      f.kn = (int64_t)(even ? y.even[0] : y.odd[0]).size();
+      n = f.kn + (int64_t)(even ? y.even[1] : y.odd[1]).size();
     }
+    if (n == 0) return (int64_t)0;
+    TriSlot t{};
+    t.n = (int32_t)n;
+    t.ld = (int32_t)round32(n);
+    t.out_off = ev_total;       ev_total += n;
+    t.a_off = total;            total += round32((int64_t)t.ld * t.ld);
+    t.rp_off = total;           total += round32((int64_t)(t.ld / kCols) * t.ld);
+    t.cp_off = total;           total += round32((int64_t)kCols * max_chunks(t.ld));
+    t.tk_off = tk_total;        tk_total += t.ld;
+    t.p_off = total;            total += round32(t.ld + kMaxGroup);
+    t.de_off = total;           total += round32(2 * n);
+    slots.push_back(t);
+    fills.push_back(f);
+    n_max = std::max(n_max, (int)n);
+    return n;
+  };
+  for (int h = 0; h < n_hx; ++h) {
+    std::vector<int> job_of(b.sectors.size(), -1);
+    for (size_t s = 0; s < b.sectors.size(); ++s) {
+      const Sector& sec = b.sectors[s];
+      if (sec.n_ns + sec.n_r == 0) continue;
+      const int64_t out = (int64_t)h * b.n_states + sec.ev_off;
+      const int p = symmetric ? b.sym[s].partner : -1;
+      if (p >= 0 && p < (int)s) {
+        MergeJob j = jobs[job_of[p]];
+        j.out = out;
+        jobs.push_back(j);
+        continue;
+      }
+      MergeJob j{out, ev_total, 0, 0, 0};
+      if (p == (int)s && b.sym[s].split) {
+        j.na = (int32_t)add(h, (int)s, 1);
+        j.b = ev_total;
+        j.nb = (int32_t)add(h, (int)s, 2);
+      } else {
+        j.na = (int32_t)add(h, (int)s, 0);
+      }
+      job_of[s] = (int)jobs.size();
+      jobs.push_back(j);
+    }
+  }
   if (slots.empty()) return TGBA_OK;
   const int B = (int)slots.size();
   int ld_max = 0;
@@ -929,7 +1060,9 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
     sm_map.resize(grid);
     for (int d = 0; d < sms; ++d) { sm_map[2 * d] = map[hi[d]]; sm_map[2 * d + 1] = map[lo[d]]; }
   }
-  const int64_t slot_doubles = round32(((int64_t)B * sizeof(TriSlot) + 7) / 8);
+  const int64_t ev_off = total;
+  total += round32(ev_total);
+  const int64_t slot_doubles = round32(((int64_t)B * (sizeof(TriSlot) + sizeof(FillSlot)) + jobs.size() * sizeof(MergeJob) + 7) / 8);
   const int64_t map_doubles = round32(((int64_t)2 * grid * sizeof(CtaWork) + 7) / 8);   // by block, by SM
   // bisection items: item_len consecutive eigenvalue indices of one matrix, 64 (a block's
   // threads) unless that gives fewer items than resident blocks, then 32.  (Items sized to fill
@@ -961,7 +1094,11 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   TriSlot* d_slots = (TriSlot*)(ws + total);
   CtaWork* d_map = (CtaWork*)(ws + total + slot_doubles);
   unsigned* d_cnt = (unsigned*)(ws + total + slot_doubles + map_doubles);
+  FillSlot* d_fill = (FillSlot*)(d_slots + B);
+  MergeJob* d_jobs = (MergeJob*)(d_fill + B);
   TGBA_CUDA(cudaMemcpyAsync(d_slots, slots.data(), B * sizeof(TriSlot), cudaMemcpyHostToDevice, st));
+  TGBA_CUDA(cudaMemcpyAsync(d_fill, fills.data(), B * sizeof(FillSlot), cudaMemcpyHostToDevice, st));
+  TGBA_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(MergeJob), cudaMemcpyHostToDevice, st));
   TGBA_CUDA(cudaMemcpyAsync(d_map, map.data(), grid * sizeof(CtaWork), cudaMemcpyHostToDevice, st));
   CtaWork* d_sm_map = nullptr;
   if (!sm_map.empty()) {
@@ -973,15 +1110,10 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   int2* d_items = (int2*)(ws + total + slot_doubles + map_doubles + cnt_doubles);
   TGBA_CUDA(cudaMemcpyAsync(d_items, items.data(), n_items * sizeof(int2), cudaMemcpyHostToDevice, st));
   TGBA_CUDA(cudaMemsetAsync(d_cnt, 0, n_cnt * sizeof(unsigned), st));
-  for (int q = 0; q < B; ++q) {
-    const Sector& sec = b.sectors[who[q].second];
-    const int64_t work = (int64_t)slots[q].ld * slots[q].ld;
-    const int fgrid = (int)std::min<int64_t>((work + 255) / 256, 152 * 16);
-    fill_sym<<<fgrid, 256, 0, st>>>(sec.n_ns, sec.n_r, slots[q].ld, b.d_E_ns + sec.ns_off, b.d_E_r + sec.r_off,
-                                    b.d_P + sec.x_off, b.d_c0, -b.L * hx[who[q].first], ws + slots[q].a_off);
-    TGBA_CUDA(cudaGetLastError());
-    ++b.launches;
-  }
+  fill_lower<<<dim3((unsigned)std::min(ld_max / kCols, std::max(1, 152 * 8 / B + 1)), (unsigned)B), 256, 0, st>>>(
+      d_slots, d_fill, b.d_c0, ws);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(per_sm == 2 ? 6 * 32 : 12 * 32);
@@ -1017,11 +1149,13 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   ++b.launches;
   TGBA_CUDA(cudaEventRecord(b.eig_ev[1], st));
   const int bis_grid = std::min(n_items, bis_per_sm * sms);
-  sturm_bisect<<<bis_grid, kSturmThreads, smem2, st>>>(d_slots, d_items, n_items, item_len, d_queue, ws, evals,
-                                                       b.d_status);
+  sturm_bisect<<<bis_grid, kSturmThreads, smem2, st>>>(d_slots, d_items, n_items, item_len, d_queue, ws,
+                                                       ws + ev_off, b.d_status);
   TGBA_CUDA(cudaGetLastError());
-  ++b.launches;
   TGBA_CUDA(cudaEventRecord(b.eig_ev[2], st));
+  merge_evals<<<(unsigned)jobs.size(), 256, 0, st>>>(d_jobs, ws + ev_off, evals);
+  TGBA_CUDA(cudaGetLastError());
+  b.launches += 2;
   b.eig_ev_recorded = true;
   double flops = 0;
   for (const TriSlot& t : slots)

@@ -1,0 +1,47 @@
+"""Eigenvalues through the reflection symmetry (mirror sectors shared, self-mirrored sectors as even and
+odd blocks) against the library solver, which takes every sector whole: all combinations of sectors
+present, truncations that are and are not closed under the reflection, one block empty."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2410_04204_gb300 import tgba
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+@pytest.mark.parametrize("L,h,sectors,mq,cut,cap", [
+    (14, 1.0, list(range(14)), 6, -1.0, 0),        # everything
+    (14, 0.7, [11, 0, 3, 7, 5], 6, -1.0, 0),       # a pair out of order, both self-mirrored, one alone
+    (16, 1.3, [8, 0], 6, -1.0, 0),
+    (16, 1.0, [0, 1, 15, 8], 8, -1.0, 101),        # capped: not closed under the reflection in general
+    (24, 1.0, [12, 6, 18], 6, 9.5, 0),
+    (12, 1.0, [0], 0, -1.0, 0),                    # the two vacua: no odd block
+    (10, 1.5, [0, 5], 4, 0.5, 0),                  # one state; an empty sector
+    (60, 1.0, [0, 59, 1], 6, 4.6, 0),
+])
+def test_against_whole_sectors(L, h, sectors, mq, cut, cap):
+    fields = [0.0, 0.13, -0.4]
+    b = tgba.tgba_build_basis(L, h, sectors, mq, cut, cap)
+    try:
+        tgba.tgba_compute_x(b)
+        n = sum(x + y for x, y in tgba.tgba_sector_sizes(b))
+        ev = [torch.full((len(fields) * n,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(3)]
+        for m in range(3):
+            tgba.tgba_eigvals(b, fields, ev[m], method=m)
+        ref = ev[2].cpu().numpy()
+        off = np.concatenate([[0], np.cumsum([x + y for x, y in tgba.tgba_sector_sizes(b)] * len(fields))])
+        for m in (0, 1):
+            got = ev[m].cpu().numpy()
+            assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max() * max(1, n) ** 0.5
+            for i, j in zip(off[:-1], off[1:]):
+                assert np.all(np.diff(got[i:j]) >= -1e-13 * np.abs(ref).max())
+    finally:
+        tgba.tgba_basis_free(b)
