@@ -11,10 +11,12 @@
 // and because sigma^x_1 is the off-diagonal part of H_eff, X~ = (D - H~)/(L h_x), so the
 // magnetisation needs only moments weighted by the diagonal:
 //   B^H X~ B = ( B^H (D - E_c) B - c~0^H (H~ - E_c) c~0 ) / (L h_x),
-//   B^H (D - E_c) B = sum_kl a_k a_l Re(i^{k-l} v_k^H (D - E_c) v_l),  a_k = (2 - d_k0) J_k(R t),
-//   c~0^H (H~ - E_c) c~0 = R Re(v_0^H v_1)      (the energy is conserved),
-// and <sigma^x>(t) = B^H X~ B / ||c0||^2.  The moments take 6 K^2 chi flops per variant instead
-// of the 2 chi^2 K of v_k^H X~ v_l.  Absolute error of <sigma^x>: about K eps R / (L |h_x|).
+//   B^H (D - E_c) B = sum_kl a_k a_l Re(i^{k-l} v_k^T (D - E_c) v_l),  a_k = (2 - d_k0) J_k(R t),
+//   c~0^T (H~ - E_c) c~0 = R v_0^T v_1          (the energy is conserved),
+// and <sigma^x>(t) = B^H X~ B / ||c0||^2.  c~0 is real (the vacuum elements C0 are real, see
+// elements.cu), so the v_k are real and only moments with k - l even contribute, with the sign
+// (-1)^{(k-l)/2}: the moments split into those of the even and of the odd k and take K^2 chi / 2
+// flops per variant.  Absolute error of <sigma^x>: about K eps R / (L |h_x|).
 //
 // The interval [E_c - R, E_c + R] comes from Lanczos: 64 steps on the union of the kept states
 // (the largest variant) for each distinct h_x give the extreme Ritz values, widened by 2%; by
@@ -23,8 +25,7 @@
 // like cosh(K acosh|x|); if the check fails the propagation is redone with Gershgorin bounds.
 //
 // Layout: all variants' vectors side by side on the union of the kept states (NS rows, then R
-// rows), two real columns (Re, Im of c~0's propagation) per variant, variants ordered by
-// decreasing kept set; entries outside a variant's set stay 0.  Every FP64 product (the
+// rows), one real column per variant, variants ordered by decreasing kept set; entries outside a variant's set stay 0.  Every FP64 product (the
 // off-diagonal blocks in each step, the Lanczos steps and the moments) runs on the tensor cores
 // through the sliced products of dgemm_tc.cu: Q is sliced once in both orientations, each
 // step slices the current vectors, and the output tiles of each step skip the (row block,
@@ -153,13 +154,13 @@ __device__ __forceinline__ bool kept(int64_t row, int64_t kn_max, const ColPrm& 
   return row < kn_max ? row < p.kn : row - kn_max < p.kr;
 }
 
-// v_0: column 2j = Re c~0, 2j + 1 = Im c~0 on the kept rows of its variant
+// v_0: c~0 (real; stored as complex) on the kept rows of each column's variant
 __global__ void cheb_init(int64_t n, int64_t kn_max, int cols, const ColPrm* __restrict__ prm,
                           const double* __restrict__ c, double* __restrict__ V) {
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n * cols; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t row = q % n;
     const int col = (int)(q / n);
-    V[q] = kept(row, kn_max, prm[col]) ? c[2 * row + (col & 1)] : 0.0;
+    V[q] = kept(row, kn_max, prm[col]) ? c[2 * row] : 0.0;
   }
 }
 
@@ -201,32 +202,21 @@ __global__ void kept_energy(int64_t kn, int64_t kr, int64_t kn_max, const double
     out[i] = i < kn ? E[i] : E[kn_max + (i - kn)];
 }
 
-// Re(v_0^H v_1) of one variant (columns c, c + 1 of v_0 and of v_1)
+// v_0^T v_1 of one variant
 __global__ void cheb_dot01(int64_t n, const double* __restrict__ v0, const double* __restrict__ v1, double* __restrict__ out) {
   __shared__ double sh[32];
   double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s = fma(v0[i], v1[i], fma(v0[n + i], v1[n + i], s));
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s = fma(v0[i], v1[i], s);
   s = block_reduce(s, sh);
   if (threadIdx.x == 0) *out = s;
 }
 
-// Gamma_kl = Re(i^{k-l} mu_kl), mu = (G_rr + G_ii) + i (G_ri - G_ri^T), G column-major K1 x K1;
-// G_rr and G_ii are symmetric and only their lower triangle (row >= column) is computed
-__global__ void cheb_gamma(int K1, const double* __restrict__ Grr, const double* __restrict__ Gii,
-                           const double* __restrict__ Gri, double* __restrict__ Gam) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)K1 * K1; q += (int64_t)gridDim.x * blockDim.x) {
-    const int l = (int)(q / K1), k = (int)(q % K1);
-    const int64_t kl = (int64_t)l * K1 + k, lk = (int64_t)k * K1 + l;
-    const int64_t low = k >= l ? kl : lk;
-    const double re = Grr[low] + Gii[low], im = Gri[kl] - Gri[lk];
-    double g;
-    switch (((k - l) % 4 + 4) % 4) {
-      case 0: g = re; break;
-      case 1: g = -im; break;
-      case 2: g = -re; break;
-      default: g = im; break;
-    }
-    Gam[kl] = g;
+// The whole of a symmetric matrix (column-major k x k) of which the tiles on or below the diagonal
+// (row >= column) were computed
+__global__ void symmetrise(int k, double* __restrict__ G) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)k * k; q += (int64_t)gridDim.x * blockDim.x) {
+    const int c = (int)(q / k), r = (int)(q % k);
+    if (r < c) G[q] = G[(int64_t)r * k + c];
   }
 }
 
@@ -237,7 +227,8 @@ __global__ void cheb_gamma(int K1, const double* __restrict__ Grr, const double*
 // in the recurrence).  When the unnormalised values pass 1e250 the recurrence is rescaled by
 // 1e-250 without touching the values already stored: an entry stored before one rescaling
 // gets the factor 1e-250 at the end, one stored before two or more is below 1e-236 of the
-// result and becomes 0, so only the positions of the last two rescalings are kept.
+// result and becomes 0, so only the positions of the last two rescalings are kept.  The sign
+// (-1)^{floor(k/2)} of the moments is put into a_k.
 __global__ void cheb_bessel(int n_t, int t0, double dt, double R, int K, int m_start, double* __restrict__ out) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n_t) return;
@@ -270,21 +261,27 @@ __global__ void cheb_bessel(int n_t, int t0, double dt, double R, int K, int m_s
   const double inv = 1.0 / norm;
   for (int q = 0; q <= K; ++q) {
     const double f = (q + 1 >= k_prev) ? 0.0 : (q + 1 >= k_last ? 1e-250 : 1.0);
-    a[q * S] *= (q == 0 ? inv : 2.0 * inv) * f;
+    const double w = (q == 0 ? inv : 2.0 * inv) * f;
+    a[q * S] *= (q & 2) ? -w : w;
   }
 }
 
-// mx[t] = (a(t)^T Gamma a(t) - e_shift) * scale, one warp per time (A = a [k][t], GA = Gamma a
-// precomputed, [t][k])
-__global__ void cheb_mx(int K1, int cnt, const double* __restrict__ A, const double* __restrict__ GA, double e_shift,
-                        double scale, double* __restrict__ mx) {
+// mx[t] = (a(t)^T Gamma a(t) - R v_0^T v_1) * scale, one warp per time (A = a [k][t]; Gamma a of the
+// even k in G0, of the odd k in G1, both [t][k / 2])
+__global__ void cheb_mx(int K1, int cnt, const double* __restrict__ A, const double* __restrict__ G0,
+                        const double* __restrict__ G1, const double* __restrict__ d01, double R, double scale,
+                        double* __restrict__ mx) {
   const int lane = threadIdx.x & 31;
   const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (col >= cnt) return;
+  const int n0 = (K1 + 1) / 2, n1 = K1 / 2;
   double acc = 0.0;
-  for (int k = lane; k < K1; k += 32) acc = fma(A[(int64_t)k * cnt + col], GA[(int64_t)col * K1 + k], acc);
+  for (int k = lane; k < K1; k += 32) {
+    const double g = (k & 1) ? G1[(int64_t)col * n1 + k / 2] : G0[(int64_t)col * n0 + k / 2];
+    acc = fma(A[(int64_t)k * cnt + col], g, acc);
+  }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) mx[col] = (acc - e_shift) * scale;
+  if (lane == 0) mx[col] = (acc - R * *d01) * scale;
 }
 
 int blocks_for(int64_t work) {
@@ -511,21 +508,20 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     }
     return TGBA_OK;
   };
-  // ---- columns: variants by decreasing kept set, Re and Im of each, padded to a tile multiple
+  // ---- columns: variants by decreasing kept set, padded to a tile multiple
   std::vector<int> ord(vars.size());
   for (size_t i = 0; i < vars.size(); ++i) ord[i] = (int)i;
   std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) {
     return vars[x].kn != vars[y].kn ? vars[x].kn > vars[y].kn : vars[x].kr > vars[y].kr;
   });
-  const int ncol = 2 * (int)vars.size();
-  const int ncolp = (ncol + TC - 1) / TC * TC;
+  const int ncol = (int)vars.size();
+  const int ncolp = (int)r16(ncol);
   std::vector<int64_t> out_ns(ncolp, 0), out_r(ncolp, 0), k_ns(ncolp, 0), k_r(ncolp, 0);
-  for (int j = 0; j < (int)ord.size(); ++j)
-    for (int h = 0; h < 2; ++h) {
-      const ChebVariant& v = vars[ord[j]];
-      out_ns[2 * j + h] = v.kn; k_ns[2 * j + h] = v.kr;
-      out_r[2 * j + h] = v.kr; k_r[2 * j + h] = v.kn;
-    }
+  for (int j = 0; j < ncol; ++j) {
+    const ChebVariant& v = vars[ord[j]];
+    out_ns[j] = v.kn; k_ns[j] = v.kr;
+    out_r[j] = v.kr; k_r[j] = v.kn;
+  }
   std::vector<EmuTile> tn = product_tiles(kn_max, ncolp, out_ns, k_ns), tr = product_tiles(kr_max, ncolp, out_r, k_r);
   const int64_t cn = emu_number_tiles(tn), cr_ = emu_number_tiles(tr);
   if (cn < 0 || cr_ < 0) return fail(TGBA_EINVAL, "quench product tiles");
@@ -573,7 +569,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     std::vector<ColPrm> hp(ncolp, ColPrm{0.0, 0.0, 0.0, 0, 0});
     for (int j = 0; j < (int)ord.size(); ++j) {
       const int v = ord[j];
-      for (int h = 0; h < 2; ++h) hp[2 * j + h] = ColPrm{-b.L * vars[v].hx * cabs, ec[v], 1.0 / R[v], vars[v].kn, vars[v].kr};
+      hp[j] = ColPrm{-b.L * vars[v].hx * cabs, ec[v], 1.0 / R[v], vars[v].kn, vars[v].kr};
     }
     TGBA_CUDA(cudaMemcpyAsync(prm, hp.data(), ncolp * sizeof(ColPrm), cudaMemcpyHostToDevice, st));
     if (!tn.empty()) TGBA_CUDA(cudaMemcpyAsync(dtl, tn.data(), tn.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
@@ -623,7 +619,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     b.q_ev_recorded = true;
     b.launches += graph_launches;
     b.quench_flops = 0;
-    for (const ChebVariant& v : vars) b.quench_flops += 8.0 * (double)K * (double)v.kn * (double)v.kr;
+    for (const ChebVariant& v : vars) b.quench_flops += 4.0 * (double)K * (double)v.kn * (double)v.kr;
     // the interval check: ||v_K|| <= ||v_0|| for every column
     cheb_norms<<<ncolp, kRedThreads, 0, st>>>(n_un, V, V + (size_t)K * S, nrm);
     TGBA_CUDA(cudaGetLastError());
@@ -643,8 +639,8 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     }
     // ---- moments and <sigma^x>(t), one variant at a time, with the variant's own number of
     // terms K_v <= K (the other columns' longer expansions cost it nothing): the Gram matrices
-    // of its first K_v + 1 vectors and the Bessel sums over the whole time grid are tensor-core
-    // FP64 products as well
+    // of its even and of its odd vectors up to K_v and the Bessel sums over the whole time grid are
+    // tensor-core FP64 products as well.  Nothing waits for the host between the variants.
     int64_t chi_max = 0;
     for (const ChebVariant& v : vars) chi_max = std::max<int64_t>(chi_max, v.kn + v.kr);
     std::vector<int> Kv(vars.size());
@@ -652,34 +648,26 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       const double xmax = R[v] * t_max;
       Kv[v] = std::min(K, (int)std::ceil(xmax + 10.0 * std::cbrt(xmax) + 30.0));
     }
-    const int64_t nt = std::max(1, dt_n);
-    const size_t sa = std::max(emu_operand_elems(K1, (int)chi_max, TR), emu_operand_elems(K1, K1, TR));
-    const size_t sb = std::max(emu_operand_elems(K1, (int)chi_max, TC), emu_operand_elems((int)nt, K1, TC));
-    const size_t n_tiles_max = (size_t)((K1 + TR - 1) / TR) * (size_t)std::max<int64_t>((K1 + TC - 1) / TC, (nt + TC - 1) / TC);
+    const int64_t nt = std::max(1, dt_n), KH = (K1 + 1) / 2;
+    const size_t sa = std::max(emu_operand_elems((int)KH, (int)chi_max, TR), emu_operand_elems((int)KH, (int)KH, TR));
+    const size_t sb = std::max(emu_operand_elems((int)KH, (int)chi_max, TC), emu_operand_elems((int)nt, (int)KH, TC));
+    const size_t n_tiles_max = (size_t)((KH + TR - 1) / TR) * (size_t)std::max<int64_t>((KH + TC - 1) / TC, (nt + TC - 1) / TC);
     DevBuf mbuf(st);
-    const size_t mdoubles = 4 * (size_t)K1 * K1 + 2 * (size_t)K1 * nt + chi_max + 8;
-    TGBA_CUDA(cudaMallocAsync(&mbuf.p, mdoubles * 8 + (2 * sa + 2 * sb) * 2 + 4 * ((size_t)K1 + nt) * 4 +
-                                           2 * n_tiles_max * sizeof(EmuTile) + 1024, st));
-    double* Grr = (double*)mbuf.p;
-    double* Gii = Grr + (size_t)K1 * K1;
-    double* Gri = Gii + (size_t)K1 * K1;
-    double* Gam = Gri + (size_t)K1 * K1;
-    double* Ab = Gam + (size_t)K1 * K1;                   // a_k(t): [K_v + 1][t]
-    double* GA = Ab + (size_t)K1 * nt;                    // Gamma a(t): column-major (K_v + 1) x n_t
-    double* Ek = GA + (size_t)K1 * nt;
+    const size_t mdoubles = (size_t)KH * KH + (size_t)K1 * nt + 2 * (size_t)KH * nt + chi_max + 8;
+    TGBA_CUDA(cudaMallocAsync(&mbuf.p, mdoubles * 8 + (sa + sb) * 2 + 2 * ((size_t)KH + nt) * 4 +
+                                           n_tiles_max * sizeof(EmuTile) + 1024, st));
+    double* Gam = (double*)mbuf.p;
+    double* Ab = Gam + (size_t)KH * KH;                   // a_k(t): [K_v + 1][t]
+    double* GA[2] = {Ab + (size_t)K1 * nt, Ab + (size_t)K1 * nt + (size_t)KH * nt};   // Gamma a(t): column-major
+    double* Ek = GA[1] + (size_t)KH * nt;
     double* d01 = Ek + chi_max;
     EmuTile* dtg = (EmuTile*)(((uintptr_t)(d01 + 8) + 15) & ~(uintptr_t)15);
-    EmuTile* dlo = dtg + n_tiles_max;                     // the lower-triangle tiles of the Gram matrices
-    __nv_bfloat16* Vr = (__nv_bfloat16*)(((uintptr_t)(dlo + n_tiles_max) + 255) & ~(uintptr_t)255);
-    __nv_bfloat16* Vi = Vr + sa;
-    __nv_bfloat16* Wr = Vi + sa;
-    __nv_bfloat16* Wi = Wr + sb;
-    int* evr = (int*)(Wi + sb);
-    int* evi = evr + K1;
-    int* ewr = evi + K1;
-    int* ewi = ewr + (K1 > nt ? K1 : nt);
+    __nv_bfloat16* Va = (__nv_bfloat16*)(((uintptr_t)(dtg + n_tiles_max) + 255) & ~(uintptr_t)255);
+    __nv_bfloat16* Wb = Va + sa;
+    int* eva = (int*)(Wb + sb);
+    int* ewb = eva + KH;
     // output tiles of a product (lower: only the tiles on or below the diagonal, for a
-    // symmetric result that is read through its lower triangle; TR == TC)
+    // symmetric result; TR == TC)
     auto grid_tiles = [&](int64_t rows, int64_t cols, int64_t kdim, int64_t& n_chunks, bool lower = false) {
       std::vector<EmuTile> t;
       for (int64_t rb = 0; rb * TR < rows; ++rb)
@@ -689,65 +677,74 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       n_chunks = emu_number_tiles(t);
       return t;
     };
+    struct Events {                                       // stage times of the moments and of the sums
+      std::vector<cudaEvent_t> e;
+      cudaError_t mark(cudaStream_t q) {
+        cudaEvent_t x;
+        cudaError_t r = cudaEventCreate(&x);
+        if (r != cudaSuccess) return r;
+        e.push_back(x);
+        return cudaEventRecord(x, q);
+      }
+      ~Events() { for (cudaEvent_t x : e) cudaEventDestroy(x); }
+    } ev;
     for (int j = 0; j < (int)ord.size(); ++j) {
       const ChebVariant& vv = vars[ord[j]];
       const int v = ord[j];
       const int k1 = Kv[v] + 1;
-      const int64_t kn = vv.kn, kr = vv.kr, chi = kn + kr;
-      const double* vre = V + (size_t)(2 * j) * n_un;       // column 2j of step 0; step k at + k S
-      TGBA_CUDA(cudaStreamSynchronize(st));
-      const auto t_gram = clk::now();
+      const int64_t kn = vv.kn, kr = vv.kr, chi = kn + kr, jump = kn_max - kn;
+      const double* vre = V + (size_t)j * n_un;             // column j of step 0; step k at + k S
+      TGBA_CUDA(ev.mark(st));
       kept_energy<<<blocks_for(chi), 256, 0, st>>>(kn, kr, kn_max, E, Ek);
       cheb_dot01<<<1, kRedThreads, 0, st>>>(n_un, vre, vre + S, d01);
-      b.launches += 2;
-      int64_t cg = 0, cl = 0;
-      const std::vector<EmuTile> tgv = grid_tiles(k1, k1, chi, cg), tlo = grid_tiles(k1, k1, chi, cl, true);
-      if (cg < 0 || cl < 0) return fail(TGBA_EINVAL, "quench moment tiles");
-      TGBA_CUDA(cudaMemcpyAsync(dtg, tgv.data(), tgv.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
-      TGBA_CUDA(cudaMemcpyAsync(dlo, tlo.data(), tlo.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
-      // rows k of V (K = the kept rows in their own order: kn NS rows, then kr R rows)
-      const int64_t jump = kn_max - kn;
-      if ((r = emu_slice(b, vre, S, 1, (int)kn, jump, nullptr, 0.0, k1, (int)chi, TR, Vr, evr, st)) != TGBA_OK) return r;
-      if ((r = emu_slice(b, vre + n_un, S, 1, (int)kn, jump, nullptr, 0.0, k1, (int)chi, TR, Vi, evi, st)) != TGBA_OK)
-        return r;
-      if ((r = emu_slice(b, vre, S, 1, (int)kn, jump, Ek, ec[v], k1, (int)chi, TC, Wr, ewr, st)) != TGBA_OK) return r;
-      if ((r = emu_slice(b, vre + n_un, S, 1, (int)kn, jump, Ek, ec[v], k1, (int)chi, TC, Wi, ewi, st)) != TGBA_OK)
-        return r;
-      if ((r = emu_gemm(b, Vr, evr, k1, (int)chi, Wr, ewr, k1, (int)chi, dlo, (int)tlo.size(), cl, Grr, k1, st)) != TGBA_OK)
-        return r;
-      if ((r = emu_gemm(b, Vi, evi, k1, (int)chi, Wi, ewi, k1, (int)chi, dlo, (int)tlo.size(), cl, Gii, k1, st)) != TGBA_OK)
-        return r;
-      if ((r = emu_gemm(b, Vr, evr, k1, (int)chi, Wi, ewi, k1, (int)chi, dtg, (int)tgv.size(), cg, Gri, k1, st)) != TGBA_OK)
-        return r;
-      cheb_gamma<<<blocks_for((int64_t)k1 * k1), 256, 0, st>>>(k1, Grr, Gii, Gri, Gam);
-      ++b.launches;
-      double h01 = 0.0;
-      TGBA_CUDA(cudaMemcpyAsync(&h01, d01, sizeof(double), cudaMemcpyDeviceToHost, st));
-      TGBA_CUDA(cudaStreamSynchronize(st));            // also: the tile list is reused below
-      b.quench_gram_ms += ms_since(t_gram);
-      const auto t_eval = clk::now();
-      // a_k(t) for the whole grid, Gamma a(t) (Gamma symmetric: its rows are its columns), the sums
+      // a_k(t) for the whole grid
       const double scale = 1.0 / (b.L * vv.hx * vv.norm2);
       const int ms = [&] {
         int m0 = Kv[v] + 30 + (int)std::ceil(std::sqrt(40.0 * Kv[v]));
         return m0 + (m0 & 1);
       }();
       cheb_bessel<<<(int)((nt + 31) / 32), 32, 0, st>>>((int)nt, 0, dt, R[v], Kv[v], ms, Ab);
-      ++b.launches;
-      int64_t ct = 0;
-      const std::vector<EmuTile> tt = grid_tiles(k1, nt, k1, ct);
-      if (ct < 0) return fail(TGBA_EINVAL, "quench time-sum tiles");
-      TGBA_CUDA(cudaMemcpyAsync(dtg, tt.data(), tt.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
-      if ((r = emu_slice(b, Gam, k1, 1, k1, 0, nullptr, 0.0, k1, k1, TR, Vr, evr, st)) != TGBA_OK) return r;
-      if ((r = emu_slice(b, Ab, 1, nt, k1, 0, nullptr, 0.0, (int)nt, k1, TC, Wr, ewi, st)) != TGBA_OK) return r;
-      if ((r = emu_gemm(b, Vr, evr, k1, k1, Wr, ewi, (int)nt, k1, dtg, (int)tt.size(), ct, GA, k1, st)) != TGBA_OK) return r;
-      cheb_mx<<<(int)((nt * 32 + 255) / 256), 256, 0, st>>>(k1, (int)nt, Ab, GA, R[v] * h01, scale,
+      b.launches += 3;
+      for (int p = 0; p < 2; ++p) {
+        const int kp = (k1 - p + 1) / 2;                    // vectors k = p, p + 2, ...
+        if (kp == 0) continue;
+        int64_t cl = 0, ct = 0;
+        const std::vector<EmuTile> tlo = grid_tiles(kp, kp, chi, cl, true);
+        if (cl < 0) return fail(TGBA_EINVAL, "quench moment tiles");
+        TGBA_CUDA(cudaMemcpyAsync(dtg, tlo.data(), tlo.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
+        // rows of V (K = the kept rows in their own order: kn NS rows, then kr R rows)
+        const double* vp = vre + (size_t)p * S;
+        if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, nullptr, 0.0, kp, (int)chi, TR, Va, eva, st)) != TGBA_OK) return r;
+        if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, Ek, ec[v], kp, (int)chi, TC, Wb, ewb, st)) != TGBA_OK) return r;
+        if ((r = emu_gemm(b, Va, eva, kp, (int)chi, Wb, ewb, kp, (int)chi, dtg, (int)tlo.size(), cl, Gam, kp, st)) != TGBA_OK)
+          return r;
+        symmetrise<<<blocks_for((int64_t)kp * kp), 256, 0, st>>>(kp, Gam);
+        ++b.launches;
+        TGBA_CUDA(ev.mark(st));
+        // Gamma a(t) (Gamma symmetric: its rows are its columns)
+        const std::vector<EmuTile> tt = grid_tiles(kp, nt, kp, ct);
+        if (ct < 0) return fail(TGBA_EINVAL, "quench time-sum tiles");
+        TGBA_CUDA(cudaMemcpyAsync(dtg, tt.data(), tt.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
+        if ((r = emu_slice(b, Gam, kp, 1, kp, 0, nullptr, 0.0, kp, kp, TR, Va, eva, st)) != TGBA_OK) return r;
+        if ((r = emu_slice(b, Ab + (size_t)p * nt, 1, 2 * nt, kp, 0, nullptr, 0.0, (int)nt, kp, TC, Wb, ewb, st)) != TGBA_OK)
+          return r;
+        if ((r = emu_gemm(b, Va, eva, kp, kp, Wb, ewb, (int)nt, kp, dtg, (int)tt.size(), ct, GA[p], kp, st)) != TGBA_OK)
+          return r;
+        TGBA_CUDA(ev.mark(st));
+      }
+      cheb_mx<<<(int)((nt * 32 + 255) / 256), 256, 0, st>>>(k1, (int)nt, Ab, GA[0], GA[1], d01, R[v], scale,
                                                               mx + (int64_t)vv.out * n_t);
-      ++b.launches;
       TGBA_CUDA(cudaGetLastError());
-      TGBA_CUDA(cudaStreamSynchronize(st));
-      b.quench_eval_ms += ms_since(t_eval);
+      ++b.launches;
     }
+    TGBA_CUDA(cudaStreamSynchronize(st));
+    // per variant: start, then (moments, sums) for the even and the odd k (K >= 1: both exist)
+    for (size_t x = 0; x + 5 <= ev.e.size(); x += 5)
+      for (int q = 0; q < 4; ++q) {
+        float ms = 0.f;
+        TGBA_CUDA(cudaEventElapsedTime(&ms, ev.e[x + q], ev.e[x + q + 1]));
+        (q % 2 ? b.quench_eval_ms : b.quench_gram_ms) += ms;
+      }
     b.quench_terms = K;
     TGBA_CUDA(cudaStreamSynchronize(st));
     return check_status(b, st);

@@ -105,6 +105,24 @@ __global__ void gather_kernel(int64_t kn, int64_t kr, const int32_t* __restrict_
   }
 }
 
+// The X block between the kept NS and R entries, column-major kr x kn; even: between even combinations of
+// mirror images (see coupling in tridiag.cu), else the entries are single states.
+__global__ void gather_even(int64_t kn, int64_t kr, const MirrorPair* __restrict__ ns, const MirrorPair* __restrict__ r,
+                            int64_t n_r, const double* __restrict__ P, bool even, double* __restrict__ Q) {
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < kn * kr; idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t a = idx / kr, b = idx - a * kr;
+    const MirrorPair x = ns[a], y = r[b];
+    const double* row = P + (int64_t)x.a * n_r;
+    double v = row[y.a];
+    if (even) {
+      const bool sx = x.a == x.b, sy = y.a == y.b;
+      if (!sx && !sy) v += row[y.b];
+      else if (sx != sy) v *= M_SQRT2;
+    }
+    Q[idx] = v;
+  }
+}
+
 // Eq. 11 at each time t: || Psi^chi(t) - Psi^chi'(t) ||^2 = sum over the larger subspace of
 // |B'_a - B_a|^2 (B_a = 0 for states the smaller one lacks).  The smaller subspace's NS and R
 // lists are prefixes of the larger one's (nested truncations in one ranking).  B, B': [Re | Im]
@@ -189,6 +207,30 @@ __global__ void gather_energy(int64_t kn, int64_t kr, const int32_t* __restrict_
 int blocks_for(int64_t work) {
   int64_t g = (work + 255) / 256;
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 32));
+}
+
+// Kept sets (lists of states of one parity) under the reflection: closed, and the mirror pairs by
+// their first member in the list.
+bool closed_under_mirror(const std::vector<int32_t>& list, const std::vector<int32_t>& img) {
+  std::vector<char> in(img.size(), 0);
+  for (int32_t q : list) in[q] = 1;
+  for (int32_t q : list)
+    if (!in[img[q]]) return false;
+  return true;
+}
+std::vector<MirrorPair> mirror_reps(const std::vector<int32_t>& list, const std::vector<int32_t>& img) {
+  std::vector<char> in(img.size(), 0);
+  std::vector<MirrorPair> v;
+  for (int32_t q : list) {
+    if (!in[img[q]]) v.push_back({q, img[q]});
+    in[q] = 1;
+  }
+  return v;
+}
+int64_t mirror_count(const std::vector<int32_t>& list, const std::vector<int32_t>& img) {   // of a closed set
+  int64_t self = 0;
+  for (int32_t q : list) self += img[q] == q;
+  return self + ((int64_t)list.size() - self) / 2;
 }
 
 tgba_status blas_fail(cublasStatus_t s, const char* what) {
@@ -513,9 +555,26 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
       if (sel_ns[v].size() > un_ns->size()) un_ns = &sel_ns[v];
       if (sel_r[v].size() > un_r->size()) un_r = &sel_r[v];
     }
-    const int64_t kn = (int64_t)un_ns->size(), kr = (int64_t)un_r->size(), n = kn + kr;
+    // The initial state is even under the reflection (its overlaps vanish unless the momenta pair up,
+    // and then a state is its own image), so it stays in the even block of H~: when every kept set is
+    // closed under the reflection (energy cutoffs are), the propagation runs on the even combinations
+    // of mirror images, half the states on each side of the X block.  One entry per pair, the first
+    // in the ranking, so that the variants stay prefixes.
+    const SectorSym& sy = b.sym[s];
+    bool even = sy.split && b.x_screen == nullptr;
+    for (int v : cheb_vars)
+      even = even && closed_under_mirror(sel_ns[v], sy.img[0]) && closed_under_mirror(sel_r[v], sy.img[1]);
+    std::vector<MirrorPair> mn, mr_;
+    if (even) {
+      mn = mirror_reps(*un_ns, sy.img[0]);
+      mr_ = mirror_reps(*un_r, sy.img[1]);
+    } else {
+      for (int32_t q : *un_ns) mn.push_back({q, q});
+      for (int32_t q : *un_r) mr_.push_back({q, q});
+    }
+    const int64_t kn = (int64_t)mn.size(), kr = (int64_t)mr_.size(), n = kn + kr;
     double* ub = nullptr;
-    const size_t udoubles = (size_t)n + 2 * n + 8 + (size_t)kn * kr + 2 * L + (n + 2) / 2 + 8;
+    const size_t udoubles = (size_t)n + 2 * n + 8 + (size_t)kn * kr + 2 * L + (n + 2) / 2 + n + 16;
     TGBA_CUDA(cudaMallocAsync(&ub, udoubles * sizeof(double), st));
     struct FreeU {
       double* p; cudaStream_t s;
@@ -526,18 +585,21 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
     double* norm2 = c + 2 * n;
     double* Q = norm2 + 8;
     double* dth_dev = Q + (size_t)kn * kr;
-    int32_t* idx = (int32_t*)(dth_dev + 2 * L);
+    MirrorPair* prs = (MirrorPair*)(dth_dev + 2 * L);
+    int32_t* idx = (int32_t*)(prs + n);
+    std::vector<int32_t> first(n);
+    for (int64_t q = 0; q < n; ++q) first[q] = q < kn ? mn[q].a : mr_[q - kn].a;
     TGBA_CUDA(cudaMemcpyAsync(dth_dev, dth.data(), 2 * L * sizeof(double), cudaMemcpyHostToDevice, st));
-    TGBA_CUDA(cudaMemcpyAsync(idx, un_ns->data(), kn * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    TGBA_CUDA(cudaMemcpyAsync(idx + kn, un_r->data(), kr * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    TGBA_CUDA(cudaMemsetAsync(norm2, 0, sizeof(double), st));
+    TGBA_CUDA(cudaMemcpyAsync(idx, first.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    TGBA_CUDA(cudaMemcpyAsync(prs, mn.data(), kn * sizeof(MirrorPair), cudaMemcpyHostToDevice, st));
+    TGBA_CUDA(cudaMemcpyAsync(prs + kn, mr_.data(), kr * sizeof(MirrorPair), cudaMemcpyHostToDevice, st));
     overlap_kernel<<<blocks_for(n), 256, 0, st>>>(kn, kr, idx, idx + kn, sec.ns_off, sec.r_off, b.d_M_ns, b.d_M_r,
                                                  b.d_modes_ns, b.d_modes_r, b.max_qp, b.d_nlab, dth_dev, base[0],
                                                  base[1], s_re, s_im, g_re, g_im, L, c, norm2);
     gather_energy<<<blocks_for(n), 256, 0, st>>>(kn, kr, idx, idx + kn, b.d_E_ns + sec.ns_off, b.d_E_r + sec.r_off, E);
     b.launches += 2;
     if (kn > 0 && kr > 0) {
-      gather_kernel<<<blocks_for(kn * kr), 256, 0, st>>>(kn, kr, idx, idx + kn, sec.n_r, b.d_P + sec.x_off, Q);
+      gather_even<<<blocks_for(kn * kr), 256, 0, st>>>(kn, kr, prs, prs + kn, sec.n_r, b.d_P + sec.x_off, even, Q);
       ++b.launches;
     }
     TGBA_CUDA(cudaGetLastError());
@@ -551,8 +613,8 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
     for (int v : cheb_vars) {
       ChebVariant x;
       x.out = v;
-      x.kn = (int64_t)sel_ns[v].size();
-      x.kr = (int64_t)sel_r[v].size();
+      x.kn = even ? mirror_count(sel_ns[v], sy.img[0]) : (int64_t)sel_ns[v].size();
+      x.kr = even ? mirror_count(sel_r[v], sy.img[1]) : (int64_t)sel_r[v].size();
       x.hx = hx[v];
       x.norm2 = pre[x.kn] + (pre[kn + x.kr] - pre[kn]);
       norms[v] = x.norm2;
