@@ -29,8 +29,7 @@
 // off-diagonal blocks in each step, the Lanczos steps and the moments) runs on the tensor cores
 // through the sliced products of dgemm_tc.cu: Q is sliced once in both orientations, each
 // step slices the current vectors, and the output tiles of each step skip the (row block,
-// column block) pairs that no variant's kept set reaches.  The K steps are captured into one
-// CUDA graph.
+// column block) pairs that no variant's kept set reaches.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -72,7 +71,22 @@ __global__ void transpose_kernel(int64_t rows, int64_t cols, const double* __res
 }
 
 // Lanczos start vectors: a fixed pseudo-random vector per column (SplitMix64 of the row), unit norm
-__global__ void lz_start(int64_t n, double* __restrict__ q) {
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+// maxima of a column's halves over the block into mb[0] (R rows) and mb[1] (NS rows)
+__device__ __forceinline__ void block_max(unsigned long long m0, unsigned long long m1, unsigned long long* mb) {
+  for (int o = 16; o > 0; o >>= 1) {
+    m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+    m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(mb, m0);
+    atomicMax(mb + 1, m1);
+  }
+}
+
+__global__ void lz_start(int64_t n, int64_t kn, double* __restrict__ q, unsigned long long* __restrict__ mb) {
   __shared__ double sh[32];
   double* col = q + (int64_t)blockIdx.x * n;
   double s = 0.0;
@@ -87,14 +101,21 @@ __global__ void lz_start(int64_t n, double* __restrict__ q) {
   }
   s = block_reduce(s, sh);
   const double inv = 1.0 / sqrt(s);
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) col[i] *= inv;
+  unsigned long long m[2] = {0ull, 0ull};
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    col[i] *= inv;
+    unsigned long long& x = i < kn ? m[1] : m[0];
+    x = max(x, abs_bits(col[i]));
+  }
+  block_max(m[0], m[1], mb + 2 * blockIdx.x);
 }
 
 // One Lanczos step per column (block): w = g Y + E q; alpha = q.w; w -= alpha q + beta q_prev;
 // beta' = ||w||; q_next = w / beta' (zero after a breakdown).  Y holds A q.
-__global__ void lz_step(int64_t n, const double* __restrict__ E, const double* __restrict__ g, const double* __restrict__ Y,
+__global__ void lz_step(int64_t n, int64_t kn, const double* __restrict__ E, const double* __restrict__ g, const double* __restrict__ Y,
                         const double* __restrict__ qp, const double* __restrict__ qc, double* __restrict__ qn,
-                        double* __restrict__ alpha, double* __restrict__ beta, int j, int m) {
+                        double* __restrict__ alpha, double* __restrict__ beta, int j, int m,
+                        unsigned long long* __restrict__ mb) {
   __shared__ double sh[32];
   const int c = blockIdx.x;
   const double gc = g[c];
@@ -118,7 +139,13 @@ __global__ void lz_step(int64_t n, const double* __restrict__ E, const double* _
   }
   const double bn = sqrt(block_reduce(s, sh));
   const double inv = bn > 1e-300 ? 1.0 / bn : 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) w[i] *= inv;
+  unsigned long long mx[2] = {0ull, 0ull};
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    w[i] *= inv;
+    unsigned long long& x = i < kn ? mx[1] : mx[0];
+    x = max(x, abs_bits(w[i]));
+  }
+  block_max(mx[0], mx[1], mb + 2 * c);
   if (threadIdx.x == 0) {
     alpha[(int64_t)c * m + j] = a;
     if (j + 1 < m) beta[(int64_t)c * m + j + 1] = bn;
@@ -154,30 +181,55 @@ __device__ __forceinline__ bool kept(int64_t row, int64_t kn_max, const ColPrm& 
   return row < kn_max ? row < p.kn : row - kn_max < p.kr;
 }
 
-// v_0: c~0 (real; stored as complex) on the kept rows of each column's variant
-__global__ void cheb_init(int64_t n, int64_t kn_max, int cols, const ColPrm* __restrict__ prm,
-                          const double* __restrict__ c, double* __restrict__ V) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n * cols; q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = q % n;
-    const int col = (int)(q / n);
-    V[q] = kept(row, kn_max, prm[col]) ? c[2 * row] : 0.0;
+// The largest magnitude (bits) of a block's entries of one column in each half (NS rows, R rows), into
+// mb[2 col + half] (half 0: R rows, half 1: NS rows), for the slicing of the next product.
+__device__ __forceinline__ void column_max(double v, bool ns, unsigned long long* mb) {
+  unsigned long long bits;
+  asm("and.b64 %0, %1, 0x7fffffffffffffff;" : "=l"(bits) : "l"((unsigned long long)__double_as_longlong(v)));
+  unsigned long long m0 = ns ? 0ull : bits, m1 = ns ? bits : 0ull;
+  for (int o = 16; o > 0; o >>= 1) {
+    m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+    m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (m0) atomicMax(mb, m0);
+    if (m1) atomicMax(mb + 1, m1);
   }
 }
 
-// v_{k+1} = alpha (g Y + (E - E_c) v_k) / R - beta v_{k-1}, 0 outside each column's kept rows
-__global__ void cheb_step(int64_t n, int64_t kn_max, int cols, const double* __restrict__ E,
-                          const ColPrm* __restrict__ prm, double alpha, double beta, const double* __restrict__ Y,
-                          const double* __restrict__ x, const double* __restrict__ prev, double* __restrict__ next) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n * cols; q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = q % n;
-    const ColPrm p = prm[q / n];
-    double v = 0.0;
+// v_0: c~0 (real; stored as complex) on the kept rows of each column's variant (blockIdx.y)
+__global__ void __launch_bounds__(256) cheb_init(int64_t n, int64_t kn_max, const ColPrm* __restrict__ prm,
+                                                 const double* __restrict__ c, double* __restrict__ V,
+                                                 unsigned long long* __restrict__ mb) {
+  const int col = blockIdx.y;
+  const int64_t row = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  double v = 0.0;
+  if (row < n) {
+    if (kept(row, kn_max, prm[col])) v = c[2 * row];
+    V[(int64_t)col * n + row] = v;
+  }
+  column_max(v, row < kn_max, mb + 2 * col);
+}
+
+// v_{k+1} = alpha (g Y + (E - E_c) v_k) / R - beta v_{k-1}, 0 outside each column's kept rows, and the
+// halves' maxima (one pass: a separate maximum per product cost two launches of 8 us per step)
+__global__ void __launch_bounds__(256) cheb_step(int64_t n, int64_t kn_max, const double* __restrict__ E,
+                                                 const ColPrm* __restrict__ prm, double alpha, double beta,
+                                                 const double* __restrict__ Y, const double* __restrict__ x,
+                                                 const double* __restrict__ prev, double* __restrict__ next,
+                                                 unsigned long long* __restrict__ mb) {
+  const int col = blockIdx.y;
+  const int64_t row = (int64_t)blockIdx.x * 256 + threadIdx.x, q = (int64_t)col * n + row;
+  const ColPrm p = prm[col];
+  double v = 0.0;
+  if (row < n) {
     if (kept(row, kn_max, p)) {
       const double h = fma(p.g, Y[q], (E[row] - p.ec) * x[q]);
       v = alpha * p.invr * h - (prev ? beta * prev[q] : 0.0);
     }
     next[q] = v;
   }
+  column_max(v, row < kn_max, mb + 2 * col);
 }
 
 // per column: ||v_0||^2 and ||v_K||^2 (one block per column)
@@ -337,7 +389,7 @@ int64_t r16(int64_t x) { return (x + 15) / 16 * 16; }
 // none).
 std::vector<EmuTile> product_tiles(int64_t rows, int64_t cols, const std::vector<int64_t>& out_c,
                                    const std::vector<int64_t>& k_c) {
-  const int TR = emu_tile_rows_a(), TC = emu_tile_rows_b(), KB = emu_k_block();
+  const int TR = emu_tile_rows_a(), TC = kEmuTileCols, KB = emu_k_block();
   std::vector<EmuTile> t;
   for (int64_t rb = 0; rb * TR < rows; ++rb)
     for (int64_t cb = 0; cb * TC < cols; ++cb) {
@@ -369,7 +421,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
                                "use method 1 for h_x = 0");
   const int64_t n_un = kn_max + kr_max;
   const double cabs = std::hypot(b.c0_host[0], b.c0_host[1]);
-  const int TR = emu_tile_rows_a(), TC = emu_tile_rows_b();
+  const int TR = emu_tile_rows_a(), TC = kEmuTileCols;
   // stage times (host clock around synchronised sections)
   using clk = std::chrono::steady_clock;
   TGBA_CUDA(cudaStreamSynchronize(st));
@@ -401,20 +453,30 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     cudaFreeAsync(Qt, st);
     if (r != TGBA_OK) return r;
   }
-  // B-operand slices of the current vectors (the columns padded to whole tiles)
-  auto vec_slices = [&](int cols) {
-    return std::max(emu_operand_elems(cols, (int)std::max<int64_t>(1, kr_max), TC),
-                    emu_operand_elems(cols, (int)std::max<int64_t>(1, kn_max), TC));
+  // B-operand slices of the current vectors: room for both halves' images
+  auto half_slices = [&](int cols, int64_t K) {
+    return emu_operand_elems(cols, (int)std::max<int64_t>(1, K), emu_tile_rows_b(cols));
   };
-  // off-diagonal product Y = A x on the union layout (x, Y: n_un x cols, ld n_un)
-  auto offdiag = [&](const double* x, double* Y, int cols, __nv_bfloat16* Bs, int* eb, EmuTile* t_ns, int n_ns,
-                     int64_t c_ns, EmuTile* t_r, int n_r, int64_t c_r, int ns) -> tgba_status {
-    tgba_status q = emu_slice(b, x + kn_max, n_un, 1, (int)kr_max, 0, nullptr, 0.0, cols, (int)kr_max, TC, Bs, eb, st);
-    if (q == TGBA_OK) q = emu_gemm(b, A_ns, e_ns, (int)kn_max, (int)kr_max, Bs, eb, cols, (int)kr_max, t_ns, n_ns, c_ns, Y, n_un, st, ns);
-    if (q == TGBA_OK) q = emu_slice(b, x, n_un, 1, (int)kn_max, 0, nullptr, 0.0, cols, (int)kn_max, TC, Bs, eb, st);
-    if (q == TGBA_OK)
-      q = emu_gemm(b, A_r, e_r, (int)kr_max, (int)kn_max, Bs, eb, cols, (int)kn_max, t_r, n_r, c_r, Y + kn_max, n_un, st, ns);
-    return q;
+  // off-diagonal product Y = A x on the union layout (x, Y: n_un x cols, ld n_un; max_bits: the halves'
+  // maxima of x): one slicing launch and one product launch for both blocks
+  auto offdiag = [&](const double* x, const unsigned long long* max_bits, double* Y, int cols, __nv_bfloat16* Bs, int* eb,
+                     EmuTile* tiles, int n_tiles, int64_t n_blocks, int ns, cudaStream_t q) -> tgba_status {
+    __nv_bfloat16* Bn = Bs + half_slices(cols, kr_max);
+    tgba_status z = emu_slice_halves(b, x, n_un, cols, (int)kn_max, (int)kr_max, max_bits, Bs, Bn, eb, eb + cols, q);
+    if (z != TGBA_OK) return z;
+    const EmuSet sets[2] = {
+        emu_set(A_ns, e_ns, (int)kn_max, (int)kr_max, Bs, eb, cols, (int)kr_max, Y, n_un),
+        emu_set(A_r, e_r, (int)kr_max, (int)kn_max, Bn, eb + cols, cols, (int)kn_max, Y + kn_max, n_un)};
+    return emu_gemm_sets(b, sets, 2, emu_tile_rows_b(cols), tiles, n_tiles, n_blocks, q, ns);
+  };
+  // the tiles of both blocks in one list
+  auto both_tiles = [&](int64_t cols, const std::vector<int64_t>& out_ns, const std::vector<int64_t>& out_r,
+                        const std::vector<int64_t>& k_ns, const std::vector<int64_t>& k_r, int64_t& blocks) {
+    std::vector<EmuTile> t = product_tiles(kn_max, cols, out_ns, k_ns), u = product_tiles(kr_max, cols, out_r, k_r);
+    for (EmuTile& e : u) e.set = 1;
+    t.insert(t.end(), u.begin(), u.end());
+    blocks = emu_number_tiles(t);
+    return t;
   };
   // ---- Lanczos bounds on the union for each distinct field.  The products take only the two
   // leading digit slices of each operand (X's relative error about 2^-16 of its row scale, a
@@ -424,20 +486,21 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
   for (const ChebVariant& v : vars)
     if (std::find(fields.begin(), fields.end(), v.hx) == fields.end()) fields.push_back(v.hx);
   const int nh = (int)fields.size();
-  const int nhp = (int)std::max<int64_t>(TC, (nh + TC - 1) / TC * TC);
+  const int nhp = (int)r16(nh);
   std::vector<double> lo(nh), hi(nh);
   {
     const int m = (int)std::min<int64_t>(kLanczosSteps, n_un);
     std::vector<int64_t> out_ns(nhp, 0), out_r(nhp, 0), k_ns(nhp, 0), k_r(nhp, 0);
     for (int i = 0; i < nh; ++i) { out_ns[i] = kn_max; k_ns[i] = kr_max; out_r[i] = kr_max; k_r[i] = kn_max; }
-    std::vector<EmuTile> tn = product_tiles(kn_max, nhp, out_ns, k_ns), tr = product_tiles(kr_max, nhp, out_r, k_r);
-    const int64_t cn = emu_number_tiles(tn), cr_ = emu_number_tiles(tr);
-    if (cn < 0 || cr_ < 0) return fail(TGBA_EINVAL, "quench product tiles");
+    int64_t blocks = 0;
+    const std::vector<EmuTile> tl = both_tiles(nhp, out_ns, out_r, k_ns, k_r, blocks);
+    if (blocks < 0) return fail(TGBA_EINVAL, "quench product tiles");
     DevBuf buf(st);
-    const size_t vs = vec_slices(nhp);
-    const size_t doubles = (size_t)4 * n_un * nhp + 2 * (size_t)m * nhp + nhp;
-    const size_t tb = (tn.size() + tr.size()) * sizeof(EmuTile);
-    TGBA_CUDA(cudaMallocAsync(&buf.p, doubles * 8 + vs * 2 + (size_t)nhp * 4 + tb + 512, st));
+    const size_t vs = half_slices(nhp, kr_max) + half_slices(nhp, kn_max);
+    const size_t n_max_bits = (size_t)(m + 1) * nhp * 2;
+    const size_t doubles = (size_t)4 * n_un * nhp + 2 * (size_t)m * nhp + nhp + n_max_bits;
+    const size_t tb = tl.size() * sizeof(EmuTile);
+    TGBA_CUDA(cudaMallocAsync(&buf.p, doubles * 8 + vs * 2 + 2 * (size_t)nhp * 4 + tb + 512, st));
     double* q0 = (double*)buf.p;
     double* q1 = q0 + n_un * nhp;
     double* q2 = q1 + n_un * nhp;
@@ -445,25 +508,25 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     double* al = Y + n_un * nhp;
     double* be = al + (size_t)m * nhp;
     double* g = be + (size_t)m * nhp;
-    EmuTile* dt = (EmuTile*)(((uintptr_t)(g + nhp) + 15) & ~(uintptr_t)15);
-    __nv_bfloat16* Bs = (__nv_bfloat16*)(((uintptr_t)(dt + tn.size() + tr.size()) + 255) & ~(uintptr_t)255);
+    unsigned long long* mb = (unsigned long long*)(g + nhp);
+    EmuTile* dt = (EmuTile*)(((uintptr_t)(mb + n_max_bits) + 15) & ~(uintptr_t)15);
+    __nv_bfloat16* Bs = (__nv_bfloat16*)(((uintptr_t)(dt + tl.size()) + 255) & ~(uintptr_t)255);
     int* eb = (int*)(Bs + vs);
     std::vector<double> gh(nhp, 0.0);
     for (int i = 0; i < nh; ++i) gh[i] = -b.L * fields[i] * cabs;
     TGBA_CUDA(cudaMemcpyAsync(g, gh.data(), nhp * sizeof(double), cudaMemcpyHostToDevice, st));
-    if (!tn.empty()) TGBA_CUDA(cudaMemcpyAsync(dt, tn.data(), tn.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
-    if (!tr.empty())
-      TGBA_CUDA(cudaMemcpyAsync(dt + tn.size(), tr.data(), tr.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
+    if (!tl.empty()) TGBA_CUDA(cudaMemcpyAsync(dt, tl.data(), tl.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
     TGBA_CUDA(cudaMemsetAsync(q0, 0, 4 * (size_t)n_un * nhp * sizeof(double), st));
     TGBA_CUDA(cudaMemsetAsync(be, 0, (size_t)m * nhp * sizeof(double), st));
-    lz_start<<<nh, kRedThreads, 0, st>>>(n_un, q1);
+    TGBA_CUDA(cudaMemsetAsync(mb, 0, n_max_bits * sizeof(*mb), st));
+    lz_start<<<nh, kRedThreads, 0, st>>>(n_un, kn_max, q1, mb);
     ++b.launches;
     double *qp = q0, *qc = q1, *qn = q2;
     for (int j = 0; j < m; ++j) {
       if (coupled) {
-        if ((r = offdiag(qc, Y, nhp, Bs, eb, dt, (int)tn.size(), cn, dt + tn.size(), (int)tr.size(), cr_, 2)) != TGBA_OK) return r;
+        if ((r = offdiag(qc, mb + (size_t)j * 2 * nhp, Y, nhp, Bs, eb, dt, (int)tl.size(), blocks, 2, st)) != TGBA_OK) return r;
       }
-      lz_step<<<nh, kRedThreads, 0, st>>>(n_un, E, g, Y, qp, qc, qn, al, be, j, m);
+      lz_step<<<nh, kRedThreads, 0, st>>>(n_un, kn_max, E, g, Y, qp, qc, qn, al, be, j, m, mb + (size_t)(j + 1) * 2 * nhp);
       ++b.launches;
       double* t = qp; qp = qc; qc = qn; qn = t;
     }
@@ -522,14 +585,11 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     out_ns[j] = v.kn; k_ns[j] = v.kr;
     out_r[j] = v.kr; k_r[j] = v.kn;
   }
-  std::vector<EmuTile> tn = product_tiles(kn_max, ncolp, out_ns, k_ns), tr = product_tiles(kr_max, ncolp, out_r, k_r);
-  const int64_t cn = emu_number_tiles(tn), cr_ = emu_number_tiles(tr);
-  if (cn < 0 || cr_ < 0) return fail(TGBA_EINVAL, "quench product tiles");
+  int64_t n_blocks = 0;
+  const std::vector<EmuTile> tl = both_tiles(ncolp, out_ns, out_r, k_ns, k_r, n_blocks);
+  if (n_blocks < 0) return fail(TGBA_EINVAL, "quench product tiles");
   const int dt_n = n_t;
   const double dt = n_t > 1 ? t_max / (n_t - 1) : 0.0;
-  cudaStream_t cap = nullptr;
-  TGBA_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-  struct StreamGuard { cudaStream_t s; ~StreamGuard() { if (s) cudaStreamDestroy(s); } } cap_guard{cap};
   for (int attempt = 0; attempt < 2; ++attempt) {
     // per variant: interval, terms
     std::vector<double> ec(vars.size()), R(vars.size());
@@ -548,10 +608,10 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     }
     const int K1 = K + 1;
     const int64_t S = n_un * ncolp;                      // one step's vectors
-    const size_t vs = vec_slices(ncolp);
-    const size_t tb = (tn.size() + tr.size()) * sizeof(EmuTile);
-    const size_t need = sizeof(double) * ((size_t)S * K1 + S + 2 * (size_t)ncolp + 8) + ncolp * sizeof(ColPrm) + vs * 2 +
-                        (size_t)ncolp * 4 + tb + 1024;
+    const size_t vs = half_slices(ncolp, kr_max) + half_slices(ncolp, kn_max);
+    const size_t tb = tl.size() * sizeof(EmuTile), n_mb = (size_t)K1 * ncolp * 2;
+    const size_t need = sizeof(double) * ((size_t)S * K1 + S + 2 * (size_t)ncolp + 8 + n_mb) + ncolp * sizeof(ColPrm) + vs * 2 +
+                        2 * (size_t)ncolp * 4 + tb + 1024;
     size_t free_b = 0, tot_b = 0;
     TGBA_CUDA(cudaMemGetInfo(&free_b, &tot_b));
     if (need + ((size_t)2 << 30) > free_b)
@@ -562,9 +622,10 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     double* V = (double*)vbuf.p;
     double* Y = V + (size_t)S * K1;
     double* nrm = Y + S;
-    ColPrm* prm = (ColPrm*)(nrm + 2 * (size_t)ncolp + 8);
+    unsigned long long* mb = (unsigned long long*)(nrm + 2 * (size_t)ncolp + 8);   // maxima per step [K1][ncolp][2]
+    ColPrm* prm = (ColPrm*)(mb + n_mb);
     EmuTile* dtl = (EmuTile*)(((uintptr_t)(prm + ncolp) + 15) & ~(uintptr_t)15);
-    __nv_bfloat16* Bs = (__nv_bfloat16*)(((uintptr_t)(dtl + tn.size() + tr.size()) + 255) & ~(uintptr_t)255);
+    __nv_bfloat16* Bs = (__nv_bfloat16*)(((uintptr_t)(dtl + tl.size()) + 255) & ~(uintptr_t)255);
     int* eb = (int*)(Bs + vs);
     std::vector<ColPrm> hp(ncolp, ColPrm{0.0, 0.0, 0.0, 0, 0});
     for (int j = 0; j < (int)ord.size(); ++j) {
@@ -572,52 +633,32 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       hp[j] = ColPrm{-b.L * vars[v].hx * cabs, ec[v], 1.0 / R[v], vars[v].kn, vars[v].kr};
     }
     TGBA_CUDA(cudaMemcpyAsync(prm, hp.data(), ncolp * sizeof(ColPrm), cudaMemcpyHostToDevice, st));
-    if (!tn.empty()) TGBA_CUDA(cudaMemcpyAsync(dtl, tn.data(), tn.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
-    if (!tr.empty())
-      TGBA_CUDA(cudaMemcpyAsync(dtl + tn.size(), tr.data(), tr.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
+    if (!tl.empty()) TGBA_CUDA(cudaMemcpyAsync(dtl, tl.data(), tl.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
     TGBA_CUDA(cudaMemsetAsync(Y, 0, S * sizeof(double), st));
-    cheb_init<<<blocks_for(S), 256, 0, st>>>(n_un, kn_max, ncolp, prm, c, V);
+    TGBA_CUDA(cudaMemsetAsync(mb, 0, n_mb * sizeof(*mb), st));
+    const dim3 vgrid((unsigned)((n_un + 255) / 256), (unsigned)ncolp);
+    cheb_init<<<vgrid, 256, 0, st>>>(n_un, kn_max, prm, c, V, mb);
     TGBA_CUDA(cudaGetLastError());
     ++b.launches;
     TGBA_CUDA(cudaStreamSynchronize(st));
     b.quench_prep_ms = ms_since(t_start);     // slicing of Q, Lanczos, set-up (last attempt)
-    // the K steps of all variants, captured once and launched as one graph
-    TGBA_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-    cudaStream_t keep = st;
-    st = cap;                                            // offdiag launches on `st`
-    tgba_status cr = TGBA_OK;
-    const int64_t launches0 = b.launches.load();
-    for (int k = 0; k < K && cr == TGBA_OK; ++k) {
-      double* vk = V + (size_t)k * S;
-      if (coupled)
-        cr = offdiag(vk, Y, ncolp, Bs, eb, dtl, (int)tn.size(), cn, dtl + tn.size(), (int)tr.size(), cr_, 6);
-      if (cr != TGBA_OK) break;
-      cheb_step<<<blocks_for(S), 256, 0, cap>>>(n_un, kn_max, ncolp, E, prm, k == 0 ? 1.0 : 2.0, 1.0, Y, vk,
-                                                 k == 0 ? nullptr : vk - S, vk + S);
-      ++b.launches;
-    }
-    st = keep;
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ce = cudaStreamEndCapture(cap, &graph);
-    const int64_t graph_launches = b.launches.load() - launches0;
-    b.launches -= graph_launches;                        // counted when the graph runs
-    if (cr != TGBA_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return cr;
-    }
-    if (ce != cudaSuccess) return cuda_fail(ce, "cudaStreamEndCapture (Chebyshev steps)");
-    cudaGraphExec_t exec = nullptr;
-    const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ie != cudaSuccess) return cuda_fail(ie, "cudaGraphInstantiate (Chebyshev steps)");
-    struct ExecGuard { cudaGraphExec_t e; ~ExecGuard() { cudaGraphExecDestroy(e); } } exec_guard{exec};
+    // the K steps of all variants, three launches each (the host enqueues them ahead of the device;
+    // capturing and instantiating a graph of them for one use took longer)
     for (int e = 0; e < 2; ++e)
       if (b.q_ev[e] == nullptr) TGBA_CUDA(cudaEventCreate(&b.q_ev[e]));
     TGBA_CUDA(cudaEventRecord(b.q_ev[0], st));
-    TGBA_CUDA(cudaGraphLaunch(exec, st));
+    for (int k = 0; k < K; ++k) {
+      double* vk = V + (size_t)k * S;
+      if (coupled &&
+          (r = offdiag(vk, mb + (size_t)k * 2 * ncolp, Y, ncolp, Bs, eb, dtl, (int)tl.size(), n_blocks, 6, st)) != TGBA_OK)
+        return r;
+      cheb_step<<<vgrid, 256, 0, st>>>(n_un, kn_max, E, prm, k == 0 ? 1.0 : 2.0, 1.0, Y, vk, k == 0 ? nullptr : vk - S,
+                                       vk + S, mb + (size_t)(k + 1) * 2 * ncolp);
+      ++b.launches;
+    }
+    TGBA_CUDA(cudaGetLastError());
     TGBA_CUDA(cudaEventRecord(b.q_ev[1], st));
     b.q_ev_recorded = true;
-    b.launches += graph_launches;
     b.quench_flops = 0;
     for (const ChebVariant& v : vars) b.quench_flops += 4.0 * (double)K * (double)v.kn * (double)v.kr;
     // the interval check: ||v_K|| <= ||v_0|| for every column
@@ -650,6 +691,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     }
     const int64_t nt = std::max(1, dt_n), KH = (K1 + 1) / 2;
     const size_t sa = std::max(emu_operand_elems((int)KH, (int)chi_max, TR), emu_operand_elems((int)KH, (int)KH, TR));
+    // every product of this stage takes B images of 128 rows (k or times), whatever its size
     const size_t sb = std::max(emu_operand_elems((int)KH, (int)chi_max, TC), emu_operand_elems((int)nt, (int)KH, TC));
     const size_t n_tiles_max = (size_t)((KH + TR - 1) / TR) * (size_t)std::max<int64_t>((KH + TC - 1) / TC, (nt + TC - 1) / TC);
     DevBuf mbuf(st);
@@ -716,7 +758,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
         const double* vp = vre + (size_t)p * S;
         if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, nullptr, 0.0, kp, (int)chi, TR, Va, eva, st)) != TGBA_OK) return r;
         if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, Ek, ec[v], kp, (int)chi, TC, Wb, ewb, st)) != TGBA_OK) return r;
-        if ((r = emu_gemm(b, Va, eva, kp, (int)chi, Wb, ewb, kp, (int)chi, dtg, (int)tlo.size(), cl, Gam, kp, st)) != TGBA_OK)
+        if ((r = emu_gemm(b, Va, eva, kp, (int)chi, Wb, ewb, kp, (int)chi, TC, dtg, (int)tlo.size(), cl, Gam, kp, st)) != TGBA_OK)
           return r;
         symmetrise<<<blocks_for((int64_t)kp * kp), 256, 0, st>>>(kp, Gam);
         ++b.launches;
@@ -728,7 +770,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
         if ((r = emu_slice(b, Gam, kp, 1, kp, 0, nullptr, 0.0, kp, kp, TR, Va, eva, st)) != TGBA_OK) return r;
         if ((r = emu_slice(b, Ab + (size_t)p * nt, 1, 2 * nt, kp, 0, nullptr, 0.0, (int)nt, kp, TC, Wb, ewb, st)) != TGBA_OK)
           return r;
-        if ((r = emu_gemm(b, Va, eva, kp, kp, Wb, ewb, (int)nt, kp, dtg, (int)tt.size(), ct, GA[p], kp, st)) != TGBA_OK)
+        if ((r = emu_gemm(b, Va, eva, kp, kp, Wb, ewb, (int)nt, kp, TC, dtg, (int)tt.size(), ct, GA[p], kp, st)) != TGBA_OK)
           return r;
         TGBA_CUDA(ev.mark(st));
       }

@@ -72,11 +72,9 @@ constexpr int kTMr = 128;                 // rows of A per tile
 constexpr int kTNr = 128;                 // rows of B per tile
 constexpr int kChunkBlocks = 8;           // K blocks per exact FP32 chunk (256 K values)
 constexpr uint32_t kASlice = kTMr * kKB * 2;          // 8 KB
-constexpr uint32_t kBSlice = kTNr * kKB * 2;          // 8 KB
-constexpr uint32_t kAStage = kS * kASlice;            // 48 KB
-constexpr uint32_t kBStage = kS * kBSlice;            // 48 KB
-constexpr int kStages = 2;
-constexpr uint32_t kSmem = 1024 + kStages * (kAStage + kBStage) + 256;
+constexpr int kMaxStages = 4;
+constexpr uint32_t kSmemStages = 221184;              // 216 KB for the stages
+constexpr uint32_t kSmemMax = 1024 + kSmemStages + 256;
 constexpr unsigned kWait = 1u << 24;                   // polls of a bounded wait
 constexpr int kThreads = 320;
 constexpr int kEpiWarps = 8;
@@ -170,47 +168,41 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
 struct GemmArgs {
   EmuTile* tiles;             // the output tiles, numbered by emu_number_tiles (arrival counters at 0)
   int n_tiles;
-  int64_t n_chunks;           // chunks of all tiles (a chunk: kChunkBlocks K blocks of one tile)
-  const __nv_bfloat16* A;     // [row block][K block][slice] tile images
-  const __nv_bfloat16* B;
-  int a_kb, b_kb;             // K blocks per row block of A / of B (the stride between row blocks)
-  const int* ea;              // row exponents of A [M]
-  const int* eb;              // row exponents of B [N]
-  int M, N;
-  double* C;                  // C[i + j ldc]
-  int64_t ldc;
+  int64_t n_blocks;           // K blocks of all tiles
+  EmuSet set[2];              // operands and outputs; a tile names its set
+  int tb;                     // rows of a B tile image: 16, 32, 64 or 128
+  int stages;                 // shared-memory stages
   double* part;               // [2 gridDim.x][kTNr][kTMr] partial tiles of the split tiles
   unsigned* status;
 };
 
-// Work split (stream-K): the chunks of all tiles, tile after tile, are cut into gridDim.x
-// contiguous ranges of equal length, one per CTA.  A tile whose chunks fall to several CTAs is
+// Work split (stream-K): the K blocks of all tiles, tile after tile, are cut into gridDim.x
+// contiguous ranges of equal length, one per CTA.  A tile whose blocks fall to several CTAs is
 // a split tile: each of them writes its partial sum to a slot of g.part, and the last to arrive
 // (an atomic counter in the tile; no CTA waits for another) adds the partials in CTA order and
 // writes C, so the result does not depend on the arrival order.
 __device__ __forceinline__ int64_t range_start(int c, int64_t T, int G) { return (int64_t)c * T / G; }
-__device__ __forceinline__ int cta_of(int64_t x, int64_t T, int G) {    // the CTA whose range holds chunk x
+__device__ __forceinline__ int cta_of(int64_t x, int64_t T, int G) {    // the CTA whose range holds block x
   return (int)(((x + 1) * G + T - 1) / T) - 1;
 }
-__device__ __forceinline__ int64_t tile_chunks(const EmuTile& t) { return (t.nkb + kChunkBlocks - 1) / kChunkBlocks; }
 
 struct Seg {
   int t;                      // tile
   int kb0, kb1;               // K blocks [kb0, kb1) of the tile
   bool whole;                 // the segment is the whole tile
 };
-// the segment of tile t from chunk c on (c inside tile t), clipped at the CTA's range end; false past it
+// the segment of tile t from block c on (c inside tile t), clipped at the CTA's range end; false past it
 __device__ __forceinline__ bool seg_at(const GemmArgs& g, int t, int64_t c, int64_t c_end, Seg& s) {
   if (t >= g.n_tiles || c >= c_end) return false;
-  const EmuTile tl = g.tiles[t];
-  const int64_t n = tile_chunks(tl), s0 = c - tl.c0, s1 = min(n, c_end - tl.c0);
+  const int64_t c0 = g.tiles[t].c0;
+  const int nkb = g.tiles[t].nkb;
   s.t = t;
-  s.kb0 = (int)(s0 * kChunkBlocks);
-  s.kb1 = (int)min((int64_t)tl.nkb, s1 * kChunkBlocks);
-  s.whole = s0 == 0 && s1 == n;
+  s.kb0 = (int)(c - c0);
+  s.kb1 = (int)min((int64_t)nkb, c_end - c0);
+  s.whole = s.kb0 == 0 && s.kb1 == nkb;
   return true;
 }
-__device__ __forceinline__ int first_tile(const GemmArgs& g, int64_t c) {   // the tile holding chunk c
+__device__ __forceinline__ int first_tile(const GemmArgs& g, int64_t c) {   // the tile holding block c
   int lo = 0, hi = g.n_tiles - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -228,29 +220,55 @@ __device__ __forceinline__ int active_cols(const EmuTile& tl, int kb) {
   return n;
 }
 
+// The MMAs of one K block: the slice pairs (p, q) with p + q < NS, each as two K = 16 steps, into the
+// accumulator of digit diagonal min(p + q, 3).  Fully unrolled: one thread issues them, and computing
+// the descriptors in loops took it longer than the MMAs take at N = 16 (measured on the L = 80 quench's
+// 2750 x 16 x 2650 products: 100 us each, 50 us per 256 K values).  `fresh`: the chunk's first block,
+// whose first MMA of each accumulator overwrites it.
+template <int NS>
+__device__ __forceinline__ void issue_block(uint32_t d0, uint32_t acc_cols, uint64_t a0, uint64_t b0, uint32_t bq,
+                                            uint32_t id, bool fresh) {
+#pragma unroll
+  for (int p = 0; p < NS; ++p)
+#pragma unroll
+    for (int q = 0; q + p < NS; ++q) {
+      const int d = p + q < 3 ? p + q : 3;
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks)
+        mma(d0 + (uint32_t)d * acc_cols, a0 + (uint64_t)((p * kASlice + ks * 32) >> 4),
+            b0 + (uint64_t)((uint32_t)q * bq + ks * 2), id, (fresh && p == 0 && q < 4 && ks == 0) ? 0u : 1u);
+    }
+}
+
 // NS: slices used per operand, kS (the FP64 product) or 2 (the two leading digits: ~2^-16)
 template <int NS>
 __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads x 168 registers, one CTA per SM
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = su32(smem_raw);
   unsigned char* base = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  unsigned char* sA = base;                                  // [stage] A slices
-  unsigned char* sB = base + kStages * kAStage;              // [stage] B slices
-  uint64_t* bars = (uint64_t*)(sB + kStages * kBStage);
-  uint64_t* full = bars;               // [kStages] stage loaded
-  uint64_t* empty = bars + kStages;    // [kStages] stage consumed by the MMAs
-  uint64_t* accf = bars + 2 * kStages; // accumulators written (one set)
-  uint64_t* acce = accf + 1;           // accumulators read
-  uint32_t* tslot = (uint32_t*)(acce + 1);
+  const uint32_t b_slice = (uint32_t)g.tb * 64u, stage_bytes = (uint32_t)NS * (kASlice + b_slice);
+  const int n_st = g.stages;
+  // two sets of accumulators when a tile's columns leave room for them in the 512 of TMEM: the fold
+  // of one chunk then overlaps the MMAs of the next
+  const int n_acc = g.tb <= 64 ? 2 : 1;
+  const uint32_t acc_cols = g.tb <= 64 ? 64u : 128u;
+  uint64_t* bars = (uint64_t*)(base + (size_t)n_st * stage_bytes);
+  uint64_t* full = bars;                   // [kMaxStages] stage loaded
+  uint64_t* empty = bars + kMaxStages;     // [kMaxStages] stage consumed by the MMAs
+  uint64_t* accf = bars + 2 * kMaxStages;  // [2] accumulators written
+  uint64_t* acce = accf + 2;               // [2] accumulators read
+  uint32_t* tslot = (uint32_t*)(acce + 2);
   __shared__ volatile int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < n_st; ++s) {
       bar_init(full + s, 1);
       bar_init(empty + s, 1);
     }
-    bar_init(accf, 1);
-    bar_init(acce, kEpiWarps);
+    for (int s = 0; s < 2; ++s) {
+      bar_init(accf + s, 1);
+      bar_init(acce + s, kEpiWarps);
+    }
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -263,75 +281,74 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
   fence_after();
   const uint32_t tmem = *tslot;
   const int G = gridDim.x;
-  const int64_t T = g.n_chunks, c_begin = range_start(blockIdx.x, T, G), c_end = range_start(blockIdx.x + 1, T, G);
+  const int64_t T = g.n_blocks, c_begin = range_start(blockIdx.x, T, G), c_end = range_start(blockIdx.x + 1, T, G);
   const int t_first = first_tile(g, c_begin);
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
     if (lane == 0) {
       uint32_t it = 0;
+      int st = 0;
+      unsigned ph = 1;                                  // parity of the wait on `empty`
       Seg sg{t_first - 1, 0, 0, false};
       for (int64_t c = c_begin; !s_abort && seg_at(g, sg.t + 1, c, c_end, sg);
-           c = g.tiles[sg.t].c0 + tile_chunks(g.tiles[sg.t])) {
-        const EmuTile tl = g.tiles[sg.t];
+           c = g.tiles[sg.t].c0 + g.tiles[sg.t].nkb) {
+        const EmuTile& tl = g.tiles[sg.t];
+        const EmuSet& op = g.set[tl.set];
+        const unsigned char* pa = (const unsigned char*)op.A + ((size_t)tl.rb * op.a_kb + sg.kb0) * (kS * kASlice);
+        const unsigned char* pb = (const unsigned char*)op.B + ((size_t)tl.cb * op.b_kb + sg.kb0) * (kS * b_slice);
         for (int kb = sg.kb0; kb < sg.kb1; ++kb, ++it) {
-          const int st = it % kStages;
-          if (!bar_wait(empty + st, ((it / kStages) & 1u) ^ 1u, &s_abort)) { atomicOr(g.status, kStTimeout); s_abort = 1; break; }
-          // the first ns slices of a K block are the first ns x 8 KB of its image
-          bar_expect(full + st, (uint32_t)NS * (kASlice + kBSlice));
-          bulk_load(sA + st * kAStage, g.A + ((size_t)tl.rb * g.a_kb + kb) * (kAStage / 2), (uint32_t)NS * kASlice,
-                    full + st);
-          bulk_load(sB + st * kBStage, g.B + ((size_t)tl.cb * g.b_kb + kb) * (kBStage / 2), (uint32_t)NS * kBSlice,
-                    full + st);
+          if (!bar_wait(empty + st, ph, &s_abort)) { atomicOr(g.status, kStTimeout); s_abort = 1; break; }
+          // the first NS slices of a K block are the first bytes of its image
+          bar_expect(full + st, stage_bytes);
+          unsigned char* dst = base + (size_t)st * stage_bytes;
+          bulk_load(dst, pa, (uint32_t)NS * kASlice, full + st);
+          bulk_load(dst + NS * kASlice, pb, (uint32_t)NS * b_slice, full + st);
+          pa += kS * kASlice;
+          pb += kS * b_slice;
+          if (++st == n_st) { st = 0; ph ^= 1u; }
         }
       }
       if (s_abort) {                                  // copies still in flight land before the CTA leaves
         const volatile int never = 0;
-        for (uint32_t j = (it >= kStages ? it - kStages : 0); j < it; ++j)
-          bar_wait(full + (j % kStages), (j / kStages) & 1u, (volatile int*)&never);
+        for (uint32_t j = (it >= (uint32_t)n_st ? it - n_st : 0); j < it; ++j)
+          bar_wait(full + (j % n_st), (j / n_st) & 1u, (volatile int*)&never);
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0) {
-      uint32_t it = 0, chunk = 0;
+      uint32_t chunk = 0;
+      int st = 0;
+      unsigned ph = 0;                                  // parity of the wait on `full`
       uint64_t* last = nullptr;
       Seg sg{t_first - 1, 0, 0, false};
       for (int64_t c = c_begin; !s_abort && seg_at(g, sg.t + 1, c, c_end, sg);
-           c = g.tiles[sg.t].c0 + tile_chunks(g.tiles[sg.t])) {
+           c = g.tiles[sg.t].c0 + g.tiles[sg.t].nkb) {
         const EmuTile tl = g.tiles[sg.t];
         for (int kb0 = sg.kb0; kb0 < sg.kb1 && !s_abort; kb0 += kChunkBlocks, ++chunk) {
-          // the epilogue has read the previous chunk's accumulators
-          if (!bar_wait(acce, (chunk & 1u) ^ 1u, &s_abort)) { atomicOr(g.status, kStTimeout); s_abort = 1; break; }
+          // the epilogue has read this set's previous chunk
+          const int as = n_acc == 2 ? (int)(chunk & 1u) : 0;
+          const unsigned use = n_acc == 2 ? chunk >> 1 : chunk;
+          if (!bar_wait(acce + as, (use & 1u) ^ 1u, &s_abort)) { atomicOr(g.status, kStTimeout); s_abort = 1; break; }
           fence_after();
           const int kb1 = min(sg.kb1, kb0 + kChunkBlocks);
-          for (int kb = kb0; kb < kb1; ++kb, ++it) {
-            const int st = it % kStages;
-            if (!bar_wait(full + st, (it / kStages) & 1u, &s_abort)) { atomicOr(g.status, kStTimeout); s_abort = 1; break; }
-            fence_after();
+          for (int kb = kb0; kb < kb1; ++kb) {
             // columns whose K extent ends before this block are skipped (their rows of B are zero
             // there); the chunk's first block touches the most columns, so its MMAs initialise
             // every column that the epilogue reads
             const uint32_t id = idesc_f16(active_cols(tl, kb));
-            const uint32_t a0 = su32(sA + st * kAStage), b0 = su32(sB + st * kBStage);
-#pragma unroll 1
-            for (int p = 0; p < NS; ++p)
-#pragma unroll 1
-              for (int q = 0; p + q < NS; ++q) {
-                const int d = min(p + q, 3);
-                // first write of accumulator d in this chunk overwrites it: pair (0, d) for d <= 2,
-                // (0, 3) for the shared one, at the chunk's first K block
-                const bool first = kb == kb0 && p == 0 && q == (d < 3 ? d : 3);
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks)
-                  mma(tmem + (uint32_t)d * 128u, desc64(a0 + p * kASlice + ks * 32), desc64(b0 + q * kBSlice + ks * 32), id,
-                      (first && ks == 0) ? 0u : 1u);
-              }
+            const uint32_t a0 = su32(base + (size_t)st * stage_bytes);
+            const uint64_t da = desc64(a0), db = desc64(a0 + NS * kASlice);
+            if (!bar_wait(full + st, ph, &s_abort)) { atomicOr(g.status, kStTimeout); s_abort = 1; break; }
+            fence_after();
+            issue_block<NS>(tmem + (uint32_t)as * 256u, acc_cols, da, db, b_slice >> 4, id, kb == kb0);
             commit(empty + st);                       // the stage's smem is free once these complete
             last = empty + st;
+            if (++st == n_st) { st = 0; ph ^= 1u; }
           }
-          commit(accf);                               // the chunk's accumulators are complete
-          last = accf;
+          commit(accf + as);                          // the chunk's accumulators are complete
+          last = accf + as;
         }
       }
       if (s_abort && last) {                          // MMAs still in flight finish before the dealloc
@@ -342,34 +359,38 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2-9)
-    constexpr int kCols = kTNr / 2;                   // columns per epilogue warp
+    constexpr int kCols = kTNr / 2;                   // most columns per epilogue warp
+    const int kc = g.tb <= 64 ? 32 : kCols;           // columns per epilogue warp
     const int quad = warp & 3;                        // TMEM lanes 32 quad .. 32 quad + 31
-    const int half = (warp - 2) >> 2;                 // columns kCols half .. kCols half + kCols - 1
+    const int half = (warp - 2) >> 2;                 // columns kc half .. kc half + kc - 1
     const int r = quad * 32 + lane;                   // row of the tile
     uint32_t chunk = 0;
     Seg sg{t_first - 1, 0, 0, false};
     for (int64_t c = c_begin; !s_abort && seg_at(g, sg.t + 1, c, c_end, sg);
-         c = g.tiles[sg.t].c0 + tile_chunks(g.tiles[sg.t])) {
+         c = g.tiles[sg.t].c0 + g.tiles[sg.t].nkb) {
       const EmuTile tl = g.tiles[sg.t];
+      const EmuSet& op = g.set[tl.set];
       float hi[kCols], lo[kCols];                     // registers: every index below is a constant
 #pragma unroll
       for (int cc = 0; cc < kCols; ++cc) { hi[cc] = 0.f; lo[cc] = 0.f; }
       for (int kb0 = sg.kb0; kb0 < sg.kb1; kb0 += kChunkBlocks, ++chunk) {
-        if (!bar_wait(accf, chunk & 1u, &s_abort)) {
+        const int as = n_acc == 2 ? (int)(chunk & 1u) : 0;
+        const unsigned use = n_acc == 2 ? chunk >> 1 : chunk;
+        if (!bar_wait(accf + as, use & 1u, &s_abort)) {
           if (lane == 0) atomicOr(g.status, kStTimeout);
           s_abort = 1;
           break;
         }
         fence_after();
         const int na = active_cols(tl, kb0);          // columns the chunk's MMAs wrote
-        const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * kCols);
+        const uint32_t lane_base = tmem + (uint32_t)as * 256u + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * kc);
 #pragma unroll
         for (int h = 0; h < kCols / 16; ++h) {
-          if (half * kCols + h * 16 < na) {
+          if (h * 16 < kc && half * kc + h * 16 < na) {
 #pragma unroll
             for (int d = 0; d < (NS < 4 ? NS : 4); ++d) {   // with 2 slices only diagonals 0 and 1 are written
               float v[16];
-              ld16(lane_base + (uint32_t)d * (uint32_t)kTNr + (uint32_t)h * 16u, v);
+              ld16(lane_base + (uint32_t)d * acc_cols + (uint32_t)h * 16u, v);
 #pragma unroll
               for (int j = 0; j < 16; ++j) two_sum_add(hi[h * 16 + j], lo[h * 16 + j], v[j]);
             }
@@ -377,19 +398,19 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
         }
         fence_before();
         __syncwarp();
-        if (lane == 0) bar_arrive(acce);
+        if (lane == 0) bar_arrive(acce + as);
       }
       if (s_abort) break;
       const int i = tl.rb * kTMr + r;
-      const int c_lo = half * kCols;
+      const int c_lo = half * kc;
       if (sg.whole) {
-        if (i < g.M) {
-          const int e_i = g.ea[i];
+        if (i < op.M) {
+          const int e_i = op.ea[i];
 #pragma unroll
           for (int cc = 0; cc < kCols; ++cc) {
             const int j = tl.cb * kTNr + c_lo + cc;
-            if (c_lo + cc < tl.n_eff && j < g.N)
-              g.C[(int64_t)i + (int64_t)j * g.ldc] = ldexp((double)hi[cc] + (double)lo[cc], e_i + g.eb[j] - 16);
+            if (cc < kc && c_lo + cc < tl.n_eff && j < op.N)
+              op.C[(int64_t)i + (int64_t)j * op.ldc] = ldexp((double)hi[cc] + (double)lo[cc], e_i + op.eb[j] - 16);
           }
         }
         continue;
@@ -399,27 +420,28 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
       double* mine = g.part + (size_t)slot * kTNr * kTMr;
 #pragma unroll
       for (int cc = 0; cc < kCols; ++cc)
-        if (c_lo + cc < tl.n_eff) mine[(size_t)(c_lo + cc) * kTMr + r] = (double)hi[cc] + (double)lo[cc];
-      // the last of the tile's CTAs to finish this warp's 32 x 64 block adds the parts (no waiting)
+        if (cc < kc && c_lo + cc < tl.n_eff) mine[(size_t)(c_lo + cc) * kTMr + r] = (double)hi[cc] + (double)lo[cc];
+      // the last of the tile's CTAs to finish this warp's block adds the parts (no waiting)
       __threadfence();
       __syncwarp();
-      const int c_a = cta_of(tl.c0, T, G), c_b = cta_of(tl.c0 + tile_chunks(tl) - 1, T, G);
+      const int c_a = cta_of(tl.c0, T, G), c_b = cta_of(tl.c0 + tl.nkb - 1, T, G);
       int last = 0;
       if (lane == 0) last = atomicAdd(&g.tiles[sg.t].arrivals[warp - 2], 1) == c_b - c_a;
       if (__shfl_sync(0xffffffffu, last, 0)) {
         __threadfence();
-        if (i < g.M) {
-          const int e_i = g.ea[i];
+        if (i < op.M) {
+          const int e_i = op.ea[i];
+          const int nc = min(kc, tl.n_eff - c_lo);
 #pragma unroll 4
-          for (int cc = 0; cc < kCols; ++cc) {
+          for (int cc = 0; cc < nc; ++cc) {
             const int j = tl.cb * kTNr + c_lo + cc;
-            if (c_lo + cc < tl.n_eff && j < g.N) {
+            if (j < op.N) {
               double v = 0.0;
               for (int cta = c_a; cta <= c_b; ++cta) {
                 const int sl = 2 * cta + (range_start(cta, T, G) >= tl.c0 ? 0 : 1);
                 v += __ldcg(g.part + (size_t)sl * kTNr * kTMr + (size_t)(c_lo + cc) * kTMr + r);
               }
-              g.C[(int64_t)i + (int64_t)j * g.ldc] = ldexp(v, e_i + g.eb[j] - 16);
+              op.C[(int64_t)i + (int64_t)j * op.ldc] = ldexp(v, e_i + op.eb[j] - 16);
             }
           }
         }
@@ -444,6 +466,12 @@ __device__ __forceinline__ double weighted(const double* __restrict__ src, int64
   return w ? x * (w[k] - w_shift) : x;
 }
 
+// smallest e with x < 2^e for the magnitude bits m of x (0 for m = 0)
+__device__ __forceinline__ int exponent_of(unsigned long long m) {
+  const int ef = (int)(m >> 52);                       // biased exponent
+  return m == 0ull ? 0 : (ef == 0 ? -1021 : ef - 1022);
+}
+
 // Row exponents: e[i] = smallest e with max_k |X(i, k)| < 2^e (0 for a zero row), from the
 // largest magnitude's exponent field (integer maximum of the magnitudes' bit patterns).  One
 // warp per row.
@@ -462,10 +490,7 @@ __global__ void row_exponents(int rows, int K, const double* __restrict__ src, i
       m = max(m, bits);
     }
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) {
-      const int ef = (int)(m >> 52);                     // biased exponent of the largest magnitude
-      e[i] = m == 0ull ? 0 : (ef == 0 ? -1021 : ef - 1022);   // max < 2^(ef - 1022)
-    }
+    if (lane == 0) e[i] = exponent_of(m);
   }
 }
 
@@ -491,10 +516,41 @@ __global__ void row_exponents_long(int rows, int K, const double* __restrict__ s
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int q = 1; q < (int)(blockDim.x >> 5); ++q) m = max(m, s_m[q]);
-      const int ef = (int)(m >> 52);
-      e[i] = m == 0ull ? 0 : (ef == 0 ? -1021 : ef - 1022);
+      e[i] = exponent_of(m);
     }
     __syncthreads();
+  }
+}
+
+// x 2^(48 - e), |x| < 2^e, as a rounded integer (from the mantissa and exponent fields)
+__device__ __forceinline__ long long fixed48(double x, int e) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+  const int ef = (int)((bits >> 52) & 0x7ff);
+  if (ef == 0) return 0;                               // subnormals are below 2^-1022: they round to 0
+  const long long mant = (long long)((bits & 0x000fffffffffffffull) | 0x0010000000000000ull);
+  // |x| = mant 2^(ef - 1075); F = |x| 2^(48 - e) = mant 2^(ef - 1027 - e), a right shift
+  const int sh = 1027 + e - ef;
+  long long f = 0;
+  if (sh <= 0) f = mant << (-sh);                      // only for |x| at the top of the range
+  else if (sh < 63) f = (mant + (1ll << (sh - 1))) >> sh;
+  return (bits >> 63) ? -f : f;
+}
+// the six digits of 8 consecutive K values, one 16-byte store per slice
+__device__ __forceinline__ void store_digits(long long (&F)[8], unsigned char* tile, uint32_t slice_bytes) {
+#pragma unroll
+  for (int p = 0; p < kS; ++p) {
+    const int shp = 40 - 8 * p;
+    uint32_t packed[4];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const long long d = shp > 0 ? ((F[u] + (1ll << (shp - 1))) >> shp) : F[u];
+      F[u] -= d << shp;
+      // d 2^(-8p): |d| <= 256, exact in FP32 and in BF16
+      const uint32_t h = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(ldexpf((float)d, -8 * p)));
+      if (u & 1) packed[u >> 1] |= h << 16;
+      else packed[u >> 1] = h;
+    }
+    *(uint4*)(tile + (size_t)p * slice_bytes) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
   }
 }
 
@@ -524,36 +580,34 @@ __global__ void slice_tiles(int rows, int K, const double* __restrict__ src, int
       F[u] = 0;
       if (i < rows && k < K) {
         const int64_t off = (int64_t)i * row_stride + (int64_t)k * k_stride + (k >= k_split ? k_jump : 0);
-        const unsigned long long bits = (unsigned long long)__double_as_longlong(weighted(src, off, w, w_shift, k));
-        const int ef = (int)((bits >> 52) & 0x7ff);
-        if (ef != 0) {                                   // subnormals are below 2^-1022: they round to 0
-          const long long mant = (long long)((bits & 0x000fffffffffffffull) | 0x0010000000000000ull);
-          // |x| = mant 2^(ef - 1075); F = |x| 2^(48 - e) = mant 2^(ef - 1027 - e), a right shift
-          const int sh = 1027 + e[i] - ef;
-          long long f = 0;
-          if (sh <= 0) f = mant << (-sh);                // only for |x| at the top of the range
-          else if (sh < 63) f = (mant + (1ll << (sh - 1))) >> sh;
-          F[u] = (bits >> 63) ? -f : f;
-        }
+        F[u] = fixed48(weighted(src, off, w, w_shift, k), e[i]);
       }
     }
-    unsigned char* tile = (unsigned char*)out + ((size_t)rb * n_kb + kb) * kS * slice_bytes + sw64(r, kk);
-#pragma unroll
-    for (int p = 0; p < kS; ++p) {
-      const int shp = 40 - 8 * p;
-      uint32_t packed[4];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const long long d = shp > 0 ? ((F[u] + (1ll << (shp - 1))) >> shp) : F[u];
-        F[u] -= d << shp;
-        // d 2^(-8p): |d| <= 256, exact in FP32 and in BF16
-        const uint32_t h = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(ldexpf((float)d, -8 * p)));
-        if (u & 1) packed[u >> 1] |= h << 16;
-        else packed[u >> 1] = h;
-      }
-      *(uint4*)(tile + (size_t)p * slice_bytes) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-    }
+    store_digits(F, (unsigned char*)out + ((size_t)rb * n_kb + kb) * kS * slice_bytes + sw64(r, kk), slice_bytes);
   }
+}
+
+// The slices of both halves of the propagation's vectors in one launch, with the exponents from the
+// magnitudes' maxima that the step kernel left (max_bits [column][half]): half 0 the rows from kn
+// on (kr of them, the operand of the NS rows' product), half 1 the first kn rows.  x: column-major,
+// leading dimension n; tile images of `tb` columns.
+__global__ void __launch_bounds__(128) slice_halves(int cols, int tb, int64_t n, int kn, int kr, const double* __restrict__ x,
+                                                    const unsigned long long* __restrict__ max_bits,
+                                                    __nv_bfloat16* __restrict__ out0, __nv_bfloat16* __restrict__ out1,
+                                                    int* __restrict__ e0, int* __restrict__ e1) {
+  const int half = blockIdx.z, K = half ? kn : kr, i = blockIdx.y;
+  const int n_kb = (K + kKB - 1) / kKB, k0 = (blockIdx.x * blockDim.x + threadIdx.x) * 8;
+  if (k0 >= n_kb * kKB) return;
+  const double* src = x + (size_t)i * n + (half ? 0 : kn);
+  const int e = i < cols ? exponent_of(max_bits[2 * i + half]) : 0;
+  long long F[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) F[u] = (i < cols && k0 + u < K) ? fixed48(src[k0 + u], e) : 0;
+  const uint32_t slice_bytes = (uint32_t)tb * kKB * 2;
+  const int rb = i / tb, r = i % tb;
+  store_digits(F, (unsigned char*)(half ? out1 : out0) + ((size_t)rb * n_kb + k0 / kKB) * kS * slice_bytes + sw64(r, k0 % kKB),
+               slice_bytes);
+  if (k0 == 0 && i < cols) (half ? e1 : e0)[i] = e;
 }
 
 }  // namespace
@@ -593,7 +647,7 @@ tgba_status emu_prepare(Basis& b) {
   if (b.device < 0 || b.device >= 64) return fail(TGBA_ELIMIT, "device index");
   if (sms_of[b.device] == 0) {
     for (const void* k : {(const void*)dgemm_tc_kernel<kS>, (const void*)dgemm_tc_kernel<2>}) {
-      TGBA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
+      TGBA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
       cudaFuncAttributes fa;
       TGBA_CUDA(cudaFuncGetAttributes(&fa, k));
       if (fa.maxThreadsPerBlock < kThreads) {
@@ -623,36 +677,69 @@ int64_t emu_number_tiles(std::vector<EmuTile>& tiles) {
       t.arrivals[q] = 0;
       if (t.gkb[q] <= 0 || t.gkb[q] > t.nkb) t.gkb[q] = (int16_t)t.nkb;   // unset: the tile's whole K
     }
-    c += (t.nkb + kChunkBlocks - 1) / kChunkBlocks;
+    c += t.nkb;
   }
   return c;
 }
 
+// rows of a B tile image for `cols` columns: the smallest of 16, 32, 64, 128 that holds them, so that
+// narrow products (the propagation of a few variants) load, and keep in a stage, only the columns
+// they have; beyond 128 columns there are several tiles of 128.
+int emu_tile_rows_b(int cols) { return cols <= 16 ? 16 : cols <= 32 ? 32 : cols <= 64 ? 64 : kTNr; }
+
+EmuSet emu_set(const __nv_bfloat16* A, const int* ea, int M, int Ka, const __nv_bfloat16* B, const int* eb, int N, int Kb,
+               double* C, int64_t ldc) {
+  EmuSet e;
+  e.A = A; e.B = B; e.ea = ea; e.eb = eb; e.M = M; e.N = N; e.C = C; e.ldc = ldc;
+  e.a_kb = (Ka + kKB - 1) / kKB;
+  e.b_kb = (Kb + kKB - 1) / kKB;
+  return e;
+}
+
 // C = A B^T for sliced operands (see emu_slice), over the given output tiles (numbered by
-// emu_number_tiles, n_chunks its result; emu_prepare first).
-tgba_status emu_gemm(Basis& b, const __nv_bfloat16* A, const int* ea, int M, int Ka, const __nv_bfloat16* B,
-                     const int* eb, int N, int Kb, EmuTile* d_tiles, int n_tiles, int64_t n_chunks, double* C,
-                     int64_t ldc, cudaStream_t st, int n_slices) {
+// emu_number_tiles, n_blocks its result; emu_prepare first).  tb: the rows of B's tile images.
+tgba_status emu_gemm_sets(Basis& b, const EmuSet* sets, int n_sets, int tb, EmuTile* d_tiles, int n_tiles,
+                          int64_t n_blocks, cudaStream_t st, int n_slices) {
   if (n_slices != 2 && n_slices != kS) return fail(TGBA_EINVAL, "emu_gemm: 2 or 6 slices");
   if (n_tiles == 0) return TGBA_OK;
   if (b.emu_sms <= 0 || !b.d_emu_part) return fail(TGBA_EINVAL, "emu_prepare was not called");
-  if (n_chunks < n_tiles) return fail(TGBA_EINVAL, "tiles not numbered (emu_number_tiles)");
+  if (n_blocks < n_tiles) return fail(TGBA_EINVAL, "tiles not numbered (emu_number_tiles)");
   GemmArgs g;
-  g.tiles = d_tiles; g.n_tiles = n_tiles; g.n_chunks = n_chunks;
-  g.A = A; g.B = B;
-  g.a_kb = (Ka + kKB - 1) / kKB;
-  g.b_kb = (Kb + kKB - 1) / kKB;
-  g.ea = ea; g.eb = eb; g.M = M; g.N = N; g.C = C; g.ldc = ldc; g.part = b.d_emu_part; g.status = b.d_status;
-  const int grid = (int)std::min<int64_t>(n_chunks, b.emu_sms);
-  if (n_slices == kS) dgemm_tc_kernel<kS><<<grid, kThreads, kSmem, st>>>(g);
-  else dgemm_tc_kernel<2><<<grid, kThreads, kSmem, st>>>(g);
+  g.tiles = d_tiles; g.n_tiles = n_tiles; g.n_blocks = n_blocks;
+  for (int i = 0; i < 2; ++i) g.set[i] = sets[i < n_sets ? i : 0];
+  g.tb = tb;
+  const uint32_t stage = (uint32_t)n_slices * (kASlice + (uint32_t)tb * 64u);
+  g.stages = std::min<int>(kMaxStages, (int)(kSmemStages / stage));
+  g.part = b.d_emu_part; g.status = b.d_status;
+  const size_t smem = 1024 + (size_t)g.stages * stage + 256;
+  const int grid = (int)std::min<int64_t>(n_blocks, b.emu_sms);
+  if (n_slices == kS) dgemm_tc_kernel<kS><<<grid, kThreads, smem, st>>>(g);
+  else dgemm_tc_kernel<2><<<grid, kThreads, smem, st>>>(g);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
+  return TGBA_OK;
+}
+
+tgba_status emu_gemm(Basis& b, const __nv_bfloat16* A, const int* ea, int M, int Ka, const __nv_bfloat16* B,
+                     const int* eb, int N, int Kb, int tb, EmuTile* d_tiles, int n_tiles, int64_t n_blocks, double* C,
+                     int64_t ldc, cudaStream_t st, int n_slices) {
+  const EmuSet e = emu_set(A, ea, M, Ka, B, eb, N, Kb, C, ldc);
+  return emu_gemm_sets(b, &e, 1, tb, d_tiles, n_tiles, n_blocks, st, n_slices);
+}
+
+tgba_status emu_slice_halves(Basis& b, const double* x, int64_t n, int cols, int kn, int kr,
+                             const unsigned long long* max_bits, __nv_bfloat16* out0, __nv_bfloat16* out1, int* e0, int* e1,
+                             cudaStream_t st) {
+  const int tb = emu_tile_rows_b(cols), rows = (cols + tb - 1) / tb * tb, K = std::max(kn, kr);
+  const int threads8 = (K + kKB - 1) / kKB * (kKB / 8);
+  slice_halves<<<dim3((unsigned)((threads8 + 127) / 128), (unsigned)rows, 2), 128, 0, st>>>(cols, tb, n, kn, kr, x, max_bits,
+                                                                                         out0, out1, e0, e1);
   TGBA_CUDA(cudaGetLastError());
   ++b.launches;
   return TGBA_OK;
 }
 
 int emu_tile_rows_a() { return kTMr; }
-int emu_tile_rows_b() { return kTNr; }
 int emu_k_block() { return kKB; }
 
 }  // namespace tgba
@@ -666,14 +753,14 @@ extern "C" tgba_status tgba_dgemm_tc(int32_t M, int32_t N, int32_t K, const doub
   cudaStream_t st = (cudaStream_t)stream;
   Basis ctx;
   TGBA_CUDA(cudaGetDevice(&ctx.device));
-  const size_t ea = emu_operand_elems(M, K, emu_tile_rows_a()), eb = emu_operand_elems(N, K, emu_tile_rows_b());
-  const int TR = emu_tile_rows_a(), TC = emu_tile_rows_b(), KB = emu_k_block();
+  const size_t ea = emu_operand_elems(M, K, emu_tile_rows_a()), eb = emu_operand_elems(N, K, emu_tile_rows_b(N));
+  const int TR = emu_tile_rows_a(), TC = kTNr, TB = emu_tile_rows_b(N), KB = emu_k_block();
   std::vector<EmuTile> tiles;
   for (int rb = 0; rb < (M + TR - 1) / TR; ++rb)
     for (int cb = 0; cb < (N + TC - 1) / TC; ++cb)
       tiles.push_back(EmuTile{rb, cb, std::min(TC, (N - cb * TC + 15) / 16 * 16), (K + KB - 1) / KB});
-  const int64_t n_chunks = emu_number_tiles(tiles);
-  if (n_chunks < 0) return fail(TGBA_EINVAL, "tile list");
+  const int64_t n_blocks = emu_number_tiles(tiles);
+  if (n_blocks < 0) return fail(TGBA_EINVAL, "tile list");
   int sms = 0;
   TGBA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx.device));
   void* buf = nullptr;
@@ -692,8 +779,8 @@ extern "C" tgba_status tgba_dgemm_tc(int32_t M, int32_t N, int32_t K, const doub
   TGBA_CUDA(cudaMemcpyAsync(dt, tiles.data(), tiles.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
   tgba_status r = emu_prepare(ctx);
   if (r == TGBA_OK) r = emu_slice(ctx, A, lda, 1, K, 0, nullptr, 0.0, M, K, TR, As, xa, st);
-  if (r == TGBA_OK) r = emu_slice(ctx, B, ldb, 1, K, 0, nullptr, 0.0, N, K, TC, Bs, xb, st);
-  if (r == TGBA_OK) r = emu_gemm(ctx, As, xa, M, K, Bs, xb, N, K, dt, (int)tiles.size(), n_chunks, C, ldc, st);
+  if (r == TGBA_OK) r = emu_slice(ctx, B, ldb, 1, K, 0, nullptr, 0.0, N, K, TB, Bs, xb, st);
+  if (r == TGBA_OK) r = emu_gemm(ctx, As, xa, M, K, Bs, xb, N, K, TB, dt, (int)tiles.size(), n_blocks, C, ldc, st);
   if (r != TGBA_OK) return r;
   unsigned w = 0;
   TGBA_CUDA(cudaMemcpyAsync(&w, ctx.d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, st));

@@ -289,23 +289,44 @@ tgba_status run_elements_big(Basis& b, cudaStream_t st);
 // arrival counters, which the kernel leaves at zero again.
 struct EmuTile {
   int32_t rb, cb, n_eff, nkb;
-  int64_t c0;                 // first chunk of the tile in the list's order
+  int64_t c0;                 // first K block of the tile in the list's order
   int32_t arrivals[8];        // CTAs done with each epilogue warp's block of a split tile
   int16_t gkb[8];             // K blocks per 16-column group
+  int32_t set = 0;            // operands of the tile in a launch with two sets
+};
+struct EmuSet {               // one product C = A B^T of a launch
+  const __nv_bfloat16* A;     // [row block][K block][slice] tile images
+  const __nv_bfloat16* B;
+  int a_kb, b_kb;             // K blocks per row block of A / of B (the stride between row blocks)
+  const int* ea;              // row exponents of A [M]
+  const int* eb;              // row exponents of B [N]
+  int M, N;
+  double* C;                  // C[i + j ldc]
+  int64_t ldc;
 };
 size_t emu_operand_elems(int rows, int K, int tile_rows);
 int emu_tile_rows_a();
-int emu_tile_rows_b();
+int emu_tile_rows_b(int cols);   // rows of B's tile images for a product of `cols` columns
+constexpr int kEmuTileCols = 128;   // columns of an output tile
 int emu_k_block();
 tgba_status emu_slice(Basis& b, const double* src, int64_t row_stride, int64_t k_stride, int k_split, int64_t k_jump,
                       const double* w, double w_shift, int rows, int K, int tile_rows, __nv_bfloat16* out, int* e,
                       cudaStream_t st);
 tgba_status emu_prepare(Basis& b);
 size_t emu_part_bytes(int sms);
-int64_t emu_number_tiles(std::vector<EmuTile>& tiles);     // total chunks; -1 for an invalid tile
+int64_t emu_number_tiles(std::vector<EmuTile>& tiles);     // total K blocks; -1 for an invalid tile
 tgba_status emu_gemm(Basis& b, const __nv_bfloat16* A, const int* ea, int M, int Ka, const __nv_bfloat16* B,
-                     const int* eb, int N, int Kb, EmuTile* d_tiles, int n_tiles, int64_t n_chunks, double* C,
+                     const int* eb, int N, int Kb, int tb, EmuTile* d_tiles, int n_tiles, int64_t n_blocks, double* C,
                      int64_t ldc, cudaStream_t st, int n_slices = 6);   // 2: only the two leading digits (~2^-16)
+EmuSet emu_set(const __nv_bfloat16* A, const int* ea, int M, int Ka, const __nv_bfloat16* B, const int* eb, int N, int Kb,
+               double* C, int64_t ldc);
+tgba_status emu_gemm_sets(Basis& b, const EmuSet* sets, int n_sets, int tb, EmuTile* d_tiles, int n_tiles,
+                          int64_t n_blocks, cudaStream_t st, int n_slices = 6);
+// slices of both halves of the vectors x (column-major n x cols): out0 the rows kn .. kn + kr - 1, out1 the
+// rows 0 .. kn - 1; max_bits [cols][2]: magnitude bits of the largest entry of each column's halves
+tgba_status emu_slice_halves(Basis& b, const double* x, int64_t n, int cols, int kn, int kr,
+                             const unsigned long long* max_bits, __nv_bfloat16* out0, __nv_bfloat16* out1, int* e0, int* e1,
+                             cudaStream_t st);
 
 // screen.cu
 struct Screen;
