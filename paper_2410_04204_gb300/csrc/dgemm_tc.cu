@@ -172,7 +172,7 @@ struct GemmArgs {
   EmuSet set[2];              // operands and outputs; a tile names its set
   int tb;                     // rows of a B tile image: 16, 32, 64 or 128
   int stages;                 // shared-memory stages
-  double* part;               // [2 gridDim.x][kTNr][kTMr] partial tiles of the split tiles
+  float2* part;               // [2 gridDim.x][kTNr][kTMr] partial tiles (hi, lo) of the split tiles
   unsigned* status;
 };
 
@@ -202,13 +202,34 @@ __device__ __forceinline__ bool seg_at(const GemmArgs& g, int t, int64_t c, int6
   s.whole = s.kb0 == 0 && s.kb1 == nkb;
   return true;
 }
-__device__ __forceinline__ int first_tile(const GemmArgs& g, int64_t c) {   // the tile holding block c
-  int lo = 0, hi = g.n_tiles - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (g.tiles[mid].c0 <= c) lo = mid; else hi = mid - 1;
+// the tile holding block c; a warp together, 32 probes a round (a thread's binary search is a chain of
+// loads from L2: 4 us for 86 tiles)
+__device__ __forceinline__ int first_tile(const GemmArgs& g, int64_t c) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = g.n_tiles;
+  while (n > 1) {
+    const int step = (n + 31) / 32, o = lane * step;
+    const unsigned b = __ballot_sync(0xffffffffu, o < n && g.tiles[lo + min(o, n - 1)].c0 <= c);
+    const int k = (__popc(b) - 1) * step;            // c0 ascends: the probes at or below c come first
+    lo += k;
+    n = min(step, n - k);
   }
   return lo;
+}
+
+// (hi + lo) 2^e as a double.  FP64 conversions and ldexp run at the FP64 pipe's rate (2 lanes per SM and
+// clock), so the floats become doubles and the exponent is added on the bit patterns: one FP64
+// addition per element.  hi and lo are zero or normal floats (multiples of 2^-80).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x);
+  const unsigned h = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20));
+  return (u << 1) == 0u ? 0.0 : __hiloint2double((int)h, (int)(u << 29));
+}
+__device__ __forceinline__ double scaled_sum(float hi, float lo, int e) {
+  const double v = widen(hi) + widen(lo);
+  const int ex = (__double2hiint(v) >> 20) & 0x7ff;
+  if (ex == 0 || ex + e <= 0 || ex + e >= 2047) return ldexp(v, e);   // zero, or out of the normal range
+  return __hiloint2double(__double2hiint(v) + (e << 20), __double2loint(v));
 }
 
 // columns of the tile that K block kb touches: the 16-column groups whose K extent reaches past it
@@ -220,38 +241,51 @@ __device__ __forceinline__ int active_cols(const EmuTile& tl, int kb) {
   return n;
 }
 
-// The MMAs of one K block: the slice pairs (p, q) with p + q < NS, each as two K = 16 steps, into the
-// accumulator of digit diagonal min(p + q, 3).  Fully unrolled: one thread issues them, and computing
-// the descriptors in loops took it longer than the MMAs take at N = 16 (measured on the L = 80 quench's
-// 2750 x 16 x 2650 products: 100 us each, 50 us per 256 K values).  `fresh`: the chunk's first block,
-// whose first MMA of each accumulator overwrites it.
-template <int NS>
+// Accumulators.  An MMA that adds to the accumulator of the one before it waits for its result
+// (measured: about 115 cycles at N = 16 and 131 at N = 128, however few columns it has), so the 42
+// MMAs of a K block should go round many accumulators.  Digit diagonal d = p + q and K step ks:
+//   AM 2 (up to 32 columns): one accumulator for each (d, ks), 12 of tb columns;
+//   AM 1 (up to 64 columns): 8 of 64: diagonals 0..3, and 4 and 5 split by ks;
+//   AM 0 (128 columns): 4 of 128: diagonals 0, 1, 2, and one for 3..5 together.
+// With 16 columns the 12 accumulators leave room for a second set, so that a chunk's fold overlaps the
+// next chunk's MMAs.  Measured with the four accumulators of AM 0 for every width, 30 of the 42
+// MMAs in one chain: 11000 x 16 x 2650 took 133 us, 4800 cycles per K block, the tensor pipe 6% busy.
+template <int AM> __host__ __device__ constexpr int acc_of(int d, int ks) {
+  return AM == 2 ? 2 * d + ks : AM == 1 ? (d < 4 ? d : 2 * d - 4 + ks) : (d < 3 ? d : 3);
+}
+template <int AM, int NS> __host__ __device__ constexpr int n_accs() {   // accumulators that NS slices use
+  return NS == 2 ? (AM == 2 ? 4 : 2) : (AM == 2 ? 12 : AM == 1 ? 8 : 4);
+}
+
+// The MMAs of one K block: the slice pairs (p, q) with p + q < NS, each as two K = 16 steps.  Fully
+// unrolled, because one thread issues them.  `fresh`: the chunk's first block, whose first MMA of each
+// accumulator (a pair (0, q)) overwrites it.
+template <int NS, int AM>
 __device__ __forceinline__ void issue_block(uint32_t d0, uint32_t acc_cols, uint64_t a0, uint64_t b0, uint32_t bq,
                                             uint32_t id, bool fresh) {
 #pragma unroll
   for (int p = 0; p < NS; ++p)
 #pragma unroll
     for (int q = 0; q + p < NS; ++q) {
-      const int d = p + q < 3 ? p + q : 3;
 #pragma unroll
-      for (int ks = 0; ks < 2; ++ks)
-        mma(d0 + (uint32_t)d * acc_cols, a0 + (uint64_t)((p * kASlice + ks * 32) >> 4),
-            b0 + (uint64_t)((uint32_t)q * bq + ks * 2), id, (fresh && p == 0 && q < 4 && ks == 0) ? 0u : 1u);
+      for (int ks = 0; ks < 2; ++ks) {
+        const bool opens = p == 0 && (AM == 2 || (ks == 0 && (AM == 1 || q <= 3)) || (AM == 1 && q >= 4));
+        mma(d0 + (uint32_t)acc_of<AM>(p + q, ks) * acc_cols, a0 + (uint64_t)((p * kASlice + ks * 32) >> 4),
+            b0 + (uint64_t)((uint32_t)q * bq + ks * 2), id, (fresh && opens) ? 0u : 1u);
+      }
     }
 }
 
 // NS: slices used per operand, kS (the FP64 product) or 2 (the two leading digits: ~2^-16)
-template <int NS>
+template <int NS, int AM>
 __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads x 168 registers, one CTA per SM
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = su32(smem_raw);
   unsigned char* base = smem_raw + (((raw + 1023u) & ~1023u) - raw);
   const uint32_t b_slice = (uint32_t)g.tb * 64u, stage_bytes = (uint32_t)NS * (kASlice + b_slice);
   const int n_st = g.stages;
-  // two sets of accumulators when a tile's columns leave room for them in the 512 of TMEM: the fold
-  // of one chunk then overlaps the MMAs of the next
-  const int n_acc = g.tb <= 64 ? 2 : 1;
-  const uint32_t acc_cols = g.tb <= 64 ? 64u : 128u;
+  const int n_acc = AM == 2 && g.tb == 16 ? 2 : 1;      // sets of accumulators
+  const uint32_t acc_cols = AM == 2 ? (uint32_t)g.tb : AM == 1 ? 64u : 128u;
   uint64_t* bars = (uint64_t*)(base + (size_t)n_st * stage_bytes);
   uint64_t* full = bars;                   // [kMaxStages] stage loaded
   uint64_t* empty = bars + kMaxStages;     // [kMaxStages] stage consumed by the MMAs
@@ -342,7 +376,7 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
             const uint64_t da = desc64(a0), db = desc64(a0 + NS * kASlice);
             if (!bar_wait(full + st, ph, &s_abort)) { atomicOr(g.status, kStTimeout); s_abort = 1; break; }
             fence_after();
-            issue_block<NS>(tmem + (uint32_t)as * 256u, acc_cols, da, db, b_slice >> 4, id, kb == kb0);
+            issue_block<NS, AM>(tmem + (uint32_t)as * 256u, acc_cols, da, db, b_slice >> 4, id, kb == kb0);
             commit(empty + st);                       // the stage's smem is free once these complete
             last = empty + st;
             if (++st == n_st) { st = 0; ph ^= 1u; }
@@ -359,8 +393,8 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
     }
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2-9)
-    constexpr int kCols = kTNr / 2;                   // most columns per epilogue warp
-    const int kc = g.tb <= 64 ? 32 : kCols;           // columns per epilogue warp
+    constexpr int kCols = AM == 0 ? 64 : AM == 1 ? 32 : 16;   // columns per epilogue warp
+    constexpr int kc = kCols;
     const int quad = warp & 3;                        // TMEM lanes 32 quad .. 32 quad + 31
     const int half = (warp - 2) >> 2;                 // columns kc half .. kc half + kc - 1
     const int r = quad * 32 + lane;                   // row of the tile
@@ -386,9 +420,9 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
         const uint32_t lane_base = tmem + (uint32_t)as * 256u + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * kc);
 #pragma unroll
         for (int h = 0; h < kCols / 16; ++h) {
-          if (h * 16 < kc && half * kc + h * 16 < na) {
+          if (half * kc + h * 16 < na) {
 #pragma unroll
-            for (int d = 0; d < (NS < 4 ? NS : 4); ++d) {   // with 2 slices only diagonals 0 and 1 are written
+            for (int d = 0; d < n_accs<AM, NS>(); ++d) {
               float v[16];
               ld16(lane_base + (uint32_t)d * acc_cols + (uint32_t)h * 16u, v);
 #pragma unroll
@@ -409,18 +443,18 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
 #pragma unroll
           for (int cc = 0; cc < kCols; ++cc) {
             const int j = tl.cb * kTNr + c_lo + cc;
-            if (cc < kc && c_lo + cc < tl.n_eff && j < op.N)
-              op.C[(int64_t)i + (int64_t)j * op.ldc] = ldexp((double)hi[cc] + (double)lo[cc], e_i + op.eb[j] - 16);
+            if (c_lo + cc < tl.n_eff && j < op.N)
+              op.C[(int64_t)i + (int64_t)j * op.ldc] = scaled_sum(hi[cc], lo[cc], e_i + op.eb[j] - 16);
           }
         }
         continue;
       }
       // split tile: this CTA's partial to its slot (0: the tile its range starts in, 1: the tile it ends in)
       const int slot = 2 * (int)blockIdx.x + (sg.t == t_first ? 0 : 1);
-      double* mine = g.part + (size_t)slot * kTNr * kTMr;
+      float2* mine = g.part + (size_t)slot * kTNr * kTMr;
 #pragma unroll
       for (int cc = 0; cc < kCols; ++cc)
-        if (cc < kc && c_lo + cc < tl.n_eff) mine[(size_t)(c_lo + cc) * kTMr + r] = (double)hi[cc] + (double)lo[cc];
+        if (c_lo + cc < tl.n_eff) mine[(size_t)(c_lo + cc) * kTMr + r] = make_float2(hi[cc], lo[cc]);
       // the last of the tile's CTAs to finish this warp's block adds the parts (no waiting)
       __threadfence();
       __syncwarp();
@@ -431,17 +465,29 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
         __threadfence();
         if (i < op.M) {
           const int e_i = op.ea[i];
-          const int nc = min(kc, tl.n_eff - c_lo);
-#pragma unroll 4
-          for (int cc = 0; cc < nc; ++cc) {
-            const int j = tl.cb * kTNr + c_lo + cc;
-            if (j < op.N) {
-              double v = 0.0;
-              for (int cta = c_a; cta <= c_b; ++cta) {
-                const int sl = 2 * cta + (range_start(cta, T, G) >= tl.c0 ? 0 : 1);
-                v += __ldcg(g.part + (size_t)sl * kTNr * kTMr + (size_t)(c_lo + cc) * kTMr + r);
+          const int nc = min(kc, tl.n_eff - c_lo);        // a multiple of 16
+          // 16 columns at a time, all loads of a part in flight together
+#pragma unroll 1
+          for (int c16 = 0; c16 < nc; c16 += 16) {
+            float h16[16], l16[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) { h16[u] = 0.f; l16[u] = 0.f; }
+            for (int cta = c_a; cta <= c_b; ++cta) {
+              const int sl = 2 * cta + (range_start(cta, T, G) >= tl.c0 ? 0 : 1);
+              const float2* src = g.part + (size_t)sl * kTNr * kTMr + (size_t)(c_lo + c16) * kTMr + r;
+              float2 v[16];
+#pragma unroll
+              for (int u = 0; u < 16; ++u) v[u] = __ldcg(src + (size_t)u * kTMr);
+#pragma unroll
+              for (int u = 0; u < 16; ++u) {
+                two_sum_add(h16[u], l16[u], v[u].x);
+                l16[u] += v[u].y;
               }
-              op.C[(int64_t)i + (int64_t)j * op.ldc] = ldexp(v, e_i + op.eb[j] - 16);
+            }
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              const int j = tl.cb * kTNr + c_lo + c16 + u;
+              if (j < op.N) op.C[(int64_t)i + (int64_t)j * op.ldc] = scaled_sum(h16[u], l16[u], e_i + op.eb[j] - 16);
             }
           }
         }
@@ -646,7 +692,9 @@ tgba_status emu_prepare(Basis& b) {
   static int sms_of[64] = {0};
   if (b.device < 0 || b.device >= 64) return fail(TGBA_ELIMIT, "device index");
   if (sms_of[b.device] == 0) {
-    for (const void* k : {(const void*)dgemm_tc_kernel<kS>, (const void*)dgemm_tc_kernel<2>}) {
+    for (const void* k : {(const void*)dgemm_tc_kernel<kS, 0>, (const void*)dgemm_tc_kernel<kS, 1>,
+                          (const void*)dgemm_tc_kernel<kS, 2>, (const void*)dgemm_tc_kernel<2, 0>,
+                          (const void*)dgemm_tc_kernel<2, 1>, (const void*)dgemm_tc_kernel<2, 2>}) {
       TGBA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
       cudaFuncAttributes fa;
       TGBA_CUDA(cudaFuncGetAttributes(&fa, k));
@@ -710,11 +758,19 @@ tgba_status emu_gemm_sets(Basis& b, const EmuSet* sets, int n_sets, int tb, EmuT
   g.tb = tb;
   const uint32_t stage = (uint32_t)n_slices * (kASlice + (uint32_t)tb * 64u);
   g.stages = std::min<int>(kMaxStages, (int)(kSmemStages / stage));
-  g.part = b.d_emu_part; g.status = b.d_status;
+  g.part = (float2*)b.d_emu_part; g.status = b.d_status;
   const size_t smem = 1024 + (size_t)g.stages * stage + 256;
   const int grid = (int)std::min<int64_t>(n_blocks, b.emu_sms);
-  if (n_slices == kS) dgemm_tc_kernel<kS><<<grid, kThreads, smem, st>>>(g);
-  else dgemm_tc_kernel<2><<<grid, kThreads, smem, st>>>(g);
+  const int am = tb <= 32 ? 2 : tb == 64 ? 1 : 0;
+  if (n_slices == kS) {
+    if (am == 2) dgemm_tc_kernel<kS, 2><<<grid, kThreads, smem, st>>>(g);
+    else if (am == 1) dgemm_tc_kernel<kS, 1><<<grid, kThreads, smem, st>>>(g);
+    else dgemm_tc_kernel<kS, 0><<<grid, kThreads, smem, st>>>(g);
+  } else {
+    if (am == 2) dgemm_tc_kernel<2, 2><<<grid, kThreads, smem, st>>>(g);
+    else if (am == 1) dgemm_tc_kernel<2, 1><<<grid, kThreads, smem, st>>>(g);
+    else dgemm_tc_kernel<2, 0><<<grid, kThreads, smem, st>>>(g);
+  }
   TGBA_CUDA(cudaGetLastError());
   ++b.launches;
   return TGBA_OK;
