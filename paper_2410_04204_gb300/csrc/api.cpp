@@ -58,7 +58,7 @@ static void release(Basis* b) {
                   b->d_theta, b->d_nlab, b->d_table, b->d_c0, b->d_const, b->d_tdd, b->d_fac_ns, b->d_fac_r, b->d_pairs_r,
                   b->d_P, b->d_status,
                   b->d_eig_a, b->d_eig_w, b->d_eig_work, b->d_eig_info, b->d_scratch,
-                  b->d_rects, b->d_heff_secs, b->d_mirror, b->d_blas_ws, b->d_emu_part};
+                  b->d_tiles, b->d_groups, b->d_heff_secs, b->d_mirror, b->d_blas_ws, b->d_emu_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int e = 0; e < 3; ++e) {
@@ -146,7 +146,8 @@ static tgba_status build(const tgba_model* model, const int32_t* sectors, int32_
   const std::vector<HeffSector> hs = heff_sectors(*b, &b->heff_tiles);
   b->n_heff_secs = (int)hs.size();
   if ((r = upload(&b->d_heff_secs, hs.data(), hs.size(), &b->upload_bytes)) != TGBA_OK) return r;
-  if ((r = upload(&b->d_rects, b->rects.data(), b->rects.size(), &b->upload_bytes)) != TGBA_OK) return r;
+  if ((r = upload(&b->d_tiles, b->tiles.data(), b->tiles.size(), &b->upload_bytes)) != TGBA_OK) return r;
+  if ((r = upload(&b->d_groups, b->groups.data(), b->groups.size(), &b->upload_bytes)) != TGBA_OK) return r;
   for (int e = 0; e < 3; ++e) TGBA_CUDA(cudaEventCreate(&b->ev[e]));
   return TGBA_OK;
 }

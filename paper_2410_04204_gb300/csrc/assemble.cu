@@ -7,6 +7,9 @@
 #include "tgba_internal.h"
 
 namespace tgba {
+
+constexpr int kHeffTile = 64;
+
 namespace {
 
 // X_ab from P_ab
@@ -20,21 +23,30 @@ __device__ __forceinline__ double2 xval(const double* c0, double p, int n) {
   }
 }
 
-// Column-major complex H of every sector in one launch.  A block of 256 threads owns one 32 x 32
-// tile: of the X block (P read once, coalesced, and written to both off-diagonal blocks of H, the
+// Column-major complex H of every sector in one launch.  A block of 256 threads owns one kHeffTile
+// square tile: of the X block (P read once, coalesced, and written to both off-diagonal blocks of H, the
 // transposed one through shared memory) or of a diagonal block (zeros and the energies).  Bound: the
-// HBM write of 16 B per entry; the streaming stores leave P in L2.  One thread per entry, with P
-// read along a column for the NS-row block and one launch per sector, took 0.56 ms for the 24
-// sectors of the L = 24 workload (1.39 GB).
-__device__ __forceinline__ double2 scaled(double s, double2 x) { return make_double2(s * x.x, s * x.y); }
+// HBM write of 16 B per entry.  Measured: L = 24, all sectors (1.39 GB) 257 us, L = 80, M <= 10 (1.70 GB) 311 us,
+// 5.4 TB/s; 504 and 754 us with complex products, see phased.
+// C0 is real (elements.cu), so an entry -L h_x X is v (-i)^{n/2}, v = -L h_x C0 P: one FP64
+// multiplication per pair, the phase and the conjugate by moving v to the real or imaginary part and
+// flipping its sign bit as an integer.  (General complex products, four FP64 multiplications per pair,
+// held the kernel at 2.8 to 3.5 TB/s whatever its tile and store hints.)
+__device__ __forceinline__ double2 phased(double v, int n, bool conj) {
+  const int k = (n >> 1) & 3;                       // (-i)^k
+  const bool im = k & 1, neg = k == 2 || (im && ((k == 1) != conj));
+  const long long b = __double_as_longlong(v) ^ (neg ? (long long)0x8000000000000000ull : 0ll);
+  return make_double2(__longlong_as_double(im ? 0ll : b), __longlong_as_double(im ? b : 0ll));
+}
 
 __global__ void __launch_bounds__(256) heff_kernel(const HeffSector* __restrict__ secs, int n_sec,
                                                    const double* __restrict__ E_ns, const double* __restrict__ E_r,
                                                    const uint8_t* __restrict__ M_ns, const uint8_t* __restrict__ M_r,
                                                    const double* __restrict__ P, const double* __restrict__ c0,
                                                    double scale, double2* __restrict__ Hall) {
-  __shared__ double t[32][33];
-  __shared__ uint8_t s_m[32];
+  constexpr int T = kHeffTile, W = T / 32;            // W: lanes' columns per warp row
+  __shared__ double t[T][T + 1];
+  __shared__ uint8_t s_m[T], s_mr[T];
   int lo = 0, hi = n_sec - 1;                         // the sector holding this tile
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -42,47 +54,56 @@ __global__ void __launch_bounds__(256) heff_kernel(const HeffSector* __restrict_
     else hi = mid - 1;
   }
   const HeffSector sc = secs[lo];
-  const int64_t n_ns = sc.n_ns, n_r = sc.n_r, n = n_ns + n_r;
-  const int64_t tn = (n_ns + 31) / 32, tr = (n_r + 31) / 32;
-  int64_t q = (int64_t)blockIdx.x - sc.tile0;
+  const int n_ns = (int)sc.n_ns, n_r = (int)sc.n_r;
+  const int64_t n = sc.n_ns + sc.n_r;
+  const int tn = (n_ns + T - 1) / T, tr = (n_r + T - 1) / T;
+  int q = (int)((int64_t)blockIdx.x - sc.tile0);
   double2* H = Hall + sc.h_off;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   if (q < tn * tr) {
-    const int64_t a0 = (q / tr) * 32, b0 = (q % tr) * 32;
-    const double* Ps = P + sc.x_off;
-    if (threadIdx.x < 32 && a0 + tx < n_ns) s_m[tx] = M_ns[sc.ns_off + a0 + tx];
-    __syncthreads();
-    const int mb = b0 + tx < n_r ? M_r[sc.r_off + b0 + tx] : 0;
-#pragma unroll
-    for (int y = ty; y < 32; y += 8) {
-      const int64_t a = a0 + y, b = b0 + tx;
-      if (a >= n_ns || b >= n_r) continue;
-      const double p = Ps[a * n_r + b];
-      t[y][tx] = p;
-      const double2 x = xval(c0, p, s_m[y] + mb);
-      __stcs(H + a * n + n_ns + b, make_double2(scale * x.x, -scale * x.y));     // R row, NS column: conj(X)
+    const int a0 = (q / tr) * T, b0 = (q % tr) * T;
+    const double* Ps = P + sc.x_off + (int64_t)a0 * n_r + b0;
+    if (threadIdx.x < T) {
+      s_m[threadIdx.x] = a0 + (int)threadIdx.x < n_ns ? M_ns[sc.ns_off + a0 + threadIdx.x] : 0;
+      s_mr[threadIdx.x] = b0 + (int)threadIdx.x < n_r ? M_r[sc.r_off + b0 + threadIdx.x] : 0;
     }
-    __syncthreads();
+    const int na = min(T, n_ns - a0), nb = min(T, n_r - b0);
+    const double cs = scale * c0[0];
 #pragma unroll
-    for (int y = ty; y < 32; y += 8) {
-      const int64_t a = a0 + tx, b = b0 + y;
-      if (a >= n_ns || b >= n_r) continue;
-      __stcs(H + (n_ns + b) * n + a, scaled(scale, xval(c0, t[tx][y], s_m[tx] + M_r[sc.r_off + b])));
-    }
+    for (int y = ty; y < T; y += 8)
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if (y < na && tx + 32 * w < nb) t[y][tx + 32 * w] = cs * Ps[(int64_t)y * n_r + tx + 32 * w];
+    __syncthreads();
+#pragma unroll 4
+    for (int y = ty; y < na; y += 8)
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const int b = tx + 32 * w;
+        if (b < nb) H[(int64_t)(a0 + y) * n + n_ns + b0 + b] = phased(t[y][b], s_m[y] + s_mr[b], true);   // R row, NS column
+      }
+#pragma unroll 4
+    for (int y = ty; y < nb; y += 8)
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const int a = tx + 32 * w;
+        if (a < na) H[(int64_t)(n_ns + b0 + y) * n + a0 + a] = phased(t[a][y], s_m[a] + s_mr[y], false);
+      }
     return;
   }
   q -= tn * tr;
   const bool ns = q < tn * tn;
   if (!ns) q -= tn * tn;
-  const int64_t nt = ns ? tn : tr, m = ns ? n_ns : n_r, o = ns ? 0 : n_ns;
+  const int nt = ns ? tn : tr, m = ns ? n_ns : n_r, o = ns ? 0 : n_ns;
   const double* E = ns ? E_ns + sc.ns_off : E_r + sc.r_off;
-  const int64_t c0_ = (q / nt) * 32, r0_ = (q % nt) * 32;
+  const int col0 = (q / nt) * T, row0 = (q % nt) * T;
+#pragma unroll 4
+  for (int y = ty; y < T; y += 8)
 #pragma unroll
-  for (int y = ty; y < 32; y += 8) {
-    const int64_t col = c0_ + y, row = r0_ + tx;
-    if (col >= m || row >= m) continue;
-    __stcs(H + (o + col) * n + o + row, make_double2(row == col ? E[row] : 0.0, 0.0));
-  }
+    for (int w = 0; w < W; ++w) {
+      const int col = col0 + y, row = row0 + tx + 32 * w;
+      if (col < m && row < m) H[(int64_t)(o + col) * n + o + row] = make_double2(row == col ? E[row] : 0.0, 0.0);
+    }
 }
 
 // Real-gauge H~ (column-major, n_k x n_k) of a subset of a sector's states.
@@ -130,7 +151,7 @@ std::vector<HeffSector> heff_sectors(const Basis& b, int64_t* tiles) {
   for (const Sector& sec : b.sectors) {
     if (sec.n_ns + sec.n_r == 0) continue;
     v.push_back(HeffSector{sec.n_ns, sec.n_r, sec.ns_off, sec.r_off, sec.x_off, sec.h_off, t});
-    const int64_t tn = (sec.n_ns + 31) / 32, tr = (sec.n_r + 31) / 32;
+    const int64_t tn = (sec.n_ns + kHeffTile - 1) / kHeffTile, tr = (sec.n_r + kHeffTile - 1) / kHeffTile;
     t += tn * tr + tn * tn + tr * tr;
   }
   *tiles = t;

@@ -25,8 +25,8 @@
 // element carries about M_b/2 + 2 roundings; the elimination it replaces lost about 1e-14.
 //
 // Measured on one GB300, table, elements and the complex H_eff: the 24 sectors of the L = 24 workload
-// (2.2e7 elements) 7.22 ms by elimination, 0.90 ms as products; L = 80, M <= 10 (2.7e7 elements of sizes
-// up to 20) 17.1 ms, 1.42 ms, its error against 64-bit values 9e-15 before, 4e-16 now; L = 12,
+// (2.2e7 elements) 7.22 ms by elimination, 0.53 ms as products; L = 80, M <= 10 (2.7e7 elements of sizes
+// up to 20) 17.1 ms, 0.65 ms, its error against 64-bit values 6e-15 before, 3e-16 now; L = 12,
 // M <= 4 (latency) 136 us, 45 us.
 #include <algorithm>
 #include <cmath>
@@ -133,13 +133,13 @@ __global__ void __launch_bounds__(128) mode_table(Tab T) {
 }
 
 // R (rounded), C0, the per-state factors A_a (NS) and B_b (R), and each R state's list of mode
-// pairs (indices into the pair tables of x_tiles).  One thread per entry or state.
+// pairs (indices into the pair tables of x_tiles).
 __global__ void __launch_bounds__(256) state_factors(Tab T, double* __restrict__ R, double* __restrict__ c0,
                                                      int64_t n_ns, int64_t n_r, int max_qp,
                                                      const uint8_t* __restrict__ sel_ns, const uint8_t* __restrict__ sel_r,
                                                      const uint8_t* __restrict__ M_ns, const uint8_t* __restrict__ M_r,
                                                      double* __restrict__ A, double* __restrict__ B,
-                                                     uint16_t* __restrict__ pairs, int hp, unsigned* __restrict__ status) {
+                                                     uint16_t* __restrict__ pairs, int hp, int lanes, unsigned* __restrict__ status) {
   const int L = T.L, n2 = 2 * L;
   if (blockIdx.x == 0 && threadIdx.x < 32) {
     const int lane = threadIdx.x;
@@ -154,27 +154,36 @@ __global__ void __launch_bounds__(256) state_factors(Tab T, double* __restrict__
       if (!(c.h > 0.0) || !isfinite(c.h)) atomicOr(status, kStTableSingular);
     }
   }
-  const int64_t total = (int64_t)n2 * n2 + n_ns + n_r;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
-    if (q < n_ns + n_r) {
-      const bool ns = q < n_ns;
-      const int64_t s = ns ? q : q - n_ns;
+  // `lanes` lanes per state (a lane multiplies the factors (i, j) with j = i + lane mod lanes), then table
+  // entries.  Few states: 8 lanes, for latency (L = 12, M <= 12: a state's 78 factors in one thread take
+  // 33 us).  Many: one, because the lanes' shuffle tree costs FP64 operations (L = 24, all sectors: 82 us with
+  // 8 lanes, 41 us with one).
+  const int64_t states = (n_ns + n_r) * lanes, total = states + (int64_t)n2 * n2;
+  for (int64_t q0 = (int64_t)blockIdx.x * blockDim.x; q0 < total; q0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t q = q0 + threadIdx.x;
+    if (q0 < states) {
+      const bool live = q < states;
+      const int64_t st = (live ? q : 0) / lanes;
+      const int l8 = (int)(q & (lanes - 1));
+      const bool ns = st < n_ns;
+      const int64_t s = ns ? st : st - n_ns;
       const uint8_t* sel = (ns ? sel_ns : sel_r) + s * max_qp;
-      const int M = ns ? M_ns[s] : M_r[s];
+      const int M = !live ? 0 : ns ? M_ns[s] : M_r[s];
       dd p{1.0, 0.0};
       for (int i = 0; i < M; ++i) {
         const int a = sel[i];
-        p = mul(p, ld(T.r + a));
-        for (int j = i + 1; j < M; ++j) p = mul(p, ld(T.t + (size_t)a * n2 + sel[j]));
+        for (int j = i + l8; j < M; j += lanes) p = mul(p, j == i ? ld(T.r + a) : ld(T.t + (size_t)a * n2 + sel[j]));
       }
-      (ns ? A : B)[s] = p.h;
-      if (!ns)
-        for (int u = 0; u < M / 2; ++u) {
-          const int q0 = sel[2 * u] - L, q1 = sel[2 * u + 1] - L;      // ascending
-          pairs[s * hp + u] = (uint16_t)(q0 * (2 * L - q0 - 1) / 2 + (q1 - q0 - 1));
+      for (int o = lanes / 2; o > 0; o >>= 1) p = mul(p, dd{__shfl_xor_sync(0xffffffffu, p.h, o), __shfl_xor_sync(0xffffffffu, p.l, o)});
+      if (live && l8 == 0) (ns ? A : B)[s] = p.h;
+      if (live && !ns)
+        for (int u = l8; u < M / 2; u += lanes) {
+          const int m0 = sel[2 * u] - L, m1 = sel[2 * u + 1] - L;      // ascending
+          pairs[s * hp + u] = (uint16_t)(m0 * (2 * L - m0 - 1) / 2 + (m1 - m0 - 1));
         }
-    } else {
-      const int64_t k = q - n_ns - n_r;
+    }
+    if (q >= states && q < total) {
+      const int64_t k = q - states;
       const int a = (int)(k / n2), b = (int)(k % n2);
       R[k] = a == b ? 0.0 : mul(mul(ld(T.r + a), ld(T.r + b)), ld(T.t + k)).h;
     }
@@ -192,11 +201,21 @@ struct Elems {
   unsigned* status;
 };
 
-// G_a(q) = prod_{i in a} t(i, L + q), rounded once
+// G_a(q) = prod_{i in a} t(i, L + q), rounded once (the running product as a head and an unnormalised
+// tail: four FP64 operations per factor)
 __device__ __forceinline__ double row_factor(const Elems& g, const uint8_t* sel, int M, int q) {
-  dd p{1.0, 0.0};
-  for (int i = 0; i < M; ++i) p = mul(p, ld(g.t + (size_t)sel[i] * (2 * g.L) + g.L + q));
-  return p.h;
+  if (M == 0) return 1.0;
+  const double2* t = g.t + g.L + q;
+  dd p = ld(t + (size_t)sel[0] * (2 * g.L));
+  for (int i = 1; i < M; ++i) {
+    const dd f = ld(t + (size_t)sel[i] * (2 * g.L));
+    const double h = __dmul_rn(p.h, f.h);
+    double l = __fma_rn(p.h, f.h, -h);
+    l = __fma_rn(p.h, f.l, l);
+    p.l = __fma_rn(p.l, f.h, l);
+    p.h = h;
+  }
+  return __dadd_rn(p.h, p.l);
 }
 __device__ __forceinline__ bool finite_bits(double x) {
   return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
@@ -213,29 +232,31 @@ __device__ __forceinline__ double x_value(const Elems& g, int64_t a, int Ma, int
   return __dmul_rn(v, __ldg(g.A + a));
 }
 
-// All elements of the listed rectangles (uniform M_a and M_b).  A block owns RB rows x kColChunk
-// columns: it forms G_a(q) of its rows, then (rc.pairs) the products of all L (L - 1)/2 mode pairs
-// in shared memory, and each thread then walks down its columns, loading a column's pair list and
-// B_b once for the RB rows: M_b/2 + 1 multiplications and M_b/2 shared-memory loads per element
-// and one coalesced 8-byte store.  Rectangles whose columns would use fewer pair products than the
-// table holds (w M_b/2 <= L (L - 1)/2, see build_rects) multiply the two factors themselves, which
-// rounds the same way.  RB is the largest of 8, 4, 2, 1 whose tables fit 100 KB (two blocks per
-// SM): 8 up to L = 56, 4 up to L = 80, 2 up to L = 112.  Bound: FP64 multiplications (2 lanes per SM and clock) for M_b >= 4.
-constexpr int kColChunk = 2048;
+// All elements of the listed row tiles.  A block owns up to RB rows (NS states of one M_a) and a range
+// of the R states' columns, whatever their M_b: it forms G_a(q) of its rows once, then (tile.pairs)
+// the products of all L (L - 1)/2 mode pairs in shared memory, and each thread then walks down its
+// columns group by group of equal M_b, loading a column's pair list and B_b once for the RB rows: M_b/2 + 1
+// multiplications and M_b/2 shared-memory loads per element and one coalesced 8-byte store.  Tiles
+// whose columns would use fewer pair products than the table holds (see row_tiles) multiply the two
+// factors themselves, which rounds the same way.  RB is the largest of 8, 4, 2, 1 whose tables fit 100 KB
+// (two blocks per SM): 8 up to L = 56, 4 up to L = 80, 2 up to L = 112.  Bound: FP64 multiplications (2
+// lanes per SM and clock).  With a block per rectangle of one M_b the factors G_a were formed again
+// for each M_b (L = 24, all sectors: 350 us, now 231 us, 63% of the rate of FP64 multiplications counting the
+// elements' alone; L = 80, M <= 10, 2.7e7 elements: 620 and 295 us).
 constexpr int kTileThreads = 256;
 
 template <int RB, int H>
-__device__ __forceinline__ void tile_columns(const Elems& g, const Rect& rc, const double* sG, const double* sG2, int np,
-                                             int r0, int nr, int c0, int c1, double* __restrict__ P) {
+__device__ __forceinline__ void tile_columns(const Elems& g, const RowTile& rt, const double* sG, const double* sG2, int np,
+                                             int c0, int c1, double* __restrict__ P) {
   double av[RB];
 #pragma unroll
-  for (int r = 0; r < RB; ++r) av[r] = __ldg(g.A + rc.ns0 + r0 + min(r, nr - 1));
+  for (int r = 0; r < RB; ++r) av[r] = __ldg(g.A + rt.ns0 + min(r, rt.rows - 1));
   bool bad = false;
   for (int c = c0 + (int)threadIdx.x; c < c1; c += kTileThreads) {
-    const int64_t b = rc.r0 + c;
+    const int64_t b = rt.r_off + c;
     const double bv = __ldg(g.B + b);
-    double* out = P + rc.out0 + (int64_t)r0 * rc.ld + c;
-    if (rc.pairs || H == 0) {
+    double* out = P + rt.out0 + c;
+    if (rt.pairs || H == 0) {
       int id[H > 0 ? H : 1];
 #pragma unroll
       for (int u = 0; u < H; ++u) id[u] = __ldg(g.pairs + b * g.hp + u);
@@ -246,7 +267,7 @@ __device__ __forceinline__ void tile_columns(const Elems& g, const Rect& rc, con
         for (int u = 0; u < H; ++u) v = __dmul_rn(v, sG2[r * np + id[u]]);
         v = __dmul_rn(v, av[r]);
         bad |= !finite_bits(v);
-        if (r < nr) out[(int64_t)r * rc.ld] = v;
+        if (r < rt.rows) out[(int64_t)r * rt.ld] = v;
       }
     } else {
       const uint8_t* sb = g.sel_r + b * g.max_qp;
@@ -261,7 +282,7 @@ __device__ __forceinline__ void tile_columns(const Elems& g, const Rect& rc, con
           v = __dmul_rn(v, __dmul_rn(sG[r * g.L + q[2 * u]], sG[r * g.L + q[2 * u + 1]]));
         v = __dmul_rn(v, av[r]);
         bad |= !finite_bits(v);
-        if (r < nr) out[(int64_t)r * rc.ld] = v;
+        if (r < rt.rows) out[(int64_t)r * rt.ld] = v;
       }
     }
   }
@@ -269,30 +290,20 @@ __device__ __forceinline__ void tile_columns(const Elems& g, const Rect& rc, con
 }
 
 template <int RB>
-__global__ void __launch_bounds__(kTileThreads) x_tiles(Elems g, const Rect* __restrict__ rects, int n_rects,
-                                                        double* __restrict__ P) {
+__global__ void __launch_bounds__(kTileThreads) x_tiles(Elems g, const RowTile* __restrict__ tiles,
+                                                        const ColGroup* __restrict__ groups, double* __restrict__ P) {
   extern __shared__ double sm[];
   const int L = g.L, np = L * (L - 1) / 2;
   double* sG = sm;                       // [RB][L]
   double* sG2 = sm + RB * L;             // [RB][np]
-  int lo = 0, hi = n_rects - 1;          // the rectangle holding this tile
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (rects[mid].tile0 <= (int64_t)blockIdx.x) lo = mid;
-    else hi = mid - 1;
-  }
-  const Rect rc = rects[lo];
-  const int lt = (int)((int64_t)blockIdx.x - rc.tile0), ncc = (rc.w + kColChunk - 1) / kColChunk;
-  const int r0 = (lt / ncc) * RB, nr = min(RB, rc.rows - r0);
-  const int c0 = (lt % ncc) * kColChunk, c1 = min(rc.w, c0 + kColChunk);
-  const int Ma = rc.Ma, H = (rc.n - rc.Ma) / 2;
-  // rows beyond the rectangle repeat its last row (never stored), so that every value is finite
+  const RowTile rt = tiles[blockIdx.x];
+  // rows beyond the tile repeat its last row (never stored), so that every value is finite
   for (int i = threadIdx.x; i < RB * L; i += kTileThreads) {
-    const int r = min(i / L, nr - 1), q = i % L;
-    sG[i] = row_factor(g, g.sel_ns + (rc.ns0 + r0 + r) * g.max_qp, Ma, q);
+    const int r = min(i / L, rt.rows - 1), q = i % L;
+    sG[i] = row_factor(g, g.sel_ns + (rt.ns0 + r) * g.max_qp, rt.Ma, q);
   }
   __syncthreads();
-  if (rc.pairs) {
+  if (rt.pairs) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int q0 = warp; q0 < L - 1; q0 += kTileThreads / 32) {
       const int base = q0 * (2 * L - q0 - 1) / 2 - (q0 + 1);
@@ -302,16 +313,21 @@ __global__ void __launch_bounds__(kTileThreads) x_tiles(Elems g, const Rect* __r
     }
     __syncthreads();
   }
-  switch (H) {
-    case 0: tile_columns<RB, 0>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    case 1: tile_columns<RB, 1>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    case 2: tile_columns<RB, 2>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    case 3: tile_columns<RB, 3>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    case 4: tile_columns<RB, 4>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    case 5: tile_columns<RB, 5>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    case 6: tile_columns<RB, 6>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    case 7: tile_columns<RB, 7>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
-    default: tile_columns<RB, 8>(g, rc, sG, sG2, np, r0, nr, c0, c1, P); break;
+  for (int k = rt.g0; k < rt.g1; ++k) {
+    const ColGroup cg = groups[k];
+    const int c0 = max(cg.c0, rt.c0), c1 = min(cg.c1, rt.c1);
+    if (c0 >= c1) continue;
+    switch (cg.H) {
+      case 0: tile_columns<RB, 0>(g, rt, sG, sG2, np, c0, c1, P); break;
+      case 1: tile_columns<RB, 1>(g, rt, sG, sG2, np, c0, c1, P); break;
+      case 2: tile_columns<RB, 2>(g, rt, sG, sG2, np, c0, c1, P); break;
+      case 3: tile_columns<RB, 3>(g, rt, sG, sG2, np, c0, c1, P); break;
+      case 4: tile_columns<RB, 4>(g, rt, sG, sG2, np, c0, c1, P); break;
+      case 5: tile_columns<RB, 5>(g, rt, sG, sG2, np, c0, c1, P); break;
+      case 6: tile_columns<RB, 6>(g, rt, sG, sG2, np, c0, c1, P); break;
+      case 7: tile_columns<RB, 7>(g, rt, sG, sG2, np, c0, c1, P); break;
+      default: tile_columns<RB, 8>(g, rt, sG, sG2, np, c0, c1, P); break;
+    }
   }
 }
 
@@ -374,7 +390,8 @@ Elems elems_of(const Basis& b) {
   return g;
 }
 
-tgba_status launch_tiles(Basis& b, const Rect* d_rects, int n_rects, int64_t n_tiles, double* P, cudaStream_t st) {
+tgba_status launch_tiles(Basis& b, const RowTile* d_tiles, const ColGroup* d_groups, int64_t n_tiles, double* P,
+                         cudaStream_t st) {
   if (n_tiles == 0) return TGBA_OK;
   if (n_tiles > 0x7fffffff) return fail(TGBA_ELIMIT, "too many element tiles");
   const Elems g = elems_of(b);
@@ -383,7 +400,7 @@ tgba_status launch_tiles(Basis& b, const Rect* d_rects, int n_rects, int64_t n_t
   auto go = [&](auto kern) -> tgba_status {
     if (smem > 48 * 1024)
       TGBA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<(unsigned)n_tiles, kTileThreads, smem, st>>>(g, d_rects, n_rects, P);
+    kern<<<(unsigned)n_tiles, kTileThreads, smem, st>>>(g, d_tiles, d_groups, P);
     TGBA_CUDA(cudaGetLastError());
     ++b.launches;
     return TGBA_OK;
@@ -391,57 +408,78 @@ tgba_status launch_tiles(Basis& b, const Rect* d_rects, int n_rects, int64_t n_t
   return rb == 8 ? go(x_tiles<8>) : rb == 4 ? go(x_tiles<4>) : rb == 2 ? go(x_tiles<2>) : go(x_tiles<1>);
 }
 
-// rectangles of uniform (M_a, M_b) of one NS group list against one R group list; X row-major from
-// out0 with row stride ld
-void add_rects(std::vector<Rect>& v, const std::vector<Group>& g_ns, int64_t ns_off, const std::vector<Group>& g_r,
-               int64_t r_off, int64_t out0, int64_t ld, int L) {
-  for (const Group& ga : g_ns)
-    for (const Group& gb : g_r) {
-      Rect r;
-      r.out0 = out0 + ga.begin * ld + gb.begin;
-      r.ns0 = ns_off + ga.begin;
-      r.r0 = r_off + gb.begin;
-      r.tile0 = 0;
-      r.ld = (int32_t)ld;
-      r.w = (int32_t)(gb.end - gb.begin);
-      r.rows = (int32_t)(ga.end - ga.begin);
-      r.n = ga.M + gb.M;
-      r.Ma = ga.M;
-      // the pair table costs L (L - 1)/2 products per row and saves one per element and pair
-      r.pairs = (int64_t)std::min(r.w, kColChunk) * (gb.M / 2) > (int64_t)L * (L - 1) / 2;
-      v.push_back(r);
+// The row tiles of one NS group list against one R group list (those pairs with M_a + M_b >= n_min);
+// X row-major from out0 with row stride ld.  `chunk`: columns per tile.
+void row_tiles(std::vector<RowTile>& v, std::vector<ColGroup>& cg, const std::vector<Group>& g_ns, int64_t ns_off,
+               const std::vector<Group>& g_r, int64_t r_off, int64_t out0, int64_t ld, int L, int n_min, int chunk) {
+  const int rb = rows_per_tile(L), k0 = (int)cg.size();
+  for (const Group& gb : g_r) cg.push_back(ColGroup{(int32_t)gb.begin, (int32_t)gb.end, gb.M / 2});
+  for (const Group& ga : g_ns) {
+    int k = 0;                                        // M ascends: the first group that counts
+    while (k < (int)g_r.size() && ga.M + g_r[k].M < n_min) ++k;
+    if (k == (int)g_r.size()) continue;
+    for (int64_t c0 = g_r[k].begin; c0 < g_r.back().end; c0 += chunk) {
+      const int64_t c1 = std::min<int64_t>(g_r.back().end, c0 + chunk);
+      int64_t used = 0;                               // pair products that the columns of a row take
+      for (const Group& gb : g_r)
+        used += std::max<int64_t>(0, std::min(c1, gb.end) - std::max(c0, gb.begin)) * (gb.M / 2);
+      for (int64_t r0 = ga.begin; r0 < ga.end; r0 += rb) {
+        RowTile t;
+        t.out0 = out0 + r0 * ld;
+        t.ns0 = ns_off + r0;
+        t.r_off = r_off;
+        t.ld = (int32_t)ld;
+        t.rows = (int32_t)std::min<int64_t>(rb, ga.end - r0);
+        t.Ma = ga.M;
+        t.c0 = (int32_t)c0;
+        t.c1 = (int32_t)c1;
+        t.g0 = k0 + k;
+        t.g1 = k0 + (int)g_r.size();
+        // the pair table costs L (L - 1)/2 products per row and saves one per element and pair
+        t.pairs = used > (int64_t)L * (L - 1) / 2;
+        v.push_back(t);
+      }
     }
+  }
 }
 
-// largest n first, tiles numbered; returns the tiles of the first `head` rectangles in *head_tiles
-int64_t number_tiles(std::vector<Rect>& v, int L, int n_head, int64_t* head_tiles) {
-  std::stable_sort(v.begin(), v.end(), [](const Rect& x, const Rect& y) { return x.n > y.n; });
-  const int rb = rows_per_tile(L);
-  int64_t t = 0;
-  if (head_tiles) *head_tiles = 0;
-  for (Rect& r : v) {
-    r.tile0 = t;
-    t += (int64_t)((r.rows + rb - 1) / rb) * ((r.w + kColChunk - 1) / kColChunk);
-    if (head_tiles && r.n >= n_head) *head_tiles = t;
-  }
-  return t;
-}
+// Columns per tile: all of a sector's when there are enough row tiles for every SM, else 512.
+int column_chunk(int64_t ns_states, int L) { return ns_states / rows_per_tile(L) >= 4 * 152 ? (1 << 30) : 512; }
 
 }  // namespace
 
-// Every rectangle of the basis, largest n first (so those the screener does not judge, n >= 16, are
-// the first b.big_rects).
+// Every row tile of the basis, those of the elements that the screener does not judge (n >= 16), and
+// the rectangles of uniform (M_a, M_b) for the screener, largest n first.
 void build_rects(Basis& b) {
   b.rects.clear();
-  for (const Sector& sec : b.sectors)
-    add_rects(b.rects, sec.g_ns, sec.ns_off, sec.g_r, sec.r_off, sec.x_off, sec.n_r, b.L);
-  b.tiles_total = number_tiles(b.rects, b.L, 16, &b.big_tiles);
-  b.big_rects = 0;
   b.x_mults = 0;
-  for (const Rect& r : b.rects) {
-    if (r.n >= 16) ++b.big_rects;
-    b.x_mults += ((r.n - r.Ma) / 2 + 1.0) * (double)r.rows * r.w;
+  for (const Sector& sec : b.sectors)
+    for (const Group& ga : sec.g_ns)
+      for (const Group& gb : sec.g_r) {
+        Rect r;
+        r.out0 = sec.x_off + ga.begin * sec.n_r + gb.begin;
+        r.ns0 = sec.ns_off + ga.begin;
+        r.r0 = sec.r_off + gb.begin;
+        r.ld = (int32_t)sec.n_r;
+        r.w = (int32_t)(gb.end - gb.begin);
+        r.rows = (int32_t)(ga.end - ga.begin);
+        r.n = ga.M + gb.M;
+        r.Ma = ga.M;
+        b.rects.push_back(r);
+        b.x_mults += (gb.M / 2 + 1.0) * (double)r.rows * r.w;
+      }
+  std::stable_sort(b.rects.begin(), b.rects.end(), [](const Rect& x, const Rect& y) { return x.n > y.n; });
+  b.big_rects = 0;
+  for (const Rect& r : b.rects) b.big_rects += r.n >= 16;
+  const int chunk = column_chunk((int64_t)b.ns.E.size(), b.L);
+  b.tiles.clear();
+  b.groups.clear();
+  for (int n_min : {0, 16}) {
+    for (const Sector& sec : b.sectors)
+      row_tiles(b.tiles, b.groups, sec.g_ns, sec.ns_off, sec.g_r, sec.r_off, sec.x_off, sec.n_r, b.L, n_min, chunk);
+    if (n_min == 0) b.tiles_total = (int64_t)b.tiles.size();
   }
+  b.big_tiles = (int64_t)b.tiles.size() - b.tiles_total;
 }
 
 // Constants of the closed form, in long double on the host (rounded to pairs of doubles).
@@ -497,10 +535,10 @@ tgba_status build_table(Basis& b, cudaStream_t st) {
   T.r = T.t + (size_t)n2 * n2;
   T.lam = T.r + n2;
   mode_table<<<n2, 128, 0, st>>>(T);
-  const int64_t nns = (int64_t)b.ns.E.size(), nr = (int64_t)b.r.E.size(), work = (int64_t)n2 * n2 + nns + nr;
+  const int64_t nns = (int64_t)b.ns.E.size(), nr = (int64_t)b.r.E.size(), work = (int64_t)n2 * n2 + (nns + nr) * (nns + nr < 16384 ? 8 : 1);
   state_factors<<<(int)std::min<int64_t>((work + 255) / 256, 152 * 8), 256, 0, st>>>(
       T, b.d_table, b.d_c0, nns, nr, b.max_qp, b.d_sel_ns, b.d_sel_r, b.d_M_ns, b.d_M_r, b.d_fac_ns, b.d_fac_r,
-      b.d_pairs_r, std::max(1, b.max_qp / 2), b.d_status);
+      b.d_pairs_r, std::max(1, b.max_qp / 2), nns + nr < 16384 ? 8 : 1, b.d_status);
   TGBA_CUDA(cudaGetLastError());
   b.launches += 2;
   b.table_valid = true;
@@ -508,11 +546,11 @@ tgba_status build_table(Basis& b, cudaStream_t st) {
 }
 
 tgba_status run_elements(Basis& b, cudaStream_t st) {
-  return launch_tiles(b, b.d_rects, (int)b.rects.size(), b.tiles_total, b.d_P, st);
+  return launch_tiles(b, b.d_tiles, b.d_groups, b.tiles_total, b.d_P, st);
 }
 
 tgba_status run_elements_big(Basis& b, cudaStream_t st) {
-  return launch_tiles(b, b.d_rects, b.big_rects, b.big_tiles, b.d_P, st);
+  return launch_tiles(b, b.d_tiles + b.tiles_total, b.d_groups, b.big_tiles, b.d_P, st);
 }
 
 tgba_status run_element_lists(Basis& b, const unsigned* counts, const int64_t* list_off, int sizes,
@@ -537,14 +575,17 @@ tgba_status run_elements_cross(Basis& b, int s_ns, int s_r, double* out, cudaStr
   const Sector& A = b.sectors[s_ns];
   const Sector& B = b.sectors[s_r];
   if (A.n_ns * B.n_r == 0) return TGBA_OK;
-  std::vector<Rect> v;
-  add_rects(v, A.g_ns, A.ns_off, B.g_r, B.r_off, 0, B.n_r, b.L);
-  const int64_t tiles = number_tiles(v, b.L, 0, nullptr);
-  Rect* d = nullptr;
-  TGBA_CUDA(cudaMallocAsync((void**)&d, v.size() * sizeof(Rect), st));
-  cudaError_t e = cudaMemcpyAsync(d, v.data(), v.size() * sizeof(Rect), cudaMemcpyHostToDevice, st);
-  tgba_status r = e == cudaSuccess ? launch_tiles(b, d, (int)v.size(), tiles, out, st)
-                                   : cuda_fail(e, "rectangles of the cross-sector elements");
+  std::vector<RowTile> v;
+  std::vector<ColGroup> cg;
+  row_tiles(v, cg, A.g_ns, A.ns_off, B.g_r, B.r_off, 0, B.n_r, b.L, 0, column_chunk(A.n_ns, b.L));
+  char* d = nullptr;
+  const size_t tb = v.size() * sizeof(RowTile), gb = cg.size() * sizeof(ColGroup);
+  TGBA_CUDA(cudaMallocAsync((void**)&d, tb + gb, st));
+  cudaError_t e = cudaMemcpyAsync(d, v.data(), tb, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d + tb, cg.data(), gb, cudaMemcpyHostToDevice, st);
+  tgba_status r = e == cudaSuccess
+                      ? launch_tiles(b, (const RowTile*)d, (const ColGroup*)(d + tb), (int64_t)v.size(), out, st)
+                      : cuda_fail(e, "tiles of the cross-sector elements");
   cudaFreeAsync(d, st);
   return r;
 }

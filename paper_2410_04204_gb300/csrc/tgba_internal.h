@@ -65,20 +65,30 @@ struct SectorSym {
   int64_t even_off[2] = {0, 0}, odd_off[2] = {0, 0};   // their places in d_mirror
 };
 
-// Work of the element stage: a rectangle of pairs with uniform (M_a, M_b), laid out row-major
-// (row = NS state, column = R state), cut into tiles (elements.cu: x_tiles).
+// A rectangle of pairs with uniform (M_a, M_b), laid out row-major (row = NS state, column = R
+// state): the screener's work.
 struct Rect {
   int64_t out0;   // element index of the rectangle's first pair in the X cache
   int64_t ns0;    // global NS state index of the rectangle's first row
   int64_t r0;     // global R state index of the rectangle's first column
-  int64_t tile0;  // index of the rectangle's first tile within its list
   int32_t ld;     // row stride of the sector's X block (n_r)
   int32_t w;      // rectangle width
   int32_t rows;   // rectangle height
   int32_t n;      // Pfaffian size M_a + M_b
   int32_t Ma;     // quasiparticles of the NS state
+};
+
+// A block's work in the element stage (elements.cu: x_tiles): a few rows of one M_a, a range of columns.
+struct RowTile {
+  int64_t out0;   // where column 0 of the first row goes in X
+  int64_t ns0;    // global index of the first NS state
+  int64_t r_off;  // global index of the R list's first state
+  int32_t ld, rows, Ma;
+  int32_t c0, c1; // columns
+  int32_t g0, g1; // groups of equal M_b that hold them
   int32_t pairs;  // 1: products of mode pairs tabulated per row
 };
+struct ColGroup { int32_t c0, c1, H; };   // columns of M_b = 2 H
 
 // A sector as the assembly kernel sees it: tile0 is its first tile in the launch.
 struct HeffSector { int64_t n_ns, n_r, ns_off, r_off, x_off, h_off, tile0; };
@@ -141,11 +151,13 @@ struct Basis {
   const void* x_screen = nullptr;
   double x_tau = 0;
   int64_t x_evaluated = 0, x_screened = 0;
-  std::vector<Rect> rects;             // all rectangles, n descending, one tile prefix
-  Rect* d_rects = nullptr;
-  int64_t tiles_total = 0;
+  std::vector<Rect> rects;             // all rectangles, n descending
   int big_rects = 0;                   // the first ones: n >= 16
-  int64_t big_tiles = 0;
+  std::vector<RowTile> tiles;          // all row tiles, then (big_tiles of them) those of n >= 16
+  std::vector<ColGroup> groups;
+  RowTile* d_tiles = nullptr;
+  ColGroup* d_groups = nullptr;
+  int64_t tiles_total = 0, big_tiles = 0;
   HeffSector* d_heff_secs = nullptr;   // non-empty sectors (assemble.cu)
   int n_heff_secs = 0;
   int64_t heff_tiles = 0;
