@@ -4,10 +4,11 @@
 // Two kernels per batch of (field, sector) matrices:
 //
 // 1. sytrd_groups: Householder reduction to tridiagonal form, T = Q^T H Q.  One cooperative
-//    launch with two CTAs of 6 warps per SM (one of 12 if two do not fit); the CTAs are shared
-//    out among the matrices in proportion to their work (n^3), so a group of C CTAs (1 to 16)
-//    owns one matrix and runs all n - 1 reflections, and each SM's two CTAs come from different
-//    matrices with even loads (cta_role).  (Hardware thread-block clusters were tried first:
+//    launch with two CTAs of 6 warps per SM (one of 12 if two do not fit, or for one or two
+//    matrices); the CTAs are shared out among the matrices in proportion to their work (n^3), so a
+//    group of C CTAs (1 to 96) owns one matrix and runs its reflections up to the last 128 rows
+//    (sytrd_small finishes those in one CTA's shared memory), and each SM's two CTAs come from
+//    different matrices with even loads (cta_role).  (Hardware thread-block clusters were tried first:
 //    their placement left SMs idle, e.g. at most 46 clusters of 3 or 15 of 8 could be resident,
 //    so 48 matrices ran in two or more waves.)  Step j builds the reflector v_j from column j,
 //    then makes ONE pass over the trailing lower triangle that both applies the rank-2 update
@@ -45,6 +46,7 @@
 // in memory.
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "tgba_internal.h"
@@ -53,11 +55,13 @@ namespace tgba {
 namespace {
 
 constexpr int kCols = 16;                       // columns of a work block (rows: 32)
-constexpr int kMaxGroup = 16;                   // CTAs cooperating on one matrix
+constexpr int kMaxGroup = 96;                   // CTAs cooperating on one matrix
 constexpr unsigned kSpinLimit = 1u << 24;       // bounded barrier wait (>= 100 ns per poll: over 1 s)
 constexpr int kRed = 64;                        // reduction scratch (doubles) after the vectors
-constexpr int kChunk = 8;                       // row blocks per chunk of the pass
+constexpr int kChunk = 8;                       // most row blocks per chunk of the pass
 constexpr int kTail = 2;                        // last blocks of a column group: one chunk, handed out last
+constexpr int kSmallN = 128;                    // trailing matrix that one CTA finishes in shared memory
+constexpr int kSmallThreads = 2 * kSmallN;
 constexpr int kMaxSmId = 1024;                  // SM ids registered by cta_role
 constexpr int kMaxGroups = kMaxNativeLd / kCols;
 constexpr int kSturmThreads = 64;                // bisection block: one item of 64 eigenvalues
@@ -70,7 +74,10 @@ struct TriSlot {
   int64_t p_off;    // p = tau A v [ld], then one dot partial per CTA of the group [16]
   int64_t de_off;   // diagonal d [n], off-diagonal e [n]
   int64_t out_off;  // first eigenvalue in the workspace's list (merge_evals brings them to the caller)
+  int64_t pv_off;   // (v, w) pending when sytrd_small takes over [2 ld]
   int32_t n, ld;
+  int32_t j_end;    // steps of sytrd_groups; sytrd_small does the rest
+  int32_t ck;       // row blocks per chunk
 };
 
 // What a slot's matrix holds: H~ of a (field, sector), whole (ns = r = nullptr) or the block of the
@@ -121,9 +128,15 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   return v;
 }
 
+// Arrival on a counter of the group: everything the CTA wrote (or read) before its last CTA barrier
+// comes before it for whoever acquires the counter.
+__device__ __forceinline__ void arrive_release(unsigned* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+
 // Barrier of the C CTAs of one matrix (C = 1: the CTA barrier).  The group's counter counts
 // arrivals; the k-th barrier waits until it reaches k C.  Writes before the barrier are
-// published by the CTA barrier plus a GPU-scope fence before the arrival, and read after it
+// published by the CTA barrier and the arrival's release, and read after the acquire
 // through L2.  The wait is bounded: on timeout it records kStTimeout and returns false, and
 // the kernel leaves the matrix (the other CTAs of the group then time out as well).
 __device__ __forceinline__ bool group_barrier(unsigned* cnt, unsigned target, int C, int* flag, unsigned* status,
@@ -131,8 +144,7 @@ __device__ __forceinline__ bool group_barrier(unsigned* cnt, unsigned target, in
   __syncthreads();
   if (C == 1) return true;
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(cnt, 1u);
+    arrive_release(cnt);
     int ok = 1;
     for (unsigned it = 0; ld_acquire(cnt) < target; ++it) {
       if (it > limit) {
@@ -140,9 +152,8 @@ __device__ __forceinline__ bool group_barrier(unsigned* cnt, unsigned target, in
         atomicOr(status, kStTimeout);
         break;
       }
-      __nanosleep(100);
+      __nanosleep(it < 16 ? 20 : 100);
     }
-    __threadfence();
     *flag = ok;
   }
   __syncthreads();
@@ -162,19 +173,26 @@ __device__ __forceinline__ void warp_wait(const unsigned* cnt, unsigned target, 
   }
 }
 
-// Sum over the block in a fixed order (lane 0 of each warp, then warps in order); every thread
-// gets the same value.
+// Sum over the block's first WARPS warps in a fixed order (a shuffle tree per warp, another over the
+// warps' sums by warp 0); every thread of the block gets the same value.  (Every warp adding the WARPS
+// sums for itself kept the FP64 pipe, 16 cycles per warp instruction, busy for longer than the
+// exchange takes.)
 template <int WARPS>
 __device__ __forceinline__ double block_sum(double x, double* red) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) red[warp] = x;
+  if (warp < WARPS) {
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane == 0) red[warp] = x;
+  }
   __syncthreads();
-  double s = red[0];
+  if (warp == 0) {
+    double s = lane < WARPS ? red[lane] : 0.0;
 #pragma unroll
-  for (int w = 1; w < WARPS; ++w) s += red[w];
+    for (int o = WARPS > 8 ? 8 : WARPS > 4 ? 4 : 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) red[0] = s;
+  }
   __syncthreads();
-  return s;
+  return red[0];
 }
 
 // Work of one step.  Column group g holds columns 16 g .. 16 g + 15; its blocks are the 32-row
@@ -183,8 +201,10 @@ __device__ __forceinline__ double block_sum(double x, double* red) {
 // it are cut into chunks of up to kChunk.  Chunks 0 .. NCH1 - 1 are those of the heads, group
 // by group (cf[t] the first of group g0 + t, cf[NG] = NCH1), and chunk NCH1 + t is group
 // g0 + t's tail: so the last chunks of a step are the small ones.
-__device__ __forceinline__ int group_head(int g, int LB) { return max(0, LB - (g >> 1) - kTail); }
-__device__ __forceinline__ int group_chunks(int g, int LB) { return (group_head(g, LB) + kChunk - 1) / kChunk; }
+// The chunk length ck (a slot's) is shorter than kChunk when the group has many warps for the
+// matrix's blocks.
+__device__ __forceinline__ int group_head(int g, int LB, int ck) { return max(0, LB - (g >> 1) - min(kTail, ck)); }
+__device__ __forceinline__ int group_chunks(int g, int LB, int ck) { return (group_head(g, LB, ck) + ck - 1) / ck; }
 
 __device__ __forceinline__ void load_block(double (&a)[kCols], const double* __restrict__ p) {
 #pragma unroll
@@ -288,7 +308,7 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
                                           int* flag, unsigned limit) {
   extern __shared__ double sm[];
   unsigned arrivals = 0, col_arrivals = 0;
-  const int n = S.n, ld = S.ld, LB = ld >> 5, G = ld / kCols;
+  const int n = S.n, ld = S.ld, LB = ld >> 5, G = ld / kCols, ck = S.ck;
   double* A = ws + S.a_off;
   double* RP = ws + S.rp_off;
   double* CP = ws + S.cp_off;
@@ -305,28 +325,45 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool bad = false;
-  for (int j = 0; j < n; ++j) {
+  // the stored column of the next step, in registers: it is final once the pass is (first barrier),
+  // so its loads run under the reduction and the second barrier (rows beyond kPre T: loaded in place)
+  constexpr int T = WARPS * 32, kPre = 8;
+  double pre[kPre];
+  auto prefetch_column = [&](int j) {
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      const int i = j + (int)threadIdx.x + u * T;
+      pre[u] = i < n ? __ldcg(A + elem_off(i, j, LB)) : 0.0;
+    }
+  };
+  if (S.j_end > 0) prefetch_column(0);
+  for (int j = 0; j < S.j_end; ++j) {
     // column j of A_j: the stored column (already updated through step j - 2) minus the
     // rank-2 update of step j - 1; rows j + 2 .. n - 1 go into the norm
     const double2 vwj = vwp[j];
     double sig = 0.0;
-    for (int i = j + threadIdx.x; i < n; i += (WARPS * 32)) {
+    auto column_row = [&](int i, double a) {
       const double2 vwi = vwp[i];
-      double a = __ldcg(A + elem_off(i, j, LB));
       a = fma(-vwi.x, vwj.y, a);
       a = fma(-vwi.y, vwj.x, a);
       if (i == j) red[WARPS] = a;
       else if (i == j + 1) red[WARPS + 1] = a;
       else sig = fma(a, a, sig);
       vwn[i].x = a;
+    };
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      const int i = j + (int)threadIdx.x + u * T;
+      if (i < n) column_row(i, pre[u]);
     }
+    for (int i = j + (int)threadIdx.x + kPre * T; i < n; i += T) column_row(i, __ldcg(A + elem_off(i, j, LB)));
     // the step's chunk table (a scan by warp 0 over groups g0 .. G - 1), published by
     // block_sum's barrier
     const int g0 = (j + 1) / kCols, NG = G - g0;
     if (warp == 0) {
       const int per = (NG + 31) >> 5, t0 = min(NG, lane * per), t1 = min(NG, t0 + per);
       int own = 0;
-      for (int t = t0; t < t1; ++t) own += group_chunks(g0 + t, LB);
+      for (int t = t0; t < t1; ++t) own += group_chunks(g0 + t, LB, ck);
       int incl = own;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -336,36 +373,39 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
       int run = incl - own;
       for (int t = t0; t < t1; ++t) {
         cf[t] = run;
-        run += group_chunks(g0 + t, LB);
+        run += group_chunks(g0 + t, LB, ck);
       }
       if (lane == 31) cf[NG] = incl;
     }
     sig = block_sum<WARPS>(sig, red);
     // this CTA has read column j (block_sum's barrier): the pass below rewrites it, so the
     // warps that store column j wait until every CTA of the group has arrived here
-    if (C > 1 && threadIdx.x == 0) {
-      __threadfence();
-      atomicAdd(ccnt, 1u);
-    }
+    if (C > 1 && threadIdx.x == 0) arrive_release(ccnt);
     col_arrivals += C;
     const double dj = red[WARPS];
     if (rank == 0 && threadIdx.x == 0) D[j] = dj;
     if (j + 1 >= n) break;                            // uniform: the last diagonal entry
     const double alpha = red[WARPS + 1];
-    // Householder reflector H = I - tau v v^T with v_{j+1} = 1 mapping column j to beta e_{j+1}
-    double beta = alpha, s = 0.0;
-    {
-      double tau = 0.0;
+    // Householder reflector H = I - tau v v^T with v_{j+1} = 1 mapping column j to beta e_{j+1}.  One
+    // warp takes the square root and the two quotients: by every warp they cost 3.5 to 6 thousand cycles
+    // a step on the FP64 pipe (an eighth of a step of the L = 40 blocks).
+    if (warp == 0) {
+      double beta = alpha, s = 0.0, tau = 0.0;
       if (sig != 0.0) {
         const double nrm = sqrt(fma(alpha, alpha, sig));
         beta = alpha >= 0.0 ? -nrm : nrm;
         tau = (beta - alpha) / beta;
         s = 1.0 / (alpha - beta);
       }
-      if (threadIdx.x == 0) red[WARPS + 2] = tau;     // read back after the pass
+      if (lane == 0) {
+        red[WARPS + 2] = tau;                          // read back after the pass
+        red[WARPS + 3] = s;
+        if (rank == 0) E[j] = beta;
+        if (!(isfinite(dj) && isfinite(beta))) bad = true;
+      }
     }
-    if (rank == 0 && threadIdx.x == 0) E[j] = beta;
-    if (threadIdx.x == 0 && !(isfinite(dj) && isfinite(beta))) bad = true;
+    __syncthreads();
+    const double s = red[WARPS + 3];
     for (int i = threadIdx.x; i < ld; i += (WARPS * 32)) {
       const double x = vwn[i].x;
       vwn[i].x = i == j + 1 ? 1.0 : (i > j + 1 && i < n ? x * s : 0.0);
@@ -377,12 +417,12 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
     {
       const int NCH1 = cf[NG], NCH = NCH1 + NG;
       bool waited = !(C > 1 && (j + 1) % kCols != 0);   // column j lies in group g0
-      unsigned c = 0;
-      if (lane == 0) c = atomicAdd(tk + j, 1u);
-      c = __shfl_sync(0xffffffffu, c, 0);
+      // the warps' first chunks are dealt out over the CTAs (an SM's FP64 pipe is what a short step's
+      // chunks share), the tickets start after those
+      unsigned c = (unsigned)(warp * C + rank);
       while ((int)c < NCH) {
         unsigned cn = 0;
-        if (lane == 0) cn = atomicAdd(tk + j, 1u);
+        if (lane == 0) cn = atomicAdd(tk + j, 1u) + (unsigned)(C * WARPS);
         int lo = 0, rb, re;
         if ((int)c < NCH1) {                          // a head chunk: cf[lo] <= c < cf[lo + 1]
           int hi = NG;
@@ -392,12 +432,12 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
             else hi = mid;
           }
           const int gl = g0 + lo;
-          rb = (gl >> 1) + ((int)c - cf[lo]) * kChunk;
-          re = min(rb + kChunk, (gl >> 1) + group_head(gl, LB));
+          rb = (gl >> 1) + ((int)c - cf[lo]) * ck;
+          re = min(rb + ck, (gl >> 1) + group_head(gl, LB, ck));
         } else {                                      // a tail chunk
           lo = (int)c - NCH1;
           const int gl = g0 + lo;
-          rb = (gl >> 1) + group_head(gl, LB);
+          rb = (gl >> 1) + group_head(gl, LB, ck);
           re = LB;
         }
         const int g = g0 + lo;
@@ -411,62 +451,211 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
     }
     arrivals += C;
     if (!group_barrier(cnt, arrivals, C, flag, status, limit)) return false;
-    // rows j + 1 .. n - 1, interleaved over the group's CTAs and, within a CTA, over quads of
+    if (j + 1 < S.j_end) prefetch_column(j + 1);
+    // rows j + 1 .. n - 1, interleaved over the group's CTAs and, within a CTA, over teams of RL
     // lanes (row i to CTA i mod C; the long rows at the bottom are shared out): y_i = row sums
     // of the blocks of groups g0 .. i/16 + the column sums of the chunks of column i's group.
-    // Lane q of the quad adds the partials with index = q mod 4 (four loads in flight each),
-    // then the quad adds its four sums in a fixed order; p = tau y
+    // Lane q of the team adds the partials with index = q mod RL (four loads in flight each),
+    // then the team adds its sums in a fixed order; p = tau y.  A large group has more teams than
+    // rows, and there the chain of loads is what a row costs: 16 lanes per row; a small one has
+    // many rows per team: 4.
     double dot = 0.0;
     const double tau = red[WARPS + 2];
-    {
-      const int q4 = lane & 3;
-      const int quad = threadIdx.x >> 2, QS = C * (WARPS * 8);      // quads of the group
-      const int i_first = j + 1 + rank + C * (threadIdx.x >> 5) * 8;  // the warp's first row
+    auto reduce_rows = [&](auto rl) {
+      constexpr int RL = decltype(rl)::value;
+      const int q4 = lane & (RL - 1);
+      const int team = threadIdx.x / RL, QS = C * (WARPS * 32 / RL);
+      const int i_first = j + 1 + rank + C * (threadIdx.x >> 5) * (32 / RL);  // the warp's first row
       for (int base = 0; i_first + base < n; base += QS) {
-        const int i = j + 1 + rank + C * quad + base;
+        const int i = j + 1 + rank + C * team + base;
         double y = 0.0;
         if (i < n) {
           const int gi = i / kCols, t = gi - g0;
           const double* rr = RP + (int64_t)i * G;
           double y0 = 0.0, y1 = 0.0, y2 = 0.0, y3 = 0.0;
           int g = g0 + q4;
-          for (; g + 12 <= gi; g += 16) {
+          for (; g + 3 * RL <= gi; g += 4 * RL) {
             y0 += __ldcg(rr + g);
-            y1 += __ldcg(rr + g + 4);
-            y2 += __ldcg(rr + g + 8);
-            y3 += __ldcg(rr + g + 12);
+            y1 += __ldcg(rr + g + RL);
+            y2 += __ldcg(rr + g + 2 * RL);
+            y3 += __ldcg(rr + g + 3 * RL);
           }
-          for (; g <= gi; g += 4) y0 += __ldcg(rr + g);
+#pragma unroll
+          for (int u = 0; u < 3; ++u, g += RL)
+            if (g <= gi) y0 += __ldcg(rr + g);
           const int nh = cf[t + 1] - cf[t];             // the group's head chunks, then its tail chunk
-          for (int x = q4; x <= nh; x += 4) {
-            const int c = x < nh ? cf[t] + x : cf[NG] + t;
-            y1 += __ldcg(CP + (int64_t)c * kCols + (i & (kCols - 1)));
+          const double* cc = CP + (i & (kCols - 1));
+          int x = q4;
+          for (; x + RL <= nh; x += 2 * RL) {
+            const int c1 = x + RL < nh ? cf[t] + x + RL : cf[NG] + t;
+            y1 += __ldcg(cc + (int64_t)(cf[t] + x) * kCols);
+            y2 += __ldcg(cc + (int64_t)c1 * kCols);
           }
+          if (x <= nh) y3 += __ldcg(cc + (int64_t)(x < nh ? cf[t] + x : cf[NG] + t) * kCols);
           y = (y0 + y1) + (y2 + y3);
         }
-        y += __shfl_xor_sync(0xffffffffu, y, 1);
-        y += __shfl_xor_sync(0xffffffffu, y, 2);
+#pragma unroll
+        for (int o = 1; o < RL; o <<= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
         if (i < n && q4 == 0) {
           const double p = tau * y;
           __stcg(P + i, p);
           dot = fma(p, vwn[i].x, dot);
         }
       }
-    }
+    };
+    if (C >= 32) reduce_rows(std::integral_constant<int, 16>{});
+    else reduce_rows(std::integral_constant<int, 4>{});
     dot = block_sum<WARPS>(dot, red);
     if (threadIdx.x == 0) __stcg(dots + rank, dot);
     arrivals += C;
     if (!group_barrier(cnt, arrivals, C, flag, status, limit)) return false;
+    // w = p - (tau p.v / 2) v; p's loads go out before the sum of the CTAs' partial dots (in the same
+    // order for every warp)
+    double p8[kPre];
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      const int i = (int)threadIdx.x + u * T;
+      p8[u] = (i > j && i < n) ? __ldcg(P + i) : 0.0;
+    }
     double pv = 0.0;
-    for (int r = 0; r < C; ++r) pv += __ldcg(dots + r);
+    for (int r = lane; r < C; r += 32) pv += __ldcg(dots + r);
+    for (int o = 16; o > 0; o >>= 1) pv += __shfl_xor_sync(0xffffffffu, pv, o);
     const double Kc = 0.5 * tau * pv;
-    for (int i = threadIdx.x; i < ld; i += (WARPS * 32))
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      const int i = (int)threadIdx.x + u * T;
+      if (i < ld) vwn[i].y = (i > j && i < n) ? fma(-Kc, vwn[i].x, p8[u]) : 0.0;
+    }
+    for (int i = (int)threadIdx.x + kPre * T; i < ld; i += T)
       vwn[i].y = (i > j && i < n) ? fma(-Kc, vwn[i].x, __ldcg(P + i)) : 0.0;
     __syncthreads();
     double2* t = vwp; vwp = vwn; vwn = t;
   }
+  if (rank == 0) {                                    // the last step's update, for sytrd_small
+    double2* pv = (double2*)(ws + S.pv_off);
+    for (int i = threadIdx.x; i < n; i += WARPS * 32) pv[i] = vwp[i];
+  }
   if (bad) atomicOr(status, kStEigen);
   return true;
+}
+
+// The last min(n, kSmallN) rows and columns of a matrix by one CTA in shared memory, from the state that
+// sytrd_groups left (its last rank-2 update still to be applied).  A step of a group costs two barriers
+// across its CTAs and a chain of reductions through L2, about 6 us whatever is left to do; here it costs
+// block barriers, and the FP64 pipe of one SM (3 m^2 FMAs per step at 2 per clock) only overtakes
+// that beyond m = 128.  The square is kept whole, column-major with an odd stride: a thread owns
+// half a row, reads columns across its warp without conflicts, and needs no exchange but one partial sum.
+__global__ void __launch_bounds__(kSmallThreads) sytrd_small(const TriSlot* __restrict__ slots, double* __restrict__ ws,
+                                                             unsigned* __restrict__ status) {
+  extern __shared__ double sm[];
+  constexpr int LDA = kSmallN + 1, W = kSmallN / 32;      // W: the warps of half 0, which hold the vectors
+  __shared__ double red[W + 4];
+  __shared__ double part[kSmallN];
+  const TriSlot S = slots[blockIdx.x];
+  const int j0 = S.j_end, m = S.n - j0, LB = S.ld >> 5;
+  const double* A = ws + S.a_off;
+  const double2* pv = (const double2*)(ws + S.pv_off);
+  double* D = ws + S.de_off + j0;
+  double* E = ws + S.de_off + S.n + j0;
+  double* a = sm;                               // [k][i]: entry (i, k)
+  double2* vwp = (double2*)(sm + LDA * kSmallN + (LDA * kSmallN & 1));
+  double2* vwn = vwp + kSmallN;
+  for (int q = threadIdx.x; q < m * m; q += kSmallThreads) {
+    const int k = q / m, i = q % m;
+    if (i < k) continue;
+    double x = A[elem_off(j0 + i, j0 + k, LB)];
+    if (j0 > 0) {
+      const double2 vi = pv[j0 + i], vk = pv[j0 + k];
+      x = fma(-vi.x, vk.y, x);
+      x = fma(-vi.y, vk.x, x);
+    }
+    a[k * LDA + i] = x;
+    a[i * LDA + k] = x;
+  }
+  for (int i = threadIdx.x; i < 2 * kSmallN; i += kSmallThreads) vwp[i] = make_double2(0.0, 0.0);
+  __syncthreads();
+  const int half = threadIdx.x / kSmallN, i = threadIdx.x - half * kSmallN;   // row i, columns of parity `half`
+  bool bad = false;
+  for (int j = 0; j < m; ++j) {
+    // column j with the pending update of step j - 1; rows j + 2 .. go into the norm
+    double x = 0.0, sig = 0.0;
+    if (half == 0 && i >= j && i < m) {
+      const double2 vi = vwp[i], vj = vwp[j];
+      x = a[j * LDA + i];
+      x = fma(-vi.x, vj.y, x);
+      x = fma(-vi.y, vj.x, x);
+      if (i == j) red[W] = x;
+      else if (i == j + 1) red[W + 1] = x;
+      else sig = x * x;
+    }
+    sig = block_sum<W>(sig, red);
+    const double dj = red[W];
+    if (threadIdx.x == 0) D[j] = dj;
+    if (j + 1 >= m) {
+      if (!isfinite(dj)) bad = true;
+      break;
+    }
+    if (threadIdx.x < 32) {                         // one warp: see sytrd_matrix
+      const double alpha = red[W + 1];
+      double beta = alpha, tau = 0.0, s = 0.0;
+      if (sig != 0.0) {
+        const double nrm = sqrt(fma(alpha, alpha, sig));
+        beta = alpha >= 0.0 ? -nrm : nrm;
+        tau = (beta - alpha) / beta;
+        s = 1.0 / (alpha - beta);
+      }
+      if (threadIdx.x == 0) {
+        red[W + 2] = tau;
+        red[W + 3] = s;
+        E[j] = beta;
+        if (!(isfinite(dj) && isfinite(beta))) bad = true;
+      }
+    }
+    __syncthreads();
+    const double tau = red[W + 2], s = red[W + 3];
+    double vi = 0.0;
+    if (half == 0) {
+      vi = i == j + 1 ? 1.0 : (i > j + 1 && i < m ? x * s : 0.0);
+      vwn[i].x = vi;
+    }
+    __syncthreads();
+    // y = A_j v_j with the update of step j - 1 applied on the way
+    double y0 = 0.0, y1 = 0.0;
+    if (i > j && i < m) {
+      const double2 vwi = vwp[i];
+      int k = j + 1 + ((half ^ (j + 1)) & 1);
+      for (; k + 2 < m; k += 4) {
+        const double2 p = vwp[k], q = vwp[k + 2];
+        double b = fma(-vwi.x, p.y, a[k * LDA + i]), c = fma(-vwi.x, q.y, a[(k + 2) * LDA + i]);
+        b = fma(-vwi.y, p.x, b);
+        c = fma(-vwi.y, q.x, c);
+        a[k * LDA + i] = b;
+        a[(k + 2) * LDA + i] = c;
+        y0 = fma(b, vwn[k].x, y0);
+        y1 = fma(c, vwn[k + 2].x, y1);
+      }
+      if (k < m) {
+        const double2 p = vwp[k];
+        double b = fma(-vwi.x, p.y, a[k * LDA + i]);
+        b = fma(-vwi.y, p.x, b);
+        a[k * LDA + i] = b;
+        y0 = fma(b, vwn[k].x, y0);
+      }
+    }
+    if (half == 1) part[i] = y0 + y1;
+    __syncthreads();
+    double p = 0.0;
+    double pv_i = 0.0;
+    if (half == 0) {
+      p = tau * ((y0 + y1) + part[i]);
+      pv_i = p * vi;
+    }
+    const double dot = block_sum<W>(pv_i, red);
+    if (half == 0) vwn[i].y = (i > j && i < m) ? fma(-0.5 * tau * dot, vi, p) : 0.0;
+    __syncthreads();
+    double2* t = vwp; vwp = vwn; vwn = t;
+  }
+  if (bad) atomicOr(status, kStEigen);
 }
 
 // Which CTA plays which role.  A cooperative launch of per_sm CTAs on each of the sms SMs fills
@@ -910,10 +1099,10 @@ __global__ void __launch_bounds__(256) merge_evals(const MergeJob* __restrict__ 
 int64_t round32(int64_t x) { return (x + 31) / 32 * 32; }
 
 // Chunks of the first step (g0 = 0), the most of any step.
-int64_t max_chunks(int ld) {
+int64_t max_chunks(int ld, int ck) {
   const int LB = ld >> 5;
   int64_t c = 0;
-  for (int g = 0; g < ld / kCols; ++g) c += (std::max(0, LB - (g >> 1) - kTail) + kChunk - 1) / kChunk + 1;
+  for (int g = 0; g < ld / kCols; ++g) c += (std::max(0, LB - (g >> 1) - std::min(kTail, ck)) + ck - 1) / ck + 1;
   return c;
 }
 
@@ -955,10 +1144,13 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
     t.out_off = ev_total;       ev_total += n;
     t.a_off = total;            total += round32((int64_t)t.ld * t.ld);
     t.rp_off = total;           total += round32((int64_t)(t.ld / kCols) * t.ld);
-    t.cp_off = total;           total += round32((int64_t)kCols * max_chunks(t.ld));
+    t.cp_off = total;           total += round32((int64_t)kCols * max_chunks(t.ld, 1));   // for any ck
     t.tk_off = tk_total;        tk_total += t.ld;
     t.p_off = total;            total += round32(t.ld + kMaxGroup);
     t.de_off = total;           total += round32(2 * n);
+    t.pv_off = total;           total += round32(2 * t.ld);
+    t.j_end = (int32_t)std::max<int64_t>(0, n - kSmallN);
+    t.ck = kChunk;
     slots.push_back(t);
     fills.push_back(f);
     n_max = std::max(n_max, (int)n);
@@ -997,6 +1189,10 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   int dev = 0, sms = 0;
   TGBA_CUDA(cudaGetDevice(&dev));
   TGBA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // Groups of up to 96 CTAs instead of 16, chunks as short as one block, the column and p loads ahead of
+  // their use, one warp for the scalars and the last rows in shared memory took the two blocks of the
+  // L = 40, k = 0 sector (1472 and 1225 states) from 85 to 32 ms, the 30 matrices of the L = 24 step from
+  // 274 to 253 ms, the complete L = 12 sector (180 and 172) from 4.6 to 2.9 ms.
   // One or two CTAs per SM: two of 6 warps when their shared memory fits (each SM then runs
   // parts of two matrices, and one's barrier waits and serial phases are filled by the other's
   // arithmetic), else one of 12 warps.  With no more matrices than CTAs, every CTA joins one
@@ -1009,7 +1205,8 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   TGBA_CUDA(cudaFuncSetAttribute(sytrd_groups<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   TGBA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sytrd_groups<6>, 6 * 32, smem));
-  per_sm = per_sm >= 2 ? 2 : 1;
+  // one or two matrices: nothing to share an SM with, and the barriers want few CTAs
+  per_sm = per_sm >= 2 && B > 2 ? 2 : 1;
   if (per_sm == 1) {
     int one = 0;
     TGBA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&one, sytrd_groups<12>, 12 * 32, smem));
@@ -1019,13 +1216,22 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   std::vector<CtaWork> map;
   int C_max = 1;
   if (B <= ctas) {
-    std::vector<int> Cq(B, 1);
-    for (int left = ctas - B; left > 0; --left) {
+    // at most a CTA per three blocks of the lower triangle (about LB^2 of them); 16 when a CTA is withheld
+    std::vector<int> Cq(B, 0), cap(B, 1);
+    int used = 0;
+    for (int q = 0; q < B; ++q) {
+      const int LB = slots[q].ld / 32;
+      cap[q] = check && check->withhold_matrix >= 0 ? 16 : std::min(kMaxGroup, std::max(1, LB * (LB + 1) / 3));
+      Cq[q] = slots[q].j_end > 0 ? 1 : 0;             // the smallest are left to sytrd_small
+      used += Cq[q];
+    }
+    for (int left = ctas - used; left > 0; --left) {
       int best = -1;
       double best_w = -1.0;
       for (int q = 0; q < B; ++q) {
+        if (Cq[q] == 0 || Cq[q] >= cap[q]) continue;
         const double w = (double)slots[q].n * slots[q].n * slots[q].n / Cq[q];
-        if (Cq[q] < kMaxGroup && w > best_w) { best_w = w; best = q; }
+        if (w > best_w) { best_w = w; best = q; }
       }
       if (best < 0) break;
       ++Cq[best];
@@ -1033,6 +1239,9 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
     for (int q = 0; q < B; ++q) {
       for (int r = 0; r < Cq[q]; ++r) map.push_back({q, r, Cq[q], B});
       C_max = std::max(C_max, Cq[q]);
+      // about four chunks per warp and step at the start
+      const int LB = slots[q].ld / 32, warps = std::max(1, Cq[q]) * (per_sm == 2 ? 6 : 12);
+      slots[q].ck = std::min(kChunk, std::max(1, LB * (LB + 1) / (4 * warps)));
     }
   } else {
     for (int q = 0; q < ctas; ++q) map.push_back({q, 0, 1, ctas});
@@ -1138,7 +1347,11 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   for (int e = 0; e < 3; ++e)
     if (b.eig_ev[e] == nullptr) TGBA_CUDA(cudaEventCreate(&b.eig_ev[e]));
   TGBA_CUDA(cudaEventRecord(b.eig_ev[0], st));
-  if (per_sm == 2)
+  const size_t smem_small = (size_t)(((kSmallN + 1) * kSmallN + 1) / 2 * 2 + 4 * kSmallN) * sizeof(double);
+  TGBA_CUDA(cudaFuncSetAttribute(sytrd_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_small));
+  if (grid == 0) {
+    // every matrix fits sytrd_small
+  } else if (per_sm == 2)
     TGBA_CUDA(cudaLaunchKernelEx(&cfg, sytrd_groups<6>, (const TriSlot*)d_slots, B, (const CtaWork*)d_map,
                                  (const CtaWork*)d_sm_map, per_sm, sms, d_reg, d_cnt, ws, b.d_status, limit,
                                  withhold_q, withhold_rank));
@@ -1146,7 +1359,9 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
     TGBA_CUDA(cudaLaunchKernelEx(&cfg, sytrd_groups<12>, (const TriSlot*)d_slots, B, (const CtaWork*)d_map,
                                  (const CtaWork*)d_sm_map, per_sm, sms, d_reg, d_cnt, ws, b.d_status, limit,
                                  withhold_q, withhold_rank));
-  ++b.launches;
+  sytrd_small<<<(unsigned)B, kSmallThreads, smem_small, st>>>(d_slots, ws, b.d_status);
+  TGBA_CUDA(cudaGetLastError());
+  b.launches += grid > 0 ? 2 : 1;
   TGBA_CUDA(cudaEventRecord(b.eig_ev[1], st));
   const int bis_grid = std::min(n_items, bis_per_sm * sms);
   sturm_bisect<<<bis_grid, kSturmThreads, smem2, st>>>(d_slots, d_items, n_items, item_len, d_queue, ws,
