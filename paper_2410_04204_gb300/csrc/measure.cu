@@ -1,0 +1,685 @@
+// Spectral measure of a tridiagonalised H~ = Q T Q^T with respect to a vector (row a8: the weights of
+// Eq. 8-9 are (u_a^T v)^2 over all eigenvectors u_a, with one v).  The eigenvectors themselves are not
+// needed, only their products with q = Q^T v:
+//  * apply_q: Q x or Q^T x from the kept reflectors, 16 at a time in compact WY form (Schreiber and Van
+//    Loan, SIAM J. Sci. Stat. Comput. 10 (1989) 53): I - V T V^T;
+//  * lowest_vector: the eigenvector of T for its lowest eigenvalue by the twisted factorisation
+//    (Parlett and Dhillon, Linear Algebra Appl. 267 (1997) 247);
+//  * spectral_rows: all eigenvalues lambda_a of T and the products s_a^T q with its eigenvectors, by
+//    divide and conquer (Cuppen, Numer. Math. 36 (1981) 177) that carries three row vectors of the
+//    eigenvector matrix S instead of S: its first and last row, which the next merge needs, and q^T S.
+//    A merge of size k then costs O(k^2): the secular equation's roots, the z vector recomputed from
+//    them so that the eigenvectors of the merge are orthogonal to working precision (Gu and Eisenstat,
+//    SIAM J. Matrix Anal. Appl. 16 (1995) 172), and three sums per root.  Near-degenerate levels are
+//    deflated by exact rotations, so their summed weights are as exact as the others.
+// The library's eigen-decomposition with vectors that this replaces took 180 ms for n = 2697 (all of S(0, w)
+// now 36 ms, most of it the tridiagonalisation).
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "tgba_internal.h"
+
+namespace tgba {
+namespace {
+
+constexpr int kWY = 16;          // reflectors per block of apply_q
+constexpr int kLeaf = 20;        // largest leaf of the divide and conquer
+constexpr double kEps = 0x1p-53;
+
+// ------------------------------------------------------------------ Q
+// T factor of reflectors j0 .. j0 + 15 (block g): H_{j0} ... = I - V T V^T, T upper triangular, from the
+// Gram matrix of the reflectors (one block of 256 threads each).
+__global__ void __launch_bounds__(256) wy_factors(int n, int ld, const double* __restrict__ v, double* __restrict__ T) {
+  __shared__ double g[kWY][kWY + 1];
+  __shared__ double t[kWY][kWY + 1];
+  const int j0 = blockIdx.x * kWY, k = min(kWY, n - 1 - j0);
+  const double* tau = v + (int64_t)ld * ld;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int p = warp; p < k * k; p += 8) {
+    const int a = p / k, c = p % k;
+    if (a >= c) continue;
+    const double *x = v + (int64_t)(j0 + a) * ld, *y = v + (int64_t)(j0 + c) * ld;
+    double s = 0.0;
+    for (int i = j0 + c + 1 + lane; i < n; i += 32) s = fma(x[i], y[i], s);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) g[a][c] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < kWY) {
+    const int a = threadIdx.x;               // row a of T, column by column
+    for (int c = 0; c < kWY; ++c) {
+      __syncwarp(0xffffu);
+      const double tc = c < k ? tau[j0 + c] : 0.0;
+      double x = 0.0;
+      if (a == c) x = tc;
+      else if (a < c && c < k) {
+        for (int b = a; b < c; ++b) x = fma(t[a][b], g[b][c], x);
+        x *= -tc;
+      }
+      t[a][c] = x;
+    }
+    for (int c = 0; c < kWY; ++c) T[(int64_t)blockIdx.x * kWY * kWY + a * kWY + c] = t[a][c];
+  }
+}
+
+// x <- Q x (blocks last to first) or Q^T x (first to last): one CTA, x in shared memory.  Bound by one
+// SM's reads of the reflectors from L2 (twice n^2/2 doubles).
+constexpr int kApplyThreads = 1024;
+__global__ void __launch_bounds__(kApplyThreads) wy_apply(int n, int ld, bool transpose, const double* __restrict__ v,
+                                                          const double* __restrict__ T, double* __restrict__ x) {
+  extern __shared__ double sx[];
+  __shared__ double part[2 * kWY], w[kWY];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nb = (n - 1 + kWY - 1) / kWY;
+  for (int i = threadIdx.x; i < n; i += kApplyThreads) sx[i] = x[i];
+  __syncthreads();
+  for (int b = 0; b < nb; ++b) {
+    const int g = transpose ? b : nb - 1 - b, j0 = g * kWY, k = min(kWY, n - 1 - j0);
+    {
+      // dots: warps 2 c and 2 c + 1 take the two halves of column c
+      const int c = warp >> 1, h = warp & 1;
+      double s0 = 0.0, s1 = 0.0;
+      if (c < k) {
+        const double* vc = v + (int64_t)(j0 + c) * ld;
+        int i = j0 + 1 + h * 32 + lane;
+        for (; i + 64 < n; i += 128) {
+          s0 = fma(vc[i], sx[i], s0);
+          s1 = fma(vc[i + 64], sx[i + 64], s1);
+        }
+        if (i < n) s0 = fma(vc[i], sx[i], s0);
+      }
+      double s = s0 + s1;
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) part[warp] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < kWY) {
+      const double* t = T + (int64_t)g * kWY * kWY;
+      double s = 0.0;
+      for (int c = 0; c < kWY; ++c) {
+        const double d = part[2 * c] + part[2 * c + 1];
+        s = fma(transpose ? t[c * kWY + threadIdx.x] : t[threadIdx.x * kWY + c], d, s);
+      }
+      w[threadIdx.x] = s;
+    }
+    __syncthreads();
+    for (int i = j0 + 1 + threadIdx.x; i < n; i += kApplyThreads) {
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+      for (int c = 0; c < kWY; c += 2) {
+        if (c < k) s0 = fma(v[(int64_t)(j0 + c) * ld + i], w[c], s0);
+        if (c + 1 < k) s1 = fma(v[(int64_t)(j0 + c + 1) * ld + i], w[c + 1], s1);
+      }
+      sx[i] -= s0 + s1;
+    }
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < n; i += kApplyThreads) x[i] = sx[i];
+}
+
+// Unit eigenvector of T for the eigenvalue *lambda: the pivots of T - lambda from both ends, the index
+// where they meet with the smallest residual, and the two recurrences from there.
+__global__ void __launch_bounds__(64) twisted(int n, const double* __restrict__ d, const double* __restrict__ lambda,
+                                              double* __restrict__ fw, double* __restrict__ bw, double* __restrict__ x) {
+  const double* e = d + n;
+  const double l = *lambda;
+  __shared__ int s_r;
+  __shared__ double s_n[64];
+  const double tiny = 1e-300;
+  if (threadIdx.x == 0) {
+    double p = d[0] - l;
+    for (int i = 0;; ++i) {
+      if (fabs(p) < tiny) p = p < 0.0 ? -tiny : tiny;
+      fw[i] = p;
+      if (i + 1 == n) break;
+      p = (d[i + 1] - l) - e[i] * (e[i] / p);
+    }
+  } else if (threadIdx.x == 32) {
+    double p = d[n - 1] - l;
+    for (int i = n - 1;; --i) {
+      if (fabs(p) < tiny) p = p < 0.0 ? -tiny : tiny;
+      bw[i] = p;
+      if (i == 0) break;
+      p = (d[i - 1] - l) - e[i - 1] * (e[i - 1] / p);
+    }
+  }
+  __syncthreads();
+  // |fw + bw - (d - l)| smallest (NaN never is)
+  double best = INFINITY;
+  int bi = 0;
+  for (int i = threadIdx.x; i < n; i += 64) {
+    const double g = fabs(fw[i] + bw[i] - (d[i] - l));
+    if (g < best) { best = g; bi = i; }
+  }
+  s_n[threadIdx.x] = best;
+  __syncthreads();
+  for (int t = 0; t < 64; ++t)
+    if (s_n[t] < best) best = s_n[t];
+  if (threadIdx.x == 0) s_r = n;
+  __syncthreads();
+  if (fabs(fw[bi] + bw[bi] - (d[bi] - l)) == best) atomicMin(&s_r, bi);
+  __syncthreads();
+  const int r = min(s_r, n - 1);
+  if (threadIdx.x == 0) {
+    x[r] = 1.0;
+    double z = 1.0;
+    for (int i = r - 1; i >= 0; --i) { z = -(e[i] / fw[i]) * z; x[i] = z; }
+  } else if (threadIdx.x == 32) {
+    double z = 1.0;
+    for (int i = r + 1; i < n; ++i) { z = -(e[i - 1] / bw[i]) * z; x[i] = z; }
+  }
+  __syncthreads();
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += 64) s = fma(x[i], x[i], s);
+  s_n[threadIdx.x] = s;
+  __syncthreads();
+  s = 0.0;
+  for (int t = 0; t < 64; ++t) s += s_n[t];
+  const double inv = 1.0 / sqrt(s);
+  for (int i = threadIdx.x; i < n; i += 64) x[i] *= inv;
+}
+
+// ------------------------------------------------------------------ divide and conquer
+// Per-index arrays of the whole matrix, each node using its own range [lo, hi).
+struct Dc {
+  int n;
+  const double* e;            // off-diagonal of T
+  double *lam, *r0, *r1, *rq; // eigenvalues and the three rows
+  double *D, *z;              // merge: not deflated values and z (ascending), then the deflated values
+  double *f0, *f1, *fq;       // rows of the sources, in the order of D
+  double *tau, *zh;           // roots relative to their origin; recomputed z
+  int *org;                   // the root's origin
+  int *K;                     // [node] not deflated
+  double *rho;                // [node]
+};
+struct Node { int lo, mid, hi; };
+
+// The tears: both diagonal entries at a cut lose |e| (dt: a copy of T's diagonal).
+__global__ void dc_tear(int n, const double* __restrict__ d, const int* __restrict__ cuts, int n_cuts,
+                        double* __restrict__ dt) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dt[i] = d[i];
+  __syncthreads();
+  for (int c = threadIdx.x; c < n_cuts; c += blockDim.x) {
+    const int m = cuts[c];
+    const double a = fabs(d[n + m - 1]);
+    dt[m - 1] -= a;                            // no index lies next to two cuts: a leaf has at least 10
+    dt[m] -= a;
+  }
+}
+
+// A leaf's eigenvalues and rows by implicit QL with Wilkinson's shift, one thread per leaf.
+__global__ void __launch_bounds__(32) dc_leaves(Dc a, const Node* __restrict__ leaves, int n_leaves,
+                                                const double* __restrict__ dt, const double* __restrict__ q) {
+  __shared__ double buf[5][kLeaf];
+  const Node nd = leaves[blockIdx.x];
+  const int lo = nd.lo, n = nd.hi - nd.lo;
+  double *d = buf[0], *e = buf[1], *z0 = buf[2], *z1 = buf[3], *zq = buf[4];
+  if (threadIdx.x != 0) return;
+  for (int i = 0; i < n; ++i) {
+    d[i] = dt[lo + i];
+    e[i] = i + 1 < n ? a.e[lo + i] : 0.0;
+    z0[i] = i == 0 ? 1.0 : 0.0;
+    z1[i] = i == n - 1 ? 1.0 : 0.0;
+    zq[i] = q[lo + i];
+  }
+  for (int l = 0; l < n; ++l) {
+    for (int it = 0; it < 60; ++it) {
+      int m = l;
+      while (m < n - 1 && fabs(e[m]) > kEps * (fabs(d[m]) + fabs(d[m + 1]))) ++m;
+      if (m == l) break;
+      double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
+      double r = sqrt(fma(g, g, 1.0));
+      g = d[m] - d[l] + e[l] / (g + (g >= 0.0 ? r : -r));
+      double s = 1.0, c = 1.0, p = 0.0;
+      int i = m - 1;
+      for (; i >= l; --i) {
+        const double f = s * e[i], b = c * e[i];
+        r = sqrt(fma(f, f, g * g));
+        e[i + 1] = r;
+        if (r == 0.0) { d[i + 1] -= p; e[m] = 0.0; break; }
+        s = f / r;
+        c = g / r;
+        g = d[i + 1] - p;
+        r = (d[i] - g) * s + 2.0 * c * b;
+        p = s * r;
+        d[i + 1] = g + p;
+        g = c * r - b;
+        double t = z0[i + 1];
+        z0[i + 1] = s * z0[i] + c * t; z0[i] = c * z0[i] - s * t;
+        t = z1[i + 1];
+        z1[i + 1] = s * z1[i] + c * t; z1[i] = c * z1[i] - s * t;
+        t = zq[i + 1];
+        zq[i + 1] = s * zq[i] + c * t; zq[i] = c * zq[i] - s * t;
+      }
+      if (r == 0.0 && i >= l) continue;
+      d[l] -= p;
+      e[l] = g;
+      e[m] = 0.0;
+    }
+  }
+  for (int i = 0; i < n; ++i) {                // selection sort, ascending
+    int k = i;
+    for (int j = i + 1; j < n; ++j)
+      if (d[j] < d[k]) k = j;
+    double t = d[i]; d[i] = d[k]; d[k] = t;
+    t = z0[i]; z0[i] = z0[k]; z0[k] = t;
+    t = z1[i]; z1[i] = z1[k]; z1[k] = t;
+    t = zq[i]; zq[i] = zq[k]; zq[k] = t;
+    a.lam[lo + i] = d[i];
+    a.r0[lo + i] = z0[i];
+    a.r1[lo + i] = z1[i];
+    a.rq[lo + i] = zq[i];
+  }
+}
+
+// Merge, first part (one block per node): the sorted values and z of both halves, and the deflation:
+// entries with a negligible z, and the first of two close values after a rotation that zeroes its z.
+// The rest (K of them) come first in D, ascending, then the deflated ones.  When no two neighbours are
+// close (tested in parallel) only the negligible entries are moved; else one thread walks the list.
+constexpr int kMergeThreads = 512;
+__global__ void __launch_bounds__(kMergeThreads) dc_deflate(Dc a, const Node* __restrict__ nodes) {
+  extern __shared__ double sm[];
+  const Node nd = nodes[blockIdx.x];
+  const int lo = nd.lo, n1 = nd.mid - nd.lo, n = nd.hi - nd.lo;
+  double* sD = sm;                                // sorted values
+  double* sZ = sm + n;                            // their z
+  int* src = (int*)(sm + 2 * n);                  // their sources
+  int* kind = src + n;                            // 0 kept, 1 deflated
+  __shared__ double s_red[kMergeThreads / 32][2];
+  __shared__ int s_any, s_scan[kMergeThreads / 32 + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double em = a.e[nd.mid - 1];
+  const double rho = 2.0 * fabs(em), sg = em < 0.0 ? -M_SQRT1_2 : M_SQRT1_2;
+  const double *la = a.lam + lo, *lb = la + n1;
+  double dmax = 0.0, zmax = 0.0;
+  for (int i = threadIdx.x; i < n; i += kMergeThreads) {
+    const bool left = i < n1;
+    const double v = la[i];
+    const double* o = left ? lb : la;
+    int p = 0, q = left ? n - n1 : n1;
+    while (p < q) {                               // ties: the left half first
+      const int mid = (p + q) >> 1;
+      if (left ? o[mid] < v : o[mid] <= v) p = mid + 1;
+      else q = mid;
+    }
+    const int pos = (left ? i : i - n1) + p;
+    const double z = left ? M_SQRT1_2 * a.r1[lo + i] : sg * a.r0[lo + i];
+    sD[pos] = v;
+    sZ[pos] = z;
+    src[pos] = i;
+    dmax = fmax(dmax, fabs(v));
+    zmax = fmax(zmax, fabs(z));
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+  }
+  if (lane == 0) { s_red[warp][0] = dmax; s_red[warp][1] = zmax; }
+  if (threadIdx.x == 0) s_any = 0;
+  __syncthreads();
+  for (int w = 0; w < kMergeThreads / 32; ++w) { dmax = fmax(dmax, s_red[w][0]); zmax = fmax(zmax, s_red[w][1]); }
+  const double tol = 8.0 * kEps * fmax(dmax, zmax);
+  // rows of the sources, in sorted order (before any rotation)
+  for (int p = threadIdx.x; p < n; p += kMergeThreads) {
+    const int i = src[p];
+    a.f0[lo + p] = i < n1 ? a.r0[lo + i] : 0.0;
+    a.f1[lo + p] = i < n1 ? 0.0 : a.r1[lo + i];
+    a.fq[lo + p] = a.rq[lo + i];
+    kind[p] = rho * fabs(sZ[p]) <= tol ? 1 : 0;
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < n; p += kMergeThreads) {
+    if (kind[p]) continue;
+    int m = p + 1;                                // the next entry that counts
+    while (m < n && kind[m]) ++m;
+    if (m < n && fabs((sD[m] - sD[p]) * sZ[m] * sZ[p]) <= tol * fma(sZ[m], sZ[m], sZ[p] * sZ[p])) s_any = 1;
+  }
+  __syncthreads();
+  if (s_any && threadIdx.x == 0) {
+    int pj = -1;
+    for (int p = 0; p < n; ++p) {
+      if (kind[p]) continue;
+      if (pj >= 0) {
+        double s = sZ[pj], c = sZ[p];
+        const double t2 = fma(c, c, s * s), t = sD[p] - sD[pj];
+        if (fabs(t * c * s) <= tol * t2) {
+          const double h = sqrt(t2);
+          c /= h;
+          s = -s / h;
+          sZ[p] = h;
+          sZ[pj] = 0.0;
+          double* rows[3] = {a.f0 + lo, a.f1 + lo, a.fq + lo};
+          for (int k = 0; k < 3; ++k) {
+            const double x = rows[k][pj], y = rows[k][p];
+            rows[k][pj] = c * x + s * y;
+            rows[k][p] = c * y - s * x;
+          }
+          const double dj = sD[pj], dp = sD[p];
+          sD[p] = dj * s * s + dp * c * c;
+          sD[pj] = dj * c * c + dp * s * s;
+          kind[pj] = 1;
+        }
+      }
+      pj = p;
+    }
+  }
+  __syncthreads();
+  // kept entries to the front, deflated behind them, both in order
+  int base = 0, K = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int p0 = 0; p0 < n; p0 += kMergeThreads) {
+      const int p = p0 + threadIdx.x;
+      const bool take = p < n && kind[p] == pass;
+      const unsigned bal = __ballot_sync(0xffffffffu, take);
+      if (lane == 0) s_scan[warp] = __popc(bal);
+      __syncthreads();
+      int before = 0, all = 0;
+      for (int w = 0; w < kMergeThreads / 32; ++w) {
+        before += w < warp ? s_scan[w] : 0;
+        all += s_scan[w];
+      }
+      if (take) {
+        const int to = base + before + __popc(bal & ((1u << lane) - 1u));
+        a.D[lo + to] = sD[p];
+        a.z[lo + to] = sZ[p];
+        src[p] = to;                              // where p goes
+      }
+      base += all;
+      __syncthreads();
+    }
+    if (pass == 0) K = base;
+  }
+  // the rows follow (through registers: source and target overlap)
+  for (double* f : {a.f0 + lo, a.f1 + lo, a.fq + lo}) {
+    for (int p = threadIdx.x; p < n; p += kMergeThreads) sZ[p] = f[p];
+    __syncthreads();
+    for (int p = threadIdx.x; p < n; p += kMergeThreads) f[src[p]] = sZ[p];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    a.K[blockIdx.x] = K;
+    a.rho[blockIdx.x] = rho;
+  }
+}
+
+__device__ __forceinline__ double recip(double x) {     // two Newton steps from the hardware's seed
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = fma(-x, y, 1.0);
+  y = fma(y, e, y);
+  e = fma(-x, y, 1.0);
+  return fma(y, e, y);
+}
+__device__ __forceinline__ double warp_sum(double x) {
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// Roots of 1 + rho sum z_i^2 / (d_i - x), a warp each: root j in (d_j, d_{j+1}), the last one up to
+// d_{K-1} + rho |z|^2.  The root is kept relative to its nearer pole, so the differences d_i - x that the
+// eigenvectors need are exact to rounding.  Steps: the two-pole rational interpolation that matches the
+// value and both halves' derivatives (Li's middle way), kept inside the bracket, else bisection.
+__global__ void __launch_bounds__(128) dc_secular(Dc a, const Node* __restrict__ nodes) {
+  const Node nd = nodes[blockIdx.y];
+  const int lo = nd.lo, K = a.K[blockIdx.y], lane = threadIdx.x & 31;
+  const double rho = a.rho[blockIdx.y];
+  const double *d = a.D + lo, *z = a.z + lo;
+  for (int j = blockIdx.x * 4 + (threadIdx.x >> 5); j < K; j += gridDim.x * 4) {
+    const bool last = j == K - 1;
+    double z2 = 0.0;
+    if (last) {
+      for (int i = lane; i < K; i += 32) z2 = fma(z[i], z[i], z2);
+      z2 = warp_sum(z2);
+    }
+    const double gap = last ? rho * z2 : d[j + 1] - d[j];
+    // which half of the interval: the function grows from -inf at d_j to +inf at d_{j+1}
+    int o = j;
+    double lo_t = 0.0, hi_t = last ? gap * (1.0 + 8.0 * kEps) : gap;
+    {
+      double f = 0.0;
+      for (int i = lane; i < K; i += 32) f = fma(z[i] * recip((d[i] - d[j]) - 0.5 * gap), z[i], f);
+      f = fma(rho, warp_sum(f), 1.0);
+      if (last) {
+        if (f < 0.0) lo_t = 0.5 * gap; else hi_t = 0.5 * gap;
+      } else if (f >= 0.0) {
+        hi_t = 0.5 * gap;
+      } else {
+        o = j + 1;
+        lo_t = -0.5 * gap;
+        hi_t = 0.0;
+      }
+    }
+    const double d_o = d[o];
+    const double p1 = d[j] - d_o, p2 = last ? 0.0 : d[j + 1] - d_o;   // the neighbouring poles
+    double t = 0.5 * (lo_t + hi_t);
+    for (int it = 0; it < 60; ++it) {
+      double ps = 0.0, dps = 0.0, ph = 0.0, dph = 0.0;
+      for (int i = lane; i < K; i += 32) {
+        const double r = recip((d[i] - d_o) - t), w = z[i] * r;
+        if (i <= j) { ps = fma(w, z[i], ps); dps = fma(w, w, dps); }
+        else { ph = fma(w, z[i], ph); dph = fma(w, w, dph); }
+      }
+      ps = rho * warp_sum(ps);
+      dps = rho * warp_sum(dps);
+      ph = rho * warp_sum(ph);
+      dph = rho * warp_sum(dph);
+      const double f = 1.0 + ps + ph;
+      if (f < 0.0) lo_t = t; else hi_t = t;
+      // converged: f is rounding (each term to a few units, plus the root's own last bits)
+      if (fabs(f) <= 8.0 * kEps * (1.0 + fabs(ps) + fabs(ph)) + kEps * fabs(t) * (dps + dph)) break;
+      if (!(hi_t - lo_t > 2.0 * kEps * fmax(fabs(lo_t), fabs(hi_t)))) break;
+      double tn;
+      const double x1 = p1 - t;
+      if (last) {
+        // one pole: f ~ c + s / (p1 - x)
+        const double s = dps * x1 * x1, c = f - dps * x1;
+        tn = c > 0.0 ? p1 + s / c : hi_t;
+      } else {
+        const double x2 = p2 - t;
+        const double c = f - x1 * dps - x2 * dph;
+        const double aa = (x1 + x2) * f - x1 * x2 * (dps + dph), bb = x1 * x2 * f;
+        const double disc = sqrt(fmax(0.0, aa * aa - 4.0 * bb * c));
+        const double eta = aa <= 0.0 ? (c != 0.0 ? (aa - disc) / (2.0 * c) : bb / aa) : 2.0 * bb / (aa + disc);
+        tn = t + eta;
+      }
+      if (!(tn > lo_t && tn < hi_t)) tn = 0.5 * (lo_t + hi_t);
+      if (tn == t) break;
+      t = tn;
+    }
+    if (lane == 0) {
+      a.tau[lo + j] = t;
+      a.org[lo + j] = o;
+    }
+  }
+}
+
+// z recomputed from the roots, a warp per entry: the z for which the roots are exact,
+// z_i^2 = prod_j (x_j - d_i) / prod_{j != i} (d_j - d_i), up to a common factor.
+__global__ void __launch_bounds__(128) dc_z(Dc a, const Node* __restrict__ nodes) {
+  const Node nd = nodes[blockIdx.y];
+  const int lo = nd.lo, K = a.K[blockIdx.y], lane = threadIdx.x & 31;
+  const double* d = a.D + lo;
+  for (int i = blockIdx.x * 4 + (threadIdx.x >> 5); i < K; i += gridDim.x * 4) {
+    const double di = d[i];
+    double p = 1.0;
+    for (int j = lane; j < K; j += 32) {
+      const double x = (d[a.org[lo + j]] - di) + a.tau[lo + j];       // x_j - d_i
+      // pair x_j with d_j (j > i: both right of d_i) or d_{j+1} (j < i: both left), x_{K-1} with none
+      if (j == K - 1) p *= i == K - 1 ? x : x * recip(d[j] - di);
+      else if (j >= i) p *= j == i ? x : x * recip(d[j] - di);
+      else p *= x * recip(d[j] - di);
+    }
+    for (int o = 16; o > 0; o >>= 1) p *= __shfl_xor_sync(0xffffffffu, p, o);
+    if (lane == 0) a.zh[lo + i] = copysign(sqrt(fabs(p)), a.z[lo + i]);
+  }
+}
+
+// The merged node's eigenvalues and rows, sorted, a warp per entry: a root's rows are the sums over
+// the kept sources of f_i z_i / (d_i - x), over its norm; a deflated entry's are its own.
+__device__ __forceinline__ double entry_value(const Dc& a, int lo, int K, int p) {
+  return p < K ? a.D[lo + a.org[lo + p]] + a.tau[lo + p] : a.D[lo + p];
+}
+__global__ void __launch_bounds__(128) dc_rows(Dc a, const Node* __restrict__ nodes) {
+  const Node nd = nodes[blockIdx.y];
+  const int lo = nd.lo, n = nd.hi - nd.lo, K = a.K[blockIdx.y], lane = threadIdx.x & 31;
+  const double* d = a.D + lo;
+  for (int p = blockIdx.x * 4 + (threadIdx.x >> 5); p < n; p += gridDim.x * 4) {
+    double s0, s1, sq;
+    const double v = entry_value(a, lo, K, p);
+    if (p < K) {
+      const double d_o = d[a.org[lo + p]], t = a.tau[lo + p];
+      double nn = 0.0;
+      s0 = s1 = sq = 0.0;
+      for (int i = lane; i < K; i += 32) {
+        const double u = a.zh[lo + i] * recip((d[i] - d_o) - t);
+        nn = fma(u, u, nn);
+        s0 = fma(u, a.f0[lo + i], s0);
+        s1 = fma(u, a.f1[lo + i], s1);
+        sq = fma(u, a.fq[lo + i], sq);
+      }
+      const double inv = rsqrt(warp_sum(nn));
+      s0 = inv * warp_sum(s0);
+      s1 = inv * warp_sum(s1);
+      sq = inv * warp_sum(sq);
+    } else {
+      s0 = a.f0[lo + p];
+      s1 = a.f1[lo + p];
+      sq = a.fq[lo + p];
+    }
+    // its place: the entries before it (the kept ones ascend; ties by index)
+    int before = 0;
+    if (p < K) {
+      before = lane == 0 ? p : 0;
+      for (int q = K + lane; q < n; q += 32) before += a.D[lo + q] < v;
+    } else {
+      for (int q = lane; q < n; q += 32) {
+        const double x = entry_value(a, lo, K, q);
+        before += x < v || (x == v && q < p);
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (lane == 0) {
+      a.lam[lo + before] = v;
+      a.r0[lo + before] = s0;
+      a.r1[lo + before] = s1;
+      a.rq[lo + before] = sq;
+    }
+  }
+}
+
+}  // namespace
+
+int64_t measure_work(int64_t n) {
+  const int64_t nodes = 2 * (n / (kLeaf / 2) + 2);
+  return (n / kWY + 2) * kWY * kWY + 16 * n + 64 + 4 * nodes + 64;
+}
+
+// x <- Q x or Q^T x.  factors: form the blocks' T factors first (they stay in the workspace).
+tgba_status apply_q(Basis& b, const TriData& t, bool transpose, double* x, double* work, bool factors, cudaStream_t st) {
+  if (t.n < 2) return TGBA_OK;
+  const int nb = (t.n - 1 + kWY - 1) / kWY;
+  if (factors) {
+    wy_factors<<<nb, 256, 0, st>>>(t.n, t.ld, t.v, work);
+    ++b.launches;
+  }
+  const size_t smem = (size_t)t.n * sizeof(double);
+  if (smem > 48 * 1024)
+    TGBA_CUDA(cudaFuncSetAttribute(wy_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  wy_apply<<<1, kApplyThreads, smem, st>>>(t.n, t.ld, transpose, t.v, work, x);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
+  return TGBA_OK;
+}
+
+// The workspace after the T factors.
+static double* dc_area(double* work, int64_t n) { return work + (n / kWY + 2) * kWY * kWY; }
+
+tgba_status lowest_vector(Basis& b, const TriData& t, const double* lambda, double* x, double* work, cudaStream_t st) {
+  double* a = dc_area(work, t.n);
+  twisted<<<1, 64, 0, st>>>(t.n, t.d, lambda, a, a + t.n, x);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
+  return TGBA_OK;
+}
+
+tgba_status spectral_rows(Basis& b, const TriData& t, const double* q, double* lambda, double* amp, double* work,
+                          cudaStream_t st) {
+  const int n = t.n;
+  // the tree: ranges halved until they fit a leaf
+  std::vector<std::vector<Node>> levels(1);
+  std::vector<Node> leaves;
+  std::vector<int> cuts;
+  {
+    std::vector<Node> cur{Node{0, 0, n}};
+    levels.clear();
+    while (!cur.empty()) {
+      std::vector<Node> next, merges;
+      for (Node x : cur) {
+        if (x.hi - x.lo <= kLeaf) { leaves.push_back(x); continue; }
+        x.mid = (x.lo + x.hi) / 2;
+        cuts.push_back(x.mid);
+        merges.push_back(x);
+        next.push_back(Node{x.lo, 0, x.mid});
+        next.push_back(Node{x.mid, 0, x.hi});
+      }
+      if (!merges.empty()) levels.push_back(merges);
+      cur.swap(next);
+    }
+  }
+  double* w = dc_area(work, n);
+  Dc a;
+  a.n = n;
+  a.e = t.d + n;
+  double* dt = w;      w += n;
+  a.lam = lambda;
+  a.r0 = w;            w += n;
+  a.r1 = w;            w += n;
+  a.rq = amp;
+  a.D = w;             w += n;
+  a.z = w;             w += n;
+  a.f0 = w;            w += n;
+  a.f1 = w;            w += n;
+  a.fq = w;            w += n;
+  a.tau = w;           w += n;
+  a.zh = w;            w += n;
+  a.rho = w;           w += leaves.size() + 1;
+  a.org = (int*)w;     w += (n + 1) / 2 + 1;
+  a.K = (int*)w;       w += (leaves.size() + 1) / 2 + 1;
+  // nodes (leaves, then the levels) and cuts
+  std::vector<Node> all(leaves);
+  for (const auto& l : levels) all.insert(all.end(), l.begin(), l.end());
+  Node* d_nodes = (Node*)w;
+  int* d_cuts = (int*)(d_nodes + all.size());
+  TGBA_CUDA(cudaMemcpyAsync(d_nodes, all.data(), all.size() * sizeof(Node), cudaMemcpyHostToDevice, st));
+  if (!cuts.empty())
+    TGBA_CUDA(cudaMemcpyAsync(d_cuts, cuts.data(), cuts.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  dc_tear<<<1, 1024, 0, st>>>(n, t.d, d_cuts, (int)cuts.size(), dt);
+  dc_leaves<<<(unsigned)leaves.size(), 32, 0, st>>>(a, d_nodes, (int)leaves.size(), dt, q);
+  TGBA_CUDA(cudaGetLastError());
+  b.launches += 2;
+  const size_t smem_max = (size_t)n * 24;
+  if (smem_max > 48 * 1024)
+    TGBA_CUDA(cudaFuncSetAttribute(dc_deflate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+  size_t off = all.size();
+  for (int l = (int)levels.size() - 1; l >= 0; --l) {
+    const std::vector<Node>& lv = levels[l];
+    off -= lv.size();
+    // the levels follow the leaves from the root down: this level's place
+    size_t at = leaves.size();
+    for (int m = 0; m < l; ++m) at += levels[m].size();
+    const Node* nd = d_nodes + at;
+    int size = 0;
+    for (const Node& x : lv) size = std::max(size, x.hi - x.lo);
+    const unsigned per = (unsigned)std::max<int>(1, std::min<int>((size + 3) / 4, 152 * 16 / (int)lv.size() + 1));
+    dc_deflate<<<(unsigned)lv.size(), kMergeThreads, (size_t)size * 24, st>>>(a, nd);
+    dc_secular<<<dim3(per, (unsigned)lv.size()), 128, 0, st>>>(a, nd);
+    dc_z<<<dim3(per, (unsigned)lv.size()), 128, 0, st>>>(a, nd);
+    dc_rows<<<dim3(per, (unsigned)lv.size()), 128, 0, st>>>(a, nd);
+    TGBA_CUDA(cudaGetLastError());
+    b.launches += 4;
+  }
+  return TGBA_OK;
+}
+
+}  // namespace tgba

@@ -243,6 +243,30 @@ struct WaitCheck {
 };
 tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double* evals, cudaStream_t st,
                                    const WaitCheck* check = nullptr);
+// one matrix of a batch: sector, kind (0 whole, 1 even, 2 odd block), field; keep the reflectors?
+// compute the eigenvalues (0: none, 1: all, 2: the lowest few)?
+struct TriBlock { int sector, kind; double hx; bool vectors; int evals; };
+struct TriData {
+  int n, ld;
+  int64_t ev;       // its eigenvalues in TriResult::evals
+  double* d;        // T: diagonal [n], off-diagonal [n - 1]
+  double* v;        // reflectors (column j: v_j, ld rows; then tau [n - 1] at ld ld), or null
+};
+struct TriResult {
+  std::vector<TriData> blocks;
+  double* evals = nullptr;
+  double* extra = nullptr;
+};
+int64_t tri_block_size(const Basis& b, int s, int kind);
+tgba_status make_ascending(Basis& b, double* v, int64_t n, cudaStream_t st);   // running maxima of a list from the bisection
+tgba_status tri_solve(Basis& b, const std::vector<TriBlock>& blocks, int64_t extra, const WaitCheck* check,
+                      cudaStream_t st, TriResult* res);
+// measure.cu: for T of a block with its reflectors, H~ = Q T Q^T
+int64_t measure_work(int64_t n);                      // doubles of workspace for the calls below
+tgba_status apply_q(Basis& b, const TriData& t, bool transpose, double* x, double* work, bool factors, cudaStream_t st);
+tgba_status lowest_vector(Basis& b, const TriData& t, const double* lambda, double* x, double* work, cudaStream_t st);
+tgba_status spectral_rows(Basis& b, const TriData& t, const double* q, double* lambda, double* amp, double* work,
+                          cudaStream_t st);
 
 // dsf.cu
 tgba_status dsf(Basis& b, int s, double h_x, double w_min, double w_max, int n_w, double eta, float* S,

@@ -75,6 +75,7 @@ struct TriSlot {
   int64_t de_off;   // diagonal d [n], off-diagonal e [n]
   int64_t out_off;  // first eigenvalue in the workspace's list (merge_evals brings them to the caller)
   int64_t pv_off;   // (v, w) pending when sytrd_small takes over [2 ld]
+  int64_t v_off;    // the reflectors v_j (column j, ld rows) and then tau [ld], kept if >= 0
   int32_t n, ld;
   int32_t j_end;    // steps of sytrd_groups; sytrd_small does the rest
   int32_t ck;       // row blocks per chunk
@@ -401,14 +402,17 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
         red[WARPS + 2] = tau;                          // read back after the pass
         red[WARPS + 3] = s;
         if (rank == 0) E[j] = beta;
+        if (rank == 0 && S.v_off >= 0) ws[S.v_off + (int64_t)ld * ld + j] = tau;
         if (!(isfinite(dj) && isfinite(beta))) bad = true;
       }
     }
     __syncthreads();
     const double s = red[WARPS + 3];
+    double* keep = rank == (j % C) && S.v_off >= 0 ? ws + S.v_off + (int64_t)j * ld : nullptr;
     for (int i = threadIdx.x; i < ld; i += (WARPS * 32)) {
-      const double x = vwn[i].x;
-      vwn[i].x = i == j + 1 ? 1.0 : (i > j + 1 && i < n ? x * s : 0.0);
+      const double x = vwn[i].x, v = i == j + 1 ? 1.0 : (i > j + 1 && i < n ? x * s : 0.0);
+      vwn[i].x = v;
+      if (keep) keep[i] = v;
     }
     __syncthreads();
     // one pass over the trailing lower triangle: update of step j - 1 and y = A_j v_j.  The
@@ -608,6 +612,7 @@ __global__ void __launch_bounds__(kSmallThreads) sytrd_small(const TriSlot* __re
         red[W + 2] = tau;
         red[W + 3] = s;
         E[j] = beta;
+        if (S.v_off >= 0) ws[S.v_off + (int64_t)S.ld * S.ld + j0 + j] = tau;
         if (!(isfinite(dj) && isfinite(beta))) bad = true;
       }
     }
@@ -617,6 +622,9 @@ __global__ void __launch_bounds__(kSmallThreads) sytrd_small(const TriSlot* __re
     if (half == 0) {
       vi = i == j + 1 ? 1.0 : (i > j + 1 && i < m ? x * s : 0.0);
       vwn[i].x = vi;
+      if (S.v_off >= 0 && i < m) ws[S.v_off + (int64_t)(j0 + j) * S.ld + j0 + i] = vi;
+      // zeros above, as far as a block of 16 reflectors that begins in sytrd_groups reads
+      if (S.v_off >= 0 && i < 16 && j0 > i) ws[S.v_off + (int64_t)(j0 + j) * S.ld + j0 - 1 - i] = 0.0;
     }
     __syncthreads();
     // y = A_j v_j with the update of step j - 1 applied on the way
@@ -1070,6 +1078,11 @@ __device__ void make_monotone(double* v, int n, double* part) {
   __syncthreads();
 }
 
+__global__ void __launch_bounds__(256) monotone_list(double* __restrict__ v, int n) {
+  __shared__ double part[256];
+  make_monotone(v, n, part);
+}
+
 __global__ void __launch_bounds__(256) merge_evals(const MergeJob* __restrict__ jobs, double* __restrict__ list,
                                                    double* __restrict__ evals) {
   __shared__ double part[256];
@@ -1116,44 +1129,15 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   // workload 11 whole sectors and 4 blocks of half the size instead of 24 sectors (table, elements
   // and both fields' eigenvalues 514 -> 274 ms); the k = 0 sector of L = 40 with 2697 states as two
   // blocks 345 -> 85 ms.
-  std::vector<TriSlot> slots;
-  std::vector<FillSlot> fills;
+  std::vector<TriBlock> blocks;
   std::vector<MergeJob> jobs;
-  int64_t total = 0, tk_total = 0, ev_total = 0;
-  int n_max = 0;
+  int64_t ev_total = 0;
   // (A withheld CTA is named by its (field, sector) matrix: then every sector is solved whole.)
   const bool symmetric = b.x_screen == nullptr && (check == nullptr || check->withhold_matrix < 0);
-  auto add = [&](int h, int s, int kind) {        // kind 0: the whole sector, 1: even, 2: odd block
-    const Sector& sec = b.sectors[s];
-    const SectorSym& y = b.sym[s];
-    FillSlot f{nullptr, nullptr, b.d_E_ns + sec.ns_off, b.d_E_r + sec.r_off, b.d_P + sec.x_off, -b.L * hx[h], 1.0,
-               sec.n_r, sec.n_ns};
-    int64_t n = sec.n_ns + sec.n_r;
-    if (kind > 0) {
-      const bool even = kind == 1;
-      f.ns = b.d_mirror + (even ? y.even_off[0] : y.odd_off[0]);
-      f.r = b.d_mirror + (even ? y.even_off[1] : y.odd_off[1]);
-      f.sgn = even ? 1.0 : -1.0;
-      f.kn = (int64_t)(even ? y.even[0] : y.odd[0]).size();
-      n = f.kn + (int64_t)(even ? y.even[1] : y.odd[1]).size();
-    }
-    if (n == 0) return (int64_t)0;
-    TriSlot t{};
-    t.n = (int32_t)n;
-    t.ld = (int32_t)round32(n);
-    t.out_off = ev_total;       ev_total += n;
-    t.a_off = total;            total += round32((int64_t)t.ld * t.ld);
-    t.rp_off = total;           total += round32((int64_t)(t.ld / kCols) * t.ld);
-    t.cp_off = total;           total += round32((int64_t)kCols * max_chunks(t.ld, 1));   // for any ck
-    t.tk_off = tk_total;        tk_total += t.ld;
-    t.p_off = total;            total += round32(t.ld + kMaxGroup);
-    t.de_off = total;           total += round32(2 * n);
-    t.pv_off = total;           total += round32(2 * t.ld);
-    t.j_end = (int32_t)std::max<int64_t>(0, n - kSmallN);
-    t.ck = kChunk;
-    slots.push_back(t);
-    fills.push_back(f);
-    n_max = std::max(n_max, (int)n);
+  auto add = [&](int h, int s, int kind) {
+    const int64_t n = tri_block_size(b, s, kind);
+    if (n > 0) blocks.push_back(TriBlock{s, kind, hx[h], false, 1});
+    ev_total += n;
     return n;
   };
   for (int h = 0; h < n_hx; ++h) {
@@ -1181,6 +1165,75 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
       jobs.push_back(j);
     }
   }
+  if (blocks.empty()) return TGBA_OK;
+  TriResult res;
+  tgba_status r = tri_solve(b, blocks, (int64_t)(jobs.size() * sizeof(MergeJob) / sizeof(double) + 8), check, st, &res);
+  if (r != TGBA_OK) return r;
+  MergeJob* d_jobs = (MergeJob*)res.extra;
+  TGBA_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(MergeJob), cudaMemcpyHostToDevice, st));
+  merge_evals<<<(unsigned)jobs.size(), 256, 0, st>>>(d_jobs, res.evals, evals);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
+  return TGBA_OK;
+}
+
+tgba_status make_ascending(Basis& b, double* v, int64_t n, cudaStream_t st) {
+  if (n == 0) return TGBA_OK;
+  monotone_list<<<1, 256, 0, st>>>(v, (int)n);
+  TGBA_CUDA(cudaGetLastError());
+  ++b.launches;
+  return TGBA_OK;
+}
+
+// The whole sector (kind 0), or its even (1) or odd (2) block under the reflection.
+int64_t tri_block_size(const Basis& b, int s, int kind) {
+  const Sector& sec = b.sectors[s];
+  const SectorSym& y = b.sym[s];
+  if (kind == 0) return sec.n_ns + sec.n_r;
+  return kind == 1 ? (int64_t)(y.even[0].size() + y.even[1].size()) : (int64_t)(y.odd[0].size() + y.odd[1].size());
+}
+
+// H~ of every block, tridiagonalised in one launch (with the reflectors kept where asked), and, where
+// asked, its eigenvalues.  The workspace is the handle's scratch; `extra` doubles of it are the caller's.
+tgba_status tri_solve(Basis& b, const std::vector<TriBlock>& blocks, int64_t extra, const WaitCheck* check,
+                      cudaStream_t st, TriResult* res) {
+  std::vector<TriSlot> slots;
+  std::vector<FillSlot> fills;
+  int64_t total = 0, tk_total = 0, ev_total = 0;
+  int n_max = 0;
+  for (const TriBlock& k : blocks) {
+    const Sector& sec = b.sectors[k.sector];
+    const SectorSym& y = b.sym[k.sector];
+    FillSlot f{nullptr, nullptr, b.d_E_ns + sec.ns_off, b.d_E_r + sec.r_off, b.d_P + sec.x_off, -b.L * k.hx, 1.0,
+               sec.n_r, sec.n_ns};
+    const int64_t n = tri_block_size(b, k.sector, k.kind);
+    if (n == 0) return fail(TGBA_EINVAL, "empty block");
+    if (k.kind > 0) {
+      const bool even = k.kind == 1;
+      f.ns = b.d_mirror + (even ? y.even_off[0] : y.odd_off[0]);
+      f.r = b.d_mirror + (even ? y.even_off[1] : y.odd_off[1]);
+      f.sgn = even ? 1.0 : -1.0;
+      f.kn = (int64_t)(even ? y.even[0] : y.odd[0]).size();
+    }
+    TriSlot t{};
+    t.n = (int32_t)n;
+    t.ld = (int32_t)round32(n);
+    t.out_off = ev_total;       ev_total += n;
+    t.a_off = total;            total += round32((int64_t)t.ld * t.ld);
+    t.rp_off = total;           total += round32((int64_t)(t.ld / kCols) * t.ld);
+    t.cp_off = total;           total += round32((int64_t)kCols * max_chunks(t.ld, 1));   // for any ck
+    t.tk_off = tk_total;        tk_total += t.ld;
+    t.p_off = total;            total += round32(t.ld + kMaxGroup);
+    t.de_off = total;           total += round32(2 * n);
+    t.pv_off = total;           total += round32(2 * t.ld);
+    t.v_off = -1;
+    if (k.vectors) { t.v_off = total; total += round32((int64_t)t.ld * t.ld + t.ld); }
+    t.j_end = (int32_t)std::max<int64_t>(0, n - kSmallN);
+    t.ck = kChunk;
+    slots.push_back(t);
+    fills.push_back(f);
+    n_max = std::max(n_max, (int)n);
+  }
   if (slots.empty()) return TGBA_OK;
   const int B = (int)slots.size();
   int ld_max = 0;
@@ -1197,7 +1250,7 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   // parts of two matrices, and one's barrier waits and serial phases are filled by the other's
   // arithmetic), else one of 12 warps.  With no more matrices than CTAs, every CTA joins one
   // matrix's group: each matrix starts with one CTA and the remaining CTAs go, one at a time,
-  // to the matrix with the most work (n^3) per CTA, at most 16 per matrix.  With more matrices
+  // to the matrix with the most work (n^3) per CTA, at most 96 per matrix.  With more matrices
   // than CTAs, CTA b takes matrices b, b + CTAs, ... alone.
   const size_t smem = (size_t)(4 * ld_max + kRed) * sizeof(double) +
                       (size_t)(kMaxGroups + 1) * sizeof(int);
@@ -1271,7 +1324,7 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   }
   const int64_t ev_off = total;
   total += round32(ev_total);
-  const int64_t slot_doubles = round32(((int64_t)B * (sizeof(TriSlot) + sizeof(FillSlot)) + jobs.size() * sizeof(MergeJob) + 7) / 8);
+  const int64_t slot_doubles = round32(((int64_t)B * (sizeof(TriSlot) + sizeof(FillSlot)) + 7) / 8);
   const int64_t map_doubles = round32(((int64_t)2 * grid * sizeof(CtaWork) + 7) / 8);   // by block, by SM
   // bisection items: item_len consecutive eigenvalue indices of one matrix, 64 (a block's
   // threads) unless that gives fewer items than resident blocks, then 32.  (Items sized to fill
@@ -1291,23 +1344,23 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   if (count_items(item_len) < (int64_t)bis_per_sm * sms) item_len = kSturmThreads / 2;
   std::vector<int2> items;
   for (int q = 0; q < B; ++q)
-    for (int k0 = 0; k0 < slots[q].n; k0 += item_len) items.push_back(make_int2(q, k0));
+    for (int k0 = 0; k0 < (blocks[q].evals == 1 ? slots[q].n : blocks[q].evals == 2 ? std::min(slots[q].n, 1) : 0); k0 += item_len)
+      items.push_back(make_int2(q, k0));
   const int n_items = (int)items.size();
   const int64_t item_doubles = round32(n_items);
   // counters: barriers, column reads, tickets, SM registration, the bisection queue
   const int64_t n_cnt = 2 * (int64_t)B + tk_total + kMaxSmId + 2 + 1;
   const int64_t cnt_doubles = round32((n_cnt + 1) / 2);
   double* ws;
-  tgba_status r = scratch(b, total + slot_doubles + map_doubles + cnt_doubles + item_doubles, &ws);
+  const int64_t extra_off = total + slot_doubles + map_doubles + cnt_doubles + item_doubles;
+  tgba_status r = scratch(b, extra_off + extra, &ws);
   if (r != TGBA_OK) return r;
   TriSlot* d_slots = (TriSlot*)(ws + total);
   CtaWork* d_map = (CtaWork*)(ws + total + slot_doubles);
   unsigned* d_cnt = (unsigned*)(ws + total + slot_doubles + map_doubles);
   FillSlot* d_fill = (FillSlot*)(d_slots + B);
-  MergeJob* d_jobs = (MergeJob*)(d_fill + B);
   TGBA_CUDA(cudaMemcpyAsync(d_slots, slots.data(), B * sizeof(TriSlot), cudaMemcpyHostToDevice, st));
   TGBA_CUDA(cudaMemcpyAsync(d_fill, fills.data(), B * sizeof(FillSlot), cudaMemcpyHostToDevice, st));
-  TGBA_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(MergeJob), cudaMemcpyHostToDevice, st));
   TGBA_CUDA(cudaMemcpyAsync(d_map, map.data(), grid * sizeof(CtaWork), cudaMemcpyHostToDevice, st));
   CtaWork* d_sm_map = nullptr;
   if (!sm_map.empty()) {
@@ -1363,14 +1416,19 @@ tgba_status eig_all_sectors_native(Basis& b, const double* hx, int n_hx, double*
   TGBA_CUDA(cudaGetLastError());
   b.launches += grid > 0 ? 2 : 1;
   TGBA_CUDA(cudaEventRecord(b.eig_ev[1], st));
-  const int bis_grid = std::min(n_items, bis_per_sm * sms);
-  sturm_bisect<<<bis_grid, kSturmThreads, smem2, st>>>(d_slots, d_items, n_items, item_len, d_queue, ws,
-                                                       ws + ev_off, b.d_status);
-  TGBA_CUDA(cudaGetLastError());
+  if (n_items > 0) {
+    const int bis_grid = std::min(n_items, bis_per_sm * sms);
+    sturm_bisect<<<bis_grid, kSturmThreads, smem2, st>>>(d_slots, d_items, n_items, item_len, d_queue, ws, ws + ev_off,
+                                                         b.d_status);
+    TGBA_CUDA(cudaGetLastError());
+    ++b.launches;
+  }
   TGBA_CUDA(cudaEventRecord(b.eig_ev[2], st));
-  merge_evals<<<(unsigned)jobs.size(), 256, 0, st>>>(d_jobs, ws + ev_off, evals);
-  TGBA_CUDA(cudaGetLastError());
-  b.launches += 2;
+  res->evals = ws + ev_off;
+  res->extra = ws + extra_off;
+  res->blocks.clear();
+  for (const TriSlot& t : slots)
+    res->blocks.push_back(TriData{t.n, t.ld, t.out_off, ws + t.de_off, t.v_off >= 0 ? ws + t.v_off : nullptr});
   b.eig_ev_recorded = true;
   double flops = 0;
   for (const TriSlot& t : slots)
