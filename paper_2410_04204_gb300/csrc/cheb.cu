@@ -232,6 +232,132 @@ __global__ void __launch_bounds__(256) cheb_step(int64_t n, int64_t kn_max, cons
   column_max(v, row < kn_max, mb + 2 * col);
 }
 
+// All K steps of a few small variants in one cooperative launch, in FP64.  Row q of the union belongs to
+// CTA q mod gridDim; a CTA keeps its rows of the X block (both orientations: its NS rows over the R
+// states and its R rows over the NS states) in shared memory for the whole run.  A step reads the
+// current vectors of all variants from L2 into shared memory, takes the rows' products (a warp per
+// row, each variant up to its own extent), writes the next vectors and ends with a barrier of the grid
+// (an arrival counter, bounded waits).  Bound: the FP64 pipe (2 kn kr FMAs per variant and step on 2
+// lanes per SM and clock) and the barrier.  The tensor-core step costs 30 to 40 us however small the
+// block is.
+constexpr int kPersistThreads = 512;
+constexpr int kPersistCols = 8;
+struct PersistArgs {
+  int kn, kr, nv, K;
+  int64_t S;                       // vectors' stride between steps
+  const double* Q;                 // col-major kr x kn
+  const double* E;
+  const ColPrm* prm;
+  double* V;                       // [K + 1][S]: v_0 given
+  unsigned* count;
+  unsigned* status;
+};
+
+__device__ __forceinline__ unsigned acquire_u32(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__global__ void __launch_bounds__(kPersistThreads, 1) cheb_persist(PersistArgs g) {
+  extern __shared__ double sm[];
+  __shared__ int s_ok;
+  const int n = g.kn + g.kr, G = gridDim.x, c0 = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int W = kPersistThreads / 32;
+  const int rn = g.kn > c0 ? (g.kn - c0 + G - 1) / G : 0;           // own NS rows: c0, c0 + G, ...
+  const int b0 = ((c0 - g.kn) % G + G) % G;                          // own R rows: b0, b0 + G, ... (row kn + b)
+  const int rr = g.kr > b0 ? (g.kr - b0 + G - 1) / G : 0;
+  double* An = sm;                                                   // [rn][kr]
+  double* Ar = An + (size_t)rn * g.kr;                               // [rr][kn]
+  double* x = Ar + (size_t)rr * g.kn;                                // [nv][n]
+  double* prev = x + (size_t)g.nv * n;                               // [rn + rr][nv]
+  for (int i = 0; i < rn; ++i)
+    for (int b = threadIdx.x; b < g.kr; b += kPersistThreads) An[(size_t)i * g.kr + b] = g.Q[(size_t)(c0 + i * G) * g.kr + b];
+  for (int q = threadIdx.x; q < rr * g.kn; q += kPersistThreads) {
+    const int i = q % rr, a = q / rr;
+    Ar[(size_t)i * g.kn + a] = g.Q[(size_t)a * g.kr + b0 + i * G];
+  }
+  for (int k = 0; k < g.K; ++k) {
+    const double* vk = g.V + (size_t)k * g.S;
+    for (int q = threadIdx.x; q < g.nv * n; q += kPersistThreads) x[q] = __ldcg(vk + q);
+    __syncthreads();
+    for (int i = warp; i < rn + rr; i += W) {
+      const bool ns = i < rn;
+      const double* row = ns ? An + (size_t)i * g.kr : Ar + (size_t)(i - rn) * g.kn;
+      const int at = ns ? c0 + i * G : g.kn + b0 + (i - rn) * G;      // row of the union
+      const double e = g.E[at];
+      for (int c = 0; c < g.nv; ++c) {
+        const ColPrm p = g.prm[c];
+        double v = 0.0;
+        if (ns ? at < p.kn : at - g.kn < p.kr) {                     // warp-uniform
+          const int ext = (int)(ns ? p.kr : p.kn);
+          const double* xc = x + (size_t)c * n + (ns ? g.kn : 0);
+          double y0 = 0.0, y1 = 0.0, y2 = 0.0, y3 = 0.0;
+          int j = lane;
+          for (; j + 96 < ext; j += 128) {
+            y0 = fma(row[j], xc[j], y0);
+            y1 = fma(row[j + 32], xc[j + 32], y1);
+            y2 = fma(row[j + 64], xc[j + 64], y2);
+            y3 = fma(row[j + 96], xc[j + 96], y3);
+          }
+          for (; j < ext; j += 32) y0 = fma(row[j], xc[j], y0);
+          double y = (y0 + y1) + (y2 + y3);
+          for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+          const double xi = x[(size_t)c * n + at];
+          const double h = fma(p.g, y, (e - p.ec) * xi);
+          v = (k == 0 ? 1.0 : 2.0) * p.invr * h - (k == 0 ? 0.0 : prev[i * g.nv + c]);
+          __syncwarp();
+          if (lane == 0) prev[i * g.nv + c] = xi;
+        }
+        if (lane == 0) __stcg(g.V + (size_t)(k + 1) * g.S + (size_t)c * n + at, v);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.count) : "memory");
+      const unsigned target = (unsigned)G * (unsigned)(k + 1);
+      int ok = 0;
+      for (unsigned it = 0; it < (1u << 24); ++it) {
+        if (acquire_u32(g.count) >= target) { ok = 1; break; }
+        if (it > 32) __nanosleep(40);
+      }
+      if (!ok) atomicOr(g.status, kStTimeout);
+      s_ok = ok;
+    }
+    __syncthreads();
+    if (!s_ok) return;
+  }
+}
+
+// B(t) times its phase e^{-i E_c t} (B as [Re | -Im] column-major n x n_t blocks), for variants whose
+// E_c differ
+__global__ void rotate_phase(int64_t n, int n_t, double dt, double ec, double* __restrict__ re, double* __restrict__ im) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n * n_t; q += (int64_t)gridDim.x * blockDim.x) {
+    double s, c;
+    sincos(ec * dt * (double)(q / n), &s, &c);
+    const double a = re[q], b = -im[q];
+    re[q] = a * c + b * s;
+    im[q] = -(b * c - a * s);
+  }
+}
+
+// max over t of || B'(t) - B(t) || (both on the union), one warp per time
+__global__ void eps_union(int64_t n, int n_t, const double* __restrict__ ra, const double* __restrict__ ia,
+                          const double* __restrict__ rb, const double* __restrict__ ib, unsigned long long* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n_t;
+       t += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    double acc = 0.0;
+    for (int64_t i = lane; i < n; i += 32) {
+      const double x = rb[i + t * n] - ra[i + t * n], y = ib[i + t * n] - ia[i + t * n];
+      acc = fma(x, x, fma(y, y, acc));
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) atomicMax(out, (unsigned long long)__double_as_longlong(sqrt(acc)));
+  }
+}
+
 // per column: ||v_0||^2 and ||v_K||^2 (one block per column)
 __global__ void cheb_norms(int64_t n, const double* __restrict__ V0, const double* __restrict__ VK,
                            double* __restrict__ out) {
@@ -413,7 +539,7 @@ std::vector<EmuTile> product_tiles(int64_t rows, int64_t cols, const std::vector
 
 tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t kr_max, const double* E,
                               const double* c, const std::vector<ChebVariant>& vars, double t_max, int n_t,
-                              double* mx, cudaStream_t st) {
+                              double* mx, double* eps, cudaStream_t st) {
   if (vars.empty()) return TGBA_OK;
   for (const ChebVariant& v : vars)
     if (!(std::fabs(v.hx) * b.L >= 1e-3))
@@ -421,7 +547,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
                                "use method 1 for h_x = 0");
   const int64_t n_un = kn_max + kr_max;
   const double cabs = std::hypot(b.c0_host[0], b.c0_host[1]);
-  const int TR = emu_tile_rows_a(), TC = kEmuTileCols;
+  const int TR = emu_tile_rows_a();
   // stage times (host clock around synchronised sections)
   using clk = std::chrono::steady_clock;
   TGBA_CUDA(cudaStreamSynchronize(st));
@@ -642,12 +768,44 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     ++b.launches;
     TGBA_CUDA(cudaStreamSynchronize(st));
     b.quench_prep_ms = ms_since(t_start);     // slicing of Q, Lanczos, set-up (last attempt)
-    // the K steps of all variants, three launches each (the host enqueues them ahead of the device;
+    // a few small variants: one launch (see cheb_persist), when the block fits the SMs' shared memory
+    // and the FP64 pipe takes less than a tensor-core step (about 30 us)
+    double fma_step = 0.0;
+    for (const ChebVariant& v : vars) fma_step += 2.0 * (double)v.kn * (double)v.kr;
+    const int G = b.emu_sms;
+    const size_t smem_p = sizeof(double) * ((size_t)((kn_max + G - 1) / G) * kr_max + (size_t)((kr_max + G - 1) / G) * kn_max +
+                                            (size_t)ncol * n_un + (size_t)((kn_max + G - 1) / G + (kr_max + G - 1) / G) * ncol);
+    const bool persist = coupled && ncol <= kPersistCols && smem_p <= 220 * 1024 && fma_step <= 30e-6 * 2.0 * G * 1.9e9;
+    // otherwise the K steps of all variants, three launches each (the host enqueues them ahead of the device;
     // capturing and instantiating a graph of them for one use took longer)
     for (int e = 0; e < 2; ++e)
       if (b.q_ev[e] == nullptr) TGBA_CUDA(cudaEventCreate(&b.q_ev[e]));
     TGBA_CUDA(cudaEventRecord(b.q_ev[0], st));
-    for (int k = 0; k < K; ++k) {
+    if (persist) {
+      TGBA_CUDA(cudaFuncSetAttribute(cheb_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_p));
+      PersistArgs pa;
+      pa.kn = (int)kn_max; pa.kr = (int)kr_max; pa.nv = ncol; pa.K = K; pa.S = S;
+      pa.Q = Q; pa.E = E; pa.prm = prm; pa.V = V;
+      pa.count = (unsigned*)(nrm + 2 * (size_t)ncolp);
+      pa.status = b.d_status;
+      TGBA_CUDA(cudaMemsetAsync(pa.count, 0, sizeof(unsigned), st));
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)G);
+      cfg.blockDim = dim3(kPersistThreads);
+      cfg.dynamicSmemBytes = smem_p;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeCooperative;       // all CTAs resident at once: the grid barrier relies on it
+      attr[0].val.cooperative = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      // the padding columns of every step are zero (the moments never read them, the norms do)
+      if (ncolp > ncol)
+        TGBA_CUDA(cudaMemset2DAsync(V + (size_t)ncol * n_un, (size_t)S * 8, 0, (size_t)(ncolp - ncol) * n_un * 8, K1, st));
+      TGBA_CUDA(cudaLaunchKernelEx(&cfg, cheb_persist, pa));
+      ++b.launches;
+    }
+    for (int k = 0; k < K && !persist; ++k) {
       double* vk = V + (size_t)k * S;
       if (coupled &&
           (r = offdiag(vk, mb + (size_t)k * 2 * ncolp, Y, ncolp, Bs, eb, dtl, (int)tl.size(), n_blocks, 6, st)) != TGBA_OK)
@@ -689,14 +847,25 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       const double xmax = R[v] * t_max;
       Kv[v] = std::min(K, (int)std::ceil(xmax + 10.0 * std::cbrt(xmax) + 30.0));
     }
+    // Tiles of 64 columns: each digit diagonal then has accumulators of its own, and the products'
+    // error is 6e-15 of sum |a||b| instead of 2e-13.
+    constexpr int TM = 64;
     const int64_t nt = std::max(1, dt_n), KH = (K1 + 1) / 2;
-    const size_t sa = std::max(emu_operand_elems((int)KH, (int)chi_max, TR), emu_operand_elems((int)KH, (int)KH, TR));
-    // every product of this stage takes B images of 128 rows (k or times), whatever its size
-    const size_t sb = std::max(emu_operand_elems((int)KH, (int)chi_max, TC), emu_operand_elems((int)nt, (int)KH, TC));
-    const size_t n_tiles_max = (size_t)((KH + TR - 1) / TR) * (size_t)std::max<int64_t>((KH + TC - 1) / TC, (nt + TC - 1) / TC);
+    const int64_t a_rows = eps ? std::max<int64_t>(KH, n_un) : KH;
+    const size_t sa = std::max({emu_operand_elems((int)KH, (int)chi_max, TR), emu_operand_elems((int)a_rows, (int)KH, TR)});
+    const size_t sb = std::max(emu_operand_elems((int)KH, (int)chi_max, TM), emu_operand_elems((int)nt, (int)KH, TM));
+    const size_t n_tiles_max = (size_t)((a_rows + TR - 1) / TR) * (size_t)std::max<int64_t>((KH + TM - 1) / TM, (nt + TM - 1) / TM);
+    DevBuf bbuf(st);                                      // B(t) of two variants, for eps
+    const size_t bt = (size_t)n_un * nt;
+    if (eps) {
+      TGBA_CUDA(cudaMallocAsync(&bbuf.p, 4 * bt * sizeof(double), st));
+      TGBA_CUDA(cudaMemsetAsync(eps, 0, (vars.size() - 1) * sizeof(double), st));
+    }
+    bool one_field = true;
+    for (const ChebVariant& v : vars) one_field = one_field && v.hx == vars[0].hx;
     DevBuf mbuf(st);
     const size_t mdoubles = (size_t)KH * KH + (size_t)K1 * nt + 2 * (size_t)KH * nt + chi_max + 8;
-    TGBA_CUDA(cudaMallocAsync(&mbuf.p, mdoubles * 8 + (sa + sb) * 2 + 2 * ((size_t)KH + nt) * 4 +
+    TGBA_CUDA(cudaMallocAsync(&mbuf.p, mdoubles * 8 + (sa + sb) * 2 + 2 * ((size_t)a_rows + nt) * 4 +
                                            n_tiles_max * sizeof(EmuTile) + 1024, st));
     double* Gam = (double*)mbuf.p;
     double* Ab = Gam + (size_t)KH * KH;                   // a_k(t): [K_v + 1][t]
@@ -707,16 +876,16 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     __nv_bfloat16* Va = (__nv_bfloat16*)(((uintptr_t)(dtg + n_tiles_max) + 255) & ~(uintptr_t)255);
     __nv_bfloat16* Wb = Va + sa;
     int* eva = (int*)(Wb + sb);
-    int* ewb = eva + KH;
-    // output tiles of a product (lower: only the tiles on or below the diagonal, for a
-    // symmetric result; TR == TC)
-    auto grid_tiles = [&](int64_t rows, int64_t cols, int64_t kdim, int64_t& n_chunks, bool lower = false) {
+    int* ewb = eva + a_rows;
+    // output tiles of a product (lower: only the tiles that reach the diagonal or lie below it, for a
+    // symmetric result)
+    auto grid_tiles = [&](int64_t rows, int64_t cols, int64_t kdim, int64_t& n_blocks_out, bool lower = false) {
       std::vector<EmuTile> t;
       for (int64_t rb = 0; rb * TR < rows; ++rb)
-        for (int64_t cb = 0; cb * TC < cols && (!lower || cb <= rb); ++cb)
-          t.push_back(EmuTile{(int32_t)rb, (int32_t)cb, (int32_t)std::min<int64_t>(TC, r16(cols - cb * TC)),
+        for (int64_t cb = 0; cb * TM < cols && (!lower || cb * TM < (rb + 1) * TR); ++cb)
+          t.push_back(EmuTile{(int32_t)rb, (int32_t)cb, (int32_t)std::min<int64_t>(TM, r16(cols - cb * TM)),
                               (int32_t)((kdim + emu_k_block() - 1) / emu_k_block())});
-      n_chunks = emu_number_tiles(t);
+      n_blocks_out = emu_number_tiles(t);
       return t;
     };
     struct Events {                                       // stage times of the moments and of the sums
@@ -730,9 +899,11 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       }
       ~Events() { for (cudaEvent_t x : e) cudaEventDestroy(x); }
     } ev;
-    for (int j = 0; j < (int)ord.size(); ++j) {
-      const ChebVariant& vv = vars[ord[j]];
-      const int v = ord[j];
+    std::vector<int> col_of(vars.size());
+    for (int j = 0; j < (int)ord.size(); ++j) col_of[ord[j]] = j;
+    for (int v = 0; v < (int)vars.size(); ++v) {
+      const ChebVariant& vv = vars[v];
+      const int j = col_of[v];
       const int k1 = Kv[v] + 1;
       const int64_t kn = vv.kn, kr = vv.kr, chi = kn + kr, jump = kn_max - kn;
       const double* vre = V + (size_t)j * n_un;             // column j of step 0; step k at + k S
@@ -757,8 +928,8 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
         // rows of V (K = the kept rows in their own order: kn NS rows, then kr R rows)
         const double* vp = vre + (size_t)p * S;
         if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, nullptr, 0.0, kp, (int)chi, TR, Va, eva, st)) != TGBA_OK) return r;
-        if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, Ek, ec[v], kp, (int)chi, TC, Wb, ewb, st)) != TGBA_OK) return r;
-        if ((r = emu_gemm(b, Va, eva, kp, (int)chi, Wb, ewb, kp, (int)chi, TC, dtg, (int)tlo.size(), cl, Gam, kp, st)) != TGBA_OK)
+        if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, Ek, ec[v], kp, (int)chi, TM, Wb, ewb, st)) != TGBA_OK) return r;
+        if ((r = emu_gemm(b, Va, eva, kp, (int)chi, Wb, ewb, kp, (int)chi, TM, dtg, (int)tlo.size(), cl, Gam, kp, st)) != TGBA_OK)
           return r;
         symmetrise<<<blocks_for((int64_t)kp * kp), 256, 0, st>>>(kp, Gam);
         ++b.launches;
@@ -768,16 +939,40 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
         if (ct < 0) return fail(TGBA_EINVAL, "quench time-sum tiles");
         TGBA_CUDA(cudaMemcpyAsync(dtg, tt.data(), tt.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
         if ((r = emu_slice(b, Gam, kp, 1, kp, 0, nullptr, 0.0, kp, kp, TR, Va, eva, st)) != TGBA_OK) return r;
-        if ((r = emu_slice(b, Ab + (size_t)p * nt, 1, 2 * nt, kp, 0, nullptr, 0.0, (int)nt, kp, TC, Wb, ewb, st)) != TGBA_OK)
+        if ((r = emu_slice(b, Ab + (size_t)p * nt, 1, 2 * nt, kp, 0, nullptr, 0.0, (int)nt, kp, TM, Wb, ewb, st)) != TGBA_OK)
           return r;
-        if ((r = emu_gemm(b, Va, eva, kp, kp, Wb, ewb, (int)nt, kp, TC, dtg, (int)tt.size(), ct, GA[p], kp, st)) != TGBA_OK)
+        if ((r = emu_gemm(b, Va, eva, kp, kp, Wb, ewb, (int)nt, kp, TM, dtg, (int)tt.size(), ct, GA[p], kp, st)) != TGBA_OK)
           return r;
+        if (eps) {
+          // B(t) on the union: its real part from the even k, minus its imaginary part from the odd ones
+          int64_t cb = 0;
+          const std::vector<EmuTile> tb = grid_tiles(n_un, nt, kp, cb);
+          if (cb < 0) return fail(TGBA_EINVAL, "quench state tiles");
+          TGBA_CUDA(cudaMemcpyAsync(dtg, tb.data(), tb.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
+          if ((r = emu_slice(b, vp, 1, 2 * S, kp, 0, nullptr, 0.0, (int)n_un, kp, TR, Va, eva, st)) != TGBA_OK) return r;
+          if ((r = emu_gemm(b, Va, eva, (int)n_un, kp, Wb, ewb, (int)nt, kp, TM, dtg, (int)tb.size(), cb,
+                            (double*)bbuf.p + (2 * (v & 1) + p) * bt, n_un, st)) != TGBA_OK)
+            return r;
+        }
         TGBA_CUDA(ev.mark(st));
       }
       cheb_mx<<<(int)((nt * 32 + 255) / 256), 256, 0, st>>>(k1, (int)nt, Ab, GA[0], GA[1], d01, R[v], scale,
                                                               mx + (int64_t)vv.out * n_t);
       TGBA_CUDA(cudaGetLastError());
       ++b.launches;
+      if (eps) {
+        double *cur = (double*)bbuf.p + 2 * (v & 1) * bt, *old = (double*)bbuf.p + 2 * ((v + 1) & 1) * bt;
+        if (!one_field) {
+          rotate_phase<<<blocks_for((int64_t)bt), 256, 0, st>>>(n_un, (int)nt, dt, ec[v], cur, cur + bt);
+          ++b.launches;
+        }
+        if (v > 0) {
+          eps_union<<<(int)std::min<int64_t>((nt * 32 + 255) / 256, 152 * 8), 256, 0, st>>>(
+              n_un, (int)nt, old, old + bt, cur, cur + bt, (unsigned long long*)(eps + v - 1));
+          ++b.launches;
+        }
+        TGBA_CUDA(cudaGetLastError());
+      }
     }
     TGBA_CUDA(cudaStreamSynchronize(st));
     // per variant: start, then (moments, sums) for the even and the odd k (K >= 1: both exist)

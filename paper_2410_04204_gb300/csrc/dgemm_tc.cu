@@ -442,7 +442,7 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
           const int e_i = op.ea[i];
 #pragma unroll
           for (int cc = 0; cc < kCols; ++cc) {
-            const int j = tl.cb * kTNr + c_lo + cc;
+            const int j = tl.cb * g.tb + c_lo + cc;
             if (c_lo + cc < tl.n_eff && j < op.N)
               op.C[(int64_t)i + (int64_t)j * op.ldc] = scaled_sum(hi[cc], lo[cc], e_i + op.eb[j] - 16);
           }
@@ -486,7 +486,7 @@ __global__ void __maxnreg__(168) dgemm_tc_kernel(GemmArgs g) {   // 320 threads 
             }
 #pragma unroll
             for (int u = 0; u < 16; ++u) {
-              const int j = tl.cb * kTNr + c_lo + c16 + u;
+              const int j = tl.cb * g.tb + c_lo + c16 + u;
               if (j < op.N) op.C[(int64_t)i + (int64_t)j * op.ldc] = scaled_sum(h16[u], l16[u], e_i + op.eb[j] - 16);
             }
           }
@@ -730,9 +730,10 @@ int64_t emu_number_tiles(std::vector<EmuTile>& tiles) {
   return c;
 }
 
-// rows of a B tile image for `cols` columns: the smallest of 16, 32, 64, 128 that holds them, so that
-// narrow products (the propagation of a few variants) load, and keep in a stage, only the columns
-// they have; beyond 128 columns there are several tiles of 128.
+// rows of a B tile image (and columns of an output tile) for `cols` columns: the smallest of 16, 32, 64, 128
+// that holds them, so that narrow products (the propagation of a few variants) load, and keep in a
+// stage, only the columns they have; beyond 128 columns there are several tiles of 128.  A caller that
+// wants the smaller error of the separate accumulators takes tiles of 64 for any number of columns.
 int emu_tile_rows_b(int cols) { return cols <= 16 ? 16 : cols <= 32 ? 32 : cols <= 64 ? 64 : kTNr; }
 
 EmuSet emu_set(const __nv_bfloat16* A, const int* ea, int M, int Ka, const __nv_bfloat16* B, const int* eb, int N, int Kb,

@@ -359,8 +359,35 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
                                "with method 0)");
     n_max = std::max(n_max, n);
   }
+  // The automatic method propagates (method 2) where that costs less than the eigen-decompositions:
+  // the expansion takes K = R t_max + ... steps of all variants together (R: half the spectrum's
+  // width, here from the kept energies), a step about 8 us and the FP64 pipe's time for the X block
+  // (cheb_persist) or about 45 us on the tensor cores; an eigen-decomposition was measured at 4 ms
+  // for n = 101, 45 at 1000, 110 at 2000, and its time sums take 6 n^2 n_t flops on the FP64 pipe.
+  // It reads <sigma^x> off the energy, with an error of about K eps R / (L |h_x|): only from
+  // L |h_x| >= 1/2 on, where that stays below the phase error E t eps of the eigen path.
+  bool auto_cheb = method == 0 && j_max == 0;
+  if (auto_cheb) {
+    double e_lo = 1e300, e_hi = -1e300, t_eig = 0.0, fma = 0.0;
+    int64_t un_n = 0, un_r = 0;
+    for (int v = 0; v < nv; ++v) {
+      const double a = (double)sel_ns[v].size(), c = (double)sel_r[v].size(), n = a + c;
+      auto_cheb = auto_cheb && std::fabs(hx[v]) * L >= 0.5 && a > 0 && c > 0;
+      for (int32_t q : sel_ns[v]) { e_lo = std::min(e_lo, energy(q)); e_hi = std::max(e_hi, energy(q)); }
+      for (int32_t q : sel_r[v]) { e_lo = std::min(e_lo, energy(sec.n_ns + q)); e_hi = std::max(e_hi, energy(sec.n_ns + q)); }
+      t_eig += 3e-3 + 35e-6 * n + 8e-9 * n * n + 6.0 * n * n * n_t / 1.1e12;
+      fma += 2.0 * a * c;
+      un_n = std::max<int64_t>(un_n, (int64_t)a);
+      un_r = std::max<int64_t>(un_r, (int64_t)c);
+    }
+    const bool small = nv <= 8 && 16.0 * un_n * un_r + 8.0 * nv * 160 * (un_n + un_r) < 150.0 * 200e3 && fma < 30e-6 * 5.8e11;
+    const double K = 0.65 * (e_hi - e_lo) * t_max + 60.0;
+    const double t_cheb = 6e-3 + K * (small ? 8e-6 + fma / 5e11 : 45e-6 + fma / 2e13) +
+                          (double)nv * (1e-3 + K * K * (double)n_t / 1e14);
+    auto_cheb = auto_cheb && t_cheb < t_eig;
+  }
   double* Bbuf[2] = {nullptr, nullptr};
-  if (eps_out) {
+  if (eps_out && !auto_cheb) {
     TGBA_CUDA(cudaMemsetAsync(eps_out, 0, std::max(0, nv - 1) * sizeof(double), st));
     TGBA_CUDA(cudaMallocAsync(&Bbuf[0], 2 * sizeof(double) * (size_t)n_max * 2 * n_t, st));
     Bbuf[1] = Bbuf[0] + (size_t)n_max * 2 * n_t;
@@ -376,7 +403,7 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
     const std::vector<int32_t>& ir = sel_r[v];
     const int64_t kn = (int64_t)ins.size(), kr = (int64_t)ir.size(), n = kn + kr;
     if (chi_out) chi_out[v] = n;
-    const bool cheb = method == 2 || (method == 0 && n > kEigenMaxStates);
+    const bool cheb = method == 2 || auto_cheb || (method == 0 && n > kEigenMaxStates);
     if (cheb) {                                     // propagated together after this loop
       cheb_vars.push_back(v);
       continue;
@@ -620,7 +647,7 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
       norms[v] = x.norm2;
       cv.push_back(x);
     }
-    tgba_status r = quench_cheb_batch(b, Q, kn, kr, E, c, cv, t_max, n_t, mx, st);
+    tgba_status r = quench_cheb_batch(b, Q, kn, kr, E, c, cv, t_max, n_t, mx, auto_cheb ? eps_out : nullptr, st);
     if (r != TGBA_OK) return r;
     if (norm_out)
       for (int v : cheb_vars) TGBA_CUDA(cudaMemcpyAsync(norm_out + v, &norms[v], sizeof(double), cudaMemcpyHostToDevice, st));
