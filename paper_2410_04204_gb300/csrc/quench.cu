@@ -155,14 +155,16 @@ __global__ void eps_kernel(int n_t, int64_t knp, int64_t krp, int64_t kn, int64_
 }
 
 // Z~ = G^H Z G for one parity block of sigma^x_1 sigma^x_{j+1} (Z row-major complex [k][k] over
-// the kept states idx): the real-gauge phase of a state depends only on M, and for two states of
+// the kept states idx, its pairs a <= c in rows of falling length: Z is Hermitian): the real-gauge phase of a state
+// depends only on M, and for two states of
 // one parity it is i^{sgn (M_a - M_b)/2} (sgn = +1 NS, -1 R).  Output: real and imaginary parts.
 __global__ void zgauge_kernel(int64_t k, const int32_t* __restrict__ idx, const uint8_t* __restrict__ M, int64_t off,
                               int sgn, const double* __restrict__ Zc, double* __restrict__ Zr, double* __restrict__ Zi) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < k * k; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t a = e / k, c = e - a * k;
     const int p = (((sgn * ((int)M[off + idx[a]] - (int)M[off + idx[c]])) / 2) % 4 + 4) % 4;
-    const double re = Zc[2 * e], im = Zc[2 * e + 1];
+    const int64_t lo = a < c ? a : c, hi = a < c ? c : a, at = lo * k - lo * (lo - 1) / 2 + (hi - lo);
+    const double re = Zc[2 * at], im = a <= c ? Zc[2 * at + 1] : -Zc[2 * at + 1];
     double xr = re, xi = im;
     if (p == 1) { xr = -im; xi = re; }
     else if (p == 2) { xr = -re; xi = -im; }
@@ -471,9 +473,11 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
           const std::vector<int32_t>& lst = par ? ir : ins;
           const int64_t k = (int64_t)lst.size();
           if (k == 0) continue;
-          std::vector<int32_t> hp(2 * (size_t)k * k);
+          const int64_t np = k * (k + 1) / 2;
+          std::vector<int32_t> hp;
+          hp.reserve(2 * (size_t)np);
           for (int64_t x = 0; x < k; ++x)
-            for (int64_t y = 0; y < k; ++y) { hp[2 * (x * k + y)] = lst[x]; hp[2 * (x * k + y) + 1] = lst[y]; }
+            for (int64_t y = x; y < k; ++y) { hp.push_back(lst[x]); hp.push_back(lst[y]); }
           TGBA_CUDA(cudaMemcpyAsync(zp, hp.data(), hp.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
           int32_t* didx = (int32_t*)(par ? idx + kn : idx);
           // the parity's contraction table of the string up to j_max (reduced form)
@@ -487,7 +491,7 @@ tgba_status quench(Basis& b, int s, double h0, const double* hx, const double* t
           double* c0z = ztab + 2 * nE * nE;
           if ((r = z_table(b, par, j_max, ztab, c0z, st)) != TGBA_OK) return r;
           for (int j = 1; j <= j_max; ++j) {
-            if ((r = z_reduced_elements(b, s, par, j, j_max, ztab, c0z, zp, k * k, Zc, st)) != TGBA_OK) return r;
+            if ((r = z_reduced_elements(b, s, par, j, j_max, ztab, c0z, zp, np, Zc, st)) != TGBA_OK) return r;
             double* zr = (par ? Zr_r : Zr_ns) + (size_t)(j - 1) * k * k;
             double* zi = (par ? Zi_r : Zi_ns) + (size_t)(j - 1) * k * k;
             zgauge_kernel<<<blocks_for(k * k), 256, 0, st>>>(k, didx, par ? b.d_M_r : b.d_M_ns, par ? sec.r_off : sec.ns_off,

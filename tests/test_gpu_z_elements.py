@@ -69,6 +69,26 @@ def test_j0_is_the_identity_and_z_is_hermitian(L, mq, cut):
         tgba.tgba_basis_free(b)
 
 
+@pytest.mark.parametrize("mq,j", [(4, 0), (4, 21), (4, 22), (4, 23), (1, 25), (1, 26), (0, 26), (0, 1)])
+def test_warp_and_block_pfaffians_at_their_border(mq, j):
+    """Operator counts 2 max_qp + 2j up to 52 take a warp per element, larger ones a block: the sizes next to
+    the border, the empty Pfaffian and the vacuum alone, against the oracle within 1e-9 (its bound everywhere)."""
+    b = tgba.tgba_build_basis(60, 1.0, [0], mq, 3.0)
+    try:
+        g = GpuSector(b, 0, mq)
+        for parity, n in ((0, g.n_ns), (1, g.n_r)):
+            if n == 0:
+                continue
+            pairs = [(0, 0), (n - 1, n - 1), (0, n - 1), (n - 1, 0), (n // 2, 0)]
+            z = _z(b, parity, j, pairs)
+            zo = (np.array([float(a == c) for a, c in pairs]) if j == 0 else
+                  oel.z_elements(60, 1.0, parity, j, [(_modes(g, parity, a), _modes(g, parity, c)) for a, c in pairs]))
+            ok, worst = x_close(z, zo, rel=1e-9)
+            assert ok, (parity, j, worst)
+    finally:
+        tgba.tgba_basis_free(b)
+
+
 def test_rejects_bad_arguments():
     b = tgba.tgba_build_basis(12, 1.0, [0], 4)
     try:
