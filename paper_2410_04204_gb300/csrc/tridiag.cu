@@ -4,7 +4,7 @@
 // Two kernels per batch of (field, sector) matrices:
 //
 // 1. sytrd_groups: Householder reduction to tridiagonal form, T = Q^T H Q.  One cooperative
-//    launch with two CTAs of 6 warps per SM (one of 12 if two do not fit, or for one or two
+//    launch with two CTAs of 6 warps per SM (one of 12 if two do not fit, or for up to six
 //    matrices); the CTAs are shared out among the matrices in proportion to their work (n^3), so a
 //    group of C CTAs (1 to 96) owns one matrix and runs its reflections up to the last 128 rows
 //    (sytrd_small finishes those in one CTA's shared memory), and each SM's two CTAs come from
@@ -18,9 +18,9 @@
 //    read and written once per step with four FMAs.  The trailing lower triangle is cut into
 //    blocks of 32 rows x 16 columns, and each column group's blocks into chunks of up to
 //    kChunk consecutive blocks, with the group's last kTail blocks as a separate tail chunk
-//    handed out after all the others.  Warps draw chunks from a per-step ticket counter of the
-//    group, so warps and CTAs that run faster (a less busy co-resident CTA, a less crowded
-//    SM sub-partition) take more of them.  In a block a lane owns one row: its row sum needs
+//    handed out after all the others.  With two CTAs on an SM warps draw chunks from a per-step ticket
+//    counter of the group, so warps and CTAs that run faster (a less busy co-resident CTA, a less
+//    crowded SM sub-partition) take more of them; with one, chunks are dealt out in turn.  In a block a lane owns one row: its row sum needs
 //    no communication, and its 16 column partial sums stay in registers over the chunk, then
 //    one transpose-reduce (16 adds per lane) sums them over the warp.  Two block buffers in
 //    registers keep the next block's loads in flight during the current block's arithmetic.
@@ -63,7 +63,6 @@ constexpr int kTail = 2;                        // last blocks of a column group
 constexpr int kSmallN = 128;                    // trailing matrix that one CTA finishes in shared memory
 constexpr int kSmallThreads = 2 * kSmallN;
 constexpr int kMaxSmId = 1024;                  // SM ids registered by cta_role
-constexpr int kMaxGroups = kMaxNativeLd / kCols;
 constexpr int kSturmThreads = 64;                // bisection block: one item of 64 eigenvalues
 
 struct TriSlot {
@@ -267,46 +266,62 @@ __device__ __forceinline__ double transpose_reduce16(double (&cs)[kCols], int la
   return cs[0] + __shfl_xor_sync(0xffffffffu, cs[0], 1);
 }
 
-// Chunk c of the step: row blocks [rb_b, rb_e) of column group g.  Two block buffers in
-// registers: the loads of the next block are in flight while the current one is computed.
-// The chunk's 16 column sums go to CP[16 c ..].
+// Chunk c of the step: row blocks [rb_b, rb_e) of column group g, the first already on its way to cur[].
+// Two block buffers in registers: the loads of the next block (after the last one, of the warp's next
+// chunk at `after`, if that is known) are in flight while the current one is computed.  The chunk's 16
+// column sums go to CP[16 c ..].
 __device__ __forceinline__ void sytrd_chunk(double* __restrict__ A, int ld, int LB, int g, int rb_b, int rb_e,
                                             int lane, int c, const double2* __restrict__ vwp,
                                             const double2* __restrict__ vwn, double* __restrict__ RP,
-                                            double* __restrict__ CP) {
+                                            double* __restrict__ CP, double (&cur)[kCols],
+                                            const double* __restrict__ after) {
   const int k0 = kCols * g;
   double* gp = A + blk_off(g, 0, LB) + lane;       // + 512 rb: the lane's row of block rb
   double* rp = RP + g;                             // row i's sum at rp[i G]
   const int G = ld / kCols;
-  double cs[kCols], cur[kCols], nxt[kCols];
+  double cs[kCols], nxt[kCols];
 #pragma unroll
   for (int kk = 0; kk < kCols; ++kk) cs[kk] = 0.0;
+  const double* last = after ? after : gp + 512 * (rb_e - 1);
+  auto next = [&](int rb) { return rb + 1 < rb_e ? gp + 512 * (rb + 1) : last; };
   int rb = rb_b;
-  load_block(cur, gp + 512 * rb);
   if (rb == (g >> 1)) {                            // the diagonal block comes first
-    load_block(nxt, gp + 512 * min(rb + 1, rb_e - 1));
+    load_block(nxt, next(rb));
     sytrd_block<true>(cur, gp + 512 * rb, 32 * rb + lane, k0, vwp, vwn, cs, rp, G);
     ++rb;
 #pragma unroll
     for (int kk = 0; kk < kCols; ++kk) cur[kk] = nxt[kk];
   }
   for (; rb + 1 < rb_e; rb += 2) {
-    load_block(nxt, gp + 512 * (rb + 1));
+    load_block(nxt, next(rb));
     sytrd_block<false>(cur, gp + 512 * rb, 32 * rb + lane, k0, vwp, vwn, cs, rp, G);
-    load_block(cur, gp + 512 * min(rb + 2, rb_e - 1));
+    load_block(cur, next(rb + 1));
     sytrd_block<false>(nxt, gp + 512 * (rb + 1), 32 * (rb + 1) + lane, k0, vwp, vwn, cs, rp, G);
   }
-  if (rb < rb_e) sytrd_block<false>(cur, gp + 512 * rb, 32 * rb + lane, k0, vwp, vwn, cs, rp, G);
+  if (rb < rb_e) {
+    if (after) load_block(nxt, after);
+    sytrd_block<false>(cur, gp + 512 * rb, 32 * rb + lane, k0, vwp, vwn, cs, rp, G);
+#pragma unroll
+    for (int kk = 0; kk < kCols; ++kk) cur[kk] = nxt[kk];
+  }
   const double colsum = transpose_reduce16(cs, lane);
   if ((lane & 1) == 0) __stcg(CP + (int64_t)c * kCols + (lane >> 1), colsum);
 }
 
-// All n - 1 reflections of one matrix, as CTA `rank` of its group of C.  Returns false if a
-// group barrier gave up.
+// The reflections of one matrix down to its last kSmallN rows, as CTA `rank` of its group of C.  Returns
+// false if a group barrier gave up.  A step is short (half its time was latency at n = 1472 on 84 CTAs),
+// so what a warp waits for goes out early: the column and p as soon as they are final, the first block of the warp's
+// first chunk before the column is formed; w of the last step and column j are formed in one loop; and the
+// square root and quotient of the reflector, taken by warp 0, run under the pass, which starts with the
+// columns that do not need them.
 template <int WARPS>
 __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsigned* cnt, unsigned* ccnt,
                                           unsigned* tk, double* __restrict__ ws, unsigned* __restrict__ status,
                                           int* flag, unsigned limit) {
+  // One CTA on an SM: all warps run alike, and chunks dealt out in turn balance the SMs to one chunk, where
+  // tickets drawn ahead leave up to a chunk per warp (27.2 against 29.7 ms for the two blocks of the L = 40,
+  // k = 0 sector).  Two CTAs: tickets (247 against 259 ms for the 30 matrices of the L = 24 step).
+  constexpr bool kTickets = WARPS < 12;
   extern __shared__ double sm[];
   unsigned arrivals = 0, col_arrivals = 0;
   const int n = S.n, ld = S.ld, LB = ld >> 5, G = ld / kCols, ck = S.ck;
@@ -320,12 +335,33 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
   double2* vwp = (double2*)sm;                   // (v_{j-1}, w_{j-1}) per index
   double2* vwn = (double2*)(sm + 2 * ld);         // (v_j, w_j)
   double* red = sm + 4 * ld;
+  volatile int* ready = (volatile int*)(red + WARPS + 4);   // j + 1 once v_j is complete
   int* cf = (int*)(red + kRed);                   // [NG + 1] first chunk of each group
+  int* cfn = cf + G + 1;                          // the next step's
   __syncthreads();                                // the previous matrix is done with sm
   for (int i = threadIdx.x; i < 4 * ld; i += (WARPS * 32)) sm[i] = 0.0;
-  __syncthreads();
+  if (threadIdx.x == 0) *ready = 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool bad = false;
+  // the chunk table of step j: a scan by one warp over groups g0 .. G - 1
+  auto chunk_table = [&](int* t_, int j) {
+    const int g0 = (j + 1) / kCols, NG = G - g0;
+    const int per = (NG + 31) >> 5, t0 = min(NG, lane * per), t1 = min(NG, t0 + per);
+    int own = 0;
+    for (int t = t0; t < t1; ++t) own += group_chunks(g0 + t, LB, ck);
+    int incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    int run = incl - own;
+    for (int t = t0; t < t1; ++t) {
+      t_[t] = run;
+      run += group_chunks(g0 + t, LB, ck);
+    }
+    if (lane == 31) t_[NG] = incl;
+  };
   // the stored column of the next step, in registers: it is final once the pass is (first barrier),
   // so its loads run under the reduction and the second barrier (rows beyond kPre T: loaded in place)
   constexpr int T = WARPS * 32, kPre = 8;
@@ -333,129 +369,174 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
   auto prefetch_column = [&](int j) {
 #pragma unroll
     for (int u = 0; u < kPre; ++u) {
-      const int i = j + (int)threadIdx.x + u * T;
-      pre[u] = i < n ? __ldcg(A + elem_off(i, j, LB)) : 0.0;
+      const int i = (int)threadIdx.x + u * T;
+      pre[u] = i >= j && i < n ? __ldcg(A + elem_off(i, j, LB)) : 0.0;
     }
   };
-  if (S.j_end > 0) prefetch_column(0);
+  // w = p - K v with K = tau p.v / 2 of the last step, the partial dots of the CTAs added in the same order
+  // by every warp
+  auto half_dot = [&]() {
+    double pv = 0.0;
+    for (int r = lane; r < C; r += 32) pv += __ldcg(dots + r);
+    for (int o = 16; o > 0; o >>= 1) pv += __shfl_xor_sync(0xffffffffu, pv, o);
+    return 0.5 * red[WARPS + 2] * pv;
+  };
+  if (S.j_end > 0) {
+    if (warp == WARPS - 1) chunk_table(cf, 0);
+    prefetch_column(0);
+  }
+  __syncthreads();
   for (int j = 0; j < S.j_end; ++j) {
-    // column j of A_j: the stored column (already updated through step j - 2) minus the
-    // rank-2 update of step j - 1; rows j + 2 .. n - 1 go into the norm
-    const double2 vwj = vwp[j];
+    const int g0 = (j + 1) / kCols, NG = G - g0, NCH1 = cf[NG], NCH = NCH1 + NG, h0 = NCH1 - cf[1];
+    // p of the last step, then the first block of the warp's first chunk
+    double p8[kPre], pj = 0.0;
+#pragma unroll
+    for (int u = 0; u < kPre; ++u) {
+      const int i = (int)threadIdx.x + u * T;
+      p8[u] = (j > 0 && i >= j && i < n) ? __ldcg(P + i) : 0.0;
+    }
+    if (j > 0) pj = __ldcg(P + j);
+    // Position x of the step's order: the head chunks of the groups after g0, those of g0 (which wait
+    // for the complete reflector and, because they rewrite column j, for the other CTAs), the tails, g0's
+    // last.  lo: the group - g0, c: the chunk's number.
+    struct Chunk { int lo, c, rb, re; };
+    auto chunk_at = [&](int x) {
+      Chunk k;
+      if (x < NCH1) {
+        k.c = x < h0 ? cf[1] + x : x - h0;
+        int lo = 0, hi = NG;                        // cf[lo] <= c < cf[lo + 1]
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (cf[mid] <= k.c) lo = mid;
+          else hi = mid;
+        }
+        k.lo = lo;
+        const int gl = g0 + lo;
+        k.rb = (gl >> 1) + (k.c - cf[lo]) * ck;
+        k.re = min(k.rb + ck, (gl >> 1) + group_head(gl, LB, ck));
+      } else {
+        k.lo = x - NCH1 + 1 < NG ? x - NCH1 + 1 : 0;
+        k.c = NCH1 + k.lo;
+        const int gl = g0 + k.lo;
+        k.rb = (gl >> 1) + group_head(gl, LB, ck);
+        k.re = LB;
+      }
+      return k;
+    };
+    auto block_ptr = [&](const Chunk& k) { return A + blk_off(g0 + k.lo, k.rb, LB) + lane; };
+    // the warps' first chunks are dealt out over the CTAs (an SM's FP64 pipe is what a short step's
+    // chunks share), the tickets start after those
+    int x = warp * C + rank;
+    Chunk ch{0, 0, 0, 0};
+    double cur[kCols];
+    if (x < NCH) {
+      ch = chunk_at(x);
+      load_block(cur, block_ptr(ch));
+    }
+    // w_{j-1}, and column j of A_j: the stored column (already updated through step j - 2) minus the
+    // rank-2 update of step j - 1; rows j + 2 .. n - 1 go into the norm.  The reflector keeps the column's
+    // own scale: v_j = (0 .. 0, alpha - beta, rows j + 2 ..).
+    const double K = j > 0 ? half_dot() : 0.0;
+    const double vj = vwp[j].x, wj = fma(-K, vj, pj);
     double sig = 0.0;
-    auto column_row = [&](int i, double a) {
-      const double2 vwi = vwp[i];
-      a = fma(-vwi.x, vwj.y, a);
-      a = fma(-vwi.y, vwj.x, a);
-      if (i == j) red[WARPS] = a;
-      else if (i == j + 1) red[WARPS + 1] = a;
-      else sig = fma(a, a, sig);
-      vwn[i].x = a;
+    double* keep = rank == (j % C) && S.v_off >= 0 ? ws + S.v_off + (int64_t)j * ld : nullptr;
+    auto column_row = [&](int i, double p, double a) {
+      double v = 0.0, w = 0.0;
+      if (i >= j && i < n) {
+        const double vi = vwp[i].x;
+        w = fma(-K, vi, p);
+        a = fma(-vi, wj, a);
+        a = fma(-w, vj, a);
+        if (i == j) red[WARPS] = a;
+        else if (i == j + 1) red[WARPS + 1] = a;
+        else {
+          sig = fma(a, a, sig);
+          v = a;
+        }
+      }
+      vwp[i].y = w;
+      vwn[i].x = v;
+      if (keep && i != j + 1) keep[i] = v;
     };
 #pragma unroll
     for (int u = 0; u < kPre; ++u) {
-      const int i = j + (int)threadIdx.x + u * T;
-      if (i < n) column_row(i, pre[u]);
+      const int i = (int)threadIdx.x + u * T;
+      if (i < ld) column_row(i, p8[u], pre[u]);
     }
-    for (int i = j + (int)threadIdx.x + kPre * T; i < n; i += T) column_row(i, __ldcg(A + elem_off(i, j, LB)));
-    // the step's chunk table (a scan by warp 0 over groups g0 .. G - 1), published by
-    // block_sum's barrier
-    const int g0 = (j + 1) / kCols, NG = G - g0;
-    if (warp == 0) {
-      const int per = (NG + 31) >> 5, t0 = min(NG, lane * per), t1 = min(NG, t0 + per);
-      int own = 0;
-      for (int t = t0; t < t1; ++t) own += group_chunks(g0 + t, LB, ck);
-      int incl = own;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      int run = incl - own;
-      for (int t = t0; t < t1; ++t) {
-        cf[t] = run;
-        run += group_chunks(g0 + t, LB, ck);
-      }
-      if (lane == 31) cf[NG] = incl;
+    for (int i = (int)threadIdx.x + kPre * T; i < ld; i += T) {
+      const bool in = i >= j && i < n;
+      column_row(i, in && j > 0 ? __ldcg(P + i) : 0.0, in ? __ldcg(A + elem_off(i, j, LB)) : 0.0);
     }
-    sig = block_sum<WARPS>(sig, red);
-    // this CTA has read column j (block_sum's barrier): the pass below rewrites it, so the
-    // warps that store column j wait until every CTA of the group has arrived here
-    if (C > 1 && threadIdx.x == 0) arrive_release(ccnt);
+    for (int o = 16; o > 0; o >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, o);
+    if (lane == 0) red[warp] = sig;
+    __syncthreads();
+    // this CTA has read column j: the pass below rewrites it, so the warps that store column j wait until
+    // every CTA of the group has arrived here
+    if (C > 1 && threadIdx.x == 32) arrive_release(ccnt);
     col_arrivals += C;
-    const double dj = red[WARPS];
-    if (rank == 0 && threadIdx.x == 0) D[j] = dj;
-    if (j + 1 >= n) break;                            // uniform: the last diagonal entry
-    const double alpha = red[WARPS + 1];
-    // Householder reflector H = I - tau v v^T with v_{j+1} = 1 mapping column j to beta e_{j+1}.  One
-    // warp takes the square root and the two quotients: by every warp they cost 3.5 to 6 thousand cycles
-    // a step on the FP64 pipe (an eighth of a step of the L = 40 blocks).
+    // Householder reflector H = I - tau v v^T mapping column j to beta e_{j+1}: v_{j+1} = alpha - beta,
+    // tau = 2 / v.v = 1 / (|beta| (|beta| + |alpha|)).  Rows whose squares vanish beside any spectrum (a norm below
+    // 1e-140) count as zero, so tau stays finite.
     if (warp == 0) {
-      double beta = alpha, s = 0.0, tau = 0.0;
-      if (sig != 0.0) {
-        const double nrm = sqrt(fma(alpha, alpha, sig));
+      double sg = lane < WARPS ? red[lane] : 0.0;
+#pragma unroll
+      for (int o = WARPS > 8 ? 8 : 4; o > 0; o >>= 1) sg += __shfl_xor_sync(0xffffffffu, sg, o);
+      sg = __shfl_sync(0xffffffffu, sg, 0);
+      const double dj = red[WARPS], alpha = red[WARPS + 1];
+      double beta = alpha, v1 = 1.0, tau = 0.0;
+      if (!(sg < 1e-280)) {
+        const double nrm = sqrt(fma(alpha, alpha, sg));
         beta = alpha >= 0.0 ? -nrm : nrm;
-        tau = (beta - alpha) / beta;
-        s = 1.0 / (alpha - beta);
+        v1 = alpha - beta;
+        tau = 1.0 / (nrm * fabs(v1));
       }
       if (lane == 0) {
+        vwn[j + 1].x = v1;
         red[WARPS + 2] = tau;                          // read back after the pass
-        red[WARPS + 3] = s;
-        if (rank == 0) E[j] = beta;
-        if (rank == 0 && S.v_off >= 0) ws[S.v_off + (int64_t)ld * ld + j] = tau;
+        if (keep) keep[j + 1] = v1;
+        __threadfence_block();
+        *ready = j + 1;
+        if (rank == 0) {
+          D[j] = dj;
+          E[j] = beta;
+          if (S.v_off >= 0) ws[S.v_off + (int64_t)ld * ld + j] = tau;
+        }
         if (!(isfinite(dj) && isfinite(beta))) bad = true;
       }
+      __syncwarp();
     }
-    __syncthreads();
-    const double s = red[WARPS + 3];
-    double* keep = rank == (j % C) && S.v_off >= 0 ? ws + S.v_off + (int64_t)j * ld : nullptr;
-    for (int i = threadIdx.x; i < ld; i += (WARPS * 32)) {
-      const double x = vwn[i].x, v = i == j + 1 ? 1.0 : (i > j + 1 && i < n ? x * s : 0.0);
-      vwn[i].x = v;
-      if (keep) keep[i] = v;
-    }
-    __syncthreads();
-    // one pass over the trailing lower triangle: update of step j - 1 and y = A_j v_j.  The
-    // chunks go out one at a time from the step's ticket counter (the next ticket is drawn
-    // while a chunk is computed), so warps and CTAs that run faster take more of them.
-    {
-      const int NCH1 = cf[NG], NCH = NCH1 + NG;
-      bool waited = !(C > 1 && (j + 1) % kCols != 0);   // column j lies in group g0
-      // the warps' first chunks are dealt out over the CTAs (an SM's FP64 pipe is what a short step's
-      // chunks share), the tickets start after those
-      unsigned c = (unsigned)(warp * C + rank);
-      while ((int)c < NCH) {
-        unsigned cn = 0;
-        if (lane == 0) cn = atomicAdd(tk + j, 1u) + (unsigned)(C * WARPS);
-        int lo = 0, rb, re;
-        if ((int)c < NCH1) {                          // a head chunk: cf[lo] <= c < cf[lo + 1]
-          int hi = NG;
-          while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (cf[mid] <= (int)c) lo = mid;
-            else hi = mid;
-          }
-          const int gl = g0 + lo;
-          rb = (gl >> 1) + ((int)c - cf[lo]) * ck;
-          re = min(rb + ck, (gl >> 1) + group_head(gl, LB, ck));
-        } else {                                      // a tail chunk
-          lo = (int)c - NCH1;
-          const int gl = g0 + lo;
-          rb = (gl >> 1) + group_head(gl, LB, ck);
-          re = LB;
-        }
-        const int g = g0 + lo;
-        if (lo == 0 && !waited) {
-          warp_wait(ccnt, col_arrivals, status, limit);
-          waited = true;
-        }
-        sytrd_chunk(A, ld, LB, g, rb, re, lane, (int)c, vwp, vwn, RP, CP);
-        c = __shfl_sync(0xffffffffu, cn, 0);
+    // one pass over the trailing lower triangle: update of step j - 1 and y = A_j v_j
+    bool waited = false;
+    while (x < NCH) {
+      unsigned xn = (unsigned)(x + C * WARPS);
+      if (kTickets && lane == 0) xn = atomicAdd(tk + j, 1u) + (unsigned)(C * WARPS);
+      Chunk chn = ch;
+      const double* after = nullptr;
+      if (!kTickets && (int)xn < NCH) {
+        chn = chunk_at((int)xn);
+        after = block_ptr(chn);
       }
+      if (ch.lo == 0 && !waited) {
+        for (unsigned it = 0; *ready != j + 1 && it < kSpinLimit; ++it) {}   // warp 0, before its own chunks
+        __threadfence_block();
+        if (C > 1 && (j + 1) % kCols != 0) warp_wait(ccnt, col_arrivals, status, limit);   // column j in g0
+        __syncwarp();
+        waited = true;
+      }
+      sytrd_chunk(A, ld, LB, g0 + ch.lo, ch.rb, ch.re, lane, ch.c, vwp, vwn, RP, CP, cur, after);
+      x = kTickets ? (int)__shfl_sync(0xffffffffu, xn, 0) : (int)xn;
+      if (kTickets && x < NCH) {
+        chn = chunk_at(x);
+        load_block(cur, block_ptr(chn));
+      }
+      ch = chn;
     }
     arrivals += C;
     if (!group_barrier(cnt, arrivals, C, flag, status, limit)) return false;
-    if (j + 1 < S.j_end) prefetch_column(j + 1);
+    if (j + 1 < S.j_end) {
+      prefetch_column(j + 1);
+      if (warp == WARPS - 1) chunk_table(cfn, j + 1);
+    }
     // rows j + 1 .. n - 1, interleaved over the group's CTAs and, within a CTA, over teams of RL
     // lanes (row i to CTA i mod C; the long rows at the bottom are shared out): y_i = row sums
     // of the blocks of groups g0 .. i/16 + the column sums of the chunks of column i's group.
@@ -513,31 +594,16 @@ __device__ __noinline__ bool sytrd_matrix(const TriSlot S, int C, int rank, unsi
     if (threadIdx.x == 0) __stcg(dots + rank, dot);
     arrivals += C;
     if (!group_barrier(cnt, arrivals, C, flag, status, limit)) return false;
-    // w = p - (tau p.v / 2) v; p's loads go out before the sum of the CTAs' partial dots (in the same
-    // order for every warp)
-    double p8[kPre];
-#pragma unroll
-    for (int u = 0; u < kPre; ++u) {
-      const int i = (int)threadIdx.x + u * T;
-      p8[u] = (i > j && i < n) ? __ldcg(P + i) : 0.0;
-    }
-    double pv = 0.0;
-    for (int r = lane; r < C; r += 32) pv += __ldcg(dots + r);
-    for (int o = 16; o > 0; o >>= 1) pv += __shfl_xor_sync(0xffffffffu, pv, o);
-    const double Kc = 0.5 * tau * pv;
-#pragma unroll
-    for (int u = 0; u < kPre; ++u) {
-      const int i = (int)threadIdx.x + u * T;
-      if (i < ld) vwn[i].y = (i > j && i < n) ? fma(-Kc, vwn[i].x, p8[u]) : 0.0;
-    }
-    for (int i = (int)threadIdx.x + kPre * T; i < ld; i += T)
-      vwn[i].y = (i > j && i < n) ? fma(-Kc, vwn[i].x, __ldcg(P + i)) : 0.0;
-    __syncthreads();
     double2* t = vwp; vwp = vwn; vwn = t;
+    int* tc = cf; cf = cfn; cfn = tc;
   }
   if (rank == 0) {                                    // the last step's update, for sytrd_small
+    const double K = S.j_end > 0 ? half_dot() : 0.0;
     double2* pv = (double2*)(ws + S.pv_off);
-    for (int i = threadIdx.x; i < n; i += WARPS * 32) pv[i] = vwp[i];
+    for (int i = threadIdx.x; i < n; i += WARPS * 32) {
+      const double v = vwp[i].x;
+      pv[i] = make_double2(v, i >= S.j_end && S.j_end > 0 ? fma(-K, v, __ldcg(P + i)) : 0.0);
+    }
   }
   if (bad) atomicOr(status, kStEigen);
   return true;
@@ -602,7 +668,7 @@ __global__ void __launch_bounds__(kSmallThreads) sytrd_small(const TriSlot* __re
     if (threadIdx.x < 32) {                         // one warp: see sytrd_matrix
       const double alpha = red[W + 1];
       double beta = alpha, tau = 0.0, s = 0.0;
-      if (sig != 0.0) {
+      if (!(sig < 1e-280)) {                         // the bound of sytrd_matrix: no quotient of subnormal squares
         const double nrm = sqrt(fma(alpha, alpha, sig));
         beta = alpha >= 0.0 ? -nrm : nrm;
         tau = (beta - alpha) / beta;
@@ -1245,7 +1311,8 @@ tgba_status tri_solve(Basis& b, const std::vector<TriBlock>& blocks, int64_t ext
   // Groups of up to 96 CTAs instead of 16, chunks as short as one block, the column and p loads ahead of
   // their use, one warp for the scalars and the last rows in shared memory took the two blocks of the
   // L = 40, k = 0 sector (1472 and 1225 states) from 85 to 32 ms, the 30 matrices of the L = 24 step from
-  // 274 to 253 ms, the complete L = 12 sector (180 and 172) from 4.6 to 2.9 ms.
+  // 274 to 253 ms, the complete L = 12 sector (180 and 172) from 4.6 to 2.9 ms; a step without the serial
+  // parts of its reflector (sytrd_matrix) these to 27.6, 247 and 2.66 ms.
   // One or two CTAs per SM: two of 6 warps when their shared memory fits (each SM then runs
   // parts of two matrices, and one's barrier waits and serial phases are filled by the other's
   // arithmetic), else one of 12 warps.  With no more matrices than CTAs, every CTA joins one
@@ -1253,13 +1320,15 @@ tgba_status tri_solve(Basis& b, const std::vector<TriBlock>& blocks, int64_t ext
   // to the matrix with the most work (n^3) per CTA, at most 96 per matrix.  With more matrices
   // than CTAs, CTA b takes matrices b, b + CTAs, ... alone.
   const size_t smem = (size_t)(4 * ld_max + kRed) * sizeof(double) +
-                      (size_t)(kMaxGroups + 1) * sizeof(int);
+                      2 * (size_t)(ld_max / kCols + 1) * sizeof(int);   // two chunk tables
   TGBA_CUDA(cudaFuncSetAttribute(sytrd_groups<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   TGBA_CUDA(cudaFuncSetAttribute(sytrd_groups<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   TGBA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sytrd_groups<6>, 6 * 32, smem));
-  // one or two matrices: nothing to share an SM with, and the barriers want few CTAs
-  per_sm = per_sm >= 2 && B > 2 ? 2 : 1;
+  // few matrices: little to share an SM with, and the barriers want few CTAs (sectors of 1950 states, two CTAs
+  // against one: 3 matrices 63.5 and 62.7 ms, 4: 73.1 and 71.5, 8: 115.3 and 115.6, 12: 157 and 166; of 340
+  // states, 4: 4.37 and 4.24, 24: 5.50 and 5.47)
+  per_sm = per_sm >= 2 && B > 6 ? 2 : 1;
   if (per_sm == 1) {
     int one = 0;
     TGBA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&one, sytrd_groups<12>, 12 * 32, smem));

@@ -45,3 +45,27 @@ def test_against_whole_sectors(L, h, sectors, mq, cut, cap):
                 assert np.all(np.diff(got[i:j]) >= -1e-13 * np.abs(ref).max())
     finally:
         tgba.tgba_basis_free(b)
+
+
+@pytest.mark.parametrize("L,sectors,mq,cut,fields", [
+    (14, [3], 6, -1.0, [0.2]),                                  # one matrix, beyond the rows one CTA finishes
+    (24, [5], 4, 9.0, [0.1 * i for i in range(1, 7)]),           # 6: one CTA on an SM
+    (24, [5], 4, 9.0, [0.1 * i for i in range(1, 8)]),           # 7: two
+    (24, [0], 4, 9.0, [1e-160, 1e-146, 1e-140, 1e-130, 1e-60]),   # columns whose squares underflow
+    (24, [5], 4, 9.0, [1e-145, 0.0, 1e3]),
+])
+def test_few_and_many_matrices(L, sectors, mq, cut, fields):
+    """Householder steps with the reflector in the column's scale, chunks dealt out (up to six matrices) and
+    drawn by ticket, against the library solver; the bound of test_against_whole_sectors."""
+    b = tgba.tgba_build_basis(L, 1.0, sectors, mq, cut)
+    try:
+        tgba.tgba_compute_x(b)
+        n = sum(x + y for x, y in tgba.tgba_sector_sizes(b))
+        assert n > 130
+        ev = [torch.empty(len(fields) * n, dtype=torch.float64, device="cuda") for _ in range(2)]
+        tgba.tgba_eigvals(b, fields, ev[0], method=1)
+        tgba.tgba_eigvals(b, fields, ev[1], method=2)
+        got, ref = (e.cpu().numpy().reshape(len(fields), n) for e in ev)
+        assert (np.abs(got - ref).max(axis=1) <= 1e-12 * np.abs(ref).max(axis=1) * n ** 0.5).all()
+    finally:
+        tgba.tgba_basis_free(b)
