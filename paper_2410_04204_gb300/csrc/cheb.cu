@@ -34,6 +34,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "tgba_internal.h"
@@ -235,11 +236,13 @@ __global__ void __launch_bounds__(256) cheb_step(int64_t n, int64_t kn_max, cons
 // All K steps of a few small variants in one cooperative launch, in FP64.  Row q of the union belongs to
 // CTA q mod gridDim; a CTA keeps its rows of the X block (both orientations: its NS rows over the R
 // states and its R rows over the NS states) in shared memory for the whole run.  A step reads the
-// current vectors of all variants from L2 into shared memory, takes the rows' products (a warp per
-// row, each variant up to its own extent), writes the next vectors and ends with a barrier of the grid
-// (an arrival counter, bounded waits).  Bound: the FP64 pipe (2 kn kr FMAs per variant and step on 2
-// lanes per SM and clock) and the barrier.  The tensor-core step costs 30 to 40 us however small the
-// block is.
+// kept entries of the current vectors from L2 into shared memory, takes the rows' products (a warp per
+// row and up to NV variants at once, each up to its own extent: a row's element is read once, and the
+// variants' lane sums are added by one exchange in which a lane keeps half of its sums at each level), writes
+// the next vectors and ends with a barrier of the grid (an arrival counter, bounded waits).  Bound: the FP64
+// pipe (2 kn kr FMAs per variant and step on 2 lanes per SM and clock: 6.2 of the us of a step at L = 60,
+// sizes 1000, 1500 and 2000 per parity), the vectors' way through L2 and the barrier.  The tensor-core step costs
+// 30 to 40 us however small the block is.
 constexpr int kPersistThreads = 512;
 constexpr int kPersistCols = 8;
 struct PersistArgs {
@@ -259,12 +262,16 @@ __device__ __forceinline__ unsigned acquire_u32(const unsigned* p) {
   return v;
 }
 
+template <int NV>
 __global__ void __launch_bounds__(kPersistThreads, 1) cheb_persist(PersistArgs g) {
   extern __shared__ double sm[];
   __shared__ int s_ok;
+  __shared__ double s_g[NV], s_ec[NV], s_ir[NV];
+  __shared__ int s_kn[NV], s_kr[NV];
   const int n = g.kn + g.kr, G = gridDim.x, c0 = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int W = kPersistThreads / 32;
+  constexpr int LV = NV == 8 ? 3 : NV == 4 ? 2 : NV == 2 ? 1 : 0, LPV = 32 >> LV;   // lanes per variant's sum
   const int rn = g.kn > c0 ? (g.kn - c0 + G - 1) / G : 0;           // own NS rows: c0, c0 + G, ...
   const int b0 = ((c0 - g.kn) % G + G) % G;                          // own R rows: b0, b0 + G, ... (row kn + b)
   const int rr = g.kr > b0 ? (g.kr - b0 + G - 1) / G : 0;
@@ -278,39 +285,114 @@ __global__ void __launch_bounds__(kPersistThreads, 1) cheb_persist(PersistArgs g
     const int i = q % rr, a = q / rr;
     Ar[(size_t)i * g.kn + a] = g.Q[(size_t)a * g.kr + b0 + i * G];
   }
+  for (int q = threadIdx.x; q < g.nv * n + (rn + rr) * g.nv; q += kPersistThreads) x[q] = 0.0;   // and prev
+  if (threadIdx.x < NV) {
+    const bool in = (int)threadIdx.x < g.nv;
+    const ColPrm p = g.prm[in ? threadIdx.x : 0];
+    s_g[threadIdx.x] = p.g;
+    s_ec[threadIdx.x] = p.ec;
+    s_ir[threadIdx.x] = p.invr;
+    s_kn[threadIdx.x] = in ? (int)p.kn : 0;
+    s_kr[threadIdx.x] = in ? (int)p.kr : 0;
+  }
+  __syncthreads();
   for (int k = 0; k < g.K; ++k) {
     const double* vk = g.V + (size_t)k * g.S;
-    for (int q = threadIdx.x; q < g.nv * n; q += kPersistThreads) x[q] = __ldcg(vk + q);
+    // the kept entries (the others stay zero), all loads of a batch in flight before the first store
+    for (int base = threadIdx.x; base < n; base += 4 * kPersistThreads) {
+      double t[NV][4];
+#pragma unroll
+      for (int c = 0; c < NV; ++c)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int at = base + u * kPersistThreads;
+          if (at < n && (at < g.kn ? at < s_kn[c] : at - g.kn < s_kr[c])) t[c][u] = __ldcg(vk + (size_t)c * n + at);
+        }
+#pragma unroll
+      for (int c = 0; c < NV; ++c)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int at = base + u * kPersistThreads;
+          if (at < n && (at < g.kn ? at < s_kn[c] : at - g.kn < s_kr[c])) x[(size_t)c * n + at] = t[c][u];
+        }
+    }
     __syncthreads();
     for (int i = warp; i < rn + rr; i += W) {
       const bool ns = i < rn;
       const double* row = ns ? An + (size_t)i * g.kr : Ar + (size_t)(i - rn) * g.kn;
       const int at = ns ? c0 + i * G : g.kn + b0 + (i - rn) * G;      // row of the union
+      const double* x0 = x + (ns ? g.kn : 0);
+      const int full = ns ? g.kr : g.kn;
       const double e = g.E[at];
-      for (int c = 0; c < g.nv; ++c) {
-        const ColPrm p = g.prm[c];
-        double v = 0.0;
-        if (ns ? at < p.kn : at - g.kn < p.kr) {                     // warp-uniform
-          const int ext = (int)(ns ? p.kr : p.kn);
-          const double* xc = x + (size_t)c * n + (ns ? g.kn : 0);
-          double y0 = 0.0, y1 = 0.0, y2 = 0.0, y3 = 0.0;
-          int j = lane;
-          for (; j + 96 < ext; j += 128) {
-            y0 = fma(row[j], xc[j], y0);
-            y1 = fma(row[j + 32], xc[j + 32], y1);
-            y2 = fma(row[j + 64], xc[j + 64], y2);
-            y3 = fma(row[j + 96], xc[j + 96], y3);
+      double y[NV], z[NV];
+      int ext[NV];                                                   // 0: the row or the variant is not there
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        y[c] = z[c] = 0.0;
+        ext[c] = (ns ? at < s_kn[c] : at - g.kn < s_kr[c]) ? (ns ? s_kr[c] : s_kn[c]) : 0;
+      }
+#pragma unroll
+      for (int c = NV - 2; c >= 0; --c) ext[c] = max(ext[c], ext[c + 1]);   // (beyond its kept set a vector is zero)
+      // the first M variants as far as the M-th reaches: a predicated FMA takes its turn on the FP64 pipe, so
+      // the variants that have ended are left out by the code, not by a predicate
+      int jb = 0;
+      auto reach = [&](auto mc) {
+        constexpr int M = decltype(mc)::value;
+        for (; jb + 64 <= full && jb < ext[M - 1]; jb += 64) {
+          const double a = row[jb + lane], b = row[jb + 32 + lane];
+#pragma unroll
+          for (int c = 0; c < M; ++c) {
+            y[c] = fma(a, x0[c * n + jb + lane], y[c]);
+            z[c] = fma(b, x0[c * n + jb + 32 + lane], z[c]);
           }
-          for (; j < ext; j += 32) y0 = fma(row[j], xc[j], y0);
-          double y = (y0 + y1) + (y2 + y3);
-          for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-          const double xi = x[(size_t)c * n + at];
-          const double h = fma(p.g, y, (e - p.ec) * xi);
-          v = (k == 0 ? 1.0 : 2.0) * p.invr * h - (k == 0 ? 0.0 : prev[i * g.nv + c]);
-          __syncwarp();
-          if (lane == 0) prev[i * g.nv + c] = xi;
         }
-        if (lane == 0) __stcg(g.V + (size_t)(k + 1) * g.S + (size_t)c * n + at, v);
+        for (; jb < ext[M - 1]; jb += 32) {
+          const int jj = jb + lane;
+          if (jj < full) {
+            const double a = row[jj];
+#pragma unroll
+            for (int c = 0; c < M; ++c) y[c] = fma(a, x0[c * n + jj], y[c]);
+          }
+        }
+      };
+      if constexpr (NV == 8) {
+        reach(std::integral_constant<int, 8>{});
+        reach(std::integral_constant<int, 7>{});
+        reach(std::integral_constant<int, 6>{});
+        reach(std::integral_constant<int, 5>{});
+      }
+      if constexpr (NV >= 4) {
+        reach(std::integral_constant<int, 4>{});
+        reach(std::integral_constant<int, 3>{});
+      }
+      if constexpr (NV >= 2) reach(std::integral_constant<int, 2>{});
+      reach(std::integral_constant<int, 1>{});
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < NV; ++c) y[c] += z[c];
+      int h = NV / 2, s = 16;
+#pragma unroll
+      for (; h >= 1; h >>= 1, s >>= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int m = 0; m < h; ++m) {
+          const double send = up ? y[m] : y[m + h], own = up ? y[m + h] : y[m];
+          y[m] = own + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+      }
+#pragma unroll
+      for (s = LPV / 2; s >= 1; s >>= 1) y[0] += __shfl_xor_sync(0xffffffffu, y[0], s);
+      const int c = lane >> (5 - LV);                                // whose sum this lane holds
+      if ((lane & (LPV - 1)) == 0 && c < g.nv) {
+        double v = 0.0;
+        if (ns ? at < s_kn[c] : at - g.kn < s_kr[c]) {
+          const double xi = x[(size_t)c * n + at];
+          const double t = fma(s_g[c], y[0], (e - s_ec[c]) * xi);
+          double* pr = prev + i * g.nv + c;
+          v = fma(k == 0 ? s_ir[c] : 2.0 * s_ir[c], t, -*pr);         // prev of step 0 is zero
+          *pr = xi;
+        }
+        __stcg(g.V + (size_t)(k + 1) * g.S + (size_t)c * n + at, v);
       }
     }
     __syncthreads();
@@ -405,42 +487,60 @@ __global__ void symmetrise(int k, double* __restrict__ G) {
 // in the recurrence).  When the unnormalised values pass 1e250 the recurrence is rescaled by
 // 1e-250 without touching the values already stored: an entry stored before one rescaling
 // gets the factor 1e-250 at the end, one stored before two or more is below 1e-236 of the
-// result and becomes 0, so only the positions of the last two rescalings are kept.  The sign
-// (-1)^{floor(k/2)} of the moments is put into a_k.
-__global__ void cheb_bessel(int n_t, int t0, double dt, double R, int K, int m_start, double* __restrict__ out) {
+// result and becomes 0, so only the positions of the last two rescalings are kept (fac: the norm's
+// reciprocal, pos: the positions).  Bound by the FP64 pipe and the recurrence's chain, about 80 cycles a term
+// with one warp on an SM, so the recurrence only stores: bessel_scale applies the factors, whose loads
+// one thread would wait for one after another (K = 4987, 400 times: 3.3 ms with both in one loop).
+__global__ void cheb_bessel(int n_t, int t0, double dt, double R, int K, int m_start, double* __restrict__ out,
+                            double* __restrict__ fac, int2* __restrict__ pos) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n_t) return;
   const double x = R * dt * (double)(t0 + c);
   double* a = out + c;                         // a_k at a[k n_t]
   const int64_t S = n_t;
+  int k_last = 1 << 30, k_prev = 1 << 30;     // the last two rescalings (entry q was stored before
+                                               // the one at k iff q + 1 >= k)
   if (x == 0.0) {
     a[0] = 1.0;
     for (int k = 1; k <= K; ++k) a[k * S] = 0.0;
+    fac[c] = 1.0;
+    pos[c] = make_int2(k_last, k_prev);
     return;
   }
   const double ix2 = 2.0 / x;
   double jp1 = 0.0, j = 1e-300, norm = 0.0;
-  int k_last = 1 << 30, k_prev = 1 << 30;     // the last two rescalings (entry q was stored before
-                                               // the one at k iff q + 1 >= k)
-  for (int k = m_start; k >= 1; --k) {
+  const int big = __double2hiint(1e250);
+  auto term = [&](int k) {
     const double jm1 = fma((double)k * ix2, j, -jp1);
     jp1 = j;
     j = jm1;                                   // j = J_{k-1} (unnormalised)
     if (k - 1 <= K) a[(k - 1) * S] = j;
-    if ((k - 1) % 2 == 0 && k - 1 > 0) norm += 2.0 * j;
-    if (fabs(j) > 1e250) {
+    if ((k - 1) % 2 == 0 && k - 1 > 0) norm = fma(2.0, j, norm);
+    if ((__double2hiint(j) & 0x7fffffff) >= big) {
       const double sc = 1e-250;
       j *= sc; jp1 *= sc; norm *= sc;
       k_prev = k_last;
       k_last = k;
     }
+  };
+  for (int k = m_start; k >= 2; k -= 2) {      // m_start is even
+    term(k);
+    term(k - 1);
   }
   norm += j;                                   // + J_0
-  const double inv = 1.0 / norm;
-  for (int q = 0; q <= K; ++q) {
-    const double f = (q + 1 >= k_prev) ? 0.0 : (q + 1 >= k_last ? 1e-250 : 1.0);
+  fac[c] = 1.0 / norm;
+  pos[c] = make_int2(k_last, k_prev);
+}
+
+// a_k <- (2 - d_k0) a_k / norm with the sign (-1)^{floor(k/2)} of the moments
+__global__ void bessel_scale(int n_t, int K, const double* __restrict__ fac, const int2* __restrict__ pos,
+                             double* __restrict__ out) {
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < (int64_t)(K + 1) * n_t; x += (int64_t)gridDim.x * blockDim.x) {
+    const int q = (int)(x / n_t), c = (int)(x - (int64_t)q * n_t);
+    const int2 p = pos[c];
+    const double inv = fac[c], f = (q + 1 >= p.y) ? 0.0 : (q + 1 >= p.x ? 1e-250 : 1.0);
     const double w = (q == 0 ? inv : 2.0 * inv) * f;
-    a[q * S] *= (q & 2) ? -w : w;
+    out[x] *= (q & 2) ? -w : w;
   }
 }
 
@@ -460,6 +560,23 @@ __global__ void cheb_mx(int K1, int cnt, const double* __restrict__ A, const dou
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) mx[col] = (acc - R * *d01) * scale;
+}
+
+// <sigma^x>(t) from the states: B^H (D - E_c) B over the union, a warp per time
+__global__ void state_mx(int64_t n, int n_t, const double* __restrict__ re, const double* __restrict__ im,
+                         const double* __restrict__ E, double ec, const double* __restrict__ d01, double R, double scale,
+                         double* __restrict__ mx) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n_t;
+       t += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    double acc = 0.0;
+    for (int64_t i = lane; i < n; i += 32) {
+      const double x = re[i + t * n], y = im[i + t * n];
+      acc = fma(E[i] - ec, fma(x, x, y * y), acc);
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) mx[t] = (acc - R * *d01) * scale;
+  }
 }
 
 int blocks_for(int64_t work) {
@@ -782,7 +899,8 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       if (b.q_ev[e] == nullptr) TGBA_CUDA(cudaEventCreate(&b.q_ev[e]));
     TGBA_CUDA(cudaEventRecord(b.q_ev[0], st));
     if (persist) {
-      TGBA_CUDA(cudaFuncSetAttribute(cheb_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_p));
+      void (*kern)(PersistArgs) = ncol > 4 ? cheb_persist<8> : ncol > 2 ? cheb_persist<4> : ncol > 1 ? cheb_persist<2> : cheb_persist<1>;
+      TGBA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_p));
       PersistArgs pa;
       pa.kn = (int)kn_max; pa.kr = (int)kr_max; pa.nv = ncol; pa.K = K; pa.S = S;
       pa.Q = Q; pa.E = E; pa.prm = prm; pa.V = V;
@@ -802,7 +920,7 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       // the padding columns of every step are zero (the moments never read them, the norms do)
       if (ncolp > ncol)
         TGBA_CUDA(cudaMemset2DAsync(V + (size_t)ncol * n_un, (size_t)S * 8, 0, (size_t)(ncolp - ncol) * n_un * 8, K1, st));
-      TGBA_CUDA(cudaLaunchKernelEx(&cfg, cheb_persist, pa));
+      TGBA_CUDA(cudaLaunchKernelEx(&cfg, kern, pa));
       ++b.launches;
     }
     for (int k = 0; k < K && !persist; ++k) {
@@ -851,26 +969,34 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
     // error is 6e-15 of sum |a||b| instead of 2e-13.
     constexpr int TM = 64;
     const int64_t nt = std::max(1, dt_n), KH = (K1 + 1) / 2;
-    const int64_t a_rows = eps ? std::max<int64_t>(KH, n_un) : KH;
-    const size_t sa = std::max({emu_operand_elems((int)KH, (int)chi_max, TR), emu_operand_elems((int)a_rows, (int)KH, TR)});
-    const size_t sb = std::max(emu_operand_elems((int)KH, (int)chi_max, TM), emu_operand_elems((int)nt, (int)KH, TM));
+    // Moments cost K^2 chi / 2 flops for the Gram matrices and K^2 n_t for their sums over the time grid; the
+    // states themselves (their real part from the even k, the imaginary part from the odd ones) cost 2 K n n_t and
+    // give <sigma^x> as it stands.  So where the union has no more than K / 2 rows, or eps wants the
+    // states anyway, there are no moments (L = 60, union of 2000, K = 4987, n_t = 4801, three variants
+    // with eps: 23.8 ms of moments, sums and states, 11.1 of states).  The buffers are then no larger either.
+    const bool states = eps != nullptr || 2 * n_un <= K;
+    const int64_t KG = states ? 0 : KH, a_rows = states ? n_un : KH;
+    const size_t sa = states ? emu_operand_elems((int)n_un, (int)KH, TR)
+                             : std::max(emu_operand_elems((int)KH, (int)chi_max, TR), emu_operand_elems((int)KH, (int)KH, TR));
+    const size_t sb = std::max(states ? (size_t)0 : emu_operand_elems((int)KH, (int)chi_max, TM), emu_operand_elems((int)nt, (int)KH, TM));
     const size_t n_tiles_max = (size_t)((a_rows + TR - 1) / TR) * (size_t)std::max<int64_t>((KH + TM - 1) / TM, (nt + TM - 1) / TM);
-    DevBuf bbuf(st);                                      // B(t) of two variants, for eps
+    DevBuf bbuf(st);                                      // B(t) of one variant, of two for eps
     const size_t bt = (size_t)n_un * nt;
+    if (states) TGBA_CUDA(cudaMallocAsync(&bbuf.p, (eps ? 4 : 2) * bt * sizeof(double), st));
     if (eps) {
-      TGBA_CUDA(cudaMallocAsync(&bbuf.p, 4 * bt * sizeof(double), st));
       TGBA_CUDA(cudaMemsetAsync(eps, 0, (vars.size() - 1) * sizeof(double), st));
     }
     bool one_field = true;
     for (const ChebVariant& v : vars) one_field = one_field && v.hx == vars[0].hx;
     DevBuf mbuf(st);
-    const size_t mdoubles = (size_t)KH * KH + (size_t)K1 * nt + 2 * (size_t)KH * nt + chi_max + 8;
+    const size_t mdoubles = (size_t)KG * KG + (size_t)(K1 + 2) * nt + 2 * (size_t)KG * nt + chi_max + 8;
     TGBA_CUDA(cudaMallocAsync(&mbuf.p, mdoubles * 8 + (sa + sb) * 2 + 2 * ((size_t)a_rows + nt) * 4 +
                                            n_tiles_max * sizeof(EmuTile) + 1024, st));
     double* Gam = (double*)mbuf.p;
-    double* Ab = Gam + (size_t)KH * KH;                   // a_k(t): [K_v + 1][t]
-    double* GA[2] = {Ab + (size_t)K1 * nt, Ab + (size_t)K1 * nt + (size_t)KH * nt};   // Gamma a(t): column-major
-    double* Ek = GA[1] + (size_t)KH * nt;
+    double* Ab = Gam + (size_t)KG * KG;                   // a_k(t): [K_v + 1][t]
+    double* bfac = Ab + (size_t)K1 * nt;                   // cheb_bessel's factors: [t], then positions [t]
+    double* GA[2] = {bfac + 2 * (size_t)nt, bfac + 2 * (size_t)nt + (size_t)KG * nt};   // Gamma a(t): column-major
+    double* Ek = GA[1] + (size_t)KG * nt;
     double* d01 = Ek + chi_max;
     EmuTile* dtg = (EmuTile*)(((uintptr_t)(d01 + 8) + 15) & ~(uintptr_t)15);
     __nv_bfloat16* Va = (__nv_bfloat16*)(((uintptr_t)(dtg + n_tiles_max) + 255) & ~(uintptr_t)255);
@@ -910,23 +1036,43 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
       TGBA_CUDA(ev.mark(st));
       kept_energy<<<blocks_for(chi), 256, 0, st>>>(kn, kr, kn_max, E, Ek);
       cheb_dot01<<<1, kRedThreads, 0, st>>>(n_un, vre, vre + S, d01);
-      // a_k(t) for the whole grid
+      // a_k(t) for the whole grid; the same as the last variant's for the same radius and order (one h_x)
       const double scale = 1.0 / (b.L * vv.hx * vv.norm2);
       const int ms = [&] {
         int m0 = Kv[v] + 30 + (int)std::ceil(std::sqrt(40.0 * Kv[v]));
         return m0 + (m0 & 1);
       }();
-      cheb_bessel<<<(int)((nt + 31) / 32), 32, 0, st>>>((int)nt, 0, dt, R[v], Kv[v], ms, Ab);
-      b.launches += 3;
+      if (v == 0 || R[v] != R[v - 1] || Kv[v] != Kv[v - 1]) {
+        cheb_bessel<<<(int)((nt + 31) / 32), 32, 0, st>>>((int)nt, 0, dt, R[v], Kv[v], ms, Ab, bfac, (int2*)(bfac + nt));
+        bessel_scale<<<blocks_for((int64_t)k1 * nt), 256, 0, st>>>((int)nt, Kv[v], bfac, (const int2*)(bfac + nt), Ab);
+        b.launches += 2;
+      }
+      b.launches += 2;
       for (int p = 0; p < 2; ++p) {
         const int kp = (k1 - p + 1) / 2;                    // vectors k = p, p + 2, ...
         if (kp == 0) continue;
+        const double* vp = vre + (size_t)p * S;
+        if (states) {
+          // B(t) on the union: its real part from the even k, minus its imaginary part from the odd ones
+          int64_t cb = 0;
+          const std::vector<EmuTile> tb = grid_tiles(n_un, nt, kp, cb);
+          if (cb < 0) return fail(TGBA_EINVAL, "quench state tiles");
+          TGBA_CUDA(ev.mark(st));
+          TGBA_CUDA(cudaMemcpyAsync(dtg, tb.data(), tb.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
+          if ((r = emu_slice(b, Ab + (size_t)p * nt, 1, 2 * nt, kp, 0, nullptr, 0.0, (int)nt, kp, TM, Wb, ewb, st)) != TGBA_OK)
+            return r;
+          if ((r = emu_slice(b, vp, 1, 2 * S, kp, 0, nullptr, 0.0, (int)n_un, kp, TR, Va, eva, st)) != TGBA_OK) return r;
+          if ((r = emu_gemm(b, Va, eva, (int)n_un, kp, Wb, ewb, (int)nt, kp, TM, dtg, (int)tb.size(), cb,
+                            (double*)bbuf.p + (2 * (eps ? v & 1 : 0) + p) * bt, n_un, st)) != TGBA_OK)
+            return r;
+          TGBA_CUDA(ev.mark(st));
+          continue;
+        }
         int64_t cl = 0, ct = 0;
         const std::vector<EmuTile> tlo = grid_tiles(kp, kp, chi, cl, true);
         if (cl < 0) return fail(TGBA_EINVAL, "quench moment tiles");
         TGBA_CUDA(cudaMemcpyAsync(dtg, tlo.data(), tlo.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
         // rows of V (K = the kept rows in their own order: kn NS rows, then kr R rows)
-        const double* vp = vre + (size_t)p * S;
         if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, nullptr, 0.0, kp, (int)chi, TR, Va, eva, st)) != TGBA_OK) return r;
         if ((r = emu_slice(b, vp, 2 * S, 1, (int)kn, jump, Ek, ec[v], kp, (int)chi, TM, Wb, ewb, st)) != TGBA_OK) return r;
         if ((r = emu_gemm(b, Va, eva, kp, (int)chi, Wb, ewb, kp, (int)chi, TM, dtg, (int)tlo.size(), cl, Gam, kp, st)) != TGBA_OK)
@@ -943,21 +1089,16 @@ tgba_status quench_cheb_batch(Basis& b, const double* Q, int64_t kn_max, int64_t
           return r;
         if ((r = emu_gemm(b, Va, eva, kp, kp, Wb, ewb, (int)nt, kp, TM, dtg, (int)tt.size(), ct, GA[p], kp, st)) != TGBA_OK)
           return r;
-        if (eps) {
-          // B(t) on the union: its real part from the even k, minus its imaginary part from the odd ones
-          int64_t cb = 0;
-          const std::vector<EmuTile> tb = grid_tiles(n_un, nt, kp, cb);
-          if (cb < 0) return fail(TGBA_EINVAL, "quench state tiles");
-          TGBA_CUDA(cudaMemcpyAsync(dtg, tb.data(), tb.size() * sizeof(EmuTile), cudaMemcpyHostToDevice, st));
-          if ((r = emu_slice(b, vp, 1, 2 * S, kp, 0, nullptr, 0.0, (int)n_un, kp, TR, Va, eva, st)) != TGBA_OK) return r;
-          if ((r = emu_gemm(b, Va, eva, (int)n_un, kp, Wb, ewb, (int)nt, kp, TM, dtg, (int)tb.size(), cb,
-                            (double*)bbuf.p + (2 * (v & 1) + p) * bt, n_un, st)) != TGBA_OK)
-            return r;
-        }
         TGBA_CUDA(ev.mark(st));
       }
-      cheb_mx<<<(int)((nt * 32 + 255) / 256), 256, 0, st>>>(k1, (int)nt, Ab, GA[0], GA[1], d01, R[v], scale,
-                                                              mx + (int64_t)vv.out * n_t);
+      if (states) {
+        const double* cur = (const double*)bbuf.p + 2 * (eps ? v & 1 : 0) * bt;
+        state_mx<<<(int)((nt * 32 + 255) / 256), 256, 0, st>>>(n_un, (int)nt, cur, cur + bt, E, ec[v], d01, R[v], scale,
+                                                                 mx + (int64_t)vv.out * n_t);
+      } else {
+        cheb_mx<<<(int)((nt * 32 + 255) / 256), 256, 0, st>>>(k1, (int)nt, Ab, GA[0], GA[1], d01, R[v], scale,
+                                                                mx + (int64_t)vv.out * n_t);
+      }
       TGBA_CUDA(cudaGetLastError());
       ++b.launches;
       if (eps) {
