@@ -281,6 +281,10 @@ tgba_status tgba_basis_free(tgba_basis h) {
 tgba_status tgba_compute_x(tgba_basis h, tgba_screen screen, double tau, double screen_hx, void* stream) {
   Basis* b = (Basis*)h;
   BASIS_OK(b);
+  // the basis' own stage events belong to the call, not to a graph of it
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  TGBA_CUDA(cudaStreamIsCapturing((cudaStream_t)stream, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return fail(TGBA_ECUDA, "tgba_compute_x cannot be captured into a graph");
   return compute_x(*b, (Screen*)screen, tau, screen_hx, (cudaStream_t)stream);
 }
 
