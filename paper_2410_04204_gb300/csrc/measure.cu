@@ -13,7 +13,7 @@
 //    SIAM J. Matrix Anal. Appl. 16 (1995) 172), and three sums per root.  Near-degenerate levels are
 //    deflated by exact rotations, so their summed weights are as exact as the others.
 // The library's eigen-decomposition with vectors that this replaces took 180 ms for n = 2697 (all of S(0, w)
-// now 36 ms, most of it the tridiagonalisation).
+// now 33 ms, most of it the tridiagonalisation).
 #include <algorithm>
 #include <cmath>
 #include <vector>
