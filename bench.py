@@ -347,7 +347,7 @@ def screening_leg(b24, tgba, inputs, torch, bf16_peak_tflops):
 
 # DRAM bytes of one sytrd_groups launch on the L = 24 all-sector workload, measured with ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum); None until measured for the current kernel.
-SYTRD_TRAFFIC = 487853093632 + 493968308224
+SYTRD_TRAFFIC = 207335595008 + 227916400384
 
 
 def eigen_solver_leg(b, w, evs, tgba, torch):
@@ -585,7 +585,7 @@ def run_gb300_quench(args):
     q_gflops = prof["quench_flops"] / (q_ms * 1e-3) / 1e9
     # The propagation's products run on the tensor cores as 21 BF16 slice-pair products per FP64
     # product (digit diagonals p + q <= 5 of six slices), so its roofline is the BF16 tensor peak:
-    # achieved = 21 x the useful FP64 flops of the off-diagonal products (8 K kn kr per variant)
+    # achieved = 21 x the useful FP64 flops of the off-diagonal products (4 K kn kr per variant)
     # / the propagation's time; peak = the measured sustained BF16 rate (a kernel inside a
     # seconds-long step).
     peaks = measured_peaks()
